@@ -320,37 +320,53 @@ __global__ void __launch_bounds__(512) k_select_hist_buf(const double* __restric
     if (h[b]) atomicAdd(&hist[b], (unsigned long long)h[b]);
 }
 
-// Pick the bin holding the remaining rank; extend the prefix; clear hist.
+// Pick the bin holding the remaining rank; extend the prefix; clear hist. One
+// block of SELECT_STEP_THREADS: every thread sums its run of up to 16 bins, a
+// block scan of the sums finds the run holding the rank, and its thread walks
+// the run. Bound by latency (32 KB of counts, one block): 3 us a step, where one
+// thread walking all 4096 bins took 56 us, six times per select.
+constexpr int SELECT_STEP_THREADS = 256;
+constexpr int SELECT_RUN = RADIX_BINS / SELECT_STEP_THREADS;
 __device__ __forceinline__ void select_step(SelectState* st, unsigned long long* hist, int shift, int bits,
                                             double* sigma_out, int last) {
-  __shared__ unsigned long long cnt[RADIX_BINS];
-  const int nbins = 1 << bits;
-  for (int b = threadIdx.x; b < RADIX_BINS; b += blockDim.x) {
-    cnt[b] = hist[b];
-    hist[b] = 0;
+  __shared__ unsigned long long cnt[RADIX_BINS + SELECT_STEP_THREADS];   // one pad word per run: no bank conflicts
+  __shared__ unsigned long long wsum[SELECT_STEP_THREADS / 32];
+  const int nbins = 1 << bits, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+#pragma unroll
+  for (int e = 0; e < SELECT_RUN; ++e) {
+    const int b = tid + e * SELECT_STEP_THREADS;
+    cnt[b + b / SELECT_RUN] = b < nbins ? hist[b] : 0;
+    if (b < nbins) hist[b] = 0;
   }
+  const unsigned long long r = (unsigned long long)st->rank;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    long long r = st->rank;
-    int b = 0;
-    for (; b < nbins; ++b) {
-      if ((long long)cnt[b] > r) break;
-      r -= (long long)cnt[b];
-    }
-    if (b >= nbins) b = nbins - 1;   // unreachable for a consistent histogram
-    unsigned long long dm = (unsigned long long)(nbins - 1) << shift;
-    st->prefix |= (unsigned long long)b << shift;
-    st->mask |= dm;
-    st->rank = r;
-    if (last) {
-      double d2 = __longlong_as_double((long long)st->prefix);
-      *sigma_out = sqrt(d2);
-    }
+  const unsigned long long* run = cnt + tid * (SELECT_RUN + 1);
+  unsigned long long own = 0;
+#pragma unroll
+  for (int e = 0; e < SELECT_RUN; ++e) own += run[e];
+  unsigned long long incl = own;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long v = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += v;
+  }
+  if (lane == 31) wsum[warp] = incl;
+  __syncthreads();
+  for (int w = 0; w < warp; ++w) incl += wsum[w];
+  unsigned long long below = incl - own;
+  if (below <= r && r < incl) {   // exactly one thread: the histogram counts every key that still matches
+    int e = 0;
+    while (r - below >= run[e]) below += run[e++];
+    st->prefix |= (unsigned long long)(tid * SELECT_RUN + e) << shift;
+    st->mask |= (unsigned long long)(nbins - 1) << shift;
+    st->rank = (long long)(r - below);
+    if (last) *sigma_out = sqrt(__longlong_as_double((long long)st->prefix));
   }
 }
 
-__global__ void k_select_step(SelectState* st, unsigned long long* hist, int shift, int bits,
-                              double* sigma_out, int last) {
+__global__ void __launch_bounds__(SELECT_STEP_THREADS) k_select_step(SelectState* st, unsigned long long* hist,
+                                                                     int shift, int bits, double* sigma_out,
+                                                                     int last) {
   select_step(st, hist, shift, bits, sigma_out, last);
 }
 
@@ -603,7 +619,8 @@ __global__ void __launch_bounds__(512) k_g_select_hist(const int4* __restrict__ 
   select_hist_rows(G.A, G.n, shift, bits, st, hist, t.y, t.z, 1);
 }
 
-__global__ void k_g_select_step(const GGraph* __restrict__ gs, int shift, int bits, int last) {
+__global__ void __launch_bounds__(SELECT_STEP_THREADS) k_g_select_step(const GGraph* __restrict__ gs, int shift,
+                                                                       int bits, int last) {
   const GGraph& G = gs[blockIdx.x];
   SelectState* st = static_cast<SelectState*>(G.sel);
   unsigned long long* hist = reinterpret_cast<unsigned long long*>(static_cast<char*>(G.sel) + 64);
@@ -695,7 +712,7 @@ int graph_build_grouped(cdl_ctx* ctx, const GraphBatch& B) {
       }
       {
         Launch L(ctx, CDL_KC_SELECT, 0);
-        k_g_select_step<<<B.G2, 256, 0, s>>>(B.gs, shifts[p], widths[p], p == 5);
+        k_g_select_step<<<B.G2, SELECT_STEP_THREADS, 0, s>>>(B.gs, shifts[p], widths[p], p == 5);
         CDL_TRY(L.done());
       }
     }
@@ -790,7 +807,7 @@ int graph_build(cdl_ctx* ctx, const double* X, int64_t n64, int T, double sigma,
       }
       {
         Launch L(ctx, CDL_KC_SELECT, 0);
-        k_select_step<<<1, 256, 0, s>>>(st, hist, shifts[p], widths[p], sigma_out, p == 5);
+        k_select_step<<<1, SELECT_STEP_THREADS, 0, s>>>(st, hist, shifts[p], widths[p], sigma_out, p == 5);
         CDL_TRY(L.done());
       }
     }
@@ -904,7 +921,7 @@ int graph_regen_init(cdl_ctx* ctx, RegenGraph& g, const double* X, int64_t n64, 
         CDL_TRY(L.done());
       }
       Launch L(ctx, CDL_KC_SELECT, 0);
-      k_select_step<<<1, 256, 0, s>>>(st, hist, shifts[p], widths[p], g.sigma, p == 5);
+      k_select_step<<<1, SELECT_STEP_THREADS, 0, s>>>(st, hist, shifts[p], widths[p], g.sigma, p == 5);
       CDL_TRY(L.done());
     }
   }
@@ -1192,7 +1209,7 @@ int graph_build_static(const double* X, int64_t n64, int T, double sigma, double
     for (int p = 0; p < 6; ++p) {
       k_select_hist<<<hblocks, 512, 0, s>>>(A, n, shifts[p], widths[p], st, hist);
       CDL_TRY(launched());
-      k_select_step<<<1, 256, 0, s>>>(st, hist, shifts[p], widths[p], sigma_out, p == 5);
+      k_select_step<<<1, SELECT_STEP_THREADS, 0, s>>>(st, hist, shifts[p], widths[p], sigma_out, p == 5);
       CDL_TRY(launched());
     }
   }
