@@ -233,7 +233,10 @@ int cdl_graph_add_edges(cdl_ctx* ctx, void* A, cdl_dtype a_dtype, int64_t n, int
  * ones vector, the only vectors the solve applies them to.
  * A (device, n x n, a_dtype = CDL_F64; weights finite and non-negative),
  * D (device, n), vol (device, 1).
- * chain_dtype: CDL_F64, CDL_F32 (CUDA-core GEMM), CDL_BF16 (tcgen05
+ * chain_dtype: CDL_F64, CDL_F32 (exact integer products through residues on
+ *   the tensor cores, one rounding per entry; a CUDA-core GEMM where that
+ *   form's workspace, 24 npad^2 bytes for CDL_F32 and 48 npad^2 for CDL_F64,
+ *   exceeds the cap or the memory), CDL_BF16 (tcgen05
  *   tensor-core GEMM, float32 accumulation, bfloat16 levels) or CDL_FP8E4M3
  *   (tcgen05 kind::f8f6f4 GEMM, float32 accumulation, e4m3 levels with one
  *   scale per level: level i stores value / s_i, s_i = m_i / 448 where m_0 =

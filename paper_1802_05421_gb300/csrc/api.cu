@@ -13,6 +13,35 @@ void set_last_error(const char* msg, const char* file, int line) {
   snprintf(g_last_error, sizeof(g_last_error), "%s (%s:%d)", msg, file, line);
 }
 
+// Buffers named crt.* only make a kernel faster (their users have a form
+// without them): they are given up before any other request is refused.
+static bool reclaimable(const std::string& name) { return name.compare(0, 4, "crt.") == 0; }
+
+bool ws_reclaim(cdl_ctx* ctx) {
+  bool any = false;
+  for (auto it = ctx->ws.begin(); it != ctx->ws.end();) {
+    if (!reclaimable(it->first)) {
+      ++it;
+      continue;
+    }
+    if (!any) cudaStreamSynchronize(ctx->stream);
+    any = true;
+    cudaFree(it->second.first);
+    ctx->ws_used -= it->second.second;
+    it = ctx->ws.erase(it);
+  }
+  return any;
+}
+
+cudaError_t malloc_reclaim(cdl_ctx* ctx, void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation && ws_reclaim(ctx)) {
+    cudaGetLastError();
+    e = cudaMalloc(p, bytes);
+  }
+  return e;
+}
+
 int ws_get(cdl_ctx* ctx, const char* name, size_t bytes, void** out) {
   if (bytes == 0) bytes = 256;
   auto it = ctx->ws.find(name);
@@ -28,9 +57,11 @@ int ws_get(cdl_ctx* ctx, const char* name, size_t bytes, void** out) {
     ctx->ws_used -= old;
     ctx->ws.erase(it);
   }
+  const bool opt = reclaimable(name);
+  if (ctx->ws_cap && ctx->ws_used + bytes > ctx->ws_cap && !opt) ws_reclaim(ctx);
   if (ctx->ws_cap && ctx->ws_used + bytes > ctx->ws_cap) return CDL_ERR_OOM;
   void* p = nullptr;
-  if (cudaMalloc(&p, bytes) != cudaSuccess) {
+  if ((opt ? cudaMalloc(&p, bytes) : malloc_reclaim(ctx, &p, bytes)) != cudaSuccess) {
     cudaGetLastError();
     return CDL_ERR_OOM;
   }
@@ -487,7 +518,12 @@ int cdl_chain_build(cdl_ctx* ctx, const void* A, cdl_dtype a_dtype, const double
     // float-float residual operand (CUDA-core chains) or exact bf16 slices (tensor chains)
     const size_t ahl_bytes = tensor ? 0 : 2 * (size_t)n * n * sizeof(float);
     const size_t slice_bytes = tensor ? 6 * (size_t)npad * npad * 2 : 0;
-    if (ctx->ws_cap && ctx->ws_used + bytes + aop_bytes + l16_bytes + ahl_bytes + slice_bytes > ctx->ws_cap) {
+    const size_t chain_bytes = bytes + aop_bytes + l16_bytes + ahl_bytes + slice_bytes;
+    size_t free_b = 0, total_b = 0;
+    if ((ctx->ws_cap && ctx->ws_used + chain_bytes > ctx->ws_cap) ||
+        (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && free_b < chain_bytes + (64u << 20)))
+      ws_reclaim(ctx);
+    if (ctx->ws_cap && ctx->ws_used + chain_bytes > ctx->ws_cap) {
       delete ch;
       return CDL_ERR_OOM;
     }
@@ -523,7 +559,8 @@ int cdl_chain_build(cdl_ctx* ctx, const void* A, cdl_dtype a_dtype, const double
   for (int i = 0; st == CDL_OK && i + 1 < d; ++i) {
     if (chain_dtype == CDL_FP8E4M3) st = fp8_level_bound(ctx, ch, i);
     if (st == CDL_OK)
-      st = fp8t ? chain_square_fp8t(ctx, ch, i) : tensor ? chain_square_tc(ctx, ch, i) : chain_square_simt(ctx, ch, i);
+      st = fp8t ? chain_square_fp8t(ctx, ch, i) : tensor ? chain_square_tc(ctx, ch, i) : chain_square_crt(ctx, ch, i);
+    if (st == CDL_ERR_UNSUPPORTED && !tensor) st = chain_square_simt(ctx, ch, i);
     if (st == CDL_OK && truncate) {
       // ||S~_{i+1}||_2 <= its max row sum; at 2^-24 or less neither it nor the
       // levels after it (their norms square) can change a float32 x + S~ x

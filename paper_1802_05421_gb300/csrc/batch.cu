@@ -319,11 +319,12 @@ int build_plan(cdl_ctx* ctx, int G, const int64_t* n, int T, const cdl_batch_opt
     }
     if (pass == 0) {
       P->bytes = c.used;
+      if (ctx->ws_cap && ctx->ws_used + P->bytes > ctx->ws_cap) ws_reclaim(ctx);
       if (ctx->ws_cap && ctx->ws_used + P->bytes > ctx->ws_cap) {
         delete P;
         return CDL_ERR_OOM;
       }
-      if (cudaMalloc(&P->mem, P->bytes) != cudaSuccess) {
+      if (malloc_reclaim(ctx, &P->mem, P->bytes) != cudaSuccess) {
         cudaGetLastError();
         delete P;
         return CDL_ERR_OOM;

@@ -1,6 +1,7 @@
 // Inverse chain (Alg. 2, ChainProduct) on CUDA cores: the deflated level-0
 // formation used by every precision, the float32/float64 symmetric squaring
-// S~_{i+1} = S~_i^2 and the chain-apply products S~_i x of the solve.
+// S~_{i+1} = S~_i^2 (only where crt.cu's tensor-core form has no workspace) and
+// the chain-apply products S~_i x of the solve.
 //
 // Deflation: S = D^{-1/2} A D^{-1/2} has eigenvalue 1 with unit eigenvector
 // u = D^{1/2} 1 / sqrt(vol). S~ = S - u u^T satisfies S~^{2^i} = S^{2^i} - u u^T

@@ -1,0 +1,357 @@
+// Float64 and float32 chain squarings S~_{i+1} = S~_i^2 (Alg. 2, ChainProduct)
+// on the bf16 tensor cores, by integer products through residues (crt.cuh):
+//
+//   k_crt_residues  row i of the level, scaled by the power of two 2^{e_i}
+//                   that brings its 2-norm to 2^(B-1) .. 2^B (B =
+//                   crt_norm_bits) and rounded to integers, as NP planes of
+//                   symmetric residues in bf16;
+//   k_tc_crt        the NP residue products (tc_gemm.cu);
+//   k_crt_combine   c_ij 2^{e_i + e_j} from its NP residues (exact), rounded
+//                   once to the level's type, and its mirror.
+//
+// The only errors are the rounding of the scaled rows, at most half a unit of
+// 2^-B of the row's norm per entry (B = 61.6 bits with 16 moduli for float64
+// levels, 30.7 with 8 for float32 ones), and the final rounding; a float64 or
+// float32 dot product rounds every partial sum. Rows with a non-finite entry
+// give NaN rows and columns.
+//
+// Bounds: the products by the tensor cores, 16 (8) times n^2 (n + 1) flop;
+// the other two kernels by integer issue (about 10 instructions per entry and
+// plane in the first, 9 in the second). Measured, one squaring: float32 n =
+// 8192 13.1 ms on the CUDA cores, here 2.52 ms of products (1.75 PFLOP/s) + 0.36
+// + 0.12; float64 n = 1024 1.07 ms on the CUDA cores (1 TFLOP/s of the float64
+// pipes), here 30 + 15 + 13 us. Relative error (Frobenius) of a square, n =
+// 300 .. 4096: float64 4.7e-17 (5e-16 .. 1.9e-15 before), float32 2.5e-8 (5e-7
+// .. 1e-6 before). One modulus less (15, 7) would pass on those graphs and
+// save 1/16 (1/8) of the products, but for levels near a multiple of the
+// identity the rounding of the rows would then exceed a dot product's.
+#include <algorithm>
+
+#include "crt.cuh"
+#include "internal.h"
+#include "tiles.cuh"
+
+namespace cdl {
+namespace {
+
+constexpr int CRT_ROW_NAN = 0x40000000;   // e_i of a row with a non-finite entry
+
+struct ResidueTab {
+  uint32_t mod[CRT_MAX], magic[CRT_MAX], c1[CRT_MAX], c2[CRT_MAX], bias[CRT_MAX];
+  float off[CRT_MAX];
+};
+// Signed x = u0 + 2^S u1 + 2^2S u2 (S = 21 for 62-bit x; S = 16 and no u2 for
+// 32-bit x): u0 + c1 u1 + c2 u2 + bias is x + floor(p / 2) modulo p and in
+// [0, 2^31); off = 2^23 + floor(p / 2).
+constexpr ResidueTab make_residue_tab(int S) {
+  ResidueTab t{};
+  for (int l = 0; l < CRT_MAX; ++l) {
+    const int p = CRT_MOD[l];
+    t.mod[l] = (uint32_t)p;
+    t.magic[l] = crt_magic(p);
+    t.c1[l] = (uint32_t)crt_pow2_mod(S, p);
+    t.c2[l] = (uint32_t)crt_pow2_mod(2 * S, p);
+    t.bias[l] = (uint32_t)(((1u << 29) + (unsigned)p - 1) / (unsigned)p * (unsigned)p + (unsigned)(p / 2));
+    t.off[l] = 8388608.0f + (float)(p / 2);
+  }
+  return t;
+}
+__constant__ ResidueTab c_res64 = make_residue_tab(21);
+__constant__ ResidueTab c_res32 = make_residue_tab(16);
+
+// P / p_l in 20-bit limbs (16 moduli: below 2^118) and 2^23 / p_l
+struct CombineTab64 {
+  uint32_t limb[6][CRT_MAX];
+  uint32_t frac[CRT_MAX];
+};
+constexpr CombineTab64 make_combine64() {
+  CombineTab64 t{};
+  const u128 P = crt_product(16);
+  for (int l = 0; l < 16; ++l) {
+    const u128 m = P / (u128)CRT_MOD[l];
+    for (int k = 0; k < 6; ++k) t.limb[k][l] = (uint32_t)(m >> (20 * k)) & 0xFFFFFu;
+    t.frac[l] = (uint32_t)(((1u << 24) + (unsigned)CRT_MOD[l]) / (2u * (unsigned)CRT_MOD[l]));
+  }
+  return t;
+}
+__constant__ CombineTab64 c_comb64 = make_combine64();
+struct CombineTab32 {
+  uint32_t lo[8], hi[8], frac[8];
+};
+constexpr CombineTab32 make_combine32() {
+  CombineTab32 t{};
+  const u128 P = crt_product(8);
+  for (int l = 0; l < 8; ++l) {
+    const u128 m = P / (u128)CRT_MOD[l];
+    t.lo[l] = (uint32_t)m;
+    t.hi[l] = (uint32_t)(m >> 32);
+    t.frac[l] = (uint32_t)(((1u << 24) + (unsigned)CRT_MOD[l]) / (2u * (unsigned)CRT_MOD[l]));
+  }
+  return t;
+}
+__constant__ CombineTab32 c_comb32 = make_combine32();
+constexpr unsigned long long P64_HI = (unsigned long long)(crt_product(16) >> 64),
+                             P64_LO = (unsigned long long)crt_product(16);
+constexpr unsigned long long P32 = (unsigned long long)crt_product(8);
+
+// The two types' bit patterns: magnitude bits, exponent field and mantissa
+// (value = m 2^(e - BIAS)), moduli.
+template <typename T>
+struct LevelType;
+template <>
+struct LevelType<double> {
+  static constexpr int NP = 16, BIAS = 1075;
+  static __device__ __forceinline__ unsigned long long mag(double x) {
+    return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
+  }
+  static __device__ __forceinline__ int exponent(unsigned long long m) { return max((int)(m >> 52), 1); }
+  static __device__ __forceinline__ unsigned long long mantissa(unsigned long long m) {
+    return (m & 0xFFFFFFFFFFFFFull) | (m >> 52 ? 1ull << 52 : 0ull);
+  }
+  static __device__ __forceinline__ bool negative(double x) { return __double_as_longlong(x) < 0; }
+  static __device__ __forceinline__ bool finite(unsigned long long m) { return (m >> 52) != 0x7FF; }
+};
+template <>
+struct LevelType<float> {
+  static constexpr int NP = 8, BIAS = 150;
+  static __device__ __forceinline__ unsigned long long mag(float x) { return __float_as_uint(x) & 0x7FFFFFFFu; }
+  static __device__ __forceinline__ int exponent(unsigned long long m) { return max((int)(m >> 23), 1); }
+  static __device__ __forceinline__ unsigned long long mantissa(unsigned long long m) {
+    return (m & 0x7FFFFFull) | (m >> 23 ? 1ull << 23 : 0ull);
+  }
+  static __device__ __forceinline__ bool negative(float x) { return __float_as_int(x) < 0; }
+  static __device__ __forceinline__ bool finite(unsigned long long m) { return (m >> 23) != 0xFF; }
+};
+
+// round(x 2^e) for |x 2^e| < 2^62, ties away from zero
+template <typename T>
+__device__ __forceinline__ long long scaled_int(T x, int e) {
+  const unsigned long long mg = LevelType<T>::mag(x);
+  const unsigned long long m = LevelType<T>::mantissa(mg);
+  const int sh = LevelType<T>::exponent(mg) - LevelType<T>::BIAS + e;
+  unsigned long long v;
+  if (sh >= 0)
+    v = m << min(sh, 63);
+  else
+    v = sh > -60 ? (m + (1ull << (-sh - 1))) >> -sh : 0;
+  return LevelType<T>::negative(x) ? -(long long)v : (long long)v;
+}
+
+// The residue of `x` modulo p_l as a bf16 bit pattern in the upper half of the
+// result: an integer of magnitude at most 128 through the float 2^23 + v.
+template <typename T>
+__device__ __forceinline__ uint32_t residue_bits(int u0, int u1, int u2, int l) {
+  const ResidueTab& t = sizeof(T) == 8 ? c_res64 : c_res32;
+  uint32_t r = (uint32_t)u0 + t.bias[l] + t.c1[l] * (uint32_t)u1;
+  if (sizeof(T) == 8) r += t.c2[l] * (uint32_t)u2;
+  r -= (__umulhi(r, t.magic[l]) >> 7) * t.mod[l];
+  return __float_as_uint(__uint_as_float(0x4B000000u | r) - t.off[l]);
+}
+
+// One block per row: the row's largest magnitude, then its 2-norm relative to
+// it (float32, a margin covers its rounding), e_i, and the residues. Columns
+// in pairs; np a multiple of 64.
+template <typename T>
+__global__ void __launch_bounds__(256) k_crt_residues(const T* __restrict__ X, int np, int* __restrict__ ex,
+                                                       uint32_t* __restrict__ planes) {
+  typedef LevelType<T> LT;
+  __shared__ unsigned long long wmax[8];
+  __shared__ float wsum[8];
+  const int row = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const T* x = X + (size_t)row * np;
+  unsigned long long mx = 0;
+  for (int j = tid; j < np; j += 256) mx = max(mx, LT::mag(x[j]));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (lane == 0) wmax[warp] = mx;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < 8; ++w) mx = max(mx, wmax[w]);
+  // |x| 2^-emax in [0, 2): emax = exponent of the largest
+  const int emax = LT::exponent(mx) - LT::BIAS + (sizeof(T) == 8 ? 52 : 23);
+  float s = 0.f;
+  for (int j = tid; j < np; j += 256) {
+    const float v = (float)(int)scaled_int(x[j], 22 - emax);   // magnitude up to 2^23, exact in float32
+    s = __fmaf_rn(v, v, s);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) wsum[warp] = s;
+  __syncthreads();
+  s = 0.f;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) s += wsum[w];
+  // norm 2^(e + 22 - emax) = sqrt(s); rounding and truncation within the 0.02 bits of margin
+  const bool fin = LT::finite(mx);
+  // (s < 1: zero, or so far below the smallest normal number that every square underflows)
+  const int e = s >= 1.f ? (int)floorf(crt_norm_bits(LT::NP) - 0.02f - 0.5f * log2f(s)) + 22 - emax : 0;
+  if (tid == 0) ex[row] = fin ? e : CRT_ROW_NAN;
+  const size_t plane = (size_t)np * np / 2;
+  uint32_t* out = planes + (size_t)row * np / 2;
+  for (int j = tid; j < np / 2; j += 256) {
+    int u[2][3];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const long long v = fin ? scaled_int(x[2 * j + h], e) : 0;
+      if (sizeof(T) == 8) {
+        u[h][0] = (int)(v & 0x1FFFFF);
+        u[h][1] = (int)(v >> 21) & 0x1FFFFF;
+        u[h][2] = (int)(v >> 42);
+      } else {
+        u[h][0] = (int)v & 0xFFFF;
+        u[h][1] = (int)v >> 16;
+        u[h][2] = 0;
+      }
+    }
+#pragma unroll
+    for (int l = 0; l < LT::NP; ++l)
+      out[l * plane + j] = __byte_perm(residue_bits<T>(u[0][0], u[0][1], u[0][2], l),
+                                       residue_bits<T>(u[1][0], u[1][1], u[1][2], l), 0x7632);
+  }
+}
+
+// v 2^-e rounded to nearest even, v a signed 128-bit integer
+__device__ __forceinline__ double i128_to_double(__int128 v, int e) {
+  if (v == 0) return 0.0;
+  const bool neg = v < 0;
+  const u128 a = neg ? (u128)(-v) : (u128)v;
+  const unsigned long long hi = (unsigned long long)(a >> 64), lo = (unsigned long long)a;
+  const int z = hi ? __clzll((long long)hi) : 64 + __clzll((long long)lo);
+  const u128 n = a << z;                                  // leading bit 127
+  const unsigned long long top = (unsigned long long)(n >> 64);
+  const bool sticky = (unsigned long long)n != 0;
+  unsigned long long q = top >> 11;
+  const unsigned long long rem = top & 0x7FFull;
+  if (rem > 0x400ull || (rem == 0x400ull && (sticky || (q & 1)))) ++q;   // may carry to 2^53: exact below
+  const int ex = 127 - z - 52 - e;                        // value q 2^ex
+  const unsigned long long sign = neg ? 1ull << 63 : 0ull;
+  const int field = ex + 52 + 1023;
+  if (field > 0 && field < 2046)                          // q in [2^52, 2^53]: adding carries into the exponent
+    return __longlong_as_double((long long)(sign | (((unsigned long long)(field - 1) << 52) + q)));
+  return ldexp(neg ? -(double)q : (double)q, ex);         // subnormal or out of range
+}
+
+template <typename T>
+struct Combine;
+template <>
+struct Combine<double> {
+  static constexpr int NP = 16;
+  // c from the bytes at bit `sh` of the 16 words
+  static __device__ __forceinline__ double value(const uint32_t (&w)[16], int sh, int e) {
+    uint32_t S[6] = {0, 0, 0, 0, 0, 0}, f = 0;
+#pragma unroll
+    for (int l = 0; l < 16; ++l) {
+      const uint32_t t = (w[l] >> sh) & 0xFFu;
+#pragma unroll
+      for (int k = 0; k < 6; ++k) S[k] += t * c_comb64.limb[k][l];   // 16 terms below 2^28
+      f += t * c_comb64.frac[l];
+    }
+    const uint32_t q = (f + (1u << 22)) >> 23;            // round(sum t_l / p_l): |c| <= P / 4 leaves no doubt
+    u128 c = (u128)S[0] + ((u128)S[1] << 20) + ((u128)S[2] << 40) + ((u128)S[3] << 60) + ((u128)S[4] << 80) +
+             ((u128)S[5] << 100);
+    c -= (u128)q * (((u128)P64_HI << 64) | P64_LO);       // modulo 2^128: |c| < 2^124
+    return i128_to_double((__int128)c, e);
+  }
+  static __device__ __forceinline__ double nan() { return __longlong_as_double(0x7FF8000000000000ll); }
+};
+template <>
+struct Combine<float> {
+  static constexpr int NP = 8;
+  static __device__ __forceinline__ float value(const uint32_t (&w)[8], int sh, int e) {
+    unsigned long long c = 0;
+    uint32_t hi = 0, f = 0;
+#pragma unroll
+    for (int l = 0; l < 8; ++l) {
+      const uint32_t t = (w[l] >> sh) & 0xFFu;
+      c += (unsigned long long)t * c_comb32.lo[l];
+      hi += t * c_comb32.hi[l];
+      f += t * c_comb32.frac[l];
+    }
+    const uint32_t q = (f + (1u << 22)) >> 23;
+    c += ((unsigned long long)hi << 32) - (unsigned long long)q * P32;   // modulo 2^64: |c| < 2^62
+    return ldexpf(__ll2float_rn((long long)c), -e);
+  }
+  static __device__ __forceinline__ float nan() { return __int_as_float(0x7FC00000); }
+};
+
+// C (np x np) from the residues t (NP planes of np x np bytes, valid on and
+// above the diagonal blocks): 64 x 64 tiles of the upper block triangle, each
+// thread four columns of a row at a time (one word per plane), the mirror
+// through shared memory.
+template <typename T>
+__global__ void __launch_bounds__(256) k_crt_combine(const uint8_t* __restrict__ t, int np,
+                                                      const int* __restrict__ ex, T* __restrict__ C) {
+  constexpr int NP = Combine<T>::NP;
+  __shared__ T tile[64][65];
+  int bi, bj;
+  block_tri_index(np / 64, bi, bj);
+  const int r0 = bi * 64, c0 = bj * 64;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const size_t plane = (size_t)np * np;
+  int ec[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) ec[e] = ex[c0 + tx * 4 + e];
+#pragma unroll 1
+  for (int m = 0; m < 4; ++m) {
+    const int r = ty + 16 * m;
+    const int er = ex[r0 + r];
+    const uint8_t* src = t + (size_t)(r0 + r) * np + c0 + tx * 4;
+    uint32_t w[NP];
+#pragma unroll
+    for (int l = 0; l < NP; ++l) w[l] = *reinterpret_cast<const uint32_t*>(src + l * plane);
+    T v[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      v[e] = (er == CRT_ROW_NAN || ec[e] == CRT_ROW_NAN) ? Combine<T>::nan() : Combine<T>::value(w, 8 * e, er + ec[e]);
+    T* dst = C + (size_t)(r0 + r) * np + c0 + tx * 4;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      dst[e] = v[e];
+      tile[tx * 4 + e][r] = v[e];
+    }
+  }
+  if (bi == bj) return;
+  __syncthreads();
+  for (int e = threadIdx.x; e < 64 * 64; e += 256) C[(size_t)(c0 + e / 64) * np + r0 + e % 64] = tile[e / 64][e % 64];
+}
+
+template <typename T>
+int square_impl(cdl_ctx* ctx, cdl_chain* ch, int level, void* planes, uint8_t* t, int* ex) {
+  constexpr int NP = Combine<T>::NP;
+  const int np = (int)ch->npad;
+  {
+    Launch L(ctx, CDL_KC_SQUARE, 0);
+    k_crt_residues<T><<<np, 256, 0, ctx->stream>>>(static_cast<const T*>(ch->level(level)), np, ex,
+                                                   static_cast<uint32_t*>(planes));
+    CDL_TRY(L.done());
+  }
+  CDL_TRY(crt_gemm(ctx, planes, np, nullptr, 0, np, NP, t, CDL_KC_SQUARE, (double)ch->n * ch->n * (ch->n + 1.0)));
+  const int nb = np / 64;
+  Launch L(ctx, CDL_KC_SQUARE, 0);
+  k_crt_combine<T><<<nb * (nb + 1) / 2, 256, 0, ctx->stream>>>(t, np, ex, static_cast<T*>(ch->level(level + 1)));
+  return L.done();
+}
+
+}  // namespace
+
+// Squares a float64 or float32 level. CDL_ERR_UNSUPPORTED (nothing launched)
+// when the order is past the exact sums' range, the device lacks the
+// tensor-core path, or its workspace (3 NP bytes per entry) is not to be had.
+int chain_square_crt(cdl_ctx* ctx, cdl_chain* ch, int level) {
+  const size_t cnt = (size_t)ch->npad * ch->npad;
+  const int planes = ch->dtype == CDL_F64 ? 16 : 8;
+  if ((ch->dtype != CDL_F64 && ch->dtype != CDL_F32) || !crt_gemm_supported(ctx, (int)ch->npad))
+    return CDL_ERR_UNSUPPORTED;
+  CDL_TRY(crt_gemm_prepare(ctx, (int)ch->npad, 0));
+  void *vp, *vt, *ve;
+  if (ws_get(ctx, "crt.planes", planes * cnt * 2, &vp) != CDL_OK || ws_get(ctx, "crt.t", planes * cnt, &vt) != CDL_OK ||
+      ws_get(ctx, "crt.e", (size_t)ch->npad * sizeof(int), &ve) != CDL_OK) {
+    ws_reclaim(ctx);
+    return CDL_ERR_UNSUPPORTED;
+  }
+  if (ch->dtype == CDL_F64)
+    return square_impl<double>(ctx, ch, level, vp, static_cast<uint8_t*>(vt), static_cast<int*>(ve));
+  return square_impl<float>(ctx, ch, level, vp, static_cast<uint8_t*>(vt), static_cast<int*>(ve));
+}
+
+}  // namespace cdl

@@ -145,6 +145,12 @@ namespace cdl {
 // Workspace: returns a device buffer of at least `bytes` for `name`,
 // reusing or growing it (respecting ctx->ws_cap).
 int ws_get(cdl_ctx* ctx, const char* name, size_t bytes, void** out);
+// Frees the buffers of faster forms that a slower one can do without (names
+// crt.*; synchronises the stream); true if there were any. ws_get does so by
+// itself before it refuses another buffer, and malloc_reclaim is a cudaMalloc
+// that does.
+bool ws_reclaim(cdl_ctx* ctx);
+cudaError_t malloc_reclaim(cdl_ctx* ctx, void** p, size_t bytes);
 
 // *out (device) = the float64 bit pattern of max |x_i| over count values
 // (asynchronous; out is zeroed first).
@@ -193,6 +199,9 @@ int graph_build_static(const double* X, int64_t n, int T, double sigma, double* 
 // chain.cu
 int chain_init(cdl_ctx* ctx, cdl_chain* ch, const double* A);
 int chain_square_simt(cdl_ctx* ctx, cdl_chain* ch, int level);
+// crt.cu: the same squaring of a float64 or float32 level on the tensor cores
+// (CDL_ERR_UNSUPPORTED: not at this size or without its workspace)
+int chain_square_crt(cdl_ctx* ctx, cdl_chain* ch, int level);
 int fp8_level_bound(cdl_ctx* ctx, cdl_chain* ch, int level);
 // Max absolute row sum of level i (an upper bound of its spectral norm, the
 // level being symmetric), as float bits in *out_bits (device).
@@ -217,6 +226,13 @@ int ooc_read_done(cdl_ctx* ctx, cdl_chain* ch, int i);
 int ooc_prefetch(cdl_ctx* ctx, cdl_chain* ch, int i);
 // tc_gemm.cu
 int chain_square_tc(cdl_ctx* ctx, cdl_chain* ch, int level);
+// Residue products (crt.cuh), see the definition.
+bool crt_gemm_supported(cdl_ctx* ctx, int K);
+// Builds crt_gemm's tile list. Call it before taking the operands' workspace:
+// a list that crt_gemm had to allocate itself could reclaim them.
+int crt_gemm_prepare(cdl_ctx* ctx, int a_rows, int b_rows);
+int crt_gemm(cdl_ctx* ctx, const void* a_planes, int a_rows, const void* b_planes, int b_rows, int K, int planes,
+             uint8_t* t, int kc, double work);
 // Number of exact-slice pairs of the residual product (s + t <= 7 of six slices).
 constexpr int RESID_PAIRS = 21;
 // A Z on the tensor cores from exact bf16 slices (A's in the chain, Z / c in

@@ -57,6 +57,7 @@ int pair_regen(cdl_ctx* ctx, const double* X1, const double* X2, int64_t n64, in
   // buffers: two float64 panels, the transposed slices of one, the series,
   // degrees, scalars, Y, Z1, Z2, F, top
   void *dP, *dS, *dX, *dvec, *dY, *dZ1, *dZ2, *dF, *dtop;
+  ws_reclaim(ctx);   // the resident levels take what device memory is free
   CDL_TRY(ws_get(ctx, "regen.panels", 2 * (size_t)P * n * sizeof(double), &dP));
   CDL_TRY(ws_get(ctx, "regen.slicesT", 6 * (size_t)npad * P * 2, &dS));
   CDL_TRY(ws_get(ctx, "regen.vec", (3 * (size_t)n + 8) * sizeof(double), &dvec));

@@ -27,6 +27,7 @@
 #include <string>
 #include <vector>
 
+#include "crt.cuh"
 #include "ff.cuh"
 #include "internal.h"
 
@@ -1901,6 +1902,231 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(S2_THREADS, 1)
   }
 }
 
+// ---------------------------------------------------------------- residue products on CTA pairs
+// t[l] = ((A_l B_l^T) mod p_l) inv_l mod p_l for the residue planes l of two
+// integer matrices (crt.cuh): the products of the float64 and float32 chains.
+// Pairs, stages and barriers as in k_tc_sq2; a unit is one 256 x bn block of
+// one plane. K runs in chunks of 1024, whose sums are exact in float32: each
+// chunk goes to one of the two TMEM accumulators, and the eight epilogue warps
+// add it to int32 registers (bn / 2 columns per thread) while the next chunk
+// multiplies; after the last chunk the sums are reduced modulo p_l and stored
+// as bytes. Bound by the tensor cores for long K (8192 cycles of MMA per chunk
+// against about 600 of draining), by the reduction and the stores for K of a
+// few hundred. Planes are numbered outermost, so one plane's panels stay in
+// L2 while its blocks are formed.
+constexpr int CR_CHUNK_KB = 16;                        // 1024 of K per exact chunk
+constexpr int CR_MAX_KBLOCKS = 62 * CR_CHUNK_KB;       // int32 sums and the modular reduction: |sum| <= 62 2^24
+
+struct CrtGemmParams {
+  const uint32_t* tiles;   // blocks I (bits 0-14), J (bits 15-29)
+  int nblocks;             // blocks per plane
+  int num_units;           // planes * nblocks
+  int kblocks;
+  int a_rows, b_rows;      // rows of one plane in the A and B maps
+  int bn;                  // MMA N = 64 NCH
+  uint32_t idesc;
+  uint8_t* t;
+  size_t tplane;           // bytes per output plane
+  int ldt;
+  unsigned* status;
+  int debug_withhold_load;
+  uint32_t mod[CRT_MAX], magic[CRT_MAX], inv[CRT_MAX], bias[CRT_MAX];
+};
+
+__device__ __forceinline__ uint32_t crt_mod31(uint32_t x, uint32_t p, uint32_t magic) {   // x mod p, x < 2^31
+  return x - (__umulhi(x, magic) >> 7) * p;
+}
+
+template <int NCH>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(S2_THREADS, 1)
+    k_tc_crt(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const CrtGemmParams p) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S2_STAGES * S2_STAGE);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + S2_NBARS);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + S2_NBARS + 1);
+  const uint32_t bar0 = smem_u32(bars);
+  auto full_bar = [&](int s) { return bar0 + 8u * s; };
+  auto empty_bar = [&](int s) { return bar0 + 8u * (S2_STAGES + s); };
+  auto tfull_bar = [&](int a) { return bar0 + 8u * (2 * S2_STAGES + a); };
+  auto tempty_bar = [&](int a) { return bar0 + 8u * (2 * S2_STAGES + 2 + a); };
+  const uint32_t drain_bar = bar0 + 8u * (2 * S2_STAGES + 4);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_rank();
+  const int cid = blockIdx.x >> 1, ncl = gridDim.x >> 1;
+  const uint32_t lead_bar0 = mapa_rank(bar0, 0);
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < S2_STAGES; ++s) {
+      mbar_init(full_bar(s), 1);
+      mbar_init(empty_bar(s), 1);
+    }
+    for (int a = 0; a < 2; ++a) {
+      mbar_init(tfull_bar(a), 1);
+      mbar_init(tempty_bar(a), 16);
+    }
+    mbar_init(drain_bar, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"(S2_TMEM_COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  cluster_sync_all();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+
+  if (warp == 0 && lane == 0) {
+    // ------------------------------------------------ TMA producer (both CTAs)
+    const uint32_t b_half = (uint32_t)(NCH * 32) * BK * 2;   // bytes of this CTA's half of B
+    int it = 0;
+    bool ok = true;
+    for (int u = cid; u < p.num_units && ok; u += ncl) {
+      const int l = u / p.nblocks;
+      const uint32_t td = p.tiles[u - l * p.nblocks];
+      const int a_row = l * p.a_rows + (int)(td & 0x7FFF) * 256 + (int)rank * 128;
+      const int b_row = l * p.b_rows + (int)((td >> 15) & 0x7FFF) * p.bn + (int)rank * (NCH * 32);
+      for (int kb = 0; kb < p.kblocks; ++kb, ++it) {
+        const int s = it % S2_STAGES;
+        if (!mbar_wait(empty_bar(s), ((uint32_t)(it / S2_STAGES) & 1) ^ 1, abort_flag, p.status)) {
+          ok = false;
+          break;
+        }
+        if (rank == 0) mbar_expect_tx(full_bar(s), 2 * (S2_HALF + b_half));
+        const uint32_t dst = smem_u32(smem + s * S2_STAGE);
+        const uint32_t fb = lead_bar0 + 8u * s;
+        if (!(p.debug_withhold_load && it == 0 && rank == 0)) tma_load_2d_pair(dst, &tmA, kb * BK, a_row, fb);
+        tma_load_2d_pair(dst + S2_HALF, &tmB, kb * BK, b_row, fb);
+      }
+    }
+    if (ok) {
+      for (int j = it; j < it + S2_STAGES && ok; ++j)
+        if (!mbar_wait(empty_bar(j % S2_STAGES), ((uint32_t)(j / S2_STAGES) & 1) ^ 1, abort_flag, p.status)) ok = false;
+    }
+    if (!ok) {   // copies already issued land within microseconds: give them time (bounded)
+      const unsigned long long t0 = globaltimer();
+      while (globaltimer() - t0 < 50000ull) {
+      }
+    }
+  } else if (warp == 1 && lane == 0 && rank == 0) {
+    // ------------------------------------------------ MMA issuer (rank 0 for the pair)
+    int it = 0, tc = 0;
+    bool ok = true, issued = false;
+    for (int u = cid; u < p.num_units && ok; u += ncl) {
+      for (int kb = 0; kb < p.kblocks && ok; ++kb, ++it) {
+        const int acc = tc & 1;
+        if (kb % CR_CHUNK_KB == 0) {   // a new chunk: its accumulator must have been drained
+          if (!mbar_wait(tempty_bar(acc), ((uint32_t)(tc >> 1) & 1) ^ 1, abort_flag, p.status)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+        }
+        const uint32_t d_tmem = tmem_base + (uint32_t)(acc * 256);
+        const int s = it % S2_STAGES;
+        if (!mbar_wait(full_bar(s), (uint32_t)(it / S2_STAGES) & 1, abort_flag, p.status)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t a_addr = smem_u32(smem + s * S2_STAGE);
+        const uint64_t adesc = smem_desc(a_addr);
+        const uint64_t bdesc = smem_desc(a_addr + S2_HALF);
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk)
+          mma_bf16_pair(d_tmem, adesc + (uint64_t)(kk * 2), bdesc + (uint64_t)(kk * 2), p.idesc,
+                        ((kb % CR_CHUNK_KB) | kk) != 0);
+        issued = true;
+        mma_commit_pair(empty_bar(s));
+        if (kb % CR_CHUNK_KB == CR_CHUNK_KB - 1 || kb == p.kblocks - 1) {
+          mma_commit_pair(tfull_bar(acc));
+          ++tc;
+        }
+      }
+    }
+    if (!ok && issued) {
+      asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(drain_bar)
+                   : "memory");
+      const unsigned long long t0 = globaltimer();
+      while (!mbar_try_wait(drain_bar, 0) && globaltimer() - t0 < WAIT_LIMIT_NS) {
+      }
+    }
+  } else if (warp >= 2) {
+    // ------------------------------------------------ epilogue (128 rows per CTA; two warps per TMEM
+    // lane quarter, 32 NCH columns each)
+    const int q = warp & 3;
+    const int half = (warp - 2) >> 2;
+    const int chunks = (p.kblocks + CR_CHUNK_KB - 1) / CR_CHUNK_KB;
+    int tc = 0;
+    bool ok = true;
+    for (int u = cid; u < p.num_units && ok; u += ncl) {
+      int sum[NCH][32];
+#pragma unroll
+      for (int c = 0; c < NCH; ++c)
+#pragma unroll
+        for (int e = 0; e < 32; ++e) sum[c][e] = 0;
+      for (int ch = 0; ch < chunks; ++ch, ++tc) {
+        const int acc = tc & 1;
+        if (!mbar_wait(tfull_bar(acc), (uint32_t)(tc >> 1) & 1, abort_flag, p.status)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t taddr = tmem_base + (uint32_t)(acc * 256 + half * (NCH * 32)) + ((uint32_t)(q * 32) << 16);
+#pragma unroll
+        for (int c = 0; c < NCH; ++c) {
+          float v[32];
+          tmem_ld32(taddr + (uint32_t)(c * 32), v);
+#pragma unroll
+          for (int e = 0; e < 32; ++e) sum[c][e] += __float2int_rn(v[e]);
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(lead_bar0 + 8u * (2 * S2_STAGES + 2 + acc));
+      }
+      if (!ok) break;
+      const int l = u / p.nblocks;
+      const uint32_t td = p.tiles[u - l * p.nblocks];
+      const uint32_t mod = p.mod[l], magic = p.magic[l], inv = p.inv[l], bias = p.bias[l];
+      const int r = (int)(td & 0x7FFF) * 256 + (int)rank * 128 + q * 32 + lane;
+      uint8_t* out = p.t + (size_t)l * p.tplane + (size_t)r * p.ldt + (size_t)((td >> 15) & 0x7FFF) * p.bn +
+                     half * (NCH * 32);
+#pragma unroll
+      for (int c = 0; c < NCH; ++c) {
+        uint32_t w[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          uint32_t b[4];
+#pragma unroll
+          for (int h = 0; h < 4; ++h)
+            b[h] = crt_mod31(crt_mod31((uint32_t)sum[c][4 * e + h] + bias, mod, magic) * inv, mod, magic);
+          w[e] = b[0] | (b[1] << 8) | (b[2] << 16) | (b[3] << 24);
+        }
+        // 32 columns: one 32-byte sector per lane and store
+        asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(out + c * 32), "r"(w[0]), "r"(w[1]),
+                     "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+                     : "memory");
+      }
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync_all();
+  tc_fence_after();
+  if (warp == 0) {
+    __syncwarp();
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(S2_TMEM_COLS)
+                 : "memory");
+  }
+}
+
 // ---------------------------------------------------------------- chain application on CTA pairs
 // x <- level x for one level, as k_tc_gemm's apply mode computes it (float
 // partial products per split of K, summed by the update kernel), with
@@ -2677,6 +2903,96 @@ int tc_square_grouped_pairs(cdl_ctx* ctx, const TcGroup* host_first, const TcGro
   // the kernel-parameter map is unused in grouped mode: pass the first graph's
   k_tc_sq2<<<2 * clusters, S2_THREADS, S2_SMEM_BYTES, ctx->stream>>>(host_first->mapA, p);
   return L.done();
+}
+
+// Residue products t[l] = ((A_l B_l^T) mod p_l) inv_l mod p_l of `planes`
+// planes. a_planes: planes x a_rows x K bf16 (a_rows a multiple of 256, K of
+// 64); b_planes: planes x b_rows x K, or null for B = A, of which only the
+// 256 x 256 blocks on and above the diagonal are formed. t: planes x a_rows x
+// (b_rows or a_rows) bytes, 32-byte aligned.
+bool crt_gemm_supported(cdl_ctx* ctx, int K) {
+  return tc_supported(ctx) && pair_clusters(ctx) > 0 && K / BK <= CR_MAX_KBLOCKS;
+}
+
+namespace {
+template <int NCH>
+int crt_launch(cdl_ctx* ctx, const CUtensorMap& ma, const CUtensorMap& mb, const CrtGemmParams& p, int clusters, int kc,
+               double work) {
+  static bool attr = false;
+  if (!attr) {
+    CDL_CUDA_TRY(cudaFuncSetAttribute(k_tc_crt<NCH>, cudaFuncAttributeMaxDynamicSharedMemorySize, S2_SMEM_BYTES));
+    attr = true;
+  }
+  Launch L(ctx, kc, work);
+  k_tc_crt<NCH><<<2 * clusters, S2_THREADS, S2_SMEM_BYTES, ctx->stream>>>(ma, mb, p);
+  return L.done();
+}
+}  // namespace
+
+namespace {
+// 256 x bn blocks of a_rows x b_rows; b_rows = 0: those on and above the diagonal of a_rows x a_rows
+int crt_tiles(cdl_ctx* ctx, int a_rows, int b_rows, int bn, const uint32_t** tiles, int* count) {
+  const int nb = a_rows / 256;
+  if (b_rows == 0)
+    return get_tiles(ctx, "tc.sq2." + std::to_string(nb), [&] { return square_pair_tiles(nb); }, tiles, count);
+  return get_tiles(ctx, "tc.crt." + std::to_string(nb) + "." + std::to_string(b_rows / bn),
+                   [&] {
+                     std::vector<uint32_t> v;
+                     for (int I = 0; I < nb; ++I)
+                       for (int J = 0; J < b_rows / bn; ++J) v.push_back((uint32_t)I | ((uint32_t)J << 15));
+                     return v;
+                   },
+                   tiles, count);
+}
+int crt_bn(int b_rows) { return b_rows % 256 == 0 ? 256 : b_rows; }
+}  // namespace
+
+int crt_gemm_prepare(cdl_ctx* ctx, int a_rows, int b_rows) {
+  const uint32_t* tiles;
+  int count;
+  return crt_tiles(ctx, a_rows, b_rows, crt_bn(b_rows), &tiles, &count);
+}
+
+int crt_gemm(cdl_ctx* ctx, const void* a_planes, int a_rows, const void* b_planes, int b_rows, int K, int planes,
+             uint8_t* t, int kc, double work) {
+  const bool sym = b_planes == nullptr;
+  const int bn = crt_bn(sym ? a_rows : b_rows);
+  if (a_rows % 256 || K % BK || planes > CRT_MAX || bn % 64 || bn > 256 || !crt_gemm_supported(ctx, K))
+    return CDL_ERR_INVALID_ARG;
+  const uint32_t* tiles;
+  int count;
+  CDL_TRY(crt_tiles(ctx, a_rows, sym ? 0 : b_rows, bn, &tiles, &count));
+  if (sym) b_rows = a_rows;
+  CUtensorMap ma, mb;
+  CDL_TRY(make_map(&ma, a_planes, (int64_t)planes * a_rows, K, 128));
+  CDL_TRY(make_map(&mb, sym ? a_planes : b_planes, (int64_t)planes * b_rows, K, bn / 2));
+  CrtGemmParams p{};
+  p.tiles = tiles;
+  p.nblocks = count;
+  p.num_units = count * planes;
+  p.kblocks = K / BK;
+  p.a_rows = a_rows;
+  p.b_rows = b_rows;
+  p.bn = bn;
+  p.idesc = make_idesc_m256(bn);
+  p.t = t;
+  p.tplane = (size_t)a_rows * b_rows;
+  p.ldt = b_rows;
+  p.status = ctx->dev_status;
+  p.debug_withhold_load = ctx->debug_flags & 1;
+  for (int l = 0; l < planes; ++l) {
+    p.mod[l] = (uint32_t)CRT_MOD[l];
+    p.magic[l] = crt_magic(CRT_MOD[l]);
+    p.inv[l] = (uint32_t)crt_inverse(planes, l);
+    p.bias[l] = (uint32_t)(((1u << 30) + CRT_MOD[l] - 1) / CRT_MOD[l] * CRT_MOD[l]);
+  }
+  const int clusters = std::min(p.num_units, pair_clusters(ctx));
+  switch (bn / 64) {
+    case 1: return crt_launch<1>(ctx, ma, mb, p, clusters, kc, work);
+    case 2: return crt_launch<2>(ctx, ma, mb, p, clusters, kc, work);
+    case 3: return crt_launch<3>(ctx, ma, mb, p, clusters, kc, work);
+    default: return crt_launch<4>(ctx, ma, mb, p, clusters, kc, work);
+  }
 }
 
 int chain_square_tc(cdl_ctx* ctx, cdl_chain* ch, int level) {

@@ -1,0 +1,110 @@
+"""Float64 and float32 chain squarings through residues on the tensor cores:
+level i + 1 against the exact square of the stored level i, at the edges of
+the 256-blocks and of the 1024-wide exact chunks, for magnitudes down to
+underflow, for non-finite levels, and against the CUDA-core form that runs
+when the workspace is not to be had."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from workloads import iid_pair   # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+# unit roundoff; half a unit of 2^-B of the row norm per entry with B >= 60.6 (16 moduli) and 29.7 (8)
+TYPES = {"f64": (np.float64, 2.0 ** -53, 2.0 ** -60), "f32": (np.float32, 2.0 ** -24, 2.0 ** -29)}
+
+
+@pytest.fixture(scope="module")
+def G():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from gpu_util import Ctx, lib
+    g = Ctx(lib())
+    yield g
+    g.close()
+
+
+def _dtype(cdl, name):
+    return {"f64": cdl.CDL_F64, "f32": cdl.CDL_F32}[name]
+
+
+def _levels(G, n, d, name, seed=0):
+    A, D, vol, _ = G.graph(iid_pair(n, 8, 1, seed=seed).X[0])
+    ch = G.chain(A, D, vol, d, _dtype(G.cdl, name))
+    try:
+        return [G.level(ch, i, TYPES[name][0]).cpu().numpy().copy() for i in range(d)]
+    finally:
+        G.cdl.cdl_chain_free(ch)
+
+
+def _check_square(S, C, name, rows):
+    """Rows `rows` of C against S S in extended precision (63 bits or more)."""
+    _, u, unit = TYPES[name]
+    n = S.shape[0]
+    scale = np.abs(S).max() or 1.0
+    W = (S.astype(np.longdouble)) / np.longdouble(scale)
+    R = W[rows] @ W
+    norm = np.sqrt((W * W).sum(1)).astype(np.float64)
+    got = C[rows].astype(np.longdouble) / np.longdouble(scale) / np.longdouble(scale)
+    bound = u * np.abs(R).astype(np.float64) + np.sqrt(n) * unit * norm[rows][:, None] * norm[None, :] + 1e-300
+    assert np.all(np.abs(got - R).astype(np.float64) <= bound)
+
+
+@pytest.mark.parametrize("name", ["f64", "f32"])
+@pytest.mark.parametrize("n", [2, 63, 256, 257, 1023, 1025, 2100])
+def test_square_is_exact_to_one_rounding(G, name, n):
+    L = _levels(G, n, 3, name, seed=n)
+    rows = np.unique(np.r_[0, 1, n // 2, n - 1, np.random.default_rng(n).integers(0, n, 8)])
+    for i in range(2):
+        _check_square(L[i], L[i + 1], name, rows)
+        assert np.array_equal(L[i + 1], L[i + 1].T)
+        assert not L[i + 1][n:].any()
+
+
+@pytest.mark.parametrize("name", ["f64", "f32"])
+def test_levels_underflow_to_zero(G, name):
+    """Well-connected graphs' levels decay like lambda^(2^i): every level stays finite, and the last are zero."""
+    L = _levels(G, 300, 12, name)
+    big = [float(np.abs(x).max()) for x in L]
+    assert all(np.isfinite(x).all() for x in L) and big[-1] == 0.0
+    for a, b in zip(big, big[1:]):
+        assert b <= a
+
+
+@pytest.mark.parametrize("name", ["f64", "f32"])
+def test_non_finite_level_stays_non_finite(G, name):
+    cdl = G.cdl
+    A, D, vol, _ = G.graph(iid_pair(300, 8, 1, seed=1).X[0])
+    A[7] = 0
+    A[:, 7] = 0
+    D[7] = 0                                          # a node without neighbours: D^(-1/2) is infinite
+    ch = G.chain(A, D, vol, 2, _dtype(cdl, name))
+    try:
+        S, C = (G.level(ch, i, TYPES[name][0]).cpu().numpy() for i in range(2))
+    finally:
+        cdl.cdl_chain_free(ch)
+    assert np.isnan(S).any() and np.array_equal(np.isnan(C), np.isnan(S @ S))   # 0 NaN is NaN: the padding too
+
+
+@pytest.mark.parametrize("name", ["f64", "f32"])
+def test_without_workspace_the_cuda_core_form_runs(G, name):
+    cdl = G.cdl
+    n, npad = 600, 768
+    A, D, vol, _ = G.graph(iid_pair(n, 8, 1, seed=2).X[0])
+    elem = np.dtype(TYPES[name][0]).itemsize
+    cap = 2 * npad * npad * elem + 12 * npad * npad + (1 << 20)   # the chain and the small buffers only
+    st, h = cdl.cdl_ctx_create(0, torch.cuda.current_stream().cuda_stream, cap)
+    assert st == 0
+    out = []
+    for ctx in (G.h, h):
+        st, ch = cdl.cdl_chain_build(ctx, A, cdl.CDL_F64, D, vol.data_ptr(), n, 2, _dtype(cdl, name))
+        assert st == 0 and cdl.cdl_sync(ctx) == 0
+        out.append(G.level(ch, 1, TYPES[name][0]).cpu().numpy().copy())
+        cdl.cdl_chain_free(ch)
+    assert cdl.cdl_ctx_destroy(h) == 0
+    S = _levels(G, n, 1, name, seed=2)[0].astype(np.float64)
+    bound = n * TYPES[name][1] * 2 * (np.abs(S) @ np.abs(S)) + 1e-300
+    assert np.all(np.abs(out[0].astype(np.float64) - out[1]) <= bound)
+    assert not np.array_equal(out[0], out[1])          # two forms did run
