@@ -536,14 +536,15 @@ int abs_max_bits(cdl_ctx* ctx, const double* x, size_t count, unsigned long long
   return L.done();
 }
 
+int chain_split_a(cdl_ctx* ctx, const cdl_chain* ch, const double* A) {
+  const size_t cnt = (size_t)ch->n * ch->n;
+  Launch L(ctx, CDL_KC_RESIDUAL, 0);
+  k_split_a<<<ctx->sm_count * 8, 256, 0, ctx->stream>>>(A, cnt, ch->ahl, ch->ahl + cnt);
+  return L.done();
+}
+
 int chain_init(cdl_ctx* ctx, cdl_chain* ch, const double* A) {
   const int n = (int)ch->n, np = (int)ch->npad;
-  if (ch->ahl) {
-    const size_t cnt = (size_t)n * n;
-    Launch L(ctx, CDL_KC_CHAIN_INIT, 16.0 * cnt);
-    k_split_a<<<ctx->sm_count * 8, 256, 0, ctx->stream>>>(A, cnt, ch->ahl, ch->ahl + cnt);
-    CDL_TRY(L.done());
-  }
   if (ch->aslices) {   // the slices' scale: max A, known before level 0 is formed
     unsigned long long* mb = reinterpret_cast<unsigned long long*>(ch->a_scale + 1);
     if (ctx->amax_hint_A == A && ctx->amax_hint_bits)

@@ -148,19 +148,21 @@ __device__ __forceinline__ uint32_t residue_bits(int u0, int u1, int u2, int l) 
   return __float_as_uint(__uint_as_float(0x4B000000u | r) - t.off[l]);
 }
 
-// One block per row: the row's largest magnitude, then its 2-norm relative to
-// it (float32, a margin covers its rounding), e_i, and the residues. Columns
-// in pairs; np a multiple of 64.
+// One block per row of a rows x cols matrix (zero beyond, to gridDim.x x np):
+// the row's largest magnitude, then its 2-norm relative to it (float32, a
+// margin covers its rounding), e_i, and the residues. Columns in pairs; np a
+// multiple of 64.
 template <typename T>
-__global__ void __launch_bounds__(256) k_crt_residues(const T* __restrict__ X, int np, int* __restrict__ ex,
-                                                       uint32_t* __restrict__ planes) {
+__global__ void __launch_bounds__(256) k_crt_residues(const T* __restrict__ X, int rows, int cols, int ldx, int np,
+                                                       int* __restrict__ ex, uint32_t* __restrict__ planes) {
   typedef LevelType<T> LT;
   __shared__ unsigned long long wmax[8];
   __shared__ float wsum[8];
   const int row = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const T* x = X + (size_t)row * np;
+  const T* x = X + (size_t)row * ldx;
+  if (row >= rows) cols = 0;
   unsigned long long mx = 0;
-  for (int j = tid; j < np; j += 256) mx = max(mx, LT::mag(x[j]));
+  for (int j = tid; j < cols; j += 256) mx = max(mx, LT::mag(x[j]));
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   if (lane == 0) wmax[warp] = mx;
@@ -170,7 +172,7 @@ __global__ void __launch_bounds__(256) k_crt_residues(const T* __restrict__ X, i
   // |x| 2^-emax in [0, 2): emax = exponent of the largest
   const int emax = LT::exponent(mx) - LT::BIAS + (sizeof(T) == 8 ? 52 : 23);
   float s = 0.f;
-  for (int j = tid; j < np; j += 256) {
+  for (int j = tid; j < cols; j += 256) {
     const float v = (float)(int)scaled_int(x[j], 22 - emax);   // magnitude up to 2^23, exact in float32
     s = __fmaf_rn(v, v, s);
   }
@@ -186,13 +188,13 @@ __global__ void __launch_bounds__(256) k_crt_residues(const T* __restrict__ X, i
   // (s < 1: zero, or so far below the smallest normal number that every square underflows)
   const int e = s >= 1.f ? (int)floorf(crt_norm_bits(LT::NP) - 0.02f - 0.5f * log2f(s)) + 22 - emax : 0;
   if (tid == 0) ex[row] = fin ? e : CRT_ROW_NAN;
-  const size_t plane = (size_t)np * np / 2;
+  const size_t plane = (size_t)gridDim.x * np / 2;
   uint32_t* out = planes + (size_t)row * np / 2;
   for (int j = tid; j < np / 2; j += 256) {
     int u[2][3];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const long long v = fin ? scaled_int(x[2 * j + h], e) : 0;
+      const long long v = fin && 2 * j + h < cols ? scaled_int(x[2 * j + h], e) : 0;
       if (sizeof(T) == 8) {
         u[h][0] = (int)(v & 0x1FFFFF);
         u[h][1] = (int)(v >> 21) & 0x1FFFFF;
@@ -315,13 +317,85 @@ __global__ void __launch_bounds__(256) k_crt_combine(const uint8_t* __restrict__
   for (int e = threadIdx.x; e < 64 * 64; e += 256) C[(size_t)(c0 + e / 64) * np + r0 + e % 64] = tile[e / 64][e % 64];
 }
 
+// X (rows x cols, leading dimension ldx) transposed to out (gridDim.y 32 rows x
+// np), zero beyond; 32 x 32 tiles.
+__global__ void __launch_bounds__(256) k_transpose_pad(const double* __restrict__ X, int rows, int cols, int ldx,
+                                                        int np, double* __restrict__ out) {
+  __shared__ double tile[32][33];
+  const int i0 = blockIdx.x * 32, c0 = blockIdx.y * 32, tx = threadIdx.x & 31;
+  for (int a = threadIdx.x >> 5; a < 32; a += 8)
+    tile[a][tx] = (i0 + a < rows && c0 + tx < cols) ? X[(size_t)(i0 + a) * ldx + c0 + tx] : 0.0;
+  __syncthreads();
+  for (int a = threadIdx.x >> 5; a < 32; a += 8) out[(size_t)(c0 + a) * np + i0 + tx] = tile[tx][a];
+}
+
+// (M x)_ir of four consecutive columns r from the residues t (16 planes of np x kpb bytes).
+__device__ __forceinline__ void product4(const uint8_t* __restrict__ t, int np, int kpb, const int* __restrict__ erow,
+                                         const int* __restrict__ ecol, int i, int r, double (&v)[4]) {
+  const uint8_t* src = t + (size_t)i * kpb + r;
+  uint32_t w[16];
+#pragma unroll
+  for (int l = 0; l < 16; ++l) w[l] = *reinterpret_cast<const uint32_t*>(src + (size_t)l * np * kpb);
+  const int er = erow[i];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const int ec = ecol[r + e];
+    v[e] = (er == CRT_ROW_NAN || ec == CRT_ROW_NAN) ? Combine<double>::nan()
+                                                    : Combine<double>::value(w, 8 * e, er + ec);
+  }
+}
+
+// x += M x (x: np x kp, kp a multiple of 4)
+__global__ void __launch_bounds__(128) k_crt_add(const uint8_t* __restrict__ t, int np, int kpb, int kp,
+                                                  const int* __restrict__ erow, const int* __restrict__ ecol,
+                                                  double* __restrict__ x) {
+  const int q = kp / 4;
+  const size_t idx = blockIdx.x * (size_t)128 + threadIdx.x;
+  if (idx >= (size_t)np * q) return;
+  const int i = (int)(idx / q), r = (int)(idx % q) * 4;
+  double v[4];
+  product4(t, np, kpb, erow, ecol, i, r, v);
+#pragma unroll
+  for (int e = 0; e < 4; ++e) x[(size_t)i * kp + r + e] += v[e];
+}
+
+// R = (Y - D o Z) + A Z, and per-block sums of R^2 (fixed order).
+__global__ void __launch_bounds__(128) k_crt_residual(const uint8_t* __restrict__ t, int np, int kpb,
+                                                       const int* __restrict__ erow, const int* __restrict__ ecol,
+                                                       const double* __restrict__ Y, const double* __restrict__ Z,
+                                                       const double* __restrict__ D, int n, int k,
+                                                       double* __restrict__ R, double* __restrict__ part) {
+  __shared__ double red[4];
+  const int q = (k + 3) / 4;
+  double sq = 0.0;
+  for (size_t idx = blockIdx.x * (size_t)128 + threadIdx.x; idx < (size_t)n * q; idx += (size_t)gridDim.x * 128) {
+    const int i = (int)(idx / q), r = (int)(idx % q) * 4;
+    double v[4];
+    product4(t, np, kpb, erow, ecol, i, r, v);
+    const double d = D[i];
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (r + e < k) {
+        const size_t o = (size_t)i * k + r + e;
+        const double x = (Y[o] - d * Z[o]) + v[e];
+        R[o] = x;
+        sq = fma(x, x, sq);
+      }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sq;
+  __syncthreads();
+  if (threadIdx.x == 0) part[blockIdx.x] = ((red[0] + red[1]) + red[2]) + red[3];
+}
+
 template <typename T>
 int square_impl(cdl_ctx* ctx, cdl_chain* ch, int level, void* planes, uint8_t* t, int* ex) {
   constexpr int NP = Combine<T>::NP;
   const int np = (int)ch->npad;
   {
     Launch L(ctx, CDL_KC_SQUARE, 0);
-    k_crt_residues<T><<<np, 256, 0, ctx->stream>>>(static_cast<const T*>(ch->level(level)), np, ex,
+    k_crt_residues<T><<<np, 256, 0, ctx->stream>>>(static_cast<const T*>(ch->level(level)), np, np, np, np, ex,
                                                    static_cast<uint32_t*>(planes));
     CDL_TRY(L.done());
   }
@@ -352,6 +426,71 @@ int chain_square_crt(cdl_ctx* ctx, cdl_chain* ch, int level) {
   if (ch->dtype == CDL_F64)
     return square_impl<double>(ctx, ch, level, vp, static_cast<uint8_t*>(vt), static_cast<int*>(ve));
   return square_impl<float>(ctx, ch, level, vp, static_cast<uint8_t*>(vt), static_cast<int*>(ve));
+}
+
+// ---------------------------------------------------------------- products with right-hand sides
+// M x for a float64 matrix M (a chain level, or the graph in the residual) and
+// k right-hand sides, through 16 residues as the squaring: the rows of M and
+// the columns of x are scaled by their 2-norms, the product is exact, one
+// rounding per entry. The float64 pipe's dot products took 0.52 ms per level
+// at n = 2000, k = 32 (its FMA rate); here the residues of M take most of the
+// time (8 n^2 bytes read, 32 n^2 written).
+int crt_apply_begin(cdl_ctx* ctx, int np, int k, CrtApply* a) {
+  if (!crt_gemm_supported(ctx, np)) return CDL_ERR_UNSUPPORTED;
+  a->np = np;
+  a->kpb = (int)round_up(k, k <= 256 ? 64 : 256);
+  CDL_TRY(crt_gemm_prepare(ctx, np, a->kpb));
+  const size_t kx = (size_t)a->kpb * np;
+  void *vp, *vx, *vxp, *vt, *ve;
+  if (ws_get(ctx, "crt.planes", (size_t)16 * np * np * 2, &vp) != CDL_OK ||
+      ws_get(ctx, "crt.xt", kx * sizeof(double), &vx) != CDL_OK ||
+      ws_get(ctx, "crt.xplanes", 16 * kx * 2, &vxp) != CDL_OK || ws_get(ctx, "crt.xprod", 16 * kx, &vt) != CDL_OK ||
+      ws_get(ctx, "crt.xe", (size_t)(np + a->kpb) * sizeof(int), &ve) != CDL_OK) {
+    ws_reclaim(ctx);
+    return CDL_ERR_UNSUPPORTED;
+  }
+  a->planes = static_cast<uint32_t*>(vp);
+  a->xt = static_cast<double*>(vx);
+  a->xplanes = static_cast<uint32_t*>(vxp);
+  a->t = static_cast<uint8_t*>(vt);
+  a->erow = static_cast<int*>(ve);
+  a->ecol = a->erow + np;
+  return CDL_OK;
+}
+
+int crt_apply_matrix(cdl_ctx* ctx, const CrtApply& a, const double* M, int n, int kc) {
+  Launch L(ctx, kc, 0);
+  k_crt_residues<double><<<a.np, 256, 0, ctx->stream>>>(M, n, n, n, a.np, a.erow, a.planes);
+  return L.done();
+}
+
+int crt_apply_product(cdl_ctx* ctx, const CrtApply& a, const double* x, int rows, int cols, int ldx, int kc,
+                      double work) {
+  {
+    Launch L(ctx, CDL_KC_MISC, 0);
+    k_transpose_pad<<<dim3(a.np / 32, a.kpb / 32), 256, 0, ctx->stream>>>(x, rows, cols, ldx, a.np, a.xt);
+    CDL_TRY(L.done());
+  }
+  {
+    Launch L(ctx, CDL_KC_MISC, 0);
+    k_crt_residues<double><<<a.kpb, 256, 0, ctx->stream>>>(a.xt, a.kpb, a.np, a.np, a.np, a.ecol, a.xplanes);
+    CDL_TRY(L.done());
+  }
+  return crt_gemm(ctx, a.planes, a.np, a.xplanes, a.kpb, a.np, 16, a.t, kc, work);
+}
+
+int crt_apply_add(cdl_ctx* ctx, const CrtApply& a, double* x, int kp) {
+  Launch L(ctx, CDL_KC_MISC, 0);
+  k_crt_add<<<(unsigned)(((size_t)a.np * (kp / 4) + 127) / 128), 128, 0, ctx->stream>>>(a.t, a.np, a.kpb, kp, a.erow,
+                                                                                         a.ecol, x);
+  return L.done();
+}
+
+int crt_apply_residual(cdl_ctx* ctx, const CrtApply& a, const double* Y, const double* Z, const double* D, int n, int k,
+                       double* R, double* part, int nblocks) {
+  Launch L(ctx, CDL_KC_RESIDUAL, 0);
+  k_crt_residual<<<nblocks, 128, 0, ctx->stream>>>(a.t, a.np, a.kpb, a.erow, a.ecol, Y, Z, D, n, k, R, part);
+  return L.done();
 }
 
 }  // namespace cdl

@@ -202,6 +202,30 @@ int chain_square_simt(cdl_ctx* ctx, cdl_chain* ch, int level);
 // crt.cu: the same squaring of a float64 or float32 level on the tensor cores
 // (CDL_ERR_UNSUPPORTED: not at this size or without its workspace)
 int chain_square_crt(cdl_ctx* ctx, cdl_chain* ch, int level);
+// crt.cu: M x for a float64 matrix M of order n (zero padded to np) and
+// float64 right-hand sides. begin takes the workspace (call it after every
+// other ws_get of the operation, which could reclaim it; CDL_ERR_UNSUPPORTED
+// where it is not to be had), matrix forms the residues of M (kept until the
+// next matrix call on the context), product those of x (rows x cols) and of
+// M x; add and residual put M x together: x += M x (x np x kp), R = Y - D o Z
+// + M Z with `nblocks` partial sums of R^2.
+struct CrtApply {
+  int np = 0, kpb = 0;
+  uint32_t *planes = nullptr, *xplanes = nullptr;
+  double* xt = nullptr;
+  uint8_t* t = nullptr;
+  int *erow = nullptr, *ecol = nullptr;
+};
+int crt_apply_begin(cdl_ctx* ctx, int np, int k, CrtApply* a);
+int crt_apply_matrix(cdl_ctx* ctx, const CrtApply& a, const double* M, int n, int kc);
+int crt_apply_product(cdl_ctx* ctx, const CrtApply& a, const double* x, int rows, int cols, int ldx, int kc,
+                      double work);
+int crt_apply_add(cdl_ctx* ctx, const CrtApply& a, double* x, int kp);
+int crt_apply_residual(cdl_ctx* ctx, const CrtApply& a, const double* Y, const double* Z, const double* D, int n, int k,
+                       double* R, double* part, int nblocks);
+// chain.cu: A as the float hi + lo planes of the chain (the residual's operand
+// where crt.cu's form has no workspace)
+int chain_split_a(cdl_ctx* ctx, const cdl_chain* ch, const double* A);
 int fp8_level_bound(cdl_ctx* ctx, cdl_chain* ch, int level);
 // Max absolute row sum of level i (an upper bound of its spectral norm, the
 // level being symmetric), as float bits in *out_bits (device).

@@ -869,6 +869,9 @@ struct SolveBlock {
   double yy = 0.0, rel = 1.0, drift = 0.0;
   int iters = 0, nparts = 0;
   bool exact_r = true;   // R was last formed in full (not recursively)
+  bool crt = false;      // CUDA-core chains: A Z (and float64 level products) through residues (crt.cu)
+  bool a_ready = false;  // float32 chains keep the residues (else the split) of A for every step of the solve
+  CrtApply ca;
   bool done = false;
 
   int ws(const char* name, int idx, size_t bytes, void** out) {
@@ -930,6 +933,7 @@ struct SolveBlock {
       CDL_TRY(ws("solve.part2", idx, (size_t)splits * np * part_cols * xe, &vpart2));
       CDL_TRY(ws("solve.dzop", idx, 2 * (size_t)kp * np * 2, &vdzop));
     }
+    if (!bf16) crt = crt_apply_begin(ctx, np, k, &ca) == CDL_OK;
     R = static_cast<double*>(vR);
     red = static_cast<double*>(vred);
     scal = static_cast<double*>(vscal);
@@ -1043,6 +1047,16 @@ struct SolveBlock {
       nparts = nb;
       return CDL_OK;
     }
+    if (crt) {
+      // the level products of a float64 chain use the same residue planes
+      if (!a_ready || ch->dtype == CDL_F64) CDL_TRY(crt_apply_matrix(ctx, ca, A, n, CDL_KC_RESIDUAL));
+      a_ready = true;
+      CDL_TRY(crt_apply_product(ctx, ca, Z, n, k, k, CDL_KC_RESIDUAL, (double)n * n * k));
+      nparts = std::min(1024, (int)blocks_for((size_t)n * ((k + 3) / 4), 128));
+      return crt_apply_residual(ctx, ca, Y, Z, ch->D, n, k, R, red, nparts);
+    }
+    if (!a_ready) CDL_TRY(chain_split_a(ctx, ch, A));
+    a_ready = true;
     {
       Launch L(ctx, CDL_KC_MISC, 0);
       k_split<<<blocks_for(nk, 256), 256, 0, st>>>(Z, nk, static_cast<float*>(vzh), static_cast<float*>(vzl));
@@ -1154,6 +1168,12 @@ struct SolveBlock {
       k_update_bf16<<<g, 256, 0, st>>>(static_cast<float*>(vx), static_cast<const float*>(vpart), splits, np, kp,
                                        static_cast<__nv_bfloat16*>(vxop), 1);
       return L.done();
+    }
+    if (crt && ch->dtype == CDL_F64) {
+      double* x = static_cast<double*>(vx);
+      CDL_TRY(crt_apply_matrix(ctx, ca, static_cast<const double*>(ch->level(lvl)), np, CDL_KC_APPLY));
+      CDL_TRY(crt_apply_product(ctx, ca, x, np, kp, kp, CDL_KC_APPLY, 8.0 * np * (double)np));
+      return crt_apply_add(ctx, ca, x, kp);
     }
     CDL_TRY(apply_simt(ctx, ch, lvl, vx, vpart, kp, splits));
     const size_t cnt = (size_t)np * kp;
@@ -1292,7 +1312,8 @@ int chain_solve(cdl_ctx* ctx, const cdl_chain* ch, const double* A, const double
     CDL_TRY(s.init(b));
   }
   // a regenerated graph keeps no A operand for the recursive update
-  const bool always_full = (opts->flags & CDL_SOLVE_FULL_RESIDUAL) != 0 || ch->regen != nullptr;
+  // (and with the residue form a full residual costs less than a float32 update)
+  const bool always_full = (opts->flags & CDL_SOLVE_FULL_RESIDUAL) != 0 || ch->regen != nullptr || B[0].crt;
   while (true) {
     std::vector<SolveBlock*> run;
     for (SolveBlock& s : B) {

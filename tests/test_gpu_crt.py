@@ -108,3 +108,33 @@ def test_without_workspace_the_cuda_core_form_runs(G, name):
     bound = n * TYPES[name][1] * 2 * (np.abs(S) @ np.abs(S)) + 1e-300
     assert np.all(np.abs(out[0].astype(np.float64) - out[1]) <= bound)
     assert not np.array_equal(out[0], out[1])          # two forms did run
+
+
+@pytest.mark.parametrize("name", ["f64", "f32"])
+@pytest.mark.parametrize("n,k", [(3, 1), (257, 65), (600, 16), (300, 300)])
+def test_solve_with_and_without_workspace(G, name, n, k):
+    """The exact-product applies and residuals against the forms that run under a workspace cap too small
+    for them: both solutions meet the tolerance, so they agree to it (times the graph's condition)."""
+    cdl = G.cdl
+    npad = (n + 255) // 256 * 256
+    A, D, vol, _ = G.graph(iid_pair(n, 16, 1, seed=n).X[0])
+    Y = G.project(A, k, 3)
+    elem = np.dtype(TYPES[name][0]).itemsize
+    cap = 4 * npad * npad * elem + 8 * n * n + 300 * npad * k + (1 << 18)
+    st, h = cdl.cdl_ctx_create(0, torch.cuda.current_stream().cuda_stream, cap)
+    assert st == 0
+    Zs = []
+    for ctx in (G.h, h):
+        st, ch = cdl.cdl_chain_build(ctx, A, cdl.CDL_F64, D, vol.data_ptr(), n, 4, _dtype(cdl, name))
+        assert st == 0
+        Z = torch.empty((n, k), dtype=torch.float64, device="cuda")
+        stats = cdl.cdl_solve_stats()
+        assert cdl.cdl_chain_solve(ctx, ch, A, cdl.CDL_F64, Y, k, cdl.cdl_solve_opts(60, 1e-12, 0), Z, stats) == 0
+        assert cdl.cdl_sync(ctx) == 0 and stats.rel_res <= 1e-12
+        Zs.append(Z.cpu().numpy())
+        cdl.cdl_chain_free(ch)
+    assert cdl.cdl_ctx_destroy(h) == 0
+    L = np.diag(D.cpu().numpy()) - A.cpu().numpy()
+    for Z in Zs:
+        assert np.linalg.norm(Y.cpu().numpy() - L @ Z) <= 3e-12 * np.linalg.norm(Y.cpu().numpy())
+    assert np.linalg.norm(Zs[0] - Zs[1]) <= 1e-10 * np.linalg.norm(Zs[0])
