@@ -229,7 +229,7 @@ int build_plan(cdl_ctx* ctx, int G, const int64_t* n, int T, const cdl_batch_opt
   }
   // projection variants: node rows per block
   std::vector<std::vector<uint32_t>> pblocks;
-  for (int rpb = project_rows_per_block(k); rpb >= 16; rpb /= 2) {
+  for (int rpb = PROJECT_ROWS_MAX; rpb >= 8; rpb /= 2) {
     std::vector<uint32_t> v;
     for (int g : P->order)
       for (int b = 0; b * rpb < gn(g); ++b) v.push_back(((uint32_t)b << 12) | (uint32_t)g);

@@ -414,7 +414,7 @@ struct PGraph {
   double* part;   // ceil(n / 256) x k column partial sums
   int n, pad;
 };
-int project_rows_per_block(int k);
+constexpr int PROJECT_ROWS_MAX = 32;   // node rows per block, a multiple of its 8 warps
 // blocks: (b << 12) | g over ceil(n / rows_per_block); chunks: 256-row
 // chunks; elem: 256-element blocks of n x k.
 int project_grouped(cdl_ctx* ctx, const PGraph* gs, int G2, BTiles blocks, int rpb, int k, uint64_t seed,
