@@ -148,13 +148,18 @@ int cdl_ctx_set_debug(cdl_ctx* ctx, int flags);
  * A:  device, n x n float64 output. D: device, n float64 output.
  * vol, sigma_out: device, one float64 each (sigma_out receives the sigma used).
  * Squared distances are exact when every x is a multiple of 2^-16 below 2^7
- * in magnitude (int64 arithmetic); otherwise they are computed in float64
- * with one rounding per subtraction, product and sum, samples in order.
+ * in magnitude (int64 arithmetic). Otherwise, for T >= 16 each is the exact
+ * squared distance of the two series rounded to 2^-61 of their distances to
+ * node 0 (or to 2^-60 of the largest sample, if that is more), correctly
+ * rounded, where that leaves it within about 2^-53 relative; the others, and
+ * all for T < 16, are computed in float64 with one rounding per subtraction,
+ * product and sum, samples in order.
  * Requires 2 <= n <= 2^20, 1 <= T <= 4096. */
 int cdl_build_graph(cdl_ctx* ctx, const double* X, int64_t n, int32_t T, double sigma,
                     cdl_dtype a_dtype, void* A, double* D, double* vol, double* sigma_out);
 
-/* Same computation and results as cdl_build_graph (float64 A), for callers
+/* Same computation and results as cdl_build_graph (float64 A; for inputs off
+ * the 2^-16 grid and T >= 16 the two round distances differently), for callers
  * that cannot let a library allocate device memory: for example a process
  * whose device memory is all handed to its own pool allocator, where an
  * extra cudaMalloc would fail or fragment the pool, or a service that must

@@ -34,8 +34,6 @@
 namespace cdl {
 namespace {
 
-constexpr int CRT_ROW_NAN = 0x40000000;   // e_i of a row with a non-finite entry
-
 struct ResidueTab {
   uint32_t mod[CRT_MAX], magic[CRT_MAX], c1[CRT_MAX], c2[CRT_MAX], bias[CRT_MAX];
   float off[CRT_MAX];
@@ -59,22 +57,6 @@ constexpr ResidueTab make_residue_tab(int S) {
 __constant__ ResidueTab c_res64 = make_residue_tab(21);
 __constant__ ResidueTab c_res32 = make_residue_tab(16);
 
-// P / p_l in 20-bit limbs (16 moduli: below 2^118) and 2^23 / p_l
-struct CombineTab64 {
-  uint32_t limb[6][CRT_MAX];
-  uint32_t frac[CRT_MAX];
-};
-constexpr CombineTab64 make_combine64() {
-  CombineTab64 t{};
-  const u128 P = crt_product(16);
-  for (int l = 0; l < 16; ++l) {
-    const u128 m = P / (u128)CRT_MOD[l];
-    for (int k = 0; k < 6; ++k) t.limb[k][l] = (uint32_t)(m >> (20 * k)) & 0xFFFFFu;
-    t.frac[l] = (uint32_t)(((1u << 24) + (unsigned)CRT_MOD[l]) / (2u * (unsigned)CRT_MOD[l]));
-  }
-  return t;
-}
-__constant__ CombineTab64 c_comb64 = make_combine64();
 struct CombineTab32 {
   uint32_t lo[8], hi[8], frac[8];
 };
@@ -90,8 +72,6 @@ constexpr CombineTab32 make_combine32() {
   return t;
 }
 __constant__ CombineTab32 c_comb32 = make_combine32();
-constexpr unsigned long long P64_HI = (unsigned long long)(crt_product(16) >> 64),
-                             P64_LO = (unsigned long long)crt_product(16);
 constexpr unsigned long long P32 = (unsigned long long)crt_product(8);
 
 // The two types' bit patterns: magnitude bits, exponent field and mantissa
@@ -212,27 +192,6 @@ __global__ void __launch_bounds__(256) k_crt_residues(const T* __restrict__ X, i
   }
 }
 
-// v 2^-e rounded to nearest even, v a signed 128-bit integer
-__device__ __forceinline__ double i128_to_double(__int128 v, int e) {
-  if (v == 0) return 0.0;
-  const bool neg = v < 0;
-  const u128 a = neg ? (u128)(-v) : (u128)v;
-  const unsigned long long hi = (unsigned long long)(a >> 64), lo = (unsigned long long)a;
-  const int z = hi ? __clzll((long long)hi) : 64 + __clzll((long long)lo);
-  const u128 n = a << z;                                  // leading bit 127
-  const unsigned long long top = (unsigned long long)(n >> 64);
-  const bool sticky = (unsigned long long)n != 0;
-  unsigned long long q = top >> 11;
-  const unsigned long long rem = top & 0x7FFull;
-  if (rem > 0x400ull || (rem == 0x400ull && (sticky || (q & 1)))) ++q;   // may carry to 2^53: exact below
-  const int ex = 127 - z - 52 - e;                        // value q 2^ex
-  const unsigned long long sign = neg ? 1ull << 63 : 0ull;
-  const int field = ex + 52 + 1023;
-  if (field > 0 && field < 2046)                          // q in [2^52, 2^53]: adding carries into the exponent
-    return __longlong_as_double((long long)(sign | (((unsigned long long)(field - 1) << 52) + q)));
-  return ldexp(neg ? -(double)q : (double)q, ex);         // subnormal or out of range
-}
-
 template <typename T>
 struct Combine;
 template <>
@@ -240,19 +199,7 @@ struct Combine<double> {
   static constexpr int NP = 16;
   // c from the bytes at bit `sh` of the 16 words
   static __device__ __forceinline__ double value(const uint32_t (&w)[16], int sh, int e) {
-    uint32_t S[6] = {0, 0, 0, 0, 0, 0}, f = 0;
-#pragma unroll
-    for (int l = 0; l < 16; ++l) {
-      const uint32_t t = (w[l] >> sh) & 0xFFu;
-#pragma unroll
-      for (int k = 0; k < 6; ++k) S[k] += t * c_comb64.limb[k][l];   // 16 terms below 2^28
-      f += t * c_comb64.frac[l];
-    }
-    const uint32_t q = (f + (1u << 22)) >> 23;            // round(sum t_l / p_l): |c| <= P / 4 leaves no doubt
-    u128 c = (u128)S[0] + ((u128)S[1] << 20) + ((u128)S[2] << 40) + ((u128)S[3] << 60) + ((u128)S[4] << 80) +
-             ((u128)S[5] << 100);
-    c -= (u128)q * (((u128)P64_HI << 64) | P64_LO);       // modulo 2^128: |c| < 2^124
-    return i128_to_double((__int128)c, e);
+    return i128_to_double(crt16_value(w, sh), e);
   }
   static __device__ __forceinline__ double nan() { return __longlong_as_double(0x7FF8000000000000ll); }
 };
@@ -315,6 +262,105 @@ __global__ void __launch_bounds__(256) k_crt_combine(const uint8_t* __restrict__
   if (bi == bj) return;
   __syncthreads();
   for (int e = threadIdx.x; e < 64 * 64; e += 256) C[(size_t)(c0 + e / 64) * np + r0 + e % 64] = tile[e / 64][e % 64];
+}
+
+// Node series for the residue distances (k_tc_distr): row i less the series of
+// node 0 (distances do not change, and the common part of all nodes costs no
+// bits), scaled by the power of two 2^{e_i} that brings its 2-norm to 2^61.65
+// at most and keeps both series below 2^61, rounded to integers (each entry
+// within one unit), as 16 residue planes (rows x kp, zero padded), with its
+// exact squared norm. One block of 128 threads per row; also clears the tile
+// flags. Series of fewer than DIST_RES_MIN_T samples flag every tile instead:
+// they stay with the float64 kernel. Nothing on the grid inputs of
+// the other kernel.
+__global__ void __launch_bounds__(128) k_series_residues(const double* __restrict__ X, int n, int T, int rows, int kp,
+                                                          const int* __restrict__ offgrid, int* __restrict__ ex,
+                                                          ulonglong2* __restrict__ norms,
+                                                          uint32_t* __restrict__ planes, uint32_t* __restrict__ bad,
+                                                          int bad_words) {
+  if (!(*offgrid & 1)) return;
+  typedef LevelType<double> LT;
+  __shared__ unsigned long long wmax[2][4];
+  __shared__ float wsum[4];
+  __shared__ ulonglong2 wn[4];
+  const int row = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t flags = T < DIST_RES_MIN_T ? 0x01010101u : 0u;
+  for (int w = row * 128 + tid; w < bad_words; w += gridDim.x * 128) bad[w] = flags;
+  if (flags) return;
+  const bool real = row < n;
+  const double* x = X + (size_t)(real ? row : 0) * T;
+  unsigned long long mx = 0, md = 0;
+  for (int t = tid; t < T; t += 128) {
+    mx = max(mx, max(LT::mag(x[t]), LT::mag(X[t])));
+    md = max(md, LT::mag(__dsub_rn(x[t], X[t])));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    md = max(md, __shfl_xor_sync(0xffffffffu, md, o));
+  }
+  if (lane == 0) {
+    wmax[0][warp] = mx;
+    wmax[1][warp] = md;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < 4; ++w) {
+    mx = max(mx, wmax[0][w]);
+    md = max(md, wmax[1][w]);
+  }
+  const bool fin = LT::finite(mx) && LT::finite(md);
+  const int emax = LT::exponent(md) - LT::BIAS + 52;
+  float s = 0.f;
+  if (fin)
+    for (int t = tid; t < T; t += 128) {
+      const float v = (float)(int)scaled_int(__dsub_rn(x[t], X[t]), 22 - emax);
+      s = __fmaf_rn(v, v, s);
+    }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) wsum[warp] = s;
+  __syncthreads();
+  s = wsum[0] + wsum[1] + wsum[2] + wsum[3];
+  const bool any = real && fin && s >= 1.f;
+  int e = CRT_ROW_ZERO;
+  if (any) {
+    e = (int)floorf(crt_norm_bits(16) - 0.02f - 0.5f * log2f(s)) + 22 - emax;
+    e = min(e, 60 - (LT::exponent(mx) - LT::BIAS + 52));
+  }
+  if (tid == 0) ex[row] = fin ? e : CRT_ROW_NAN;
+  const size_t plane = (size_t)rows * kp / 2;
+  uint32_t* out = planes + (size_t)row * kp / 2;
+  u128 nn = 0;
+  for (int j = tid; j < kp / 2; j += 128) {
+    int u[2][3];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int t = 2 * j + h;
+      const long long v = any && t < T ? scaled_int(x[t], e) - scaled_int(X[t], e) : 0;
+      nn += (u128)((__int128)v * v);
+      u[h][0] = (int)(v & 0x1FFFFF);
+      u[h][1] = (int)(v >> 21) & 0x1FFFFF;
+      u[h][2] = (int)(v >> 42);
+    }
+#pragma unroll
+    for (int l = 0; l < 16; ++l)
+      out[l * plane + j] = __byte_perm(residue_bits<double>(u[0][0], u[0][1], u[0][2], l),
+                                       residue_bits<double>(u[1][0], u[1][1], u[1][2], l), 0x7632);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long lo = __shfl_xor_sync(0xffffffffu, (unsigned long long)nn, o);
+    const unsigned long long hi = __shfl_xor_sync(0xffffffffu, (unsigned long long)(nn >> 64), o);
+    nn += ((u128)hi << 64) | lo;
+  }
+  if (lane == 0) wn[warp] = make_ulonglong2((unsigned long long)nn, (unsigned long long)(nn >> 64));
+  __syncthreads();
+  if (tid == 0) {
+    nn = 0;
+    for (int w = 0; w < 4; ++w) nn += ((u128)wn[w].y << 64) | wn[w].x;
+    norms[row] = make_ulonglong2((unsigned long long)nn, (unsigned long long)(nn >> 64));
+  }
 }
 
 // X (rows x cols, leading dimension ldx) transposed to out (gridDim.y 32 rows x
@@ -490,6 +536,15 @@ int crt_apply_residual(cdl_ctx* ctx, const CrtApply& a, const double* Y, const d
                        double* R, double* part, int nblocks) {
   Launch L(ctx, CDL_KC_RESIDUAL, 0);
   k_crt_residual<<<nblocks, 128, 0, ctx->stream>>>(a.t, a.np, a.kpb, a.erow, a.ecol, Y, Z, D, n, k, R, part);
+  return L.done();
+}
+
+int series_residues(cdl_ctx* ctx, const double* X, int n, int T, int rows, int kp, const int* offgrid, int* ex,
+                    void* norms, void* planes, void* bad, int bad_words) {
+  Launch L(ctx, CDL_KC_DISTANCE, 0);
+  k_series_residues<<<rows, 128, 0, ctx->stream>>>(X, n, T, rows, kp, offgrid, ex, static_cast<ulonglong2*>(norms),
+                                                   static_cast<uint32_t*>(planes), static_cast<uint32_t*>(bad),
+                                                   bad_words);
   return L.done();
 }
 

@@ -60,47 +60,50 @@ __global__ void k_to_fixed(const double* __restrict__ X, int* __restrict__ Xt, i
   if (__syncthreads_or(off) && threadIdx.x == 0) atomicOr(&st->flags, 1);
 }
 
-// Three signed base-256 digit planes of a = x 2^16 for the tensor-core
-// distances (rows x tp bf16 each, zero padded): a = d0 + 2^8 d1 + 2^16 d2 with
-// |d| <= 128, exact in bf16. Inputs off the grid give zeros (the float64
-// kernel handles them).
-__global__ void __launch_bounds__(256) k_slice_x(const double* __restrict__ X, int n, int T, int rows, int tp,
-                                                  __nv_bfloat16* __restrict__ planes) {
-  const size_t plane = (size_t)rows * tp;
-  for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < plane; idx += (size_t)gridDim.x * blockDim.x) {
-    const int i = (int)(idx / tp), t = (int)(idx % tp);
-    int a = 0;
-    if (i < n && t < T) {
-      const double v = X[(size_t)i * T + t] * 65536.0;
-      if (v == rint(v) && fabs(v) < 8388608.0) a = (int)v;
-    }
-    const int d0 = ((a + 128) & 255) - 128;
-    const int a1 = (a - d0) >> 8;                         // exact: a - d0 is a multiple of 256
-    const int d1 = ((a1 + 128) & 255) - 128;
-    const int d2 = (a1 - d1) >> 8;
-    planes[idx] = __int2bfloat16_rn(d0);
-    planes[plane + idx] = __int2bfloat16_rn(d1);
-    planes[2 * plane + idx] = __int2bfloat16_rn(d2);
-  }
-}
-
-// |a_i|^2 = sum_t a_it^2 in int64 (exact), one warp per row; padded rows 0.
-__global__ void __launch_bounds__(256) k_row_norms(const double* __restrict__ X, int n, int T, int rows,
-                                                    long long* __restrict__ norms) {
+// For the tensor-core distances, one warp per row and one pass over X: three
+// signed base-256 digit planes of a = x 2^16 (rows x tp bf16 each, zero padded: a
+// = d0 + 2^8 d1 + 2^16 d2 with |d| <= 128, exact in bf16), |a_i|^2 = sum_t a_it^2 in
+// int64 (exact), and the flag of input off the grid (whose digits are zero:
+// other kernels handle it). Bound by memory: 8 bytes read and 6 written per
+// sample; three kernels with a pass each (one an int32 copy that nothing
+// read) took 238 us at n = 20011, T = 365.
+__global__ void __launch_bounds__(256) k_prepare_series(const double* __restrict__ X, int n, int T, int rows, int tp,
+                                                         __nv_bfloat162* __restrict__ planes,
+                                                         long long* __restrict__ norms, SelectState* st) {
   const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (row >= rows) return;
+  const size_t plane = (size_t)rows * tp / 2;
+  const double* x = X + (size_t)min(row, n - 1) * T;
   long long acc = 0;
-  if (row < n)
-    for (int t = lane; t < T; t += 32) {
-      const double v = X[(size_t)row * T + t] * 65536.0;
-      const long long a = (v == rint(v) && fabs(v) < 8388608.0) ? (long long)v : 0;
-      acc += a * a;
+  bool off = false;
+  for (int t2 = lane; t2 < tp / 2; t2 += 32) {
+    int d[3][2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int t = 2 * t2 + h;
+      int a = 0;
+      if (row < n && t < T) {
+        const double v = x[t] * 65536.0;                    // exact scaling by a power of two
+        if (v == rint(v) && fabs(v) < 8388608.0)
+          a = (int)v;
+        else
+          off = true;
+      }
+      acc += (long long)a * a;
+      d[0][h] = ((a + 128) & 255) - 128;
+      const int a1 = (a - d[0][h]) >> 8;                    // exact: a - d0 is a multiple of 256
+      d[1][h] = ((a1 + 128) & 255) - 128;
+      d[2][h] = (a1 - d[1][h]) >> 8;
     }
+    const size_t o = (size_t)row * tp / 2 + t2;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) planes[q * plane + o] = __floats2bfloat162_rn((float)d[q][0], (float)d[q][1]);
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if (lane == 0) norms[row] = acc;
+  if (__any_sync(0xffffffffu, off) && lane == 0) atomicOr(&st->flags, 1);
 }
-
 
 // Exact squared distances on the 2^-16 grid: int64 sums of squared int32
 // differences, written as float64 multiples of 2^-32 to both (i,j) and (j,i).
@@ -212,13 +215,21 @@ __device__ __forceinline__ void dist_f64_tile(const double* __restrict__ X, int 
   }
 }
 
+// `bad` (may be null: every tile): only the 64 x 64 tiles that dist_residues_tc flagged.
 __global__ void __launch_bounds__(256) k_dist_f64(const double* __restrict__ X, int n, int T,
-                                                   double* __restrict__ A, const SelectState* st) {
+                                                   double* __restrict__ A, const SelectState* st,
+                                                   const unsigned char* __restrict__ bad, int bad_stride) {
   if (!(st->flags & 1)) return;
+  __shared__ int tile[2];
   const int nb = (n + DT - 1) / DT;
-  int bi, bj;
-  block_tri_index(nb, bi, bj);
-  dist_f64_tile(X, n, T, A, bi, bj);
+  const long long tiles = (long long)nb * (nb + 1) / 2;
+  for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
+    if (threadIdx.x == 0) tri_index(t, nb, tile[0], tile[1]);
+    __syncthreads();
+    const int bi = tile[0], bj = tile[1];
+    if (!bad || bad[(size_t)bi * bad_stride + bj]) dist_f64_tile(X, n, T, A, bi, bj);
+    __syncthreads();
+  }
 }
 
 __global__ void k_select_init(SelectState* st, long long rank) {
@@ -731,8 +742,7 @@ int graph_build(cdl_ctx* ctx, const double* X, int64_t n64, int T, double sigma,
                 double* D, double* vol, double* sigma_out, int kernel, unsigned long long* amax_bits) {
   const int n = (int)n64;
   cudaStream_t s = ctx->stream;
-  void *wsXi, *wsSt, *wsHist;
-  CDL_TRY(ws_get(ctx, "graph.Xi", (size_t)n * T * sizeof(int), &wsXi));
+  void *wsSt, *wsHist;
   CDL_TRY(ws_get(ctx, "graph.state", sizeof(SelectState), &wsSt));
   CDL_TRY(ws_get(ctx, "graph.hist", RADIX_BINS * sizeof(unsigned long long), &wsHist));
   SelectState* st = static_cast<SelectState*>(wsSt);
@@ -744,13 +754,6 @@ int graph_build(cdl_ctx* ctx, const double* X, int64_t n64, int T, double sigma,
     CDL_TRY(L.done());
   }
   CDL_CUDA_TRY(cudaMemsetAsync(hist, 0, RADIX_BINS * sizeof(unsigned long long), s));
-  {
-    size_t total = (size_t)n * T;
-    int blocks = (int)std::min<size_t>((total + 255) / 256, (size_t)ctx->sm_count * 8);
-    Launch L(ctx, CDL_KC_DISTANCE, 0);
-    k_to_fixed<<<blocks, 256, 0, s>>>(X, static_cast<int*>(wsXi), n, T, st);
-    CDL_TRY(L.done());
-  }
   const int nb = (n + DT - 1) / DT;
   const long long tiles = (long long)nb * (nb + 1) / 2;
   if (tiles > 0x7fffffffLL) return CDL_ERR_INVALID_ARG;
@@ -762,22 +765,32 @@ int graph_build(cdl_ctx* ctx, const double* X, int64_t n64, int T, double sigma,
     CDL_TRY(ws_get(ctx, "graph.norms", (size_t)rows * sizeof(long long), &wsNo));
     {
       Launch L(ctx, CDL_KC_DISTANCE, 0);
-      const size_t cnt = (size_t)rows * tp;
-      k_slice_x<<<(unsigned)std::min<size_t>((cnt + 255) / 256, (size_t)ctx->sm_count * 8), 256, 0, s>>>(
-          X, n, T, rows, tp, static_cast<__nv_bfloat16*>(wsPl));
-      CDL_TRY(L.done());
-    }
-    {
-      Launch L(ctx, CDL_KC_DISTANCE, 0);
-      k_row_norms<<<rows / 8, 256, 0, s>>>(X, n, T, rows, static_cast<long long*>(wsNo));
+      k_prepare_series<<<rows / 8, 256, 0, s>>>(X, n, T, rows, tp, static_cast<__nv_bfloat162*>(wsPl),
+                                                static_cast<long long*>(wsNo), st);
       CDL_TRY(L.done());
     }
     CDL_TRY(dist_tc(ctx, wsPl, static_cast<const long long*>(wsNo), n, rows, tp, A, &st->flags,
                     0.5 * (double)n * (double)(n - 1) * T));
   }
+  // off the grid: through residues on the tensor cores, and what that leaves over in float64
+  const unsigned char* bad = nullptr;
+  const int rows = (n + 127) / 128 * 128, kp = (T + 63) / 64 * 64, nb64 = rows / 64;
+  const size_t bad_bytes = ((size_t)nb64 * nb64 + 3) / 4 * 4;
+  void *wsRp, *wsRn, *wsRe, *wsBad;
+  if (ws_get(ctx, "crt.dist.planes", T < DIST_RES_MIN_T ? 0 : (size_t)16 * rows * kp * 2, &wsRp) == CDL_OK &&
+      ws_get(ctx, "crt.dist.norms", (size_t)rows * 16, &wsRn) == CDL_OK &&
+      ws_get(ctx, "crt.dist.e", (size_t)rows * sizeof(int), &wsRe) == CDL_OK &&
+      ws_get(ctx, "crt.dist.bad", bad_bytes, &wsBad) == CDL_OK) {
+    CDL_TRY(series_residues(ctx, X, n, T, rows, kp, &st->flags, static_cast<int*>(wsRe), wsRn, wsRp, wsBad,
+                            (int)(bad_bytes / 4)));
+    CDL_TRY(dist_residues_tc(ctx, wsRp, static_cast<const int*>(wsRe), wsRn, n, T, rows, kp, A, &st->flags, wsBad));
+    bad = static_cast<const unsigned char*>(wsBad);
+  } else {
+    ws_reclaim(ctx);
+  }
   {
     Launch L(ctx, CDL_KC_DISTANCE, 0);
-    k_dist_f64<<<(unsigned)tiles, 256, 0, s>>>(X, n, T, A, st);
+    k_dist_f64<<<(unsigned)std::min<long long>(tiles, ctx->sm_count * 6), 256, 0, s>>>(X, n, T, A, st, bad, nb64);
     CDL_TRY(L.done());
   }
   if (sigma > 0) {
@@ -856,8 +869,7 @@ int graph_regen_init(cdl_ctx* ctx, RegenGraph& g, const double* X, int64_t n64, 
   g.rows = (n + 127) / 128 * 128;
   g.tp = (T + 63) / 64 * 64;
   const std::string tag = "regen." + std::to_string(g.id) + ".";
-  void *wsXi, *wsSt, *wsHist, *wsPl, *wsNo, *wsSc;
-  CDL_TRY(ws_get(ctx, (tag + "Xi").c_str(), (size_t)n * T * sizeof(int), &wsXi));
+  void *wsSt, *wsHist, *wsPl, *wsNo, *wsSc;
   CDL_TRY(ws_get(ctx, (tag + "state").c_str(), sizeof(SelectState), &wsSt));
   CDL_TRY(ws_get(ctx, (tag + "hist").c_str(), RADIX_BINS * sizeof(unsigned long long), &wsHist));
   CDL_TRY(ws_get(ctx, (tag + "planes").c_str(), 3 * (size_t)g.rows * g.tp * 2, &wsPl));
@@ -877,22 +889,9 @@ int graph_regen_init(cdl_ctx* ctx, RegenGraph& g, const double* X, int64_t n64, 
   }
   CDL_CUDA_TRY(cudaMemsetAsync(hist, 0, RADIX_BINS * sizeof(unsigned long long), s));
   {
-    const size_t total = (size_t)n * T;
     Launch L(ctx, CDL_KC_DISTANCE, 0);
-    k_to_fixed<<<(int)std::min<size_t>((total + 255) / 256, (size_t)ctx->sm_count * 8), 256, 0, s>>>(
-        X, static_cast<int*>(wsXi), n, T, st);
-    CDL_TRY(L.done());
-  }
-  {
-    Launch L(ctx, CDL_KC_DISTANCE, 0);
-    const size_t cnt = (size_t)g.rows * g.tp;
-    k_slice_x<<<(unsigned)std::min<size_t>((cnt + 255) / 256, (size_t)ctx->sm_count * 8), 256, 0, s>>>(
-        X, n, T, g.rows, g.tp, static_cast<__nv_bfloat16*>(wsPl));
-    CDL_TRY(L.done());
-  }
-  {
-    Launch L(ctx, CDL_KC_DISTANCE, 0);
-    k_row_norms<<<g.rows / 8, 256, 0, s>>>(X, n, T, g.rows, static_cast<long long*>(wsNo));
+    k_prepare_series<<<g.rows / 8, 256, 0, s>>>(X, n, T, g.rows, g.tp, static_cast<__nv_bfloat162*>(wsPl),
+                                                static_cast<long long*>(wsNo), st);
     CDL_TRY(L.done());
   }
   int flags = 0;
@@ -1197,7 +1196,7 @@ int graph_build_static(const double* X, int64_t n64, int T, double sigma, double
   const long long tiles = (long long)nb * (nb + 1) / 2;
   k_dist_int<<<(unsigned)tiles, 256, 0, s>>>(Xt, n, T, A, st);
   CDL_TRY(launched());
-  k_dist_f64<<<(unsigned)tiles, 256, 0, s>>>(X, n, T, A, st);
+  k_dist_f64<<<(unsigned)std::min<long long>(tiles, sm_count * 6), 256, 0, s>>>(X, n, T, A, st, nullptr, 0);
   CDL_TRY(launched());
   if (sigma > 0) {
     k_set_scalar<<<1, 1, 0, s>>>(sigma_out, sigma);

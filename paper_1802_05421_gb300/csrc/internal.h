@@ -290,6 +290,21 @@ int resid_tc_grouped(cdl_ctx* ctx, const ResidGroup* dgroups, const uint32_t* un
 // recorded for the launch.
 int dist_tc(cdl_ctx* ctx, const void* planes, const long long* norms, int n, int rows, int tp, double* A,
             const int* offgrid, double terms);
+// Squared distances of off-grid inputs (*offgrid & 1; nothing otherwise)
+// through residues: series_residues forms 16 planes (rows x kp bf16), the row
+// exponents and the exact squared norms (16 bytes each) and clears the flags of
+// the 64 x 64 blocks; dist_residues_tc writes A and flags the blocks (byte bi
+// nb64 + bj, bi <= bj, nb64 = rows / 64) that the float64 kernel must form.
+// Series of fewer samples stay with the float64 kernel (whole builds at n =
+// 8192: T = 2 1.27 ms, T = 4 1.61, T = 8 2.37, T = 15 3.75; with residues 1.70
+// up to T = 64): the lines cross near T = 5, and up to 15 samples the bits of
+// the allocation-free and batched builds, which have only that kernel, are
+// worth more than the difference.
+constexpr int DIST_RES_MIN_T = 16;
+int series_residues(cdl_ctx* ctx, const double* X, int n, int T, int rows, int kp, const int* offgrid, int* ex,
+                    void* norms, void* planes, void* bad, int bad_words);
+int dist_residues_tc(cdl_ctx* ctx, const void* planes, const int* ex, const void* norms, int n, int T, int rows, int kp,
+                     double* A, const int* offgrid, void* bad);
 // Pair partials of the CAD scores with the Gram on the tensor cores: uplanes,
 // vplanes = six bf16 slice planes each (rows x k2p, zero padded) of u / c and
 // v / c; dint = d_i in units of c^2 2^-48; oscale = c^2 2^-48 (device);

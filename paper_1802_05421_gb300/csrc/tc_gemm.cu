@@ -904,6 +904,14 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
   }
 }
 
+// ---------------------------------------------------------------- sums of residue products
+constexpr int CR_CHUNK_KB = 16;                        // 1024 of K per exact chunk
+constexpr int CR_MAX_KBLOCKS = 62 * CR_CHUNK_KB;       // int32 sums and the modular reduction: |sum| <= 62 2^24
+
+__device__ __forceinline__ uint32_t crt_mod31(uint32_t x, uint32_t p, uint32_t magic) {   // x mod p, x < 2^31
+  return x - (__umulhi(x, magic) >> 7) * p;
+}
+
 // ---------------------------------------------------------------- exact squared distances
 // d2_ij = |a_i|^2 + |a_j|^2 - 2 a_i . a_j for node series on the 2^-16 grid
 // (a = x 2^16, integers below 2^23 in magnitude). Each a is written as three
@@ -1172,6 +1180,262 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
   if (warp == 0) {
     __syncwarp();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(DS_TMEM_COLS)
+                 : "memory");
+  }
+}
+
+// ---------------------------------------------------------------- distances of series on no grid
+// d2_ij of float64 series off the 2^-16 grid, through residues (crt.cuh): row i
+// of the series less the series of node 0 is 2^-e_i times integers x'_i of norm
+// 2^61.65 at most, rounded to one unit (k_series_residues); the Gram entry x'_i .
+// x'_j is formed exactly from 16 residue products on the bf16 tensor cores, and
+// d2' = |x'_i|^2 + |x'_j|^2 - 2 x'_i . x'_j in 128-bit integers, in units of the
+// coarser of the two rows, rounded once to float64. With d2' >= 2^109 the
+// rounding of the series is below 2^-54 of d2 (rms 0.6 units per sample and
+// pair, so 1.2 / sqrt(d2') relative), where a float64 sum of rounded squares
+// has about sqrt(T) 2^-54: tiles with a smaller entry (a distance below 2^-7
+// of the nodes' distances to node 0, duplicates, non-finite series) are
+// flagged and formed by the float64 kernel, as before.
+//
+// 128 x 64 tiles of the upper block triangle, warp roles as in k_tc_dist. Planes
+// run one after the other through a ring of eight 64-column accumulators (at
+// most 1024 samples each: exact); an epilogue thread reduces its 16 columns of
+// one row modulo p_l into bytes kept in shared memory, and after the last
+// plane puts its entries together four columns at a time. Bound by the
+// epilogue's integer arithmetic (about 11 operations per entry and plane to
+// reduce, 10 to combine). n = 8192, T = 128: 0.97 ms, and 0.03 for the series'
+// residues, where the float64 pipe took 24.9 ms.
+constexpr int DR_STAGES = 3;
+constexpr int DR_STAGE_BYTES = DS_A + DS_B;
+constexpr int DR_WORDS = 16 * 4 * 32;                  // per epilogue warp: 16 columns of 32 rows, 16 planes
+constexpr int DR_SMEM_BYTES = DR_STAGES * DR_STAGE_BYTES + 512 + 16 * DR_WORDS * 4 + 1024;
+constexpr int DR_NBUF = 8;
+
+struct DistResParams {
+  int nb128, nb64, num_tiles;
+  int rows;                   // of one plane
+  int kblocks;                // 0: nothing to do (every tile is flagged)
+  int n;
+  const int* ex;
+  const ulonglong2* norms;
+  double* A;
+  const int* offgrid;
+  unsigned char* bad;         // per 64 x 64 block (bi, bj), bi <= bj: at bi nb64 + bj
+  uint32_t idesc;
+  unsigned* status;
+  uint32_t mod[CRT_MAX], magic[CRT_MAX], inv[CRT_MAX], bias[CRT_MAX];
+};
+
+__global__ void __launch_bounds__(T8_THREADS, 1)
+    k_tc_distr(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+               const DistResParams p) {
+  if (!(*p.offgrid & 1) || p.kblocks == 0) return;       // uniform: before any barrier or allocation
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + DR_STAGES * DR_STAGE_BYTES);
+  uint32_t* words = reinterpret_cast<uint32_t*>(smem + DR_STAGES * DR_STAGE_BYTES + 512);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * DR_STAGES + 2 * DR_NBUF + 2);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 2 * DR_STAGES + 2 * DR_NBUF + 3);
+  const uint32_t bar0 = smem_u32(bars);
+  auto full_bar = [&](int s) { return bar0 + 8u * s; };
+  auto empty_bar = [&](int s) { return bar0 + 8u * (DR_STAGES + s); };
+  auto pfull_bar = [&](int b) { return bar0 + 8u * (2 * DR_STAGES + b); };
+  auto pempty_bar = [&](int b) { return bar0 + 8u * (2 * DR_STAGES + DR_NBUF + b); };
+  const uint32_t drain_bar = bar0 + 8u * (2 * DR_STAGES + 2 * DR_NBUF);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nchunks = (p.kblocks + CR_CHUNK_KB - 1) / CR_CHUNK_KB;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < DR_STAGES; ++s) {
+      mbar_init(full_bar(s), 1);
+      mbar_init(empty_bar(s), 1);
+    }
+    for (int b = 0; b < DR_NBUF; ++b) {
+      mbar_init(pfull_bar(b), 1);
+      mbar_init(pempty_bar(b), T8_EPI);
+    }
+    mbar_init(drain_bar, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"(DR_NBUF * DS_N)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+
+  if (warp == 0 && lane == 0) {
+    // ------------------------------------------------ TMA producer
+    int it = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < p.num_tiles && ok; t += gridDim.x) {
+      int I, J;
+      dist_tile(t, p.nb128, p.nb64, I, J);
+      for (int l = 0; l < 16 && ok; ++l)
+        for (int kb = 0; kb < p.kblocks; ++kb, ++it) {
+          const int s = it % DR_STAGES;
+          if (!mbar_wait(empty_bar(s), ((uint32_t)(it / DR_STAGES) & 1) ^ 1, abort_flag, p.status)) {
+            ok = false;
+            break;
+          }
+          const uint32_t dst = smem_u32(smem + s * DR_STAGE_BYTES);
+          mbar_expect_tx(full_bar(s), DR_STAGE_BYTES);
+          tma_load_2d(dst, &tmA, kb * 64, l * p.rows + I * 128, full_bar(s));
+          tma_load_2d(dst + DS_A, &tmB, kb * 64, l * p.rows + J * DS_N, full_bar(s));
+        }
+    }
+    if (!ok) {
+      for (int j = (it > DR_STAGES ? it - DR_STAGES : 0); j < it; ++j) {
+        const unsigned long long t0 = globaltimer();
+        while (!mbar_try_wait(full_bar(j % DR_STAGES), (uint32_t)(j / DR_STAGES) & 1) &&
+               globaltimer() - t0 < WAIT_LIMIT_NS) {
+        }
+      }
+    }
+  } else if (warp == 1 && lane == 0) {
+    // ------------------------------------------------ MMA issuer: one accumulator per plane and chunk
+    int it = 0, pc = 0;
+    bool ok = true, issued = false;
+    for (int t = blockIdx.x; t < p.num_tiles && ok; t += gridDim.x)
+      for (int l = 0; l < 16 && ok; ++l)
+        for (int kb = 0; kb < p.kblocks; ++kb, ++it) {
+          const int b = pc % DR_NBUF;
+          if (kb % CR_CHUNK_KB == 0) {
+            if (!mbar_wait(pempty_bar(b), ((uint32_t)(pc / DR_NBUF) & 1) ^ 1, abort_flag, p.status)) {
+              ok = false;
+              break;
+            }
+          }
+          const int s = it % DR_STAGES;
+          if (!mbar_wait(full_bar(s), (uint32_t)(it / DR_STAGES) & 1, abort_flag, p.status)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t base = smem_u32(smem + s * DR_STAGE_BYTES);
+          const uint64_t adesc = smem_desc(base), bdesc = smem_desc(base + DS_A);
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk)
+            mma_bf16(tmem_base + (uint32_t)(b * DS_N), adesc + (uint64_t)(kk * 2), bdesc + (uint64_t)(kk * 2), p.idesc,
+                     ((kb % CR_CHUNK_KB) | kk) != 0);
+          issued = true;
+          mma_commit(empty_bar(s));
+          if (kb % CR_CHUNK_KB == CR_CHUNK_KB - 1 || kb == p.kblocks - 1) {
+            mma_commit(pfull_bar(b));
+            ++pc;
+          }
+        }
+    if (!ok && issued) {
+      mma_commit(drain_bar);
+      const unsigned long long t0 = globaltimer();
+      while (!mbar_try_wait(drain_bar, 0) && globaltimer() - t0 < WAIT_LIMIT_NS) {
+      }
+    }
+  } else if (warp >= 2) {
+    // ------------------------------------------------ epilogue
+    const int q = warp & 3;                              // TMEM lane quarter
+    const int part = (warp - 2) >> 2;                    // 16-column part of the tile
+    const uint32_t lane_off = (uint32_t)(q * 32) << 16;
+    uint32_t* tw = words + (warp - 2) * DR_WORDS;        // [quad of columns][plane][lane]
+    int pc = 0;
+    bool failed = false;
+    for (int t = blockIdx.x; t < p.num_tiles; t += gridDim.x) {
+      int I, J;
+      dist_tile(t, p.nb128, p.nb64, I, J);
+      for (int l = 0; l < 16; ++l) {
+        int sum[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) sum[e] = 0;
+        for (int c = 0; c < nchunks; ++c, ++pc) {
+          if (failed) continue;
+          const int b = pc % DR_NBUF;
+          if (!mbar_wait(pfull_bar(b), (uint32_t)(pc / DR_NBUF) & 1, abort_flag, p.status)) {
+            failed = true;
+            continue;
+          }
+          tc_fence_after();
+          float v[16];
+          tmem_ld16(tmem_base + lane_off + (uint32_t)(b * DS_N + part * 16), v);
+          tc_fence_before();
+          mbar_arrive(pempty_bar(b));
+#pragma unroll
+          for (int e = 0; e < 16; ++e) sum[e] += __float2int_rn(v[e]);
+        }
+        const uint32_t mod = p.mod[l], magic = p.magic[l], inv = p.inv[l], bias = p.bias[l];
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+          uint32_t b4 = 0;
+#pragma unroll
+          for (int h = 0; h < 4; ++h)
+            b4 |= crt_mod31(crt_mod31((uint32_t)sum[4 * w + h] + bias, mod, magic) * inv, mod, magic) << (8 * h);
+          tw[(w * 16 + l) * 32 + lane] = b4;
+        }
+      }
+      if (__any_sync(0xffffffffu, failed)) continue;
+      const int row = I * 128 + q * 32 + lane, col0 = J * DS_N + part * 16;
+      const bool rowok = row < p.n, mirror = J >= 2 * I + 2;
+      const int er = p.ex[row];
+      const ulonglong2 nr2 = p.norms[row];
+      const u128 nr = ((u128)nr2.y << 64) | nr2.x;
+      bool low = false;
+#pragma unroll 1
+      for (int w = 0; w < 4; ++w) {
+        uint32_t tv[16];
+#pragma unroll
+        for (int l = 0; l < 16; ++l) tv[l] = tw[(w * 16 + l) * 32 + lane];
+        double* res = reinterpret_cast<double*>(tw + w * 512);   // the quad's words are read: 4 columns x 32 rows
+        __syncwarp();
+#pragma unroll 1
+        for (int h = 0; h < 4; ++h) {
+          const int col = col0 + 4 * w + h;
+          double d2 = 0.0;
+          if (rowok && col < p.n && row != col) {
+            const int ec = p.ex[col];
+            const ulonglong2 nc2 = p.norms[col];
+            u128 a = nr, c = ((u128)nc2.y << 64) | nc2.x;
+            __int128 g2 = crt16_value(tv, 8 * h) * 2;
+            const int d = er - ec, ad = min(d < 0 ? -d : d, 127);   // to the coarser row's units
+            if (d > 0)
+              a = 2 * ad > 127 ? 0 : a >> (2 * ad);
+            else
+              c = 2 * ad > 127 ? 0 : c >> (2 * ad);
+            g2 >>= ad;
+            const __int128 v = (__int128)(a + c) - g2;
+            if (er == CRT_ROW_NAN || ec == CRT_ROW_NAN || v < ((__int128)1 << 109))
+              low = true;
+            else
+              d2 = i128_to_double(v, 2 * min(er, ec));
+            if (mirror) p.A[(size_t)col * p.n + row] = d2;   // lanes write 32 consecutive entries
+          }
+          res[h * 32 + lane] = d2;
+        }
+      }
+      const int bi = 2 * I + (q >> 1);                   // 64-row block of this warp
+      if (__any_sync(0xffffffffu, low) && lane == 0) p.bad[(size_t)min(bi, J) * p.nb64 + max(bi, J)] = 1;
+      __syncwarp();
+      // the warp's 32 x 16 block row-wise, two 128-byte row segments per store
+#pragma unroll 4
+      for (int it = 0; it < 16; ++it) {
+        const int rr = 2 * it + (lane >> 4), c = lane & 15;
+        const int grow = I * 128 + q * 32 + rr, gcol = col0 + c;
+        if (grow < p.n && gcol < p.n)
+          p.A[(size_t)grow * p.n + gcol] = reinterpret_cast<const double*>(tw + (c >> 2) * 512)[(c & 3) * 32 + rr];
+      }
+      __syncwarp();
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 0) {
+    __syncwarp();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(DR_NBUF * DS_N)
                  : "memory");
   }
 }
@@ -1914,9 +2178,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(S2_THREADS, 1)
 // against about 600 of draining), by the reduction and the stores for K of a
 // few hundred. Planes are numbered outermost, so one plane's panels stay in
 // L2 while its blocks are formed.
-constexpr int CR_CHUNK_KB = 16;                        // 1024 of K per exact chunk
-constexpr int CR_MAX_KBLOCKS = 62 * CR_CHUNK_KB;       // int32 sums and the modular reduction: |sum| <= 62 2^24
-
 struct CrtGemmParams {
   const uint32_t* tiles;   // blocks I (bits 0-14), J (bits 15-29)
   int nblocks;             // blocks per plane
@@ -1932,10 +2193,6 @@ struct CrtGemmParams {
   int debug_withhold_load;
   uint32_t mod[CRT_MAX], magic[CRT_MAX], inv[CRT_MAX], bias[CRT_MAX];
 };
-
-__device__ __forceinline__ uint32_t crt_mod31(uint32_t x, uint32_t p, uint32_t magic) {   // x mod p, x < 2^31
-  return x - (__umulhi(x, magic) >> 7) * p;
-}
 
 template <int NCH>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(S2_THREADS, 1)
@@ -3337,6 +3594,44 @@ int dist_tc(cdl_ctx* ctx, const void* planes, const long long* norms, int n, int
   p.offgrid = offgrid;
   // algorithmic work: n (n - 1) T / 2 squared differences
   return dist_launch(ctx, planes, rows, tp, p, terms);
+}
+
+int dist_residues_tc(cdl_ctx* ctx, const void* planes, const int* ex, const void* norms, int n, int T, int rows, int kp,
+                     double* A, const int* offgrid, void* bad) {
+  if (rows % 128 || kp % 64 || rows < n || kp / 64 > CR_MAX_KBLOCKS) return CDL_ERR_INVALID_ARG;
+  DistResParams p{};
+  p.nb128 = rows / 128;
+  p.nb64 = 2 * p.nb128;
+  const long long tiles = (long long)p.nb128 * p.nb64 - (long long)p.nb128 * (p.nb128 - 1);
+  if (tiles > 0x7fffffffLL) return CDL_ERR_INVALID_ARG;
+  p.num_tiles = (int)tiles;
+  p.rows = rows;
+  p.kblocks = T < DIST_RES_MIN_T ? 0 : kp / 64;
+  p.n = n;
+  p.ex = ex;
+  p.norms = static_cast<const ulonglong2*>(norms);
+  p.A = A;
+  p.offgrid = offgrid;
+  p.bad = static_cast<unsigned char*>(bad);
+  p.idesc = make_idesc(DS_N);
+  p.status = ctx->dev_status;
+  for (int l = 0; l < 16; ++l) {
+    p.mod[l] = (uint32_t)CRT_MOD[l];
+    p.magic[l] = crt_magic(CRT_MOD[l]);
+    p.inv[l] = (uint32_t)crt_inverse(16, l);
+    p.bias[l] = (uint32_t)(((1u << 30) + CRT_MOD[l] - 1) / CRT_MOD[l] * CRT_MOD[l]);
+  }
+  CUtensorMap ma, mb;
+  CDL_TRY(make_map(&ma, planes, (int64_t)16 * rows, kp, 128));
+  CDL_TRY(make_map(&mb, planes, (int64_t)16 * rows, kp, DS_N));
+  static bool attr = false;
+  if (!attr) {
+    CDL_CUDA_TRY(cudaFuncSetAttribute(k_tc_distr, cudaFuncAttributeMaxDynamicSharedMemorySize, DR_SMEM_BYTES));
+    attr = true;
+  }
+  Launch L(ctx, CDL_KC_DISTANCE, 0);
+  k_tc_distr<<<std::min(p.num_tiles, ctx->sm_count), T8_THREADS, DR_SMEM_BYTES, ctx->stream>>>(ma, mb, p);
+  return L.done();
 }
 
 int dist_tc_panel(cdl_ctx* ctx, const void* planes, const long long* norms, int n, int rows, int tp, double* panel,
