@@ -149,7 +149,7 @@ int cdl_ctx_set_debug(cdl_ctx* ctx, int flags);
  * vol, sigma_out: device, one float64 each (sigma_out receives the sigma used).
  * Squared distances are exact when every x is a multiple of 2^-16 below 2^7
  * in magnitude (int64 arithmetic). Otherwise, for T >= 16 each is the exact
- * squared distance of the two series rounded to 2^-61 of their distances to
+ * squared distance of the two series rounded to 2^-60 of their distances to
  * node 0 (or to 2^-60 of the largest sample, if that is more), correctly
  * rounded, where that leaves it within about 2^-53 relative; the others, and
  * all for T < 16, are computed in float64 with one rounding per subtraction,
@@ -424,10 +424,10 @@ int cdl_cad_score(cdl_ctx* ctx, const void* A1, const void* A2, cdl_dtype a_dtyp
  * Delta E_ij = |A1_ij - A2_ij| |c2(i,j) - c1(i,j)| (the per-edge term of
  * cdl_cad_score). Taking edges in descending Delta E, ties to the lower
  * (i, j), is optimal for this cardinality problem; S = {Delta E > tau} plus
- * the first ties at tau, tau found by bisection on the float64 bit patterns
- * with fixed-order sums (deterministic). The remaining sum is decided in
- * float64 (a different summation order than a sequential sum: decisions
- * within about 1e-15 relative of delta can differ from one).
+ * the first ties at tau, tau found by a radix search on the float64 bit
+ * patterns with exact integer sums (deterministic; scores below 2^-80 of the
+ * largest lose their bits below that): decisions within about 1e-15 relative
+ * of delta can differ from those of a float64 sum.
  * Outputs: edge_ij (device, 2 x max_edges int64, (i, j) pairs in (i, j)
  * order) and edge_dE (device, max_edges) receive the first min(|S|,
  * max_edges) edges of S; for each of the n_nodes nodes in `nodes` (device

@@ -21,6 +21,7 @@
 #include <climits>
 #include <cmath>
 #include <cstring>
+#include <vector>
 
 #include "internal.h"
 #include "tiles.cuh"
@@ -423,66 +424,87 @@ __global__ void __launch_bounds__(256) k_tcs_diag(const double* __restrict__ Z1,
   if (lane == 0) dint[row] = llrint(acc / cs[1]);           // division by a power of two: exact
 }
 
+// float64 values as integers in the same order (0: a NaN, which is never
+// picked; -0 as 0), and back: comparisons leave the float64 pipe alone.
+__device__ __forceinline__ unsigned long long order_key(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  if ((b << 1) == 0) return 1ull << 63;
+  if ((b << 1) > (0x7FFull << 53)) return 0;
+  return b >> 63 ? ~b : b | 1ull << 63;
+}
+__device__ __forceinline__ double order_value(unsigned long long k) {
+  return __longlong_as_double((long long)(k >> 63 ? k & ~(1ull << 63) : ~k));
+}
 // (v, i) precedes (w, j) in the anomaly order: larger score first, then the
 // lower index.
-__device__ __forceinline__ bool better(double v, int i, double w, int j) {
+__device__ __forceinline__ bool better(unsigned long long v, int i, unsigned long long w, int j) {
   return v > w || (v == w && i < j);
 }
 
-__device__ __forceinline__ void topk_block(const double* __restrict__ F, int n, int topk,
-                                           int64_t* __restrict__ out) {
-  __shared__ double sv[32];
+// The `m` best of val(0) .. val(n - 1) in the anomaly order (entries with
+// skip(i) left out) to put(rank, value, index), index -1 past the end. Every
+// thread keeps the best of its own strided entries; a block reduction picks
+// the overall best, and only the thread that held it looks through its
+// entries again. Bound by the latency of the m reductions: n = 8192, m = 10
+// 23 us, where 110 went when every round read all entries and compared on the
+// float64 pipe (2 lanes a clock); the top 20 of ten nodes at n = 4001, from
+// columns of E, 153 -> 34 us.
+template <typename V, typename S, typename P>
+__device__ __forceinline__ void topk_rounds(int n, int m, V val, S skip, P put) {
+  __shared__ unsigned long long sv[32];
   __shared__ int si[32];
-  double pv = INFINITY;
-  int pi = -1;
-  for (int t = 0; t < topk; ++t) {
-    double bv = -INFINITY;
-    int bidx = INT_MAX;
+  unsigned long long bv = 0, pv = ~0ull;
+  int bidx = INT_MAX, pi = -1;
+  auto scan = [&]() {   // the best of this thread's entries after (pv, pi)
+    bv = 0;
+    bidx = INT_MAX;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      const double v = F[i];
-      const bool after = v < pv || (v == pv && i > pi);
-      if (after && better(v, i, bv, bidx)) {
+      if (skip(i)) continue;
+      const unsigned long long v = order_key(val(i));
+      if (better(pv, pi, v, i) && v != 0 && better(v, i, bv, bidx)) {
         bv = v;
         bidx = i;
       }
     }
+  };
+  auto reduce = [](unsigned long long& v, int& i) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-      const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bidx, o);
-      if (better(ov, oi, bv, bidx)) {
-        bv = ov;
-        bidx = oi;
+      const unsigned long long ov = __shfl_xor_sync(0xffffffffu, v, o);
+      const int oi = __shfl_xor_sync(0xffffffffu, i, o);
+      if (better(ov, oi, v, i)) {
+        v = ov;
+        i = oi;
       }
     }
+  };
+  scan();
+  for (int t = 0; t < m; ++t) {
+    unsigned long long v = bv;
+    int i = bidx;
+    reduce(v, i);
     if ((threadIdx.x & 31) == 0) {
-      sv[threadIdx.x >> 5] = bv;
-      si[threadIdx.x >> 5] = bidx;
+      sv[threadIdx.x >> 5] = v;
+      si[threadIdx.x >> 5] = i;
     }
     __syncthreads();
-    if (threadIdx.x < 32) {
-      bv = threadIdx.x < (blockDim.x >> 5) ? sv[threadIdx.x] : -INFINITY;
-      bidx = threadIdx.x < (blockDim.x >> 5) ? si[threadIdx.x] : INT_MAX;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bidx, o);
-        if (better(ov, oi, bv, bidx)) {
-          bv = ov;
-          bidx = oi;
-        }
-      }
-      if (threadIdx.x == 0) {
-        sv[0] = bv;
-        si[0] = bidx;
-        out[t] = bidx == INT_MAX ? -1 : bidx;
-      }
+    v = (threadIdx.x & 31) < (blockDim.x >> 5) ? sv[threadIdx.x & 31] : 0;
+    i = (threadIdx.x & 31) < (blockDim.x >> 5) ? si[threadIdx.x & 31] : INT_MAX;
+    reduce(v, i);   // in every warp: the result without another barrier
+    if (threadIdx.x == 0) put(t, order_value(v), i == INT_MAX ? -1 : i);
+    if (i == bidx && i != INT_MAX) {
+      pv = v;
+      pi = i;
+      scan();
     }
-    __syncthreads();
-    pv = sv[0];
-    pi = si[0];
-    __syncthreads();
+    __syncthreads();                     // sv, si are read by every warp
   }
+}
+
+__device__ __forceinline__ void topk_block(const double* __restrict__ F, int n, int topk,
+                                           int64_t* __restrict__ out) {
+  topk_rounds(
+      n, topk, [&](int i) { return F[i]; }, [](int) { return false; }, [&](int t, double, int i) { out[t] = i; });
 }
 
 __global__ void __launch_bounds__(1024) k_topk(const double* __restrict__ F, int n, int topk,
@@ -496,9 +518,10 @@ __global__ void __launch_bounds__(1024) k_topk(const double* __restrict__ F, int
 // descending Delta E (ties by (i, j)) is optimal for that cardinality
 // problem, so the set is {Delta E > tau} plus the first c edges equal to
 // tau, for the largest tau whose set {Delta E >= tau} already suffices. tau
-// is found by bisection on the float64 bit patterns (non-negative doubles
-// order like their bits), each step a fixed-order sum over the upper
-// triangle, so the result does not depend on scheduling.
+// is found by a radix search on the float64 bit patterns (non-negative doubles
+// order like their bits), 16 bins a pass. Sums are exact: values in units of
+// 2^-80 of the largest one's binade, added in 128-bit integers, so they
+// depend neither on scheduling nor on how the passes split them.
 
 __global__ void __launch_bounds__(256) k_edge_pairs(const double* __restrict__ A1, const double* __restrict__ A2,
                                                      const void* __restrict__ ab, int n, int k, int fp64,
@@ -518,57 +541,6 @@ __global__ void __launch_bounds__(256) k_edge_pairs(const double* __restrict__ A
 
 __device__ __forceinline__ unsigned long long dkey(double v) { return (unsigned long long)__double_as_longlong(v); }
 
-// Per-block sums and counts of the upper-triangle entries with key >= tau
-// (rows i = block, block + grid, ...; fixed order).
-__global__ void __launch_bounds__(256) k_edge_mass(const double* __restrict__ E, int n, unsigned long long tau,
-                                                    double* __restrict__ psum, unsigned long long* __restrict__ pcnt) {
-  __shared__ double rs[8];
-  __shared__ unsigned long long rc[8];
-  double s = 0.0;
-  unsigned long long c = 0;
-  for (int i = blockIdx.x; i < n - 1; i += gridDim.x)
-    for (int j = i + 1 + threadIdx.x; j < n; j += 256) {
-      const double v = E[(size_t)i * n + j];
-      if (dkey(v) >= tau) {
-        s += v;
-        ++c;
-      }
-    }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    s += __shfl_xor_sync(0xffffffffu, s, o);
-    c += __shfl_xor_sync(0xffffffffu, c, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    rs[threadIdx.x >> 5] = s;
-    rc[threadIdx.x >> 5] = c;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    unsigned long long u = 0;
-    for (int w = 0; w < 8; ++w) {
-      t += rs[w];
-      u += rc[w];
-    }
-    psum[blockIdx.x] = t;
-    pcnt[blockIdx.x] = u;
-  }
-}
-
-__global__ void k_edge_mass_total(const double* __restrict__ psum, const unsigned long long* __restrict__ pcnt, int nb,
-                                  double* __restrict__ out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double t = 0.0;
-  unsigned long long u = 0;
-  for (int b = 0; b < nb; ++b) {
-    t += psum[b];
-    u += pcnt[b];
-  }
-  out[0] = t;
-  reinterpret_cast<unsigned long long*>(out)[1] = u;
-}
-
 // Largest key of the upper triangle (atomicMax on the bit patterns).
 __global__ void __launch_bounds__(256) k_edge_maxkey(const double* __restrict__ E, int n,
                                                       unsigned long long* __restrict__ out) {
@@ -578,6 +550,236 @@ __global__ void __launch_bounds__(256) k_edge_maxkey(const double* __restrict__ 
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
   if ((threadIdx.x & 31) == 0) atomicMax(out, m);
+}
+
+// State of the cut search. The cut's key lies in [lo, lo + 16 2^sh): 16 bins
+// of 2^sh keys each, next to be summed (sh = 52: a window of binades from the
+// largest key down; sh < 0: found, lo alone); `above` = the sum of all entries
+// with larger keys.
+struct U128 {
+  unsigned long long lo, hi;
+};
+struct EdgeCut {
+  unsigned long long kmax;
+  U128 total, above;
+  unsigned long long lo;
+  unsigned long long cnt;     // entries in the range
+  int sh;
+  int have_total;
+  int none;                   // total < delta: no edge is needed
+  unsigned nbuf;              // entries collected
+  unsigned long long tau;     // result of k_edge_cut
+  unsigned long long ties;
+  U128 gt;                    // sum of the entries above tau
+};
+constexpr int EC_BINS = 17;       // 16 bins and, for the total, the entries below them
+constexpr int EC_BLOCKS_PER_SM = 2;
+constexpr int EC_BUF = 2048;      // entries the last step sorts in shared memory
+constexpr size_t EC_SMEM = (size_t)EC_BINS * 256 * 20;
+
+__device__ __forceinline__ unsigned __int128 u128_of(U128 v) { return ((unsigned __int128)v.hi << 64) | v.lo; }
+__device__ __forceinline__ U128 u128_to(unsigned __int128 v) {
+  return {(unsigned long long)v, (unsigned long long)(v >> 64)};
+}
+
+// The value of `key` in units of 2^(emax - 1075 - 28), emax the exponent field
+// of the largest key (truncated below one unit): less than 2^81.
+__host__ __device__ __forceinline__ unsigned __int128 edge_units(unsigned long long key, int emax) {
+  const int f = (int)(key >> 52), e = f > 1 ? f : 1;
+  const unsigned long long m = (key & 0xFFFFFFFFFFFFFull) | (f ? 1ull << 52 : 0ull);
+  const int s = 28 - (emax - e);
+  if (s >= 0) return (unsigned __int128)m << s;
+  return s > -53 ? (unsigned __int128)(m >> -s) : 0;
+}
+__host__ __device__ __forceinline__ int edge_emax(unsigned long long kmax) {
+  const int f = (int)(kmax >> 52);
+  return f > 1 ? f : 1;
+}
+// delta in the same units, rounded up (an integer sum is below delta iff it is below this)
+__host__ __device__ __forceinline__ unsigned __int128 edge_delta_units(double delta, int emax) {
+  unsigned long long key;
+  memcpy(&key, &delta, 8);
+  const int f = (int)(key >> 52), e = f > 1 ? f : 1;
+  const unsigned long long m = (key & 0xFFFFFFFFFFFFFull) | (f ? 1ull << 52 : 0ull);
+  const int s = 28 - (emax - e);
+  if (s > 70) return (unsigned __int128)1 << 126;
+  if (s >= 0) return (unsigned __int128)m << s;
+  if (s <= -54) return 1;
+  return (m + (1ull << -s) - 1) >> -s;
+}
+
+// One pass: per-block sums and counts of the entries in each bin. A thread adds
+// to its own column of the bins in shared memory (no conflicts, no atomics).
+// Bound by integer issue and the reads of E (about 20 us at n = 4001, 8 million
+// entries).
+__global__ void __launch_bounds__(256) k_edge_bins(const double* __restrict__ E, int n, const EdgeCut* __restrict__ c,
+                                                    U128* __restrict__ psum, unsigned long long* __restrict__ pcnt) {
+  extern __shared__ unsigned long long ecsm[];
+  unsigned long long* slo = ecsm;
+  unsigned long long* shi = slo + EC_BINS * 256;
+  unsigned* scn = reinterpret_cast<unsigned*>(shi + EC_BINS * 256);
+  const int tid = threadIdx.x;
+  if (c->sh < 0 || c->none) return;
+  for (int b = 0; b < EC_BINS; ++b) {
+    slo[b * 256 + tid] = shi[b * 256 + tid] = 0;
+    scn[b * 256 + tid] = 0;
+  }
+  const unsigned long long lo = c->lo;
+  const int sh = c->sh, emax = edge_emax(c->kmax);
+  const bool rest = !c->have_total;
+  for (int i = blockIdx.x; i < n - 1; i += gridDim.x) {
+    const double* row = E + (size_t)i * n;
+#pragma unroll 4
+    for (int j = i + 1 + tid; j < n; j += 256) {
+      const unsigned long long key = dkey(row[j]);
+      const unsigned long long d = (key - lo) >> sh;
+      const int b = key < lo ? (rest ? 16 : 17) : d < 16 ? (int)d : 17;
+      if (b < EC_BINS) {
+        const unsigned __int128 v = u128_of({slo[b * 256 + tid], shi[b * 256 + tid]}) + edge_units(key, emax);
+        slo[b * 256 + tid] = (unsigned long long)v;
+        shi[b * 256 + tid] = (unsigned long long)(v >> 64);
+        ++scn[b * 256 + tid];
+      }
+    }
+  }
+  __syncthreads();
+  for (int b = tid >> 5; b < EC_BINS; b += 8) {
+    unsigned __int128 v = 0;
+    unsigned long long u = 0;
+    for (int t = tid & 31; t < 256; t += 32) {
+      v += u128_of({slo[b * 256 + t], shi[b * 256 + t]});
+      u += scn[b * 256 + t];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      v += u128_of({__shfl_xor_sync(0xffffffffu, (unsigned long long)v, o),
+                    __shfl_xor_sync(0xffffffffu, (unsigned long long)(v >> 64), o)});
+      u += __shfl_xor_sync(0xffffffffu, u, o);
+    }
+    if ((tid & 31) == 0) {
+      psum[(size_t)b * gridDim.x + blockIdx.x] = u128_to(v);
+      pcnt[(size_t)b * gridDim.x + blockIdx.x] = u;
+    }
+  }
+}
+
+__global__ void k_edge_cut_init(EdgeCut* c) {
+  const unsigned long long binade = c->kmax >> 52;
+  c->lo = binade > 15 ? (binade - 15) << 52 : 0;
+  c->sh = 52;
+}
+
+// The bin of the cut from the per-block sums: one warp per bin, then one thread.
+__global__ void __launch_bounds__(32 * EC_BINS) k_edge_step(const U128* __restrict__ psum,
+                                                            const unsigned long long* __restrict__ pcnt, int nblocks,
+                                                            double delta, EdgeCut* __restrict__ c) {
+  __shared__ U128 bs[EC_BINS];
+  __shared__ unsigned long long bc[EC_BINS];
+  const int b = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (c->sh < 0 || c->none) return;
+  unsigned __int128 v = 0;
+  unsigned long long u = 0;
+  for (int q = lane; q < nblocks; q += 32) {
+    v += u128_of(psum[(size_t)b * nblocks + q]);
+    u += pcnt[(size_t)b * nblocks + q];
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    v += u128_of({__shfl_xor_sync(0xffffffffu, (unsigned long long)v, o),
+                  __shfl_xor_sync(0xffffffffu, (unsigned long long)(v >> 64), o)});
+    u += __shfl_xor_sync(0xffffffffu, u, o);
+  }
+  if (lane == 0) {
+    bs[b] = u128_to(v);
+    bc[b] = u;
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  const unsigned __int128 need = edge_delta_units(delta, edge_emax(c->kmax));
+  if (!c->have_total) {
+    unsigned __int128 t = 0;
+    for (int q = 0; q < EC_BINS; ++q) t += u128_of(bs[q]);
+    c->total = u128_to(t);
+    c->have_total = 1;
+    if (t < need) {
+      c->none = 1;
+      return;
+    }
+  }
+  const unsigned __int128 total = u128_of(c->total);
+  unsigned __int128 above = u128_of(c->above);
+  int d = 15;
+  for (; d >= 0; --d) {
+    const unsigned __int128 ge = above + u128_of(bs[d]);
+    if (total - ge < need) break;   // taking everything from this bin on suffices
+    above = ge;
+  }
+  c->above = u128_to(above);
+  if (d < 0) {                       // below this window of binades (only the first passes)
+    const unsigned long long step = 16ull << 52;
+    c->lo = c->lo > step ? c->lo - step : 0;
+    return;
+  }
+  c->lo += (unsigned long long)d << c->sh;
+  c->cnt = bc[d];
+  c->sh -= 4;
+}
+
+// The entries of the cut's range, in any order.
+__global__ void __launch_bounds__(256) k_edge_collect(const double* __restrict__ E, int n, EdgeCut* __restrict__ c,
+                                                       unsigned long long* __restrict__ buf) {
+  if (c->sh < 0 || c->sh == 52 || c->none || c->cnt > EC_BUF) return;
+  const unsigned long long lo = c->lo;
+  const int sh = c->sh + 4;
+  for (int i = blockIdx.x; i < n - 1; i += gridDim.x) {
+    const double* row = E + (size_t)i * n;
+#pragma unroll 4
+    for (int j = i + 1 + threadIdx.x; j < n; j += 256) {
+      const unsigned long long key = dkey(row[j]);
+      if (key >= lo && ((key - lo) >> sh) == 0) {
+        const unsigned p = atomicAdd(&c->nbuf, 1u);
+        if (p < EC_BUF) buf[p] = key;
+      }
+    }
+  }
+}
+
+// The cut among the collected entries: a bitonic sort of their keys, then the
+// distinct ones from the largest down.
+__global__ void __launch_bounds__(1024) k_edge_cut(const unsigned long long* __restrict__ buf, double delta,
+                                                    EdgeCut* __restrict__ c) {
+  __shared__ unsigned long long key[EC_BUF];
+  if (c->sh < 0 || c->sh == 52 || c->none || c->cnt > EC_BUF) return;
+  const int m = (int)c->cnt;
+  for (int e = threadIdx.x; e < EC_BUF; e += 1024) key[e] = e < m ? buf[e] : 0ull;
+  for (int w = 2; w <= EC_BUF; w <<= 1)
+    for (int o = w >> 1; o > 0; o >>= 1) {
+      __syncthreads();
+      const int e = 2 * threadIdx.x - (threadIdx.x & (o - 1)), f = e + o;
+      const unsigned long long x = key[e], y = key[f];
+      if ((x < y) == ((e & w) == 0)) {
+        key[e] = y;
+        key[f] = x;
+      }
+    }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  const int emax = edge_emax(c->kmax);
+  const unsigned __int128 need = edge_delta_units(delta, emax), total = u128_of(c->total);
+  unsigned __int128 s = u128_of(c->above);
+  for (int e = 0; e < m;) {
+    int f = e;
+    while (f < m && key[f] == key[e]) ++f;
+    const unsigned __int128 ge = s + edge_units(key[e], emax) * (unsigned)(f - e);
+    if (total - ge < need || f == m) {
+      c->tau = key[e];
+      c->ties = (unsigned long long)(f - e);
+      c->gt = u128_to(s);
+      return;
+    }
+    s = ge;
+    e = f;
+  }
 }
 
 // Per row i: entries j > i with key > tau, and with key == tau.
@@ -724,61 +926,13 @@ __global__ void __launch_bounds__(256) k_edge_write(const double* __restrict__ E
 __global__ void __launch_bounds__(1024) k_node_top_edges(const double* __restrict__ E, int n,
                                                           const long long* __restrict__ nodes, int m,
                                                           long long* __restrict__ partner, double* __restrict__ pval) {
-  __shared__ double sv[32];
-  __shared__ int si[32];
   const int i = (int)nodes[blockIdx.x];
-  double pv = INFINITY;
-  int pi = -1;
-  for (int t = 0; t < m; ++t) {
-    double bv = -INFINITY;
-    int bidx = INT_MAX;
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-      if (j == i) continue;
-      const double v = i < j ? E[(size_t)i * n + j] : E[(size_t)j * n + i];
-      const bool after = v < pv || (v == pv && j > pi);
-      if (after && better(v, j, bv, bidx)) {
-        bv = v;
-        bidx = j;
-      }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bidx, o);
-      if (better(ov, oi, bv, bidx)) {
-        bv = ov;
-        bidx = oi;
-      }
-    }
-    if ((threadIdx.x & 31) == 0) {
-      sv[threadIdx.x >> 5] = bv;
-      si[threadIdx.x >> 5] = bidx;
-    }
-    __syncthreads();
-    if (threadIdx.x < 32) {
-      bv = threadIdx.x < (blockDim.x >> 5) ? sv[threadIdx.x] : -INFINITY;
-      bidx = threadIdx.x < (blockDim.x >> 5) ? si[threadIdx.x] : INT_MAX;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bidx, o);
-        if (better(ov, oi, bv, bidx)) {
-          bv = ov;
-          bidx = oi;
-        }
-      }
-      if (threadIdx.x == 0) {
-        sv[0] = bv;
-        si[0] = bidx;
-        partner[(size_t)blockIdx.x * m + t] = bidx == INT_MAX ? -1 : bidx;
-        pval[(size_t)blockIdx.x * m + t] = bidx == INT_MAX ? 0.0 : bv;
-      }
-    }
-    __syncthreads();
-    pv = sv[0];
-    pi = si[0];
-    __syncthreads();
-  }
+  topk_rounds(
+      n, m, [&](int j) { return i < j ? E[(size_t)i * n + j] : E[(size_t)j * n + i]; }, [&](int j) { return j == i; },
+      [&](int t, double v, int j) {
+        partner[(size_t)blockIdx.x * m + t] = j;
+        pval[(size_t)blockIdx.x * m + t] = j < 0 ? 0.0 : v;
+      });
 }
 
 // ---------------------------------------------------------------- changed edges only
@@ -1148,21 +1302,22 @@ int cad_edges(cdl_ctx* ctx, const double* A1, const double* A2, const double* Z1
   const int n = (int)n64;
   cudaStream_t st = ctx->stream;
   const int nb = (n + ST - 1) / ST;
-  void *vab, *vc, *vE, *vF, *vp, *vs, *vcnt, *voff;
+  void *vab, *vc, *vE, *vF, *vp, *vs, *vbuf, *vcnt, *voff;
   CDL_TRY(score_prepare(ctx, Z1, Z2, vol1, vol2, n, k, fp64, &vab));
   CDL_TRY(ws_get(ctx, "score.contrib", (size_t)nb * n * sizeof(double), &vc));
   CDL_TRY(ws_get(ctx, "edges.E", (size_t)n * n * sizeof(double), &vE));
   CDL_TRY(ws_get(ctx, "edges.F", (size_t)n * sizeof(double), &vF));
   const int mb = std::min(n, ctx->sm_count * 8);
-  CDL_TRY(ws_get(ctx, "edges.part", (size_t)mb * 16, &vp));
-  CDL_TRY(ws_get(ctx, "edges.scal", 64, &vs));
+  const int eb = std::min(n, ctx->sm_count * EC_BLOCKS_PER_SM);
+  CDL_TRY(ws_get(ctx, "edges.part", (size_t)eb * EC_BINS * 24, &vp));
+  CDL_TRY(ws_get(ctx, "edges.cut", sizeof(EdgeCut), &vs));
+  CDL_TRY(ws_get(ctx, "edges.buf", EC_BUF * sizeof(unsigned long long), &vbuf));
   CDL_TRY(ws_get(ctx, "edges.rowcnt", 2 * (size_t)n * sizeof(int), &vcnt));
   CDL_TRY(ws_get(ctx, "edges.rowoff", 2 * (size_t)n * sizeof(long long) + 16, &voff));
   double* E = static_cast<double*>(vE);
   double* Fw = F ? F : static_cast<double*>(vF);
-  double* scal = static_cast<double*>(vs);
-  double* psum = static_cast<double*>(vp);
-  unsigned long long* pcnt = reinterpret_cast<unsigned long long*>(psum + mb);
+  U128* psum = static_cast<U128*>(vp);
+  unsigned long long* pcnt = reinterpret_cast<unsigned long long*>(psum + (size_t)eb * EC_BINS);
   const long long tiles = (long long)nb * (nb + 1) / 2;
   {
     Launch L(ctx, CDL_KC_SCORE, 8.0 * (double)n * (n - 1));
@@ -1174,73 +1329,92 @@ int cad_edges(cdl_ctx* ctx, const double* A1, const double* A2, const double* Z1
     k_score_reduce<<<(n + 255) / 256, 256, 0, st>>>(static_cast<const double*>(vc), nb, n, Fw);
     CDL_TRY(L.done());
   }
-  // masses: total (tau = 0 counts every entry) and the largest key
-  auto mass = [&](unsigned long long tau, double* sum, unsigned long long* cnt) -> int {
-    {
-      Launch L(ctx, CDL_KC_MISC, 0);
-      k_edge_mass<<<mb, 256, 0, st>>>(E, n, tau, psum, pcnt);
-      CDL_TRY(L.done());
-    }
-    {
-      Launch L(ctx, CDL_KC_MISC, 0);
-      k_edge_mass_total<<<1, 32, 0, st>>>(psum, pcnt, mb, scal);
-      CDL_TRY(L.done());
-    }
-    double h[2];
-    CDL_CUDA_TRY(cudaMemcpyAsync(h, scal, 16, cudaMemcpyDeviceToHost, st));
-    CDL_CUDA_TRY(cudaStreamSynchronize(st));
-    *sum = h[0];
-    std::memcpy(cnt, &h[1], 8);
-    return CDL_OK;
-  };
-  double total;
-  unsigned long long m_all;
-  CDL_TRY(mass(0ull, &total, &m_all));
-  unsigned long long* dmax = reinterpret_cast<unsigned long long*>(scal + 4);
-  CDL_CUDA_TRY(cudaMemsetAsync(dmax, 0, 8, st));
+  EdgeCut* cut = static_cast<EdgeCut*>(vs);
+  CDL_CUDA_TRY(cudaMemsetAsync(cut, 0, sizeof(EdgeCut), st));
   {
     Launch L(ctx, CDL_KC_MISC, 0);
-    k_edge_maxkey<<<mb, 256, 0, st>>>(E, n, dmax);
+    k_edge_maxkey<<<mb, 256, 0, st>>>(E, n, &cut->kmax);
     CDL_TRY(L.done());
   }
-  unsigned long long kmax = 0;
-  CDL_CUDA_TRY(cudaMemcpyAsync(&kmax, dmax, 8, cudaMemcpyDeviceToHost, st));
-  CDL_CUDA_TRY(cudaStreamSynchronize(st));
-  res->total = total;
+  {
+    Launch L(ctx, CDL_KC_MISC, 0);
+    k_edge_cut_init<<<1, 1, 0, st>>>(cut);
+    CDL_TRY(L.done());
+  }
+  static bool attr = false;
+  if (!attr) {
+    CDL_CUDA_TRY(cudaFuncSetAttribute(k_edge_bins, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)EC_SMEM));
+    attr = true;
+  }
+  auto pass = [&]() -> int {
+    {
+      Launch L(ctx, CDL_KC_MISC, 0);
+      k_edge_bins<<<eb, 256, EC_SMEM, st>>>(E, n, cut, psum, pcnt);
+      CDL_TRY(L.done());
+    }
+    Launch L(ctx, CDL_KC_MISC, 0);
+    k_edge_step<<<1, 32 * EC_BINS, 0, st>>>(psum, pcnt, eb, delta, cut);
+    return L.done();
+  };
+  // the binade and 16 bits of the mantissa leave a few entries in all but
+  // degenerate cases (many ties, a cut far below the largest entry): those
+  // take more passes, each with a look at the state
+  for (int q = 0; q < 5; ++q) CDL_TRY(pass());
+  EdgeCut h;
+  while (true) {
+    {
+      Launch L(ctx, CDL_KC_MISC, 0);
+      k_edge_collect<<<mb, 256, 0, st>>>(E, n, cut, static_cast<unsigned long long*>(vbuf));
+      CDL_TRY(L.done());
+    }
+    {
+      Launch L(ctx, CDL_KC_MISC, 0);
+      k_edge_cut<<<1, 1024, 0, st>>>(static_cast<const unsigned long long*>(vbuf), delta, cut);
+      CDL_TRY(L.done());
+    }
+    CDL_CUDA_TRY(cudaMemcpyAsync(&h, cut, sizeof(h), cudaMemcpyDeviceToHost, st));
+    CDL_CUDA_TRY(cudaStreamSynchronize(st));
+    if (h.none || h.sh < 0 || (h.sh < 52 && h.cnt <= EC_BUF) || (h.kmax >> 52) >= 0x7FF)
+      break;
+    CDL_TRY(pass());
+  }
+  typedef unsigned __int128 u128;
+  const int emax = edge_emax(h.kmax);
+  auto u = [](U128 v) { return ((u128)v.hi << 64) | v.lo; };
+  // truncated to float64, so that a remaining sum below delta stays below it
+  auto value = [&](u128 v) {
+    int up = 0;
+    while (v >> 53) {
+      v >>= 1;
+      ++up;
+    }
+    return std::ldexp((double)(unsigned long long)v, up + emax - 1075 - 28);
+  };
   unsigned long long tau = 0;
   long long c = 0;
-  bool none = total < delta;
-  if (!none) {
-    // largest tau in [0, kmax] with total - mass(>= tau) < delta (tau = 0 qualifies)
-    unsigned long long lo = 0, hi = kmax;
-    while (lo < hi) {
-      const unsigned long long mid = lo + (hi - lo + 1) / 2;
-      double s;
-      unsigned long long cn;
-      CDL_TRY(mass(mid, &s, &cn));
-      if (total - s < delta)
-        lo = mid;
-      else
-        hi = mid - 1;
-    }
-    tau = lo;
+  const bool none = h.none != 0;
+  const bool finite = (h.kmax >> 52) < 0x7FF;
+  if (!finite) {   // no sum is below delta: every entry, the zeros as ties
+    res->total = h.kmax << 12 ? NAN : INFINITY;
+    res->remaining = NAN;
+    res->threshold = 0.0;
+    c = (long long)n * n;
+  } else if (!none) {
+    tau = h.sh < 0 ? h.lo : h.tau;
+    const long long ties = (long long)(h.sh < 0 ? h.cnt : h.ties);
+    const u128 gt = h.sh < 0 ? u(h.above) : u(h.gt), v = edge_units(tau, emax), need = edge_delta_units(delta, emax);
     // entries above tau are taken; ties at tau one by one in (i, j) order
-    double s_gt = 0.0, s_ge = 0.0;
-    unsigned long long c_gt = 0, c_ge = 0;
-    CDL_TRY(mass(tau + 1, &s_gt, &c_gt));
-    CDL_TRY(mass(tau, &s_ge, &c_ge));
-    const long long ties = (long long)(c_ge - c_gt);
-    double v;
-    std::memcpy(&v, &tau, 8);
-    double rem = total - s_gt;
-    while (!(rem < delta) && c < ties) {
-      rem -= v;
-      ++c;
+    u128 rem = u(h.total) - gt;
+    if (rem >= need) {
+      const u128 more = v ? (rem - need) / v + 1 : (u128)ties;
+      c = more < (u128)ties ? (long long)more : ties;
+      rem -= v * (u128)c;
     }
-    res->remaining = rem;
-    res->threshold = v;
+    res->total = value(u(h.total));
+    res->remaining = value(rem);
+    std::memcpy(&res->threshold, &tau, 8);
   } else {
-    res->remaining = total;
+    res->total = res->remaining = value(u(h.total));
     res->threshold = INFINITY;
     tau = ~0ull;   // nothing is above it
   }
@@ -1254,6 +1428,14 @@ int cad_edges(cdl_ctx* ctx, const double* A1, const double* A2, const double* Z1
     Launch L(ctx, CDL_KC_MISC, 0);
     k_edge_rowcount<<<mb, 256, 0, st>>>(E, n, tau, cgt, ceq);
     CDL_TRY(L.done());
+  }
+  if (!finite) {
+    std::vector<int> eq(n);
+    CDL_CUDA_TRY(cudaMemcpyAsync(eq.data(), ceq, (size_t)n * sizeof(int), cudaMemcpyDeviceToHost, st));
+    CDL_CUDA_TRY(cudaStreamSynchronize(st));
+    c = 0;
+    for (int e : eq) c += e;
+    res->n_ties_taken = c;
   }
   {
     Launch L(ctx, CDL_KC_MISC, 0);

@@ -127,3 +127,37 @@ def test_edges_whole_pair(G):
     assert np.array_equal(ij, O.anomalous_edges(E, delta)["edges"])
     planted = set(wl.planted[0].tolist())
     assert all(i in planted or j in planted for i, j in ij)
+
+
+@pytest.mark.parametrize("case", ["spread", "ties", "cut_far_below", "all_equal", "one_edge"])
+def test_edge_cut_of_given_scores(G, case):
+    """The cut search itself: Z makes every commute-time change 1 or a chosen value, so Delta E is |A1 - A2|
+    times it, with scores spread over hundreds of binades, more ties than the sorted buffer holds, or a
+    cut many windows of binades below the largest score. The oracle takes edges one by one from a sort."""
+    cdl = G.cdl
+    n = 200
+    rng = np.random.default_rng(3)
+    iu, ju = np.triu_indices(n, 1)
+    e = {"spread": 2.0 ** rng.uniform(-300, 0, iu.size), "ties": rng.integers(1, 4, iu.size) / 4.0,
+         "cut_far_below": np.where(np.arange(iu.size) == 77, 1.0, 2.0 ** -90), "all_equal": np.full(iu.size, 0.75),
+         "one_edge": np.where(np.arange(iu.size) == 5, 0.5, 0.0)}[case]
+    A1 = np.zeros((n, n))
+    A1[iu, ju] = e
+    A1 += A1.T
+    # k = 2, vol = 1, Z1 = 0: c2 - c1 = |z_i - z_j|^2 = 1 off the diagonal needs n points at mutual distance 1;
+    # use one-hot rows over n columns scaled by sqrt(1/2)
+    Z2 = np.sqrt(0.5) * np.eye(n)
+    Z1 = np.zeros((n, n))
+    E = np.zeros((n, n))
+    E[iu, ju] = e
+    total = e.sum()
+    for frac in (0.9999, 0.5, 1e-3):
+        delta = {"cut_far_below": 0.5 * iu.size * 2.0 ** -90}.get(case, total * frac)
+        out = O.anomalous_edges(E, delta)
+        res, ij, val, part, pv, F = _edges(G, _t(A1), _t(np.zeros((n, n))), _t(Z1), _t(Z2), 1.0, 1.0, delta,
+                                           cdl.CDL_F64, [0, 7, n - 1], 5, cap=iu.size)
+        assert res.n_edges == len(out["edges"]) and res.remaining < delta
+        assert np.array_equal(ij, out["edges"])
+        np.testing.assert_allclose(res.total, total, rtol=1e-13)
+    po, _ = O.node_top_edges(E, [0, 7, n - 1], 5)
+    assert np.array_equal(part[:3], po)
