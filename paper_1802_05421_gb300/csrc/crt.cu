@@ -10,8 +10,8 @@
 //                   once to the level's type, and its mirror.
 //
 // The only errors are the rounding of the scaled rows, at most half a unit of
-// 2^-B of the row's norm per entry (B = 61.6 bits with 16 moduli for float64
-// levels, 30.7 with 8 for float32 ones), and the final rounding; a float64 or
+// 2^-B of the row's norm per entry (B = 60.9 bits with 16 moduli for float64
+// levels, 30.5 with 8 for float32 ones), and the final rounding; a float64 or
 // float32 dot product rounds every partial sum. Rows with a non-finite entry
 // give NaN rows and columns.
 //
@@ -62,17 +62,14 @@ struct CombineTab32 {
 };
 constexpr CombineTab32 make_combine32() {
   CombineTab32 t{};
-  const u128 P = crt_product(8);
   for (int l = 0; l < 8; ++l) {
-    const u128 m = P / (u128)CRT_MOD[l];
-    t.lo[l] = (uint32_t)m;
-    t.hi[l] = (uint32_t)(m >> 32);
-    t.frac[l] = (uint32_t)(((1u << 24) + (unsigned)CRT_MOD[l]) / (2u * (unsigned)CRT_MOD[l]));
+    t.lo[l] = (uint32_t)crt_weight(8, l);
+    t.hi[l] = (uint32_t)(crt_weight(8, l) >> 32);
+    t.frac[l] = crt_frac(8, l);
   }
   return t;
 }
 __constant__ CombineTab32 c_comb32 = make_combine32();
-constexpr unsigned long long P32 = (unsigned long long)crt_product(8);
 
 // The two types' bit patterns: magnitude bits, exponent field and mantissa
 // (value = m 2^(e - BIAS)), moduli.
@@ -207,6 +204,8 @@ template <>
 struct Combine<float> {
   static constexpr int NP = 8;
   static __device__ __forceinline__ float value(const uint32_t (&w)[8], int sh, int e) {
+    constexpr unsigned long long P = (unsigned long long)crt_product(8), off = (unsigned long long)crt_offset(8);
+    constexpr uint32_t f0 = crt_frac_offset(8);
     unsigned long long c = 0;
     uint32_t hi = 0, f = 0;
 #pragma unroll
@@ -216,8 +215,8 @@ struct Combine<float> {
       hi += t * c_comb32.hi[l];
       f += t * c_comb32.frac[l];
     }
-    const uint32_t q = (f + (1u << 22)) >> 23;
-    c += ((unsigned long long)hi << 32) - (unsigned long long)q * P32;   // modulo 2^64: |c| < 2^62
+    const int q = (int)(f - f0 + (1u << 18)) >> 19;
+    c += ((unsigned long long)hi << 32) - off - (unsigned long long)(long long)q * P;   // modulo 2^64: |c| < 2^62
     return ldexpf(__ll2float_rn((long long)c), -e);
   }
   static __device__ __forceinline__ float nan() { return __int_as_float(0x7FC00000); }
@@ -266,7 +265,7 @@ __global__ void __launch_bounds__(256) k_crt_combine(const uint8_t* __restrict__
 
 // Node series for the residue distances (k_tc_distr): row i less the series of
 // node 0 (distances do not change, and the common part of all nodes costs no
-// bits), scaled by the power of two 2^{e_i} that brings its 2-norm to 2^61.65
+// bits), scaled by the power of two 2^{e_i} that brings its 2-norm to 2^60.96
 // at most and keeps both series below 2^61, rounded to integers (each entry
 // within one unit), as 16 residue planes (rows x kp, zero padded), with its
 // exact squared norm. One block of 128 threads per row; also clears the tile

@@ -17,8 +17,9 @@
 namespace cdl {
 
 constexpr int CRT_MAX = 16;
-// (pairwise coprime: 255 = 3 5 17, 253 = 11 23, 247 = 13 19, 217 = 7 31, the others primes and 2^8)
-constexpr int CRT_MOD[CRT_MAX] = {256, 255, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197, 193};
+// Pairwise coprime (247 = 13 19, 217 = 7 31, the others primes and 2^8), and none of 251 .. 255, for
+// which crt_reduce could leave a byte's range.
+constexpr int CRT_MOD[CRT_MAX] = {256, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197, 193, 191, 181, 179};
 
 typedef unsigned __int128 u128;
 
@@ -49,9 +50,9 @@ constexpr int crt_pow2_mod(int k, int p) {
   return r;
 }
 
-// 2^B with 2 B <= log2(P / 4) less a rounding margin: log2 P is 63.575 for 8
-// moduli and 125.376 for 16
-constexpr float crt_norm_bits(int np) { return np == 8 ? 30.75f : 61.65f; }
+// 2^B with 2 B <= log2(P / 4) less a rounding margin: log2 P is 63.09 for 8
+// moduli and 123.98 for 16
+constexpr float crt_norm_bits(int np) { return np == 8 ? 30.52f : 60.96f; }
 
 constexpr int CRT_ROW_NAN = 0x40000000;   // e_i of a row with a non-finite entry
 constexpr int CRT_ROW_ZERO = 0x4000;      // of a zero row, where no other row's units may be coarsened by it
@@ -59,39 +60,70 @@ constexpr int CRT_ROW_ZERO = 0x4000;      // of a zero row, where no other row's
 #ifdef __CUDACC__
 namespace {
 
-// P / p_l in 20-bit limbs (16 moduli: below 2^118) and 2^23 / p_l
+// The weights W_l = (P / p_l) ((P / p_l)^-1 mod p_l), 1 modulo p_l and 0 modulo the others
+constexpr u128 crt_weight(int np, int l) { return crt_product(np) / (u128)CRT_MOD[l] * (u128)crt_inverse(np, l); }
+// round(2^19 W_l / P), without overflow: W_l / P = inv_l / p_l
+constexpr uint32_t crt_frac(int np, int l) {
+  return (uint32_t)(((unsigned)crt_inverse(np, l) * (1u << 20) + (unsigned)CRT_MOD[l]) / (2u * (unsigned)CRT_MOD[l]));
+}
+
+// 16 moduli: W_l in 32-bit limbs (below 2^124) and as fractions; the constants
+// that take out the bytes' offset of 128
 struct CombineTab64 {
-  uint32_t limb[6][CRT_MAX];
+  uint32_t limb[4][CRT_MAX];
   uint32_t frac[CRT_MAX];
 };
 constexpr CombineTab64 make_combine64() {
   CombineTab64 t{};
-  const u128 P = crt_product(16);
   for (int l = 0; l < 16; ++l) {
-    const u128 m = P / (u128)CRT_MOD[l];
-    for (int k = 0; k < 6; ++k) t.limb[k][l] = (uint32_t)(m >> (20 * k)) & 0xFFFFFu;
-    t.frac[l] = (uint32_t)(((1u << 24) + (unsigned)CRT_MOD[l]) / (2u * (unsigned)CRT_MOD[l]));
+    for (int k = 0; k < 4; ++k) t.limb[k][l] = (uint32_t)(crt_weight(16, l) >> (32 * k));
+    t.frac[l] = crt_frac(16, l);
   }
   return t;
 }
+constexpr u128 crt_offset(int np) {   // 128 sum W_l modulo 2^128
+  u128 s = 0;
+  for (int l = 0; l < np; ++l) s += crt_weight(np, l) * 128;
+  return s;
+}
+constexpr uint32_t crt_frac_offset(int np) {
+  uint32_t s = 0;
+  for (int l = 0; l < np; ++l) s += 128 * crt_frac(np, l);
+  return s;
+}
 __constant__ CombineTab64 c_comb64 = make_combine64();
-constexpr unsigned long long P64_HI = (unsigned long long)(crt_product(16) >> 64),
-                             P64_LO = (unsigned long long)crt_product(16);
 
-// The integer whose 16 t values (k_tc_crt) are the bytes at bit `sh` of the words
+// v modulo p as the nearest representative, v an integer of at most 2^24 in
+// magnitude: the quotient is off by at most 2 / p from v / p, so the result is
+// within 0.511 p of zero (p <= 247: 126; p = 256: 128, exactly).
+__device__ __forceinline__ float crt_reduce(float v, float p, float rp) {
+  const float q = __fsub_rn(__fadd_rn(__fmul_rn(v, rp), 12582912.0f), 12582912.0f);   // rint, |q| < 2^17
+  return __fmaf_rn(-q, p, v);
+}
+// r + 128 in the low byte
+__device__ __forceinline__ uint32_t crt_byte(float r) { return __float_as_uint(__fadd_rn(r, 12582912.0f + 128.0f)); }
+__device__ __forceinline__ uint32_t crt_pack(uint32_t b0, uint32_t b1, uint32_t b2, uint32_t b3) {
+  return __byte_perm(__byte_perm(b0, b1, 0x0040), __byte_perm(b2, b3, 0x0040), 0x5410);
+}
+
+// The integer c, |c| <= P / 4, from the bytes (residue + 128) at bit `sh` of the words
 __device__ __forceinline__ __int128 crt16_value(const uint32_t (&w)[16], int sh) {
-  uint32_t S[6] = {0, 0, 0, 0, 0, 0}, f = 0;
+  constexpr u128 P = crt_product(16), off = crt_offset(16);
+  constexpr unsigned long long PH = (unsigned long long)(P >> 64), PL = (unsigned long long)P,
+                               OH = (unsigned long long)(off >> 64), OL = (unsigned long long)off;
+  constexpr uint32_t f0 = crt_frac_offset(16);
+  unsigned long long S[4] = {0, 0, 0, 0};
+  uint32_t f = 0;
 #pragma unroll
   for (int l = 0; l < 16; ++l) {
     const uint32_t t = (w[l] >> sh) & 0xFFu;
 #pragma unroll
-    for (int k = 0; k < 6; ++k) S[k] += t * c_comb64.limb[k][l];   // 16 terms below 2^28
+    for (int k = 0; k < 4; ++k) S[k] += (unsigned long long)t * c_comb64.limb[k][l];   // below 2^44
     f += t * c_comb64.frac[l];
   }
-  const uint32_t q = (f + (1u << 22)) >> 23;            // round(sum t_l / p_l): |c| <= P / 4 leaves no doubt
-  u128 c = (u128)S[0] + ((u128)S[1] << 20) + ((u128)S[2] << 40) + ((u128)S[3] << 60) + ((u128)S[4] << 80) +
-           ((u128)S[5] << 100);
-  c -= (u128)q * (((u128)P64_HI << 64) | P64_LO);       // modulo 2^128: |c| < 2^124
+  const int q = (int)(f - f0 + (1u << 18)) >> 19;   // round(sum r_l W_l / P): |c| <= P / 4 leaves no doubt
+  u128 c = (u128)S[0] + ((u128)S[1] << 32) + ((u128)S[2] << 64) + ((u128)S[3] << 96);
+  c -= (((u128)OH << 64) | OL) + (u128)(__int128)q * (((u128)PH << 64) | PL);   // modulo 2^128: |c| < 2^122
   return (__int128)c;
 }
 

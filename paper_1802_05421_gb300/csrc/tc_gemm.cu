@@ -906,11 +906,7 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
 
 // ---------------------------------------------------------------- sums of residue products
 constexpr int CR_CHUNK_KB = 16;                        // 1024 of K per exact chunk
-constexpr int CR_MAX_KBLOCKS = 62 * CR_CHUNK_KB;       // int32 sums and the modular reduction: |sum| <= 62 2^24
-
-__device__ __forceinline__ uint32_t crt_mod31(uint32_t x, uint32_t p, uint32_t magic) {   // x mod p, x < 2^31
-  return x - (__umulhi(x, magic) >> 7) * p;
-}
+constexpr int CR_MAX_KBLOCKS = 62 * CR_CHUNK_KB;       // int32 sums: |sum| <= 62 2^24 < 2^30
 
 // ---------------------------------------------------------------- exact squared distances
 // d2_ij = |a_i|^2 + |a_j|^2 - 2 a_i . a_j for node series on the 2^-16 grid
@@ -1187,13 +1183,13 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
 // ---------------------------------------------------------------- distances of series on no grid
 // d2_ij of float64 series off the 2^-16 grid, through residues (crt.cuh): row i
 // of the series less the series of node 0 is 2^-e_i times integers x'_i of norm
-// 2^61.65 at most, rounded to one unit (k_series_residues); the Gram entry x'_i .
+// 2^60.96 at most, rounded to one unit (k_series_residues); the Gram entry x'_i .
 // x'_j is formed exactly from 16 residue products on the bf16 tensor cores, and
 // d2' = |x'_i|^2 + |x'_j|^2 - 2 x'_i . x'_j in 128-bit integers, in units of the
 // coarser of the two rows, rounded once to float64. With d2' >= 2^109 the
 // rounding of the series is below 2^-54 of d2 (rms 0.6 units per sample and
 // pair, so 1.2 / sqrt(d2') relative), where a float64 sum of rounded squares
-// has about sqrt(T) 2^-54: tiles with a smaller entry (a distance below 2^-7
+// has about sqrt(T) 2^-54: tiles with a smaller entry (a distance below 2^-6
 // of the nodes' distances to node 0, duplicates, non-finite series) are
 // flagged and formed by the float64 kernel, as before.
 //
@@ -1223,7 +1219,7 @@ struct DistResParams {
   unsigned char* bad;         // per 64 x 64 block (bi, bj), bi <= bj: at bi nb64 + bj
   uint32_t idesc;
   unsigned* status;
-  uint32_t mod[CRT_MAX], magic[CRT_MAX], inv[CRT_MAX], bias[CRT_MAX];
+  float mod[CRT_MAX], rmod[CRT_MAX];   // p_l and 1 / p_l
 };
 
 __global__ void __launch_bounds__(T8_THREADS, 1)
@@ -1348,9 +1344,10 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
       int I, J;
       dist_tile(t, p.nb128, p.nb64, I, J);
       for (int l = 0; l < 16; ++l) {
-        int sum[16];
+        const float mod = p.mod[l], rmod = p.rmod[l];
+        float sum[16];
 #pragma unroll
-        for (int e = 0; e < 16; ++e) sum[e] = 0;
+        for (int e = 0; e < 16; ++e) sum[e] = 0.f;
         for (int c = 0; c < nchunks; ++c, ++pc) {
           if (failed) continue;
           const int b = pc % DR_NBUF;
@@ -1364,17 +1361,16 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
           tc_fence_before();
           mbar_arrive(pempty_bar(b));
 #pragma unroll
-          for (int e = 0; e < 16; ++e) sum[e] += __float2int_rn(v[e]);
+          for (int e = 0; e < 16; ++e) sum[e] = __fadd_rn(sum[e], crt_reduce(v[e], mod, rmod));
         }
-        const uint32_t mod = p.mod[l], magic = p.magic[l], inv = p.inv[l], bias = p.bias[l];
+        if (nchunks > 1) {
 #pragma unroll
-        for (int w = 0; w < 4; ++w) {
-          uint32_t b4 = 0;
-#pragma unroll
-          for (int h = 0; h < 4; ++h)
-            b4 |= crt_mod31(crt_mod31((uint32_t)sum[4 * w + h] + bias, mod, magic) * inv, mod, magic) << (8 * h);
-          tw[(w * 16 + l) * 32 + lane] = b4;
+          for (int e = 0; e < 16; ++e) sum[e] = crt_reduce(sum[e], mod, rmod);
         }
+#pragma unroll
+        for (int w = 0; w < 4; ++w)
+          tw[(w * 16 + l) * 32 + lane] = crt_pack(crt_byte(sum[4 * w]), crt_byte(sum[4 * w + 1]),
+                                                  crt_byte(sum[4 * w + 2]), crt_byte(sum[4 * w + 3]));
       }
       if (__any_sync(0xffffffffu, failed)) continue;
       const int row = I * 128 + q * 32 + lane, col0 = J * DS_N + part * 16;
@@ -1390,7 +1386,7 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
         for (int l = 0; l < 16; ++l) tv[l] = tw[(w * 16 + l) * 32 + lane];
         double* res = reinterpret_cast<double*>(tw + w * 512);   // the quad's words are read: 4 columns x 32 rows
         __syncwarp();
-#pragma unroll 1
+#pragma unroll
         for (int h = 0; h < 4; ++h) {
           const int col = col0 + 4 * w + h;
           double d2 = 0.0;
@@ -2167,16 +2163,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(S2_THREADS, 1)
 }
 
 // ---------------------------------------------------------------- residue products on CTA pairs
-// t[l] = ((A_l B_l^T) mod p_l) inv_l mod p_l for the residue planes l of two
+// t[l] = (A_l B_l^T mod p_l) + 128 as bytes for the residue planes l of two
 // integer matrices (crt.cuh): the products of the float64 and float32 chains.
 // Pairs, stages and barriers as in k_tc_sq2; a unit is one 256 x bn block of
 // one plane. K runs in chunks of 1024, whose sums are exact in float32: each
 // chunk goes to one of the two TMEM accumulators, and the eight epilogue warps
 // add it to int32 registers (bn / 2 columns per thread) while the next chunk
 // multiplies; after the last chunk the sums are reduced modulo p_l and stored
-// as bytes. Bound by the tensor cores for long K (8192 cycles of MMA per chunk
-// against about 600 of draining), by the reduction and the stores for K of a
-// few hundred. Planes are numbered outermost, so one plane's panels stay in
+// as bytes (reducing every chunk in float32 instead costs 9 % at n = 8192). Bound by the
+// tensor cores for long K, by the epilogue and the stores for K of a few
+// hundred. Planes are numbered outermost, so one plane's panels stay in
 // L2 while its blocks are formed.
 struct CrtGemmParams {
   const uint32_t* tiles;   // blocks I (bits 0-14), J (bits 15-29)
@@ -2191,8 +2187,15 @@ struct CrtGemmParams {
   int ldt;
   unsigned* status;
   int debug_withhold_load;
-  uint32_t mod[CRT_MAX], magic[CRT_MAX], inv[CRT_MAX], bias[CRT_MAX];
+  uint32_t mod[CRT_MAX], magic[CRT_MAX], bias[CRT_MAX];
 };
+
+// The byte (residue + 128) of an int32 sum, |sum| < 2^30; bias a multiple of p not below 2^30
+__device__ __forceinline__ uint32_t crt_byte_of_sum(int sum, uint32_t p, uint32_t magic, uint32_t bias) {
+  const uint32_t x = (uint32_t)sum + bias;
+  const uint32_t t = x - (__umulhi(x, magic) >> 7) * p;   // sum mod p
+  return t + 128u - (t > 127u ? p : 0u);
+}
 
 template <int NCH>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(S2_THREADS, 1)
@@ -2323,6 +2326,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(S2_THREADS, 1)
     int tc = 0;
     bool ok = true;
     for (int u = cid; u < p.num_units && ok; u += ncl) {
+      const int l = u / p.nblocks;
       int sum[NCH][32];
 #pragma unroll
       for (int c = 0; c < NCH; ++c)
@@ -2348,9 +2352,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(S2_THREADS, 1)
         if (lane == 0) mbar_arrive_cluster(lead_bar0 + 8u * (2 * S2_STAGES + 2 + acc));
       }
       if (!ok) break;
-      const int l = u / p.nblocks;
-      const uint32_t td = p.tiles[u - l * p.nblocks];
-      const uint32_t mod = p.mod[l], magic = p.magic[l], inv = p.inv[l], bias = p.bias[l];
+      const uint32_t td = p.tiles[u - l * p.nblocks], mod = p.mod[l], magic = p.magic[l], bias = p.bias[l];
       const int r = (int)(td & 0x7FFF) * 256 + (int)rank * 128 + q * 32 + lane;
       uint8_t* out = p.t + (size_t)l * p.tplane + (size_t)r * p.ldt + (size_t)((td >> 15) & 0x7FFF) * p.bn +
                      half * (NCH * 32);
@@ -2361,9 +2363,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(S2_THREADS, 1)
         for (int e = 0; e < 8; ++e) {
           uint32_t b[4];
 #pragma unroll
-          for (int h = 0; h < 4; ++h)
-            b[h] = crt_mod31(crt_mod31((uint32_t)sum[c][4 * e + h] + bias, mod, magic) * inv, mod, magic);
-          w[e] = b[0] | (b[1] << 8) | (b[2] << 16) | (b[3] << 24);
+          for (int h = 0; h < 4; ++h) b[h] = crt_byte_of_sum(sum[c][4 * e + h], mod, magic, bias);
+          w[e] = crt_pack(b[0], b[1], b[2], b[3]);
         }
         // 32 columns: one 32-byte sector per lane and store
         asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(out + c * 32), "r"(w[0]), "r"(w[1]),
@@ -3162,8 +3163,7 @@ int tc_square_grouped_pairs(cdl_ctx* ctx, const TcGroup* host_first, const TcGro
   return L.done();
 }
 
-// Residue products t[l] = ((A_l B_l^T) mod p_l) inv_l mod p_l of `planes`
-// planes. a_planes: planes x a_rows x K bf16 (a_rows a multiple of 256, K of
+// Residue products t[l] = (A_l B_l^T mod p_l) + 128 of `planes` planes. a_planes: planes x a_rows x K bf16 (a_rows a multiple of 256, K of
 // 64); b_planes: planes x b_rows x K, or null for B = A, of which only the
 // 256 x 256 blocks on and above the diagonal are formed. t: planes x a_rows x
 // (b_rows or a_rows) bytes, 32-byte aligned.
@@ -3240,7 +3240,6 @@ int crt_gemm(cdl_ctx* ctx, const void* a_planes, int a_rows, const void* b_plane
   for (int l = 0; l < planes; ++l) {
     p.mod[l] = (uint32_t)CRT_MOD[l];
     p.magic[l] = crt_magic(CRT_MOD[l]);
-    p.inv[l] = (uint32_t)crt_inverse(planes, l);
     p.bias[l] = (uint32_t)(((1u << 30) + CRT_MOD[l] - 1) / CRT_MOD[l] * CRT_MOD[l]);
   }
   const int clusters = std::min(p.num_units, pair_clusters(ctx));
@@ -3616,10 +3615,8 @@ int dist_residues_tc(cdl_ctx* ctx, const void* planes, const int* ex, const void
   p.idesc = make_idesc(DS_N);
   p.status = ctx->dev_status;
   for (int l = 0; l < 16; ++l) {
-    p.mod[l] = (uint32_t)CRT_MOD[l];
-    p.magic[l] = crt_magic(CRT_MOD[l]);
-    p.inv[l] = (uint32_t)crt_inverse(16, l);
-    p.bias[l] = (uint32_t)(((1u << 30) + CRT_MOD[l] - 1) / CRT_MOD[l] * CRT_MOD[l]);
+    p.mod[l] = (float)CRT_MOD[l];
+    p.rmod[l] = 1.0f / (float)CRT_MOD[l];
   }
   CUtensorMap ma, mb;
   CDL_TRY(make_map(&ma, planes, (int64_t)16 * rows, kp, 128));

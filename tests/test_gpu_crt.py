@@ -12,7 +12,8 @@ from workloads import iid_pair   # noqa: E402
 
 pytestmark = pytest.mark.gpu
 
-# unit roundoff; half a unit of 2^-B of the row norm per entry with B >= 60.6 (16 moduli) and 29.7 (8)
+# unit roundoff; a bound on the rows' rounding, half a unit of 2^-59.9 (16 moduli) or 2^-29.5 (8) of the row
+# norm at most per entry (errors of one sign in every entry do not occur)
 TYPES = {"f64": (np.float64, 2.0 ** -53, 2.0 ** -60), "f32": (np.float32, 2.0 ** -24, 2.0 ** -29)}
 
 
