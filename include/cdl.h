@@ -395,13 +395,16 @@ int cdl_chain_solve(cdl_ctx* ctx, const cdl_chain* chain, const void* A, cdl_dty
  * The commute-time difference is formed as (a_i - a_j).(b_i - b_j) with
  * a = sqrt(vol2) Z2 - sqrt(vol1) Z1 and b = sqrt(vol2) Z2 + sqrt(vol1) Z1,
  * which avoids cancelling two large commute times.
- * score_dtype: CDL_F64 forms the k-term products and sums in float64;
- *   CDL_F32 forms them on the float32 pipes (much faster on this GPU):
- *   a and b split per column into hi + lo with hi on a fixed grid (23 bits
- *   of the column maximum, so hi_i - hi_j is exact), products made exact by
- *   fused multiply-add and the k-term sum compensated (TwoSum); each
- *   difference c_2 - c_1 is within about 2^-44 sum_r |a_ir - a_jr||b_ir -
- *   b_jr| even where the k terms cancel. Scores accumulate in float64.
+ * score_dtype: CDL_F64 and CDL_F32 round the rows [g a | b] (g a power of
+ *   two) to 2^-60 and 2^-49 of their 2-norm and form c_2 - c_1 of the rounded
+ *   rows exactly, through residues on the tensor cores; edge scores and sums
+ *   in float64. Where that form's workspace is not to be had, and in
+ *   cdl_cad_score_changed: CDL_F64 forms the k-term products and sums in
+ *   float64; CDL_F32 forms them on the float32 pipes, a and b split per column
+ *   into hi + lo with hi on a fixed grid (23 bits of the column maximum, so
+ *   hi_i - hi_j is exact), products made exact by fused multiply-add and the
+ *   k-term sum compensated (TwoSum): within about 2^-44 sum_r |a_ir - a_jr|
+ *   |b_ir - b_jr| even where the k terms cancel. Scores accumulate in float64.
  *   CDL_BF16 forms the k-term sums on the bf16 tensor cores, exactly:
  *   c_2 - c_1 = d_i + d_j - M_ij with d_i = a_i.b_i and M_ij = a_i.b_j +
  *   b_i.a_j, M from six exact bf16 slices of [a/g | b g] and [b g | a/g] (g a

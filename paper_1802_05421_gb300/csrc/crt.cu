@@ -27,6 +27,8 @@
 // identity the rounding of the rows would then exceed a dot product's.
 #include <algorithm>
 
+#include <cuda_bf16.h>
+
 #include "crt.cuh"
 #include "internal.h"
 #include "tiles.cuh"
@@ -196,7 +198,7 @@ struct Combine<double> {
   static constexpr int NP = 16;
   // c from the bytes at bit `sh` of the 16 words
   static __device__ __forceinline__ double value(const uint32_t (&w)[16], int sh, int e) {
-    return i128_to_double(crt16_value(w, sh), e);
+    return i128_to_double(crt_value<16>(w, sh), e);
   }
   static __device__ __forceinline__ double nan() { return __longlong_as_double(0x7FF8000000000000ll); }
 };
@@ -359,6 +361,134 @@ __global__ void __launch_bounds__(128) k_series_residues(const double* __restric
     nn = 0;
     for (int w = 0; w < 4; ++w) nn += ((u128)wn[w].y << 64) | wn[w].x;
     norms[row] = make_ulonglong2((unsigned long long)nn, (unsigned long long)(nn >> 64));
+  }
+}
+
+// ---- CAD scores (k_tc_gramr): a = sqrt(vol2) Z2 - sqrt(vol1) Z1, b = sqrt(vol2)
+// Z2 + sqrt(vol1) Z1 in float64.
+__device__ __forceinline__ void score_ab(const double* __restrict__ Z1, const double* __restrict__ Z2, double s1,
+                                         double s2, size_t o, double& a, double& b) {
+  const double w = s2 * Z2[o], v = s1 * Z1[o];
+  a = w - v;
+  b = w + v;
+}
+
+// Largest |a| and |b| (exponents of their float64 bit patterns): mx[0], mx[1].
+__global__ void __launch_bounds__(256) k_score_maxima(const double* __restrict__ Z1, const double* __restrict__ Z2,
+                                                       const double* __restrict__ vol1,
+                                                       const double* __restrict__ vol2, size_t cnt,
+                                                       int* __restrict__ mx) {
+  const double s1 = sqrt(*vol1), s2 = sqrt(*vol2);
+  int ea = 0, eb = 0;
+  for (size_t o = blockIdx.x * (size_t)256 + threadIdx.x; o < cnt; o += (size_t)gridDim.x * 256) {
+    double a, b;
+    score_ab(Z1, Z2, s1, s2, o, a, b);
+    ea = max(ea, (int)(LevelType<double>::mag(a) >> 52));
+    eb = max(eb, (int)(LevelType<double>::mag(b) >> 52));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    ea = max(ea, __shfl_xor_sync(0xffffffffu, ea, o));
+    eb = max(eb, __shfl_xor_sync(0xffffffffu, eb, o));
+  }
+  if ((threadIdx.x & 31) == 0) {
+    atomicMax(mx, ea);
+    atomicMax(mx + 1, eb);
+  }
+}
+
+// Row i: u_i = [g a_i | b_i] of 2-norm 2^B at most (B = crt_norm_bits) after the
+// power of two 2^{e_i}, rounded to integers, as NP residue planes of u and of v
+// = [b_i | g a_i] (rows x kp, zero padded), and d'_i = (g a_i) . b_i of the
+// integers, exact. g = 2^gexp brings the largest |a| to the binade of the
+// largest |b| (gexp = mx[1] - mx[0] is left in mx[2]). A block of 128 per row.
+template <int NP>
+__global__ void __launch_bounds__(128) k_score_residues(const double* __restrict__ Z1, const double* __restrict__ Z2,
+                                                         const double* __restrict__ vol1,
+                                                         const double* __restrict__ vol2, int n, int k, int rows,
+                                                         int kp, int* __restrict__ mx, int* __restrict__ ex,
+                                                         ulonglong2* __restrict__ dself,
+                                                         __nv_bfloat16* __restrict__ up,
+                                                         __nv_bfloat16* __restrict__ vp) {
+  typedef LevelType<double> LT;
+  __shared__ unsigned long long wmax[4];
+  __shared__ float wsum[4];
+  __shared__ ulonglong2 wn[4];
+  const int row = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const double s1 = sqrt(*vol1), s2 = sqrt(*vol2);
+  // zero or non-finite maxima: no balancing
+  const int ea = mx[0], eb = mx[1], ge = ea > 0 && eb > 0 && ea < 0x7FF && eb < 0x7FF ? eb - ea : 0;
+  if (row == 0 && tid == 0) mx[2] = ge;
+  const int cols = row < n ? k : 0;
+  // magnitudes as exponents relative to g: |g a| is compared through the exponent field
+  unsigned long long m = 0;
+  for (int r = tid; r < cols; r += 128) {
+    double a, b;
+    score_ab(Z1, Z2, s1, s2, (size_t)row * k + r, a, b);
+    m = max(m, max(LT::mag(scalbn(a, ge)), LT::mag(b)));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (lane == 0) wmax[warp] = m;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < 4; ++w) m = max(m, wmax[w]);
+  const bool fin = LT::finite(m);
+  const int emax = LT::exponent(m) - LT::BIAS + 52;
+  float s = 0.f;
+  if (fin)
+    for (int r = tid; r < cols; r += 128) {
+      double a, b;
+      score_ab(Z1, Z2, s1, s2, (size_t)row * k + r, a, b);
+      const float x = (float)(int)scaled_int(a, 22 - emax + ge), y = (float)(int)scaled_int(b, 22 - emax);
+      s = __fmaf_rn(x, x, __fmaf_rn(y, y, s));
+    }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) wsum[warp] = s;
+  __syncthreads();
+  s = wsum[0] + wsum[1] + wsum[2] + wsum[3];
+  const bool any = fin && s >= 1.f;
+  const int e = any ? (int)floorf(crt_norm_bits(NP) - 0.02f - 0.5f * log2f(s)) + 22 - emax : CRT_ROW_ZERO;
+  if (tid == 0) ex[row] = fin ? e : CRT_ROW_NAN;
+  const size_t plane = (size_t)rows * kp;
+  __nv_bfloat16 *u = up + (size_t)row * kp, *v = vp + (size_t)row * kp;
+  __int128 dd = 0;
+  for (int r = tid; r < k; r += 128) {
+    long long x = 0, y = 0;
+    if (any && r < cols) {
+      double a, b;
+      score_ab(Z1, Z2, s1, s2, (size_t)row * k + r, a, b);
+      x = scaled_int(a, e + ge);
+      y = scaled_int(b, e);
+      dd += (__int128)x * y;
+    }
+#pragma unroll
+    for (int l = 0; l < NP; ++l) {
+      const uint32_t rx = residue_bits<double>((int)(x & 0x1FFFFF), (int)(x >> 21) & 0x1FFFFF, (int)(x >> 42), l),
+                     ry = residue_bits<double>((int)(y & 0x1FFFFF), (int)(y >> 21) & 0x1FFFFF, (int)(y >> 42), l);
+      const __nv_bfloat16 bx = __ushort_as_bfloat16((unsigned short)(rx >> 16)),
+                          by = __ushort_as_bfloat16((unsigned short)(ry >> 16));
+      u[l * plane + r] = bx;
+      u[l * plane + k + r] = by;
+      v[l * plane + r] = by;
+      v[l * plane + k + r] = bx;
+    }
+  }
+  for (int r = 2 * k + tid; r < kp; r += 128)
+    for (int l = 0; l < NP; ++l) u[l * plane + r] = v[l * plane + r] = __ushort_as_bfloat16(0);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long lo = __shfl_xor_sync(0xffffffffu, (unsigned long long)(u128)dd, o);
+    const unsigned long long hi = __shfl_xor_sync(0xffffffffu, (unsigned long long)((u128)dd >> 64), o);
+    dd += (__int128)(((u128)hi << 64) | lo);
+  }
+  if (lane == 0) wn[warp] = make_ulonglong2((unsigned long long)(u128)dd, (unsigned long long)((u128)dd >> 64));
+  __syncthreads();
+  if (tid == 0) {
+    u128 t = 0;
+    for (int w = 0; w < 4; ++w) t += ((u128)wn[w].y << 64) | wn[w].x;
+    dself[row] = make_ulonglong2((unsigned long long)t, (unsigned long long)(t >> 64));
   }
 }
 
@@ -545,6 +675,47 @@ int series_residues(cdl_ctx* ctx, const double* X, int n, int T, int rows, int k
                                                    static_cast<uint32_t*>(planes), static_cast<uint32_t*>(bad),
                                                    bad_words);
   return L.done();
+}
+
+int score_pairs_residues(cdl_ctx* ctx, const double* Z1, const double* Z2, const double* vol1, const double* vol2,
+                         int n, int k, bool fp64, const double* A1, const double* A2, double* contrib, double* E) {
+  const int planes = fp64 ? 16 : 13;
+  const int rows = (n + 127) / 128 * 128, kp = (2 * k + 63) / 64 * 64;
+  if (!tc_supported(ctx)) return CDL_ERR_UNSUPPORTED;
+  const size_t cnt = (size_t)planes * rows * kp;
+  void *vu, *vv, *vd, *ve, *vm;
+  if (ws_get(ctx, "crt.score.u", cnt * 2, &vu) != CDL_OK || ws_get(ctx, "crt.score.v", cnt * 2, &vv) != CDL_OK ||
+      ws_get(ctx, "crt.score.d", (size_t)rows * 16, &vd) != CDL_OK ||
+      ws_get(ctx, "crt.score.e", (size_t)rows * sizeof(int), &ve) != CDL_OK ||
+      ws_get(ctx, "crt.score.max", 16, &vm) != CDL_OK) {
+    ws_reclaim(ctx);
+    return CDL_ERR_UNSUPPORTED;
+  }
+  int *mx = static_cast<int*>(vm), *ex = static_cast<int*>(ve);
+  CDL_CUDA_TRY(cudaMemsetAsync(mx, 0, 16, ctx->stream));
+  {
+    Launch L(ctx, CDL_KC_MISC, 0);
+    const size_t nk = (size_t)n * k;
+    k_score_maxima<<<(unsigned)std::min<size_t>((nk + 255) / 256, (size_t)ctx->sm_count * 8), 256, 0, ctx->stream>>>(
+        Z1, Z2, vol1, vol2, nk, mx);
+    CDL_TRY(L.done());
+  }
+  {
+    Launch L(ctx, CDL_KC_MISC, 0);
+    if (fp64)
+      k_score_residues<16><<<rows, 128, 0, ctx->stream>>>(Z1, Z2, vol1, vol2, n, k, rows, kp, mx, ex,
+                                                          static_cast<ulonglong2*>(vd),
+                                                          static_cast<__nv_bfloat16*>(vu),
+                                                          static_cast<__nv_bfloat16*>(vv));
+    else
+      k_score_residues<13><<<rows, 128, 0, ctx->stream>>>(Z1, Z2, vol1, vol2, n, k, rows, kp, mx, ex,
+                                                          static_cast<ulonglong2*>(vd),
+                                                          static_cast<__nv_bfloat16*>(vu),
+                                                          static_cast<__nv_bfloat16*>(vv));
+    CDL_TRY(L.done());
+  }
+  return score_residues_tc(ctx, vu, vv, planes, ex, vd, mx + 2, n, rows, kp, A1, A2, contrib, E,
+                           8.0 * (double)n * (n - 1));
 }
 
 }  // namespace cdl

@@ -51,8 +51,8 @@ constexpr int crt_pow2_mod(int k, int p) {
 }
 
 // 2^B with 2 B <= log2(P / 4) less a rounding margin: log2 P is 63.09 for 8
-// moduli and 123.98 for 16
-constexpr float crt_norm_bits(int np) { return np == 8 ? 30.52f : 60.96f; }
+// moduli, 101.42 for 13 and 123.98 for 16
+constexpr float crt_norm_bits(int np) { return np == 8 ? 30.52f : np == 13 ? 49.68f : 60.96f; }
 
 constexpr int CRT_ROW_NAN = 0x40000000;   // e_i of a row with a non-finite entry
 constexpr int CRT_ROW_ZERO = 0x4000;      // of a zero row, where no other row's units may be coarsened by it
@@ -67,17 +67,19 @@ constexpr uint32_t crt_frac(int np, int l) {
   return (uint32_t)(((unsigned)crt_inverse(np, l) * (1u << 20) + (unsigned)CRT_MOD[l]) / (2u * (unsigned)CRT_MOD[l]));
 }
 
-// 16 moduli: W_l in 32-bit limbs (below 2^124) and as fractions; the constants
-// that take out the bytes' offset of 128
-struct CombineTab64 {
-  uint32_t limb[4][CRT_MAX];
-  uint32_t frac[CRT_MAX];
+// W_l in 32-bit limbs (16 moduli: below 2^124; 13: below 2^102) and as fractions;
+// the constants that take out the bytes' offset of 128
+template <int NP>
+struct CombineTab {
+  uint32_t limb[4][NP];
+  uint32_t frac[NP];
 };
-constexpr CombineTab64 make_combine64() {
-  CombineTab64 t{};
-  for (int l = 0; l < 16; ++l) {
-    for (int k = 0; k < 4; ++k) t.limb[k][l] = (uint32_t)(crt_weight(16, l) >> (32 * k));
-    t.frac[l] = crt_frac(16, l);
+template <int NP>
+constexpr CombineTab<NP> make_combine() {
+  CombineTab<NP> t{};
+  for (int l = 0; l < NP; ++l) {
+    for (int k = 0; k < 4; ++k) t.limb[k][l] = (uint32_t)(crt_weight(NP, l) >> (32 * k));
+    t.frac[l] = crt_frac(NP, l);
   }
   return t;
 }
@@ -91,7 +93,8 @@ constexpr uint32_t crt_frac_offset(int np) {
   for (int l = 0; l < np; ++l) s += 128 * crt_frac(np, l);
   return s;
 }
-__constant__ CombineTab64 c_comb64 = make_combine64();
+__constant__ CombineTab<16> c_comb16 = make_combine<16>();
+__constant__ CombineTab<13> c_comb13 = make_combine<13>();
 
 // v modulo p as the nearest representative, v an integer of at most 2^24 in
 // magnitude: the quotient is off by at most 2 / p from v / p, so the result is
@@ -107,19 +110,22 @@ __device__ __forceinline__ uint32_t crt_pack(uint32_t b0, uint32_t b1, uint32_t 
 }
 
 // The integer c, |c| <= P / 4, from the bytes (residue + 128) at bit `sh` of the words
-__device__ __forceinline__ __int128 crt16_value(const uint32_t (&w)[16], int sh) {
-  constexpr u128 P = crt_product(16), off = crt_offset(16);
+template <int NP>
+__device__ __forceinline__ __int128 crt_value(const uint32_t (&w)[NP], int sh) {
+  static_assert(NP == 16 || NP == 13, "tables of 16 and 13 moduli");
+  constexpr u128 P = crt_product(NP), off = crt_offset(NP);
   constexpr unsigned long long PH = (unsigned long long)(P >> 64), PL = (unsigned long long)P,
                                OH = (unsigned long long)(off >> 64), OL = (unsigned long long)off;
-  constexpr uint32_t f0 = crt_frac_offset(16);
+  constexpr uint32_t f0 = crt_frac_offset(NP);
   unsigned long long S[4] = {0, 0, 0, 0};
   uint32_t f = 0;
 #pragma unroll
-  for (int l = 0; l < 16; ++l) {
+  for (int l = 0; l < NP; ++l) {
     const uint32_t t = (w[l] >> sh) & 0xFFu;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) S[k] += (unsigned long long)t * c_comb64.limb[k][l];   // below 2^44
-    f += t * c_comb64.frac[l];
+    for (int k = 0; k < 4; ++k)   // below 2^44
+      S[k] += (unsigned long long)t * (NP == 16 ? c_comb16.limb[k][l] : c_comb13.limb[k][l]);
+    f += t * (NP == 16 ? c_comb16.frac[l] : c_comb13.frac[l]);
   }
   const int q = (int)(f - f0 + (1u << 18)) >> 19;   // round(sum r_l W_l / P): |c| <= P / 4 leaves no doubt
   u128 c = (u128)S[0] + ((u128)S[1] << 32) + ((u128)S[2] << 64) + ((u128)S[3] << 96);
@@ -127,16 +133,31 @@ __device__ __forceinline__ __int128 crt16_value(const uint32_t (&w)[16], int sh)
   return (__int128)c;
 }
 
+// v >> s for 0 <= s < 32, the sign kept
+__device__ __forceinline__ __int128 i128_shr(__int128 v, int s) {
+  const unsigned w0 = (unsigned)v, w1 = (unsigned)(v >> 32), w2 = (unsigned)(v >> 64), w3 = (unsigned)(v >> 96);
+  const unsigned long long lo =
+      (unsigned long long)__funnelshift_r(w1, w2, s) << 32 | __funnelshift_r(w0, w1, s);
+  const unsigned long long hi = (unsigned long long)(unsigned)((int)w3 >> s) << 32 | __funnelshift_r(w2, w3, s);
+  return (__int128)(((u128)hi << 64) | lo);
+}
+
 // v 2^-e rounded to nearest even, v a signed 128-bit integer
 __device__ __forceinline__ double i128_to_double(__int128 v, int e) {
   if (v == 0) return 0.0;
   const bool neg = v < 0;
   const u128 a = neg ? (u128)(-v) : (u128)v;
-  const unsigned long long hi = (unsigned long long)(a >> 64), lo = (unsigned long long)a;
-  const int z = hi ? __clzll((long long)hi) : 64 + __clzll((long long)lo);
-  const u128 n = a << z;                                  // leading bit 127
-  const unsigned long long top = (unsigned long long)(n >> 64);
-  const bool sticky = (unsigned long long)n != 0;
+  unsigned long long hi = (unsigned long long)(a >> 64), lo = (unsigned long long)a;
+  int z = 0;
+  if (hi == 0) {
+    hi = lo;
+    lo = 0;
+    z = 64;
+  }
+  const int y = __clzll((long long)hi);                   // leading bit to 127
+  z += y;
+  const unsigned long long top = (hi << y) | ((lo >> 1) >> (63 - y));
+  const bool sticky = (lo << y) != 0;
   unsigned long long q = top >> 11;
   const unsigned long long rem = top & 0x7FFull;
   if (rem > 0x400ull || (rem == 0x400ull && (sticky || (q & 1)))) ++q;   // may carry to 2^53: exact below

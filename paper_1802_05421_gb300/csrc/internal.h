@@ -303,6 +303,14 @@ int dist_tc(cdl_ctx* ctx, const void* planes, const long long* norms, int n, int
 constexpr int DIST_RES_MIN_T = 16;
 int series_residues(cdl_ctx* ctx, const double* X, int n, int T, int rows, int kp, const int* offgrid, int* ex,
                     void* norms, void* planes, void* bad, int bad_words);
+// Pair partials of the CAD scores (as score_tc's contrib) and, if E is given,
+// the edge scores of the upper triangle, with the products through residues
+// (crt.cu); CDL_ERR_UNSUPPORTED where its workspace is not to be had.
+int score_pairs_residues(cdl_ctx* ctx, const double* Z1, const double* Z2, const double* vol1, const double* vol2,
+                         int n, int k, bool fp64, const double* A1, const double* A2, double* contrib, double* E);
+int score_residues_tc(cdl_ctx* ctx, const void* u, const void* v, int planes, const int* ex, const void* dself,
+                      const int* gexp, int n, int rows, int kp, const double* A1, const double* A2, double* contrib,
+                      double* E, double work);
 int dist_residues_tc(cdl_ctx* ctx, const void* planes, const int* ex, const void* norms, int n, int T, int rows, int kp,
                      double* A, const int* offgrid, void* bad);
 // Pair partials of the CAD scores with the Gram on the tensor cores: uplanes,

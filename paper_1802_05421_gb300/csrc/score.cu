@@ -1267,20 +1267,22 @@ int cad_score(cdl_ctx* ctx, const double* A1, const double* A2, const double* Z1
     CDL_TRY(tc_score_prepare(ctx, Z1, Z2, vol1, vol2, n, k, q));
     CDL_TRY(score_tc(ctx, q.u, q.v, q.d, q.oscale, n, q.rows, q.k2p, A1, A2, static_cast<double*>(vc)));
   } else {
-  CDL_TRY(score_prepare(ctx, Z1, Z2, vol1, vol2, n, k, fp64, &vab));
-  const long long tiles = (long long)nb * (nb + 1) / 2;
-  if (fp64) {
-    const double* aT = static_cast<const double*>(vab);
-    Launch L(ctx, CDL_KC_SCORE, 8.0 * (double)n * (n - 1));
-    k_score_pairs64<<<(unsigned)tiles, 256, 0, st>>>(A1, A2, aT, aT + nk, n, k, static_cast<double*>(vc));
-    CDL_TRY(L.done());
-  } else {
-    const float* ah = static_cast<const float*>(vab);
-    Launch L(ctx, CDL_KC_SCORE, 8.0 * (double)n * (n - 1));
-    k_score_pairs<<<(unsigned)tiles, 256, 0, st>>>(A1, A2, ah, ah + nk, ah + 2 * nk, ah + 3 * nk, n, k,
-                                                   static_cast<double*>(vc));
-    CDL_TRY(L.done());
-  }
+    const int rc = score_pairs_residues(ctx, Z1, Z2, vol1, vol2, n, k, fp64, A1, A2, static_cast<double*>(vc), nullptr);
+    if (rc != CDL_ERR_UNSUPPORTED) CDL_TRY(rc);
+    if (rc == CDL_ERR_UNSUPPORTED) {   // no workspace: on the CUDA cores
+      CDL_TRY(score_prepare(ctx, Z1, Z2, vol1, vol2, n, k, fp64, &vab));
+      const long long tiles = (long long)nb * (nb + 1) / 2;
+      Launch L(ctx, CDL_KC_SCORE, 8.0 * (double)n * (n - 1));
+      if (fp64) {
+        const double* aT = static_cast<const double*>(vab);
+        k_score_pairs64<<<(unsigned)tiles, 256, 0, st>>>(A1, A2, aT, aT + nk, n, k, static_cast<double*>(vc));
+      } else {
+        const float* ah = static_cast<const float*>(vab);
+        k_score_pairs<<<(unsigned)tiles, 256, 0, st>>>(A1, A2, ah, ah + nk, ah + 2 * nk, ah + 3 * nk, n, k,
+                                                       static_cast<double*>(vc));
+      }
+      CDL_TRY(L.done());
+    }
   }
   {
     Launch L(ctx, CDL_KC_MISC, 0);
@@ -1303,7 +1305,6 @@ int cad_edges(cdl_ctx* ctx, const double* A1, const double* A2, const double* Z1
   cudaStream_t st = ctx->stream;
   const int nb = (n + ST - 1) / ST;
   void *vab, *vc, *vE, *vF, *vp, *vs, *vbuf, *vcnt, *voff;
-  CDL_TRY(score_prepare(ctx, Z1, Z2, vol1, vol2, n, k, fp64, &vab));
   CDL_TRY(ws_get(ctx, "score.contrib", (size_t)nb * n * sizeof(double), &vc));
   CDL_TRY(ws_get(ctx, "edges.E", (size_t)n * n * sizeof(double), &vE));
   CDL_TRY(ws_get(ctx, "edges.F", (size_t)n * sizeof(double), &vF));
@@ -1318,8 +1319,11 @@ int cad_edges(cdl_ctx* ctx, const double* A1, const double* A2, const double* Z1
   double* Fw = F ? F : static_cast<double*>(vF);
   U128* psum = static_cast<U128*>(vp);
   unsigned long long* pcnt = reinterpret_cast<unsigned long long*>(psum + (size_t)eb * EC_BINS);
-  const long long tiles = (long long)nb * (nb + 1) / 2;
-  {
+  const int rc = score_pairs_residues(ctx, Z1, Z2, vol1, vol2, n, k, fp64, A1, A2, static_cast<double*>(vc), E);
+  if (rc != CDL_ERR_UNSUPPORTED) CDL_TRY(rc);
+  if (rc == CDL_ERR_UNSUPPORTED) {   // no workspace: on the CUDA cores
+    CDL_TRY(score_prepare(ctx, Z1, Z2, vol1, vol2, n, k, fp64, &vab));
+    const long long tiles = (long long)nb * (nb + 1) / 2;
     Launch L(ctx, CDL_KC_SCORE, 8.0 * (double)n * (n - 1));
     k_edge_pairs<<<(unsigned)tiles, 256, 0, st>>>(A1, A2, vab, n, k, fp64 ? 1 : 0, static_cast<double*>(vc), E);
     CDL_TRY(L.done());

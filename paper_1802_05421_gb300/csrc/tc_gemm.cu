@@ -1180,75 +1180,110 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
   }
 }
 
-// ---------------------------------------------------------------- distances of series on no grid
-// d2_ij of float64 series off the 2^-16 grid, through residues (crt.cuh): row i
-// of the series less the series of node 0 is 2^-e_i times integers x'_i of norm
-// 2^60.96 at most, rounded to one unit (k_series_residues); the Gram entry x'_i .
-// x'_j is formed exactly from 16 residue products on the bf16 tensor cores, and
-// d2' = |x'_i|^2 + |x'_j|^2 - 2 x'_i . x'_j in 128-bit integers, in units of the
-// coarser of the two rows, rounded once to float64. With d2' >= 2^109 the
-// rounding of the series is below 2^-54 of d2 (rms 0.6 units per sample and
-// pair, so 1.2 / sqrt(d2') relative), where a float64 sum of rounded squares
-// has about sqrt(T) 2^-54: tiles with a smaller entry (a distance below 2^-6
-// of the nodes' distances to node 0, duplicates, non-finite series) are
-// flagged and formed by the float64 kernel, as before.
+// ---------------------------------------------------------------- Gram matrices through residues
+// Exact integer Gram matrices g_ij = x_i . y_j over the upper block triangle,
+// from NP residue planes of the rows x (U) and y (V) on the bf16 tensor cores
+// (crt.cuh), and what is made of them in the epilogue:
 //
-// 128 x 64 tiles of the upper block triangle, warp roles as in k_tc_dist. Planes
-// run one after the other through a ring of eight 64-column accumulators (at
-// most 1024 samples each: exact); an epilogue thread reduces its 16 columns of
-// one row modulo p_l into bytes kept in shared memory, and after the last
-// plane puts its entries together four columns at a time. Bound by the
-// epilogue's integer arithmetic (about 11 operations per entry and plane to
-// reduce, 10 to combine). n = 8192, T = 128: 0.97 ms, and 0.03 for the series'
-// residues, where the float64 pipe took 24.9 ms.
-constexpr int DR_STAGES = 3;
-constexpr int DR_STAGE_BYTES = DS_A + DS_B;
-constexpr int DR_WORDS = 16 * 4 * 32;                  // per epilogue warp: 16 columns of 32 rows, 16 planes
-constexpr int DR_SMEM_BYTES = DR_STAGES * DR_STAGE_BYTES + 512 + 16 * DR_WORDS * 4 + 1024;
-constexpr int DR_NBUF = 8;
+// GR_DIST  squared distances of float64 series off the 2^-16 grid. Row i of the
+//   series less the series of node 0 is 2^-e_i times integers x'_i of norm
+//   2^60.96 at most, rounded to one unit (k_series_residues); d2' = |x'_i|^2 +
+//   |x'_j|^2 - 2 x'_i . x'_j in 128-bit integers, in units of the coarser of the
+//   two rows, rounded once to float64. With d2' >= 2^109 the rounding of the
+//   series is below 2^-54 of d2 (rms 0.6 units per sample and pair, so 1.2 /
+//   sqrt(d2') relative), where a float64 sum of rounded squares has about
+//   sqrt(T) 2^-54: tiles with a smaller entry (a distance below 2^-6 of the
+//   nodes' distances to node 0, duplicates, non-finite series) are flagged and
+//   formed by the float64 kernel.
+//
+// GR_SCORE  CAD edge scores and their sums. With a and b as in k_tc_score, u_i =
+//   [g a_i | b_i] and v_i = [b_i | g a_i] (g one power of two that balances the
+//   halves) as integers of one exponent per row (k_score_residues), Delta c_ij =
+//   d_i + d_j - u_i . v_j with d_i = g a_i . b_i exact, in 128-bit integers, rounded
+//   once; E_ij = |A1_ij - A2_ij| |Delta c_ij| and its row and column sums in
+//   float64. 16 moduli for float64 scores (rows to 2^-60 of their norm), 13
+//   for float32 ones (2^-49; 12, 2^-45, came out up to four times further off
+//   than the float32 pipes' split).
+//
+// 128 x 64 tiles, warp roles as in k_tc_dist. Planes run one after the other
+// through a ring of four 64-column accumulators (at most 1024 of K each:
+// exact); an epilogue thread reduces its 16 columns of one row modulo p_l into
+// bytes, kept in the other half of TMEM (256 columns: 16 words per plane and
+// lane for the four column parts), so that shared memory holds six operand
+// stages; after the last plane it puts its entries together four columns at a
+// time. Bound by the epilogue: of 950 us for the distances at n = 8192, K = 128,
+// 260 went to the sums over the moduli, 120 to 128-bit shifts and the
+// conversion, 70 to the reduction; three or six operand stages make no
+// difference. Measured: distances n = 8192, T = 128 912 us (24.9 ms on the
+// float64 pipe); float32 scores n = 8192, k = 64 969 us (1460 on the float32
+// pipes), float64 edge scores n = 4001, k = 32 266 us (1594 on the float64 pipe).
+enum { GR_DIST = 0, GR_SCORE = 1 };
+constexpr int GR_STAGES = 6;
+constexpr int GR_STAGE_BYTES = DS_A + DS_B;
+constexpr int GR_NBUF = 4;
+constexpr int GR_WORDS_COL = GR_NBUF * DS_N;              // TMEM columns 256 .. 511
+constexpr int GR_XP = 16 * 33;                            // per epilogue warp: 16 columns x 32 rows, padded
+constexpr int GR_PARTS = 128 * 4 + 4 * DS_N;              // row and column partials of a tile, double-buffered
+constexpr int GR_SMEM_BYTES = GR_STAGES * GR_STAGE_BYTES + 512 + (16 * GR_XP + 2 * GR_PARTS) * 8 + 1024;
+static_assert(GR_SMEM_BYTES <= 232448, "shared memory of a block");
 
-struct DistResParams {
+struct GramParams {
   int nb128, nb64, num_tiles;
   int rows;                   // of one plane
   int kblocks;                // 0: nothing to do (every tile is flagged)
   int n;
-  const int* ex;
-  const ulonglong2* norms;
-  double* A;
-  const int* offgrid;
-  unsigned char* bad;         // per 64 x 64 block (bi, bj), bi <= bj: at bi nb64 + bj
+  const int* ex;              // row exponents
+  const ulonglong2* self;     // |x'_i|^2 (GR_DIST) or d'_i (GR_SCORE, signed), 128 bits
   uint32_t idesc;
   unsigned* status;
   float mod[CRT_MAX], rmod[CRT_MAX];   // p_l and 1 / p_l
+  // GR_DIST
+  double* A;
+  const int* offgrid;
+  unsigned char* bad;         // per 64 x 64 block (bi, bj), bi <= bj: at bi nb64 + bj
+  // GR_SCORE
+  const double* A1;
+  const double* A2;
+  const int* gexp;            // log2 g
+  double* contrib;            // 64-node partner blocks x n, as k_tc_score
+  double* E;                  // edge scores of the upper triangle, or null
 };
 
+__device__ __forceinline__ void tmem_st1(uint32_t taddr, uint32_t v) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};" ::"r"(taddr), "r"(v) : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ __int128 i128_of(ulonglong2 v) { return (__int128)(((u128)v.y << 64) | v.x); }
+
+template <int MODE, int NP>
 __global__ void __launch_bounds__(T8_THREADS, 1)
-    k_tc_distr(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-               const DistResParams p) {
-  if (!(*p.offgrid & 1) || p.kblocks == 0) return;       // uniform: before any barrier or allocation
+    k_tc_gramr(const __grid_constant__ CUtensorMap tmU, const __grid_constant__ CUtensorMap tmV, const GramParams p) {
+  // uniform: before any barrier or allocation
+  if (MODE == GR_DIST && (!(*p.offgrid & 1) || p.kblocks == 0)) return;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + DR_STAGES * DR_STAGE_BYTES);
-  uint32_t* words = reinterpret_cast<uint32_t*>(smem + DR_STAGES * DR_STAGE_BYTES + 512);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * DR_STAGES + 2 * DR_NBUF + 2);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 2 * DR_STAGES + 2 * DR_NBUF + 3);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + GR_STAGES * GR_STAGE_BYTES);
+  double* xps = reinterpret_cast<double*>(smem + GR_STAGES * GR_STAGE_BYTES + 512);
+  double* parts = xps + 16 * GR_XP;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * GR_STAGES + 2 * GR_NBUF + 2);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 2 * GR_STAGES + 2 * GR_NBUF + 3);
   const uint32_t bar0 = smem_u32(bars);
   auto full_bar = [&](int s) { return bar0 + 8u * s; };
-  auto empty_bar = [&](int s) { return bar0 + 8u * (DR_STAGES + s); };
-  auto pfull_bar = [&](int b) { return bar0 + 8u * (2 * DR_STAGES + b); };
-  auto pempty_bar = [&](int b) { return bar0 + 8u * (2 * DR_STAGES + DR_NBUF + b); };
-  const uint32_t drain_bar = bar0 + 8u * (2 * DR_STAGES + 2 * DR_NBUF);
+  auto empty_bar = [&](int s) { return bar0 + 8u * (GR_STAGES + s); };
+  auto pfull_bar = [&](int b) { return bar0 + 8u * (2 * GR_STAGES + b); };
+  auto pempty_bar = [&](int b) { return bar0 + 8u * (2 * GR_STAGES + GR_NBUF + b); };
+  const uint32_t drain_bar = bar0 + 8u * (2 * GR_STAGES + 2 * GR_NBUF);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nchunks = (p.kblocks + CR_CHUNK_KB - 1) / CR_CHUNK_KB;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < DR_STAGES; ++s) {
+    for (int s = 0; s < GR_STAGES; ++s) {
       mbar_init(full_bar(s), 1);
       mbar_init(empty_bar(s), 1);
     }
-    for (int b = 0; b < DR_NBUF; ++b) {
+    for (int b = 0; b < GR_NBUF; ++b) {
       mbar_init(pfull_bar(b), 1);
-      mbar_init(pempty_bar(b), T8_EPI);
+      mbar_init(pempty_bar(b), 16);   // the epilogue warps
     }
     mbar_init(drain_bar, 1);
     *abort_flag = 0;
@@ -1256,7 +1291,7 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                 "r"(DR_NBUF * DS_N)
+                 "r"(512)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -1272,23 +1307,23 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
     for (int t = blockIdx.x; t < p.num_tiles && ok; t += gridDim.x) {
       int I, J;
       dist_tile(t, p.nb128, p.nb64, I, J);
-      for (int l = 0; l < 16 && ok; ++l)
+      for (int l = 0; l < NP && ok; ++l)
         for (int kb = 0; kb < p.kblocks; ++kb, ++it) {
-          const int s = it % DR_STAGES;
-          if (!mbar_wait(empty_bar(s), ((uint32_t)(it / DR_STAGES) & 1) ^ 1, abort_flag, p.status)) {
+          const int s = it % GR_STAGES;
+          if (!mbar_wait(empty_bar(s), ((uint32_t)(it / GR_STAGES) & 1) ^ 1, abort_flag, p.status)) {
             ok = false;
             break;
           }
-          const uint32_t dst = smem_u32(smem + s * DR_STAGE_BYTES);
-          mbar_expect_tx(full_bar(s), DR_STAGE_BYTES);
-          tma_load_2d(dst, &tmA, kb * 64, l * p.rows + I * 128, full_bar(s));
-          tma_load_2d(dst + DS_A, &tmB, kb * 64, l * p.rows + J * DS_N, full_bar(s));
+          const uint32_t dst = smem_u32(smem + s * GR_STAGE_BYTES);
+          mbar_expect_tx(full_bar(s), GR_STAGE_BYTES);
+          tma_load_2d(dst, &tmU, kb * 64, l * p.rows + I * 128, full_bar(s));
+          tma_load_2d(dst + DS_A, &tmV, kb * 64, l * p.rows + J * DS_N, full_bar(s));
         }
     }
     if (!ok) {
-      for (int j = (it > DR_STAGES ? it - DR_STAGES : 0); j < it; ++j) {
+      for (int j = (it > GR_STAGES ? it - GR_STAGES : 0); j < it; ++j) {
         const unsigned long long t0 = globaltimer();
-        while (!mbar_try_wait(full_bar(j % DR_STAGES), (uint32_t)(j / DR_STAGES) & 1) &&
+        while (!mbar_try_wait(full_bar(j % GR_STAGES), (uint32_t)(j / GR_STAGES) & 1) &&
                globaltimer() - t0 < WAIT_LIMIT_NS) {
         }
       }
@@ -1298,22 +1333,22 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
     int it = 0, pc = 0;
     bool ok = true, issued = false;
     for (int t = blockIdx.x; t < p.num_tiles && ok; t += gridDim.x)
-      for (int l = 0; l < 16 && ok; ++l)
+      for (int l = 0; l < NP && ok; ++l)
         for (int kb = 0; kb < p.kblocks; ++kb, ++it) {
-          const int b = pc % DR_NBUF;
+          const int b = pc % GR_NBUF;
           if (kb % CR_CHUNK_KB == 0) {
-            if (!mbar_wait(pempty_bar(b), ((uint32_t)(pc / DR_NBUF) & 1) ^ 1, abort_flag, p.status)) {
+            if (!mbar_wait(pempty_bar(b), ((uint32_t)(pc / GR_NBUF) & 1) ^ 1, abort_flag, p.status)) {
               ok = false;
               break;
             }
           }
-          const int s = it % DR_STAGES;
-          if (!mbar_wait(full_bar(s), (uint32_t)(it / DR_STAGES) & 1, abort_flag, p.status)) {
+          const int s = it % GR_STAGES;
+          if (!mbar_wait(full_bar(s), (uint32_t)(it / GR_STAGES) & 1, abort_flag, p.status)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t base = smem_u32(smem + s * DR_STAGE_BYTES);
+          const uint32_t base = smem_u32(smem + s * GR_STAGE_BYTES);
           const uint64_t adesc = smem_desc(base), bdesc = smem_desc(base + DS_A);
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk)
@@ -1337,21 +1372,23 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
     const int q = warp & 3;                              // TMEM lane quarter
     const int part = (warp - 2) >> 2;                    // 16-column part of the tile
     const uint32_t lane_off = (uint32_t)(q * 32) << 16;
-    uint32_t* tw = words + (warp - 2) * DR_WORDS;        // [quad of columns][plane][lane]
-    int pc = 0;
+    const uint32_t words = tmem_base + lane_off + (uint32_t)(GR_WORDS_COL + part * 64);   // + 16 quad + plane
+    double* xp = xps + (warp - 2) * GR_XP;
+    const int ge = MODE == GR_SCORE ? *p.gexp : 0;
+    int pc = 0, tpar = 0;
     bool failed = false;
     for (int t = blockIdx.x; t < p.num_tiles; t += gridDim.x) {
       int I, J;
       dist_tile(t, p.nb128, p.nb64, I, J);
-      for (int l = 0; l < 16; ++l) {
+#pragma unroll 1
+      for (int l = 0; l < NP; ++l) {
         const float mod = p.mod[l], rmod = p.rmod[l];
         float sum[16];
-#pragma unroll
-        for (int e = 0; e < 16; ++e) sum[e] = 0.f;
         for (int c = 0; c < nchunks; ++c, ++pc) {
           if (failed) continue;
-          const int b = pc % DR_NBUF;
-          if (!mbar_wait(pfull_bar(b), (uint32_t)(pc / DR_NBUF) & 1, abort_flag, p.status)) {
+          const int b = pc % GR_NBUF;
+          if (!mbar_wait(pfull_bar(b), (uint32_t)(pc / GR_NBUF) & 1, abort_flag, p.status)) failed = true;
+          if (__any_sync(0xffffffffu, failed)) {
             failed = true;
             continue;
           }
@@ -1359,68 +1396,147 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
           float v[16];
           tmem_ld16(tmem_base + lane_off + (uint32_t)(b * DS_N + part * 16), v);
           tc_fence_before();
-          mbar_arrive(pempty_bar(b));
+          __syncwarp();
+          if (lane == 0) mbar_arrive(pempty_bar(b));
 #pragma unroll
-          for (int e = 0; e < 16; ++e) sum[e] = __fadd_rn(sum[e], crt_reduce(v[e], mod, rmod));
+          for (int e = 0; e < 16; ++e) {
+            const float r = crt_reduce(v[e], mod, rmod);
+            sum[e] = c == 0 ? r : __fadd_rn(sum[e], r);
+          }
         }
+        if (failed) continue;
         if (nchunks > 1) {
 #pragma unroll
           for (int e = 0; e < 16; ++e) sum[e] = crt_reduce(sum[e], mod, rmod);
         }
 #pragma unroll
         for (int w = 0; w < 4; ++w)
-          tw[(w * 16 + l) * 32 + lane] = crt_pack(crt_byte(sum[4 * w]), crt_byte(sum[4 * w + 1]),
-                                                  crt_byte(sum[4 * w + 2]), crt_byte(sum[4 * w + 3]));
+          tmem_st1(words + (uint32_t)(w * 16 + l), crt_pack(crt_byte(sum[4 * w]), crt_byte(sum[4 * w + 1]),
+                                                            crt_byte(sum[4 * w + 2]), crt_byte(sum[4 * w + 3])));
       }
-      if (__any_sync(0xffffffffu, failed)) continue;
+      if (MODE == GR_DIST && failed) continue;
+      if (!failed) tmem_st_wait();
       const int row = I * 128 + q * 32 + lane, col0 = J * DS_N + part * 16;
-      const bool rowok = row < p.n, mirror = J >= 2 * I + 2;
+      const int br = 2 * I + (q >> 1);                   // 64-row block of the row
+      const bool rowok = !failed && row < p.n && (MODE == GR_DIST || br <= J);
+      const bool mirror = J >= 2 * I + 2;
       const int er = p.ex[row];
-      const ulonglong2 nr2 = p.norms[row];
-      const u128 nr = ((u128)nr2.y << 64) | nr2.x;
+      const __int128 nr = i128_of(p.self[row]);
       bool low = false;
+      double rsum = 0.0;
 #pragma unroll 1
       for (int w = 0; w < 4; ++w) {
-        uint32_t tv[16];
+        uint32_t tv[NP];
+        {
+          float f[16];
+          tmem_ld16(words + (uint32_t)(w * 16), f);
 #pragma unroll
-        for (int l = 0; l < 16; ++l) tv[l] = tw[(w * 16 + l) * 32 + lane];
-        double* res = reinterpret_cast<double*>(tw + w * 512);   // the quad's words are read: 4 columns x 32 rows
-        __syncwarp();
+          for (int l = 0; l < NP; ++l) tv[l] = __float_as_uint(f[l]);
+        }
+        double da[4];
+        if (MODE == GR_SCORE) {
+          // |A1 - A2| of 32 rows x 4 columns: loaded with lanes along the columns (32-byte row
+          // segments), passed through shared memory to the row-per-lane layout
+#pragma unroll
+          for (int h = 0; h < 4; ++h) {
+            const int rr = h * 8 + (lane >> 2), grow = I * 128 + q * 32 + rr, gcol = col0 + 4 * w + (lane & 3);
+            double x = 0.0;
+            if (grow < p.n && gcol < p.n) {
+              const size_t o = (size_t)grow * p.n + gcol;
+              x = fabs(p.A1[o] - p.A2[o]);
+            }
+            xp[(4 * w + (lane & 3)) * 33 + rr] = x;
+          }
+          __syncwarp();
+#pragma unroll
+          for (int h = 0; h < 4; ++h) da[h] = xp[(4 * w + h) * 33 + lane];
+          __syncwarp();
+        }
 #pragma unroll
         for (int h = 0; h < 4; ++h) {
           const int col = col0 + 4 * w + h;
-          double d2 = 0.0;
-          if (rowok && col < p.n && row != col) {
+          double out = 0.0;
+          if (rowok && col < p.n && (MODE == GR_DIST ? row != col : (br < J || row < col))) {
             const int ec = p.ex[col];
-            const ulonglong2 nc2 = p.norms[col];
-            u128 a = nr, c = ((u128)nc2.y << 64) | nc2.x;
-            __int128 g2 = crt16_value(tv, 8 * h) * 2;
-            const int d = er - ec, ad = min(d < 0 ? -d : d, 127);   // to the coarser row's units
-            if (d > 0)
-              a = 2 * ad > 127 ? 0 : a >> (2 * ad);
-            else
-              c = 2 * ad > 127 ? 0 : c >> (2 * ad);
-            g2 >>= ad;
-            const __int128 v = (__int128)(a + c) - g2;
-            if (er == CRT_ROW_NAN || ec == CRT_ROW_NAN || v < ((__int128)1 << 109))
-              low = true;
-            else
-              d2 = i128_to_double(v, 2 * min(er, ec));
-            if (mirror) p.A[(size_t)col * p.n + row] = d2;   // lanes write 32 consecutive entries
+            __int128 a = nr, c = i128_of(p.self[col]), g = crt_value<NP>(tv, 8 * h);
+            if (MODE == GR_DIST) g *= 2;
+            const int d = er - ec, ad = d < 0 ? -d : d;   // to the coarser row's units
+            if (ad < 16) {
+              a = i128_shr(a, d > 0 ? 2 * ad : 0);
+              c = i128_shr(c, d > 0 ? 0 : 2 * ad);
+              g = i128_shr(g, ad);
+            } else {
+              const int s1 = min(ad, 127), s2 = min(2 * ad, 127);
+              if (d > 0)
+                a >>= s2;
+              else
+                c >>= s2;
+              g >>= s1;
+            }
+            const __int128 v = a + c - g;
+            const bool nan = er == CRT_ROW_NAN || ec == CRT_ROW_NAN;
+            if (MODE == GR_DIST) {
+              if (nan || v < ((__int128)1 << 109))
+                low = true;
+              else
+                out = i128_to_double(v, 2 * min(er, ec));
+              if (mirror) p.A[(size_t)col * p.n + row] = out;   // lanes write 32 consecutive entries
+            } else {
+              const double dc =
+                  nan ? __longlong_as_double(0x7FF8000000000000ll) : i128_to_double(v, 2 * min(er, ec) + ge);
+              out = da[h] * fabs(dc);
+              rsum += out;
+            }
           }
-          res[h * 32 + lane] = d2;
+          xp[(4 * w + h) * 33 + lane] = out;
         }
       }
-      const int bi = 2 * I + (q >> 1);                   // 64-row block of this warp
-      if (__any_sync(0xffffffffu, low) && lane == 0) p.bad[(size_t)min(bi, J) * p.nb64 + max(bi, J)] = 1;
+      if (MODE == GR_DIST) {
+        if (__any_sync(0xffffffffu, low) && lane == 0) p.bad[(size_t)min(br, J) * p.nb64 + max(br, J)] = 1;
+      }
       __syncwarp();
-      // the warp's 32 x 16 block row-wise, two 128-byte row segments per store
+      double* dst = MODE == GR_DIST ? p.A : p.E;
+      if (dst) {
+        // the warp's 32 x 16 block row-wise, two 128-byte row segments per store
 #pragma unroll 4
-      for (int it = 0; it < 16; ++it) {
-        const int rr = 2 * it + (lane >> 4), c = lane & 15;
-        const int grow = I * 128 + q * 32 + rr, gcol = col0 + c;
-        if (grow < p.n && gcol < p.n)
-          p.A[(size_t)grow * p.n + gcol] = reinterpret_cast<const double*>(tw + (c >> 2) * 512)[(c & 3) * 32 + rr];
+        for (int it = 0; it < 16; ++it) {
+          const int rr = 2 * it + (lane >> 4), c = lane & 15;
+          const int grow = I * 128 + q * 32 + rr, gcol = col0 + c;
+          if (grow < p.n && gcol < p.n && (MODE == GR_DIST || (!failed && grow < gcol)))
+            dst[(size_t)grow * p.n + gcol] = xp[c * 33 + rr];
+        }
+      }
+      if (MODE == GR_SCORE) {
+        // sums: rows over the warp's 16 columns (rsum), columns over its 32 rows (a lane per
+        // column and half), then the tile's 64-node blocks as in k_tc_score
+        const int c = lane & 15, r0 = (lane >> 4) * 16;
+        double csum = 0.0;
+#pragma unroll
+        for (int r = 0; r < 16; ++r) csum += xp[c * 33 + r0 + r];
+        csum += __shfl_xor_sync(0xffffffffu, csum, 16);
+        double* rowpart = parts + tpar * GR_PARTS;        // [128][4]
+        double* colpart = rowpart + 128 * 4;              // [4][64]
+        tpar ^= 1;
+        rowpart[(q * 32 + lane) * 4 + part] = rsum;
+        if (lane < 16) colpart[q * DS_N + part * 16 + c] = csum;
+        asm volatile("bar.sync 1, 512;" ::: "memory");
+        const int et = threadIdx.x - 64;                  // epilogue thread 0 .. 511
+        if (et < 128 && !failed) {
+          const int r2 = I * 128 + et, b2 = 2 * I + (et >> 6);
+          if (r2 < p.n && b2 <= J && J * DS_N < p.n) {
+            double v = ((rowpart[et * 4] + rowpart[et * 4 + 1]) + rowpart[et * 4 + 2]) + rowpart[et * 4 + 3];
+            if (b2 == J) {                                // diagonal 64-block: add the column sum of the same node
+              const int hh = et >> 6, cc = et - 64 * hh;
+              v += colpart[(2 * hh) * DS_N + cc] + colpart[(2 * hh + 1) * DS_N + cc];
+            }
+            p.contrib[(size_t)J * p.n + r2] = v;
+          }
+        } else if (et < 256 && !failed) {
+          const int x = et - 128, hh = x >> 6, cc = x & 63;
+          const int col = J * DS_N + cc, b2 = 2 * I + hh;
+          if (col < p.n && b2 < J)
+            p.contrib[(size_t)b2 * p.n + col] = colpart[(2 * hh) * DS_N + cc] + colpart[(2 * hh + 1) * DS_N + cc];
+        }
       }
       __syncwarp();
     }
@@ -1431,8 +1547,7 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
   tc_fence_after();
   if (warp == 0) {
     __syncwarp();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(DR_NBUF * DS_N)
-                 : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");
   }
 }
 
@@ -3595,40 +3710,67 @@ int dist_tc(cdl_ctx* ctx, const void* planes, const long long* norms, int n, int
   return dist_launch(ctx, planes, rows, tp, p, terms);
 }
 
-int dist_residues_tc(cdl_ctx* ctx, const void* planes, const int* ex, const void* norms, int n, int T, int rows, int kp,
-                     double* A, const int* offgrid, void* bad) {
+namespace {
+template <int MODE, int NP>
+int gram_launch(cdl_ctx* ctx, const void* u, const void* v, int n, int rows, int kp, int kblocks, GramParams& p, int kc,
+                double work) {
   if (rows % 128 || kp % 64 || rows < n || kp / 64 > CR_MAX_KBLOCKS) return CDL_ERR_INVALID_ARG;
-  DistResParams p{};
   p.nb128 = rows / 128;
   p.nb64 = 2 * p.nb128;
   const long long tiles = (long long)p.nb128 * p.nb64 - (long long)p.nb128 * (p.nb128 - 1);
   if (tiles > 0x7fffffffLL) return CDL_ERR_INVALID_ARG;
   p.num_tiles = (int)tiles;
   p.rows = rows;
-  p.kblocks = T < DIST_RES_MIN_T ? 0 : kp / 64;
+  p.kblocks = kblocks;
   p.n = n;
-  p.ex = ex;
-  p.norms = static_cast<const ulonglong2*>(norms);
-  p.A = A;
-  p.offgrid = offgrid;
-  p.bad = static_cast<unsigned char*>(bad);
   p.idesc = make_idesc(DS_N);
   p.status = ctx->dev_status;
-  for (int l = 0; l < 16; ++l) {
+  for (int l = 0; l < NP; ++l) {
     p.mod[l] = (float)CRT_MOD[l];
     p.rmod[l] = 1.0f / (float)CRT_MOD[l];
   }
-  CUtensorMap ma, mb;
-  CDL_TRY(make_map(&ma, planes, (int64_t)16 * rows, kp, 128));
-  CDL_TRY(make_map(&mb, planes, (int64_t)16 * rows, kp, DS_N));
+  CUtensorMap mu, mv;
+  CDL_TRY(make_map(&mu, u, (int64_t)NP * rows, kp, 128));
+  CDL_TRY(make_map(&mv, v, (int64_t)NP * rows, kp, DS_N));
   static bool attr = false;
   if (!attr) {
-    CDL_CUDA_TRY(cudaFuncSetAttribute(k_tc_distr, cudaFuncAttributeMaxDynamicSharedMemorySize, DR_SMEM_BYTES));
+    CDL_CUDA_TRY(
+        cudaFuncSetAttribute(k_tc_gramr<MODE, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, GR_SMEM_BYTES));
     attr = true;
   }
-  Launch L(ctx, CDL_KC_DISTANCE, 0);
-  k_tc_distr<<<std::min(p.num_tiles, ctx->sm_count), T8_THREADS, DR_SMEM_BYTES, ctx->stream>>>(ma, mb, p);
+  Launch L(ctx, kc, work);
+  k_tc_gramr<MODE, NP>
+      <<<std::min(p.num_tiles, ctx->sm_count), T8_THREADS, GR_SMEM_BYTES, ctx->stream>>>(mu, mv, p);
   return L.done();
+}
+}  // namespace
+
+int dist_residues_tc(cdl_ctx* ctx, const void* planes, const int* ex, const void* norms, int n, int T, int rows, int kp,
+                     double* A, const int* offgrid, void* bad) {
+  GramParams p{};
+  p.ex = ex;
+  p.self = static_cast<const ulonglong2*>(norms);
+  p.A = A;
+  p.offgrid = offgrid;
+  p.bad = static_cast<unsigned char*>(bad);
+  return gram_launch<GR_DIST, 16>(ctx, planes, planes, n, rows, kp, T < DIST_RES_MIN_T ? 0 : kp / 64, p,
+                                  CDL_KC_DISTANCE, 0);
+}
+
+int score_residues_tc(cdl_ctx* ctx, const void* u, const void* v, int planes, const int* ex, const void* dself,
+                      const int* gexp, int n, int rows, int kp, const double* A1, const double* A2, double* contrib,
+                      double* E, double work) {
+  GramParams p{};
+  p.ex = ex;
+  p.self = static_cast<const ulonglong2*>(dself);
+  p.A1 = A1;
+  p.A2 = A2;
+  p.gexp = gexp;
+  p.contrib = contrib;
+  p.E = E;
+  if (planes == 16) return gram_launch<GR_SCORE, 16>(ctx, u, v, n, rows, kp, kp / 64, p, CDL_KC_SCORE, work);
+  if (planes == 13) return gram_launch<GR_SCORE, 13>(ctx, u, v, n, rows, kp, kp / 64, p, CDL_KC_SCORE, work);
+  return CDL_ERR_INVALID_ARG;
 }
 
 int dist_tc_panel(cdl_ctx* ctx, const void* planes, const long long* norms, int n, int rows, int tp, double* panel,

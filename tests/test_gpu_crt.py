@@ -139,3 +139,34 @@ def test_solve_with_and_without_workspace(G, name, n, k):
     for Z in Zs:
         assert np.linalg.norm(Y.cpu().numpy() - L @ Z) <= 3e-12 * np.linalg.norm(Y.cpu().numpy())
     assert np.linalg.norm(Zs[0] - Zs[1]) <= 1e-10 * np.linalg.norm(Zs[0])
+
+
+@pytest.mark.parametrize("name,tol", [("f64", 1e-12), ("f32", 1e-10)])
+@pytest.mark.parametrize("n,k", [(2, 1), (65, 33), (129, 16), (300, 200), (130, 1024)])
+def test_scores_with_and_without_workspace(G, name, tol, n, k):
+    """Residue scores against the CUDA-core ones that run under a workspace cap too small for the planes,
+    with rows of very different scales, a node without an embedding, and equal embeddings."""
+    cdl = G.cdl
+    rng = np.random.default_rng(n + k)
+    A = [rng.uniform(0, 1, (n, n)) for _ in range(2)]
+    A = [torch.from_numpy(np.triu(a, 1) + np.triu(a, 1).T).cuda() for a in A]
+    Z1 = rng.standard_normal((n, k)) * 10.0 ** rng.uniform(-3, 0, (n, 1))
+    Z2 = Z1 + 0.05 * rng.standard_normal((n, k)) * np.abs(Z1)
+    Z1[n // 2] = Z2[n // 2] = 0
+    Z2[n - 1] = Z1[n - 1]
+    Zt = [torch.from_numpy(z).cuda() for z in (Z1, Z2)]
+    vol = [torch.full((1,), v, dtype=torch.float64, device="cuda") for v in (3.0, 4.0)]
+    nb = (n + 63) // 64
+    cap = 32 * n * k + 8 * nb * n + 4 * n + 16 * k + 8192       # the float planes and the partial sums only
+    st, h = cdl.cdl_ctx_create(0, torch.cuda.current_stream().cuda_stream, cap)
+    assert st == 0
+    Fs = []
+    for ctx in (G.h, h):
+        F = torch.empty(n, dtype=torch.float64, device="cuda")
+        top = torch.empty(2, dtype=torch.int64, device="cuda")
+        st = cdl.cdl_cad_score(ctx, A[0], A[1], cdl.CDL_F64, Zt[0], Zt[1], vol[0], vol[1], n, k, _dtype(cdl, name), 2,
+                               F, top)
+        assert st == 0 and cdl.cdl_sync(ctx) == 0
+        Fs.append(F.cpu().numpy())
+    assert cdl.cdl_ctx_destroy(h) == 0
+    np.testing.assert_allclose(Fs[0], Fs[1], rtol=tol, atol=tol * Fs[1].max())
