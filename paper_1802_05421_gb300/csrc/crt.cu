@@ -16,8 +16,8 @@
 // give NaN rows and columns.
 //
 // Bounds: the products by the tensor cores, 16 (8) times n^2 (n + 1) flop;
-// the other two kernels by integer issue (about 10 instructions per entry and
-// plane in the first, 9 in the second). Measured, one squaring: float32 n =
+// the other two kernels by instruction issue (about 8 instructions per entry
+// and plane in the first, 7 in the second). Measured, one squaring: float32 n =
 // 8192 13.1 ms on the CUDA cores, here 2.52 ms of products (1.75 PFLOP/s) + 0.36
 // + 0.12; float64 n = 1024 1.07 ms on the CUDA cores (1 TFLOP/s of the float64
 // pipes), here 30 + 15 + 13 us. Relative error (Frobenius) of a square, n =
@@ -36,28 +36,24 @@
 namespace cdl {
 namespace {
 
+// 2^16, 2^32, 2^48 modulo p_l, nearest to zero, and 1 / p_l
 struct ResidueTab {
-  uint32_t mod[CRT_MAX], magic[CRT_MAX], c1[CRT_MAX], c2[CRT_MAX], bias[CRT_MAX];
-  float off[CRT_MAX];
+  float c[3][CRT_MAX], mod[CRT_MAX], rmod[CRT_MAX];
 };
-// Signed x = u0 + 2^S u1 + 2^2S u2 (S = 21 for 62-bit x; S = 16 and no u2 for
-// 32-bit x): u0 + c1 u1 + c2 u2 + bias is x + floor(p / 2) modulo p and in
-// [0, 2^31); off = 2^23 + floor(p / 2).
-constexpr ResidueTab make_residue_tab(int S) {
+constexpr ResidueTab make_residue_tab() {
   ResidueTab t{};
   for (int l = 0; l < CRT_MAX; ++l) {
     const int p = CRT_MOD[l];
-    t.mod[l] = (uint32_t)p;
-    t.magic[l] = crt_magic(p);
-    t.c1[l] = (uint32_t)crt_pow2_mod(S, p);
-    t.c2[l] = (uint32_t)crt_pow2_mod(2 * S, p);
-    t.bias[l] = (uint32_t)(((1u << 29) + (unsigned)p - 1) / (unsigned)p * (unsigned)p + (unsigned)(p / 2));
-    t.off[l] = 8388608.0f + (float)(p / 2);
+    for (int k = 0; k < 3; ++k) {
+      const int r = crt_pow2_mod(16 * (k + 1), p);
+      t.c[k][l] = (float)(2 * r > p ? r - p : r);
+    }
+    t.mod[l] = (float)p;
+    t.rmod[l] = 1.0f / (float)p;
   }
   return t;
 }
-__constant__ ResidueTab c_res64 = make_residue_tab(21);
-__constant__ ResidueTab c_res32 = make_residue_tab(16);
+__constant__ ResidueTab c_res = make_residue_tab();
 
 struct CombineTab32 {
   uint32_t lo[8], hi[8], frac[8];
@@ -116,15 +112,31 @@ __device__ __forceinline__ long long scaled_int(T x, int e) {
   return LevelType<T>::negative(x) ? -(long long)v : (long long)v;
 }
 
-// The residue of `x` modulo p_l as a bf16 bit pattern in the upper half of the
-// result: an integer of magnitude at most 128 through the float 2^23 + v.
-template <typename T>
-__device__ __forceinline__ uint32_t residue_bits(int u0, int u1, int u2, int l) {
-  const ResidueTab& t = sizeof(T) == 8 ? c_res64 : c_res32;
-  uint32_t r = (uint32_t)u0 + t.bias[l] + t.c1[l] * (uint32_t)u1;
-  if (sizeof(T) == 8) r += t.c2[l] * (uint32_t)u2;
-  r -= (__umulhi(r, t.magic[l]) >> 7) * t.mod[l];
-  return __float_as_uint(__uint_as_float(0x4B000000u | r) - t.off[l]);
+// x = d_0 + 2^16 d_1 + .. in ND balanced digits of 16 bits, as floats (|x| < 2^(16
+// ND - 2)): the unsigned digits of x + 0x8000.. through the float 2^23 + u.
+template <int ND>
+__device__ __forceinline__ void digits16(long long x, float (&d)[ND]) {
+  const unsigned long long w = (unsigned long long)x + (ND == 4 ? 0x8000800080008000ull : 0x80008000ull);
+  const uint32_t lo = (uint32_t)w, hi = (uint32_t)(w >> 32);
+#pragma unroll
+  for (int k = 0; k < ND; ++k) {
+    const uint32_t u = __byte_perm(k < 2 ? lo : hi, 0x4B000000u, k & 1 ? 0x7632u : 0x7610u);
+    d[k] = __fsub_rn(__uint_as_float(u), 8421376.0f);   // 2^23 + 2^15
+  }
+}
+
+// The residue modulo p_l as float bits (an integer of magnitude at most 128: the
+// upper half is its bf16): sum d_k (2^16k mod p) is exact in float32 (three
+// terms of at most 2^15 123, below 2^24), then as crt_reduce. All at the
+// float32 rate; 32-bit multiplications and their high halves run at half of it
+// and less.
+template <int ND>
+__device__ __forceinline__ uint32_t residue_bits(const float (&d)[ND], int l) {
+  float r = d[0];
+#pragma unroll
+  for (int k = 1; k < ND; ++k) r = __fmaf_rn(d[k], c_res.c[k - 1][l], r);
+  const float q = __fsub_rn(__fmaf_rn(r, c_res.rmod[l], 12582912.0f), 12582912.0f);
+  return __float_as_uint(__fmaf_rn(-q, c_res.mod[l], r));
 }
 
 // One block per row of a rows x cols matrix (zero beyond, to gridDim.x x np):
@@ -170,24 +182,13 @@ __global__ void __launch_bounds__(256) k_crt_residues(const T* __restrict__ X, i
   const size_t plane = (size_t)gridDim.x * np / 2;
   uint32_t* out = planes + (size_t)row * np / 2;
   for (int j = tid; j < np / 2; j += 256) {
-    int u[2][3];
+    constexpr int ND = sizeof(T) == 8 ? 4 : 2;
+    float d[2][ND];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const long long v = fin && 2 * j + h < cols ? scaled_int(x[2 * j + h], e) : 0;
-      if (sizeof(T) == 8) {
-        u[h][0] = (int)(v & 0x1FFFFF);
-        u[h][1] = (int)(v >> 21) & 0x1FFFFF;
-        u[h][2] = (int)(v >> 42);
-      } else {
-        u[h][0] = (int)v & 0xFFFF;
-        u[h][1] = (int)v >> 16;
-        u[h][2] = 0;
-      }
-    }
+    for (int h = 0; h < 2; ++h) digits16<ND>(fin && 2 * j + h < cols ? scaled_int(x[2 * j + h], e) : 0, d[h]);
 #pragma unroll
     for (int l = 0; l < LT::NP; ++l)
-      out[l * plane + j] = __byte_perm(residue_bits<T>(u[0][0], u[0][1], u[0][2], l),
-                                       residue_bits<T>(u[1][0], u[1][1], u[1][2], l), 0x7632);
+      out[l * plane + j] = __byte_perm(residue_bits<ND>(d[0], l), residue_bits<ND>(d[1], l), 0x7632);
   }
 }
 
@@ -334,20 +335,17 @@ __global__ void __launch_bounds__(128) k_series_residues(const double* __restric
   uint32_t* out = planes + (size_t)row * kp / 2;
   u128 nn = 0;
   for (int j = tid; j < kp / 2; j += 128) {
-    int u[2][3];
+    float d[2][4];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int t = 2 * j + h;
       const long long v = any && t < T ? scaled_int(x[t], e) - scaled_int(X[t], e) : 0;
       nn += (u128)((__int128)v * v);
-      u[h][0] = (int)(v & 0x1FFFFF);
-      u[h][1] = (int)(v >> 21) & 0x1FFFFF;
-      u[h][2] = (int)(v >> 42);
+      digits16<4>(v, d[h]);
     }
 #pragma unroll
     for (int l = 0; l < 16; ++l)
-      out[l * plane + j] = __byte_perm(residue_bits<double>(u[0][0], u[0][1], u[0][2], l),
-                                       residue_bits<double>(u[1][0], u[1][1], u[1][2], l), 0x7632);
+      out[l * plane + j] = __byte_perm(residue_bits<4>(d[0], l), residue_bits<4>(d[1], l), 0x7632);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -463,10 +461,12 @@ __global__ void __launch_bounds__(128) k_score_residues(const double* __restrict
       y = scaled_int(b, e);
       dd += (__int128)x * y;
     }
+    float dx[4], dy[4];
+    digits16<4>(x, dx);
+    digits16<4>(y, dy);
 #pragma unroll
     for (int l = 0; l < NP; ++l) {
-      const uint32_t rx = residue_bits<double>((int)(x & 0x1FFFFF), (int)(x >> 21) & 0x1FFFFF, (int)(x >> 42), l),
-                     ry = residue_bits<double>((int)(y & 0x1FFFFF), (int)(y >> 21) & 0x1FFFFF, (int)(y >> 42), l);
+      const uint32_t rx = residue_bits<4>(dx, l), ry = residue_bits<4>(dy, l);
       const __nv_bfloat16 bx = __ushort_as_bfloat16((unsigned short)(rx >> 16)),
                           by = __ushort_as_bfloat16((unsigned short)(ry >> 16));
       u[l * plane + r] = bx;
