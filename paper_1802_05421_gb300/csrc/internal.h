@@ -354,10 +354,29 @@ int tc_square_grouped_pairs(cdl_ctx* ctx, const TcGroup* host_first, const TcGro
 int pair_clusters(cdl_ctx* ctx);
 int tc_apply_grouped(cdl_ctx* ctx, const TcGroup* host_first, const TcGroup* dgroups, const uint32_t* dtiles,
                      int ntiles, int kp, int gate_mask, int kc, double work);
-int apply_tc(cdl_ctx* ctx, const cdl_chain* ch, int level, const void* xop, float* partial,
-             int k, int splits);
+// How the K range of a chain application is split. On CTA pairs (clusters >
+// 0) cluster c of `clusters` takes the k-blocks [bound(c), bound(c + 1)) of the
+// row-major order (256-row block, k-block), `kblocks` to a row block: equal
+// shares whatever the order, and a row block gets one partial product from
+// each cluster that reaches into it (two or three; equal splits that fill the last round of clusters
+// wrote up to ten). Without pairs every row block has `slots` equal splits.
+struct ApplySplit {
+  int clusters = 0, kblocks = 0, rowblocks = 0, slots = 1;   // slots: the most partials of a row block
+  __host__ __device__ int bound(int c) const { return (int)((long long)c * rowblocks * kblocks / clusters); }
+  // the cluster that takes position x of the order
+  __host__ __device__ int cluster_of(int x) const {
+    return (int)((((long long)x + 1) * clusters - 1) / ((long long)rowblocks * kblocks));
+  }
+  // partials of 256-row block m
+  __host__ __device__ int slots_of(int m) const {
+    return clusters == 0 ? slots : cluster_of((m + 1) * kblocks - 1) - cluster_of(m * kblocks) + 1;
+  }
+};
+ApplySplit apply_split(cdl_ctx* ctx, int np, int kp);
+int apply_tc(cdl_ctx* ctx, const cdl_chain* ch, int level, const void* xop, float* partial, int kp,
+             const ApplySplit& sp);
 int apply_tc_mat(cdl_ctx* ctx, const void* amat, int np, const void* xop, float* partial, int kp,
-                 int splits);
+                 const ApplySplit& sp);
 bool tc_supported(cdl_ctx* ctx);
 // Anomalous edge set and per-node top edges (score.cu).
 int cad_edges(cdl_ctx* ctx, const double* A1, const double* A2, const double* Z1, const double* Z2,

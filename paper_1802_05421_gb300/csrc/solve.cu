@@ -84,21 +84,43 @@ __global__ void k_precond_in(const double* __restrict__ R, const double* __restr
   x[idx] = (T)v;
 }
 
-// Z += dZ with dZ = D^{-1/2} x; dZ is also kept in float32 (npad x kp, zero
-// padded) for the recursive residual update.
+// Z += dZ with dZ = D^{-1/2} x (dZ is also kept in float32, npad x kp, zero
+// padded, for the recursive residual update), and the column sums of D o Z over
+// the block's 32 rows for the centring (part[block][r], fixed order). Lanes along
+// the columns, a warp every eighth row.
 template <typename T>
-__global__ void k_precond_out(const T* __restrict__ x, const double* __restrict__ rsd, int n, int k,
-                              int np, int kp, double* __restrict__ Z, float* __restrict__ dZ) {
-  size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (idx >= (size_t)np * kp) return;
-  int i = (int)(idx / kp), r = (int)(idx % kp);
-  float dzf = 0.f;
-  if (i < n && r < k) {
-    const double dz = (double)x[idx] * rsd[i];
-    Z[(size_t)i * k + r] += dz;
-    dzf = (float)dz;
+__global__ void __launch_bounds__(256) k_precond_out(const T* __restrict__ x, const double* __restrict__ rsd,
+                                                      const double* __restrict__ D, int n, int k, int kp,
+                                                      double* __restrict__ Z, float* __restrict__ dZ,
+                                                      double* __restrict__ part) {
+  __shared__ double red[8][33];
+  const int i0 = blockIdx.x * 32, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int c0 = 0; c0 < kp; c0 += 32) {
+    const int r = c0 + lane;
+    double acc = 0.0;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      const int i = i0 + w + 8 * a;
+      float dzf = 0.f;
+      if (i < n && r < k) {
+        const double dz = (double)x[(size_t)i * kp + r] * rsd[i];
+        const double z = Z[(size_t)i * k + r] + dz;
+        Z[(size_t)i * k + r] = z;
+        acc = fma(D[i], z, acc);
+        dzf = (float)dz;
+      }
+      if (r < kp) dZ[(size_t)i * kp + r] = dzf;
+    }
+    red[w][lane] = acc;
+    __syncthreads();
+    if (w == 0 && r < k) {
+      double t = red[0][lane];
+#pragma unroll
+      for (int q = 1; q < 8; ++q) t += red[q][lane];
+      part[(size_t)blockIdx.x * k + r] = t;
+    }
+    __syncthreads();
   }
-  dZ[idx] = dzf;
 }
 
 // x[i][r] += sum_s part[s][i][r] (CUDA-core chains)
@@ -115,10 +137,11 @@ __global__ void k_update_simt(T* __restrict__ x, const T* __restrict__ part, int
 // lo halves of the right-hand side), then the tensor-core operand
 // xop[r][i] = bf16(x[i][r]), xop[kp + r][i] = bf16(x[i][r] - hi). 32 x 32 tiles.
 __global__ void __launch_bounds__(256) k_update_bf16(float* __restrict__ x, const float* __restrict__ part,
-                                                      int splits, int np, int kp,
+                                                      ApplySplit sp, int np, int kp,
                                                       __nv_bfloat16* __restrict__ xop, int accumulate) {
   __shared__ float tile[32][33];
   const int i0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
+  const int splits = accumulate ? sp.slots_of(i0 / 256) : 0;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 32 x 8
   for (int a = ty; a < 32; a += 8) {
     const int i = i0 + a, r = r0 + tx;
@@ -148,31 +171,57 @@ __global__ void __launch_bounds__(256) k_update_bf16(float* __restrict__ x, cons
   }
 }
 
-// Column sums s_r = sum_i D_i Z[i][r] in fixed-order per-block partials.
-__global__ void __launch_bounds__(256) k_colsum_dz(const double* __restrict__ Z, const double* __restrict__ D,
-                                                    int n, int k, int rows_per_block, double* __restrict__ part) {
-  const int r = blockIdx.y * blockDim.x + threadIdx.x;
-  if (r >= k) return;
-  const int i0 = blockIdx.x * rows_per_block, i1 = min(n, i0 + rows_per_block);
-  double acc = 0.0;
-  for (int i = i0; i < i1; ++i) acc = fma(D[i], Z[(size_t)i * k + r], acc);
-  part[(size_t)blockIdx.x * k + r] = acc;
-}
-
-// shift[r] = (sum of the column's partial sums, in order) / vol, once per column.
-__global__ void k_center_shift(const double* __restrict__ part, int nparts, int k, const double* __restrict__ vol,
-                               double* __restrict__ shift) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= k) return;
+// shift[r] = (sum of the column's partial sums, fixed order) / vol, once per
+// column; mbits[r] = 0 for k_center. 32 columns per block, a warp every eighth
+// part.
+__global__ void __launch_bounds__(256) k_center_shift(const double* __restrict__ part, int nparts, int k,
+                                                       const double* __restrict__ vol, double* __restrict__ shift,
+                                                       unsigned long long* __restrict__ mbits) {
+  __shared__ double red[8][33];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, r = blockIdx.x * 32 + lane;
   double s = 0.0;
-  for (int p = 0; p < nparts; ++p) s += part[(size_t)p * k + r];
-  shift[r] = s / *vol;
+  if (r < k)
+    for (int p = w; p < nparts; p += 8) s += part[(size_t)p * k + r];
+  red[w][lane] = s;
+  __syncthreads();
+  if (w == 0 && r < k) {
+    for (int q = 1; q < 8; ++q) s += red[q][lane];
+    shift[r] = s / *vol;
+    mbits[r] = 0;
+  }
 }
 
-__global__ void k_center(double* __restrict__ Z, const double* __restrict__ shift, int n, int k) {
-  size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (idx >= (size_t)n * k) return;
-  Z[idx] -= shift[idx % k];
+// Z -= shift, and each column's largest |Z| as float64 bits (for the slices of
+// the exact residual): 64 rows per block, lanes along the columns, one atomic
+// per block and column.
+__global__ void __launch_bounds__(256) k_center(double* __restrict__ Z, const double* __restrict__ shift, int n, int k,
+                                                 unsigned long long* __restrict__ mbits) {
+  __shared__ unsigned long long red[8][32];
+  const int i0 = blockIdx.x * 64, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int c0 = 0; c0 < k; c0 += 32) {
+    const int r = c0 + lane;
+    unsigned long long m = 0;
+    if (r < k) {
+      const double s = shift[r];
+#pragma unroll
+      for (int a = 0; a < 8; ++a) {
+        const int i = i0 + w + 8 * a;
+        if (i < n) {
+          const double z = Z[(size_t)i * k + r] - s;
+          Z[(size_t)i * k + r] = z;
+          m = max(m, (unsigned long long)__double_as_longlong(z) & 0x7FFFFFFFFFFFFFFFull);
+        }
+      }
+    }
+    red[w][lane] = m;
+    __syncthreads();
+    if (w == 0 && r < k) {
+#pragma unroll
+      for (int q = 1; q < 8; ++q) m = max(m, red[q][lane]);
+      atomicMax(mbits + r, m);
+    }
+    __syncthreads();
+  }
 }
 
 // Z (float64) -> float hi + lo pair for the float-float residual.
@@ -399,7 +448,7 @@ __device__ __forceinline__ float bf16_pair_value(float v) {
 // about 16 significant bits of A and of dZ); R -= D o dZ - (sum of the four
 // products) with dZ as the products see it; per-block sums of the new R^2.
 __global__ void __launch_bounds__(256) k_residual_update_tc(const float* __restrict__ pa, const float* __restrict__ pb,
-                                                             int splits, int np, const float* __restrict__ dZ,
+                                                             ApplySplit sp, int np, const float* __restrict__ dZ,
                                                              const double* __restrict__ D, int n, int k, int kp,
                                                              double* __restrict__ R, double* __restrict__ part) {
   __shared__ double red[8];
@@ -408,12 +457,20 @@ __global__ void __launch_bounds__(256) k_residual_update_tc(const float* __restr
   for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
        idx += (size_t)gridDim.x * blockDim.x) {
     const int i = (int)(idx / k), c = (int)(idx % k);
-    double az = 0.0;
+    const int splits = sp.slots_of(i / 256);
+    // the partials in float-float (float64 additions and conversions were most of this kernel's time)
+    ff az = {0.f, 0.f};
     for (int s = 0; s < splits; ++s) {
       const size_t o = ((size_t)s * np + i) * (2 * kp);
-      az += (double)pa[o + c] + (double)pa[o + kp + c] + (double)pb[o + c] + (double)pb[o + kp + c];
+      const float v[4] = {pa[o + c], pa[o + kp + c], pb[o + c], pb[o + kp + c]};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const ff t = two_sum(az.hi, v[q]);
+        az = {t.hi, __fadd_rn(az.lo, t.lo)};
+      }
     }
-    const double r = R[idx] - (D[i] * (double)bf16_pair_value(dZ[(size_t)i * kp + c]) - az);
+    const double dz = D[i] * (double)bf16_pair_value(dZ[(size_t)i * kp + c]);
+    const double r = R[idx] - (dz - ((double)az.hi + (double)az.lo));
     R[idx] = r;
     sq = fma(r, r, sq);
   }
@@ -431,11 +488,6 @@ __global__ void __launch_bounds__(256) k_residual_update_tc(const float* __restr
 
 // ---- exact-slice residual (tensor chains): Z / c_r in six bf16 slices,
 // c_r the power of two just above column r's largest |Z|.
-__global__ void k_zcolmax(const double* __restrict__ Z, size_t count, int k, unsigned long long* __restrict__ mbits) {
-  for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < count; idx += (size_t)gridDim.x * blockDim.x)
-    atomicMax(mbits + idx % k, (unsigned long long)__double_as_longlong(fabs(Z[idx])));
-}
-
 __device__ __forceinline__ double pow2_above(unsigned long long bits) {
   if (bits == 0) return 1.0;
   const int e = (int)((bits >> 52) & 0x7FF);
@@ -859,12 +911,14 @@ struct SolveBlock {
   double* Z = nullptr;
   cdl_solve_stats* stats = nullptr;
   cudaStream_t st = nullptr;
-  int n = 0, np = 0, k = 0, kp = 0, splits = 1;
+  int n = 0, np = 0, k = 0, kp = 0, splits = 1;   // splits: CUDA-core chains; sp: tensor chains
+  ApplySplit sp;
   bool bf16 = false;
   size_t xe = 4, nk = 0;
-  int res_gx = 0, res_gy = 0, upd_gx = 0, upd_gy = 0, cs_rows = 256, cs_parts = 0;
+  int res_gx = 0, res_gy = 0, upd_gx = 0, upd_gy = 0, cs_parts = 0;
   void *vR = nullptr, *vx = nullptr, *vxop = nullptr, *vpart = nullptr, *vred = nullptr, *vscal = nullptr;
   void *vzh = nullptr, *vzl = nullptr, *vcs = nullptr, *vdz = nullptr, *vpart2 = nullptr, *vdzop = nullptr;
+  void* vzmax = nullptr;
   double *R = nullptr, *red = nullptr, *scal = nullptr;
   double yy = 0.0, rel = 1.0, drift = 0.0;
   int iters = 0, nparts = 0;
@@ -885,27 +939,12 @@ struct SolveBlock {
     st = ctx->stream;
     n = (int)ch->n;
     np = (int)ch->npad;
-    kp = (int)round_up(k, 16);   // tensor-core N = 2 kp: multiple of 32
     bf16 = ch->dtype == CDL_BF16 || ch->dtype == CDL_FP8E4M3 || ch->dtype == CDL_FP8E4M3_T128;   // tensor-core apply
     xe = ch->dtype == CDL_F64 ? 8 : 4;
-    const int kblocks = np / 64;
+    kp = (int)round_up(k, bf16 ? 32 : 16);   // tensor-core N = 2 kp: a multiple of 64 (the CTA pairs' halves)
     if (bf16) {
-      // split-K of the persistent apply (one CTA per SM over np / 128 row tiles x
-      // splits): the fewest splits (a divisor of the K blocks, at most 16) whose
-      // tiles fill the last round of CTAs to 95 %, else the best filling
-      const int mb = np / 128, sm = ctx->sm_count;
-      splits = 1;
-      double best = 0.0;
-      for (int sp = 1; sp <= 16 && sp <= kblocks; ++sp) {
-        if (kblocks % sp) continue;
-        const long long tl = (long long)mb * sp;
-        const double fill = (double)tl / (double)(((tl + sm - 1) / sm) * sm);
-        if (fill > best + 1e-9) {
-          best = fill;
-          splits = sp;
-        }
-        if (fill >= 0.95) break;
-      }
+      sp = apply_split(ctx, np, kp);
+      splits = sp.slots;
     } else {
       const int bm = ch->dtype == CDL_F32 ? 128 : 64;
       const int cols = (kp + 63) / 64;
@@ -918,7 +957,7 @@ struct SolveBlock {
     upd_gx = (n + RU_M - 1) / RU_M;
     upd_gy = (k + RU_N - 1) / RU_N;
     const int nred = std::max(res_gx * res_gy, std::max(1024, ctx->sm_count * 4));
-    cs_parts = (n + cs_rows - 1) / cs_rows;
+    cs_parts = np / 32;
     CDL_TRY(ws("solve.R", idx, (size_t)n * k * 8, &vR));
     CDL_TRY(ws("solve.x", idx, (size_t)np * kp * xe, &vx));
     if (bf16) CDL_TRY(ws("solve.xop", idx, 2 * (size_t)kp * np * 2, &vxop));
@@ -929,6 +968,7 @@ struct SolveBlock {
     CDL_TRY(ws("solve.zl", idx, (size_t)n * k * 4, &vzl));
     CDL_TRY(ws("solve.colsum", idx, (size_t)(cs_parts + 1) * k * 8, &vcs));   // partial sums, then the shift
     CDL_TRY(ws("solve.dz", idx, (size_t)np * kp * 4, &vdz));
+    CDL_TRY(ws("solve.zmax", idx, (size_t)k * 8, &vzmax));   // of the current Z, left by k_center
     if (bf16) {
       CDL_TRY(ws("solve.part2", idx, (size_t)splits * np * part_cols * xe, &vpart2));
       CDL_TRY(ws("solve.dzop", idx, 2 * (size_t)kp * np * 2, &vdzop));
@@ -973,18 +1013,10 @@ struct SolveBlock {
       // exact slices are one K range of A Z (A symmetric), added into G
       const RegenSource& rs = *ch->regen;
       const int ngroups = (k + 127) / 128;
-      void *vzs, *vG, *vmb, *vcz;
+      void *vzs, *vG, *vcz;
       CDL_TRY(ws_get(ctx, "solve.zslices", 6 * (size_t)128 * np * 2, &vzs));
       CDL_TRY(ws_get(ctx, "solve.G", (size_t)ngroups * RESID_PAIRS * np * 128 * sizeof(double), &vG));
-      CDL_TRY(ws_get(ctx, "solve.zmax", (size_t)k * 8, &vmb));
       CDL_TRY(ws_get(ctx, "solve.zc", (size_t)k * 8, &vcz));
-      CDL_CUDA_TRY(cudaMemsetAsync(vmb, 0, (size_t)k * 8, st));
-      {
-        Launch L(ctx, CDL_KC_MISC, 0);
-        k_zcolmax<<<std::min<size_t>(blocks_for(nk, 256), (size_t)ctx->sm_count * 8), 256, 0, st>>>(
-            Z, nk, k, static_cast<unsigned long long*>(vmb));
-        CDL_TRY(L.done());
-      }
       for (int g = 0; g < ngroups; ++g) {
         const int c0 = g * 128;
         const int kg = std::min(128, (k - c0 + 31) / 32 * 32);
@@ -992,7 +1024,7 @@ struct SolveBlock {
         {
           Launch L(ctx, CDL_KC_MISC, 0);
           k_zslice<<<ctx->sm_count * 4, 256, 0, st>>>(Z, n, k, np, c0, kg,
-                                                       static_cast<const unsigned long long*>(vmb),
+                                                       static_cast<const unsigned long long*>(vzmax),
                                                        static_cast<__nv_bfloat16*>(vzs), static_cast<double*>(vcz));
           CDL_TRY(L.done());
         }
@@ -1015,25 +1047,17 @@ struct SolveBlock {
     if (ch->aslices) {
       // A Z from exact bf16 slices on the tensor cores, in column groups of <= 128
       const int ngroups = (k + 127) / 128;
-      void *vzs, *vG, *vmb, *vcz;
+      void *vzs, *vG, *vcz;
       CDL_TRY(ws_get(ctx, "solve.zslices", 6 * (size_t)128 * np * 2, &vzs));
       CDL_TRY(ws_get(ctx, "solve.G", (size_t)ngroups * RESID_PAIRS * np * 128 * sizeof(double), &vG));
-      CDL_TRY(ws_get(ctx, "solve.zmax", (size_t)k * 8, &vmb));
       CDL_TRY(ws_get(ctx, "solve.zc", (size_t)k * 8, &vcz));
-      CDL_CUDA_TRY(cudaMemsetAsync(vmb, 0, (size_t)k * 8, st));
-      {
-        Launch L(ctx, CDL_KC_MISC, 0);
-        k_zcolmax<<<std::min<size_t>(blocks_for(nk, 256), (size_t)ctx->sm_count * 8), 256, 0, st>>>(
-            Z, nk, k, static_cast<unsigned long long*>(vmb));
-        CDL_TRY(L.done());
-      }
       for (int g = 0; g < ngroups; ++g) {
         const int c0 = g * 128;
         const int kg = std::min(128, (k - c0 + 31) / 32 * 32);
         {
           Launch L(ctx, CDL_KC_MISC, 0);
           k_zslice<<<ctx->sm_count * 4, 256, 0, st>>>(Z, n, k, np, c0, kg,
-                                                       static_cast<const unsigned long long*>(vmb),
+                                                       static_cast<const unsigned long long*>(vzmax),
                                                        static_cast<__nv_bfloat16*>(vzs), static_cast<double*>(vcz));
           CDL_TRY(L.done());
         }
@@ -1080,17 +1104,17 @@ struct SolveBlock {
       {
         dim3 g((np + 31) / 32, (kp + 31) / 32);
         Launch L(ctx, CDL_KC_MISC, 0);
-        k_update_bf16<<<g, 256, 0, st>>>(static_cast<float*>(vdz), nullptr, 0, np, kp,
+        k_update_bf16<<<g, 256, 0, st>>>(static_cast<float*>(vdz), nullptr, sp, np, kp,
                                          static_cast<__nv_bfloat16*>(vdzop), 0);
         CDL_TRY(L.done());
       }
       const __nv_bfloat16* ahi = static_cast<const __nv_bfloat16*>(ch->aop);
-      CDL_TRY(apply_tc_mat(ctx, ahi, np, vdzop, static_cast<float*>(vpart), kp, splits));
-      CDL_TRY(apply_tc_mat(ctx, ahi + (size_t)np * np, np, vdzop, static_cast<float*>(vpart2), kp, splits));
+      CDL_TRY(apply_tc_mat(ctx, ahi, np, vdzop, static_cast<float*>(vpart), kp, sp));
+      CDL_TRY(apply_tc_mat(ctx, ahi + (size_t)np * np, np, vdzop, static_cast<float*>(vpart2), kp, sp));
       const int nb = (int)std::min<size_t>((nk + 255) / 256, (size_t)ctx->sm_count * 4);
       Launch L(ctx, CDL_KC_RESIDUAL, 0);
       k_residual_update_tc<<<nb, 256, 0, st>>>(static_cast<const float*>(vpart), static_cast<const float*>(vpart2),
-                                               splits, np, static_cast<const float*>(vdz), ch->D, n, k, kp, R, red);
+                                               sp, np, static_cast<const float*>(vdz), ch->D, n, k, kp, R, red);
       nparts = nb;
       return L.done();
     }
@@ -1152,7 +1176,7 @@ struct SolveBlock {
     if (bf16) {
       dim3 g((np + 31) / 32, (kp + 31) / 32);
       Launch L(ctx, CDL_KC_MISC, 0);
-      k_update_bf16<<<g, 256, 0, st>>>(static_cast<float*>(vx), nullptr, 0, np, kp,
+      k_update_bf16<<<g, 256, 0, st>>>(static_cast<float*>(vx), nullptr, sp, np, kp,
                                        static_cast<__nv_bfloat16*>(vxop), 0);
       CDL_TRY(L.done());
     }
@@ -1162,10 +1186,10 @@ struct SolveBlock {
   // x <- (I + S~_lvl) x
   int apply_level(int lvl) {
     if (bf16) {
-      CDL_TRY(apply_tc(ctx, ch, lvl, vxop, static_cast<float*>(vpart), kp, splits));
+      CDL_TRY(apply_tc(ctx, ch, lvl, vxop, static_cast<float*>(vpart), kp, sp));
       dim3 g((np + 31) / 32, (kp + 31) / 32);
       Launch L(ctx, CDL_KC_MISC, 0);
-      k_update_bf16<<<g, 256, 0, st>>>(static_cast<float*>(vx), static_cast<const float*>(vpart), splits, np, kp,
+      k_update_bf16<<<g, 256, 0, st>>>(static_cast<float*>(vx), static_cast<const float*>(vpart), sp, np, kp,
                                        static_cast<__nv_bfloat16*>(vxop), 1);
       return L.done();
     }
@@ -1192,29 +1216,26 @@ struct SolveBlock {
   int finish_step(bool always_full) {
     {
       Launch L(ctx, CDL_KC_MISC, 0);
+      double* cs = static_cast<double*>(vcs);
       if (ch->dtype == CDL_F64)
-        k_precond_out<double><<<blocks_for((size_t)np * kp, 256), 256, 0, st>>>(
-            static_cast<const double*>(vx), ch->rsqrt_d, n, k, np, kp, Z, static_cast<float*>(vdz));
+        k_precond_out<double><<<cs_parts, 256, 0, st>>>(static_cast<const double*>(vx), ch->rsqrt_d, ch->D, n, k, kp, Z,
+                                                        static_cast<float*>(vdz), cs);
       else
-        k_precond_out<float><<<blocks_for((size_t)np * kp, 256), 256, 0, st>>>(
-            static_cast<const float*>(vx), ch->rsqrt_d, n, k, np, kp, Z, static_cast<float*>(vdz));
-      CDL_TRY(L.done());
-    }
-    {
-      dim3 g(cs_parts, (k + 255) / 256);
-      Launch L(ctx, CDL_KC_MISC, 0);
-      k_colsum_dz<<<g, 256, 0, st>>>(Z, ch->D, n, k, cs_rows, static_cast<double*>(vcs));
+        k_precond_out<float><<<cs_parts, 256, 0, st>>>(static_cast<const float*>(vx), ch->rsqrt_d, ch->D, n, k, kp, Z,
+                                                       static_cast<float*>(vdz), cs);
       CDL_TRY(L.done());
     }
     {
       double* shift = static_cast<double*>(vcs) + (size_t)cs_parts * k;
+      unsigned long long* zmax = static_cast<unsigned long long*>(vzmax);
       {
         Launch L(ctx, CDL_KC_MISC, 0);
-        k_center_shift<<<(k + 255) / 256, 256, 0, st>>>(static_cast<const double*>(vcs), cs_parts, k, ch->vol, shift);
+        k_center_shift<<<(k + 31) / 32, 256, 0, st>>>(static_cast<const double*>(vcs), cs_parts, k, ch->vol, shift,
+                                                      zmax);
         CDL_TRY(L.done());
       }
       Launch L(ctx, CDL_KC_MISC, 0);
-      k_center<<<blocks_for(nk, 256), 256, 0, st>>>(Z, shift, n, k);
+      k_center<<<(n + 63) / 64, 256, 0, st>>>(Z, shift, n, k, zmax);
       CDL_TRY(L.done());
     }
     ++iters;

@@ -2502,22 +2502,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(S2_THREADS, 1)
 
 // ---------------------------------------------------------------- chain application on CTA pairs
 // x <- level x for one level, as k_tc_gemm's apply mode computes it (float
-// partial products per split of K, summed by the update kernel), with
+// partial products, summed by the update kernel), with
 // tcgen05.mma.cta_group::2: the two CTAs of a cluster compute a 256-row block
-// of one split, each CTA's 128 rows in its TMEM. Per 64-wide k-block CTA rank
+// over a range of K, each CTA's 128 rows in its TMEM. Per 64-wide k-block CTA rank
 // r stages its 128 rows of the level (16 KB) and rows r bn / 2 .. (r + 1)
 // bn / 2 of the right-hand-side operand (the pair's B operand is split
 // between the two CTAs, at most 16 KB), so a stage is at most 32 KB and six
 // stages fit: twice the level bytes in flight of the one-CTA kernel's four
-// 48 KB stages (the level streams from HBM). Barriers as in k_tc_sq2.
+// 48 KB stages (the level streams from HBM). Each cluster takes an equal share
+// of all k-blocks (ApplySplit), so that none waits for a last round and few
+// partial products are written. Barriers as in k_tc_sq2.
 struct Apply2Params {
-  int num_units;   // 256-row blocks x splits (block-major)
-  int splits;
-  int kblocks;     // k-blocks per split
+  ApplySplit sp;
   int npad;
   int bn;          // N = 2 kp (hi and lo halves of the right-hand sides)
   uint32_t idesc;  // kind::f16, M = 256, N = bn
-  float* out;      // splits x npad x bn partial products
+  float* out;      // slots x npad x bn partial products
   unsigned* status;
 };
 
@@ -2536,7 +2536,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(S2_THREADS, 1)
   const uint32_t drain_bar = bar0 + 8u * (2 * S2_STAGES + 4);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();
-  const int cid = blockIdx.x >> 1, ncl = gridDim.x >> 1;
+  const int cid = blockIdx.x >> 1;
+  const int x0 = p.sp.bound(cid), x1 = p.sp.bound(cid + 1);   // this cluster's k-blocks
   const uint32_t lead_bar0 = mapa_rank(bar0, 0);   // the rank-0 CTA's barriers, cluster addresses
   const int bhalf = p.bn / 2;
   const uint32_t b_bytes = (uint32_t)bhalf * 128;
@@ -2569,10 +2570,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(S2_THREADS, 1)
     // ------------------------------------------------ TMA producer (both CTAs)
     int it = 0;
     bool ok = true;
-    for (int u = cid; u < p.num_units && ok; u += ncl) {
-      const int m = u / p.splits, split = u % p.splits;
+    for (int x = x0; x < x1 && ok;) {
+      const int m = x / p.sp.kblocks, k0 = x - m * p.sp.kblocks, k1 = min(p.sp.kblocks, k0 + x1 - x);
+      x += k1 - k0;
       const int a_row = m * 256 + (int)rank * 128, b_row = (int)rank * bhalf;
-      for (int kb = 0; kb < p.kblocks; ++kb, ++it) {
+      for (int kb = k0; kb < k1; ++kb, ++it) {
         const int s = it % S2_STAGES;
         if (!mbar_wait(empty_bar(s), ((uint32_t)(it / S2_STAGES) & 1) ^ 1, abort_flag, p.status)) {
           ok = false;
@@ -2581,9 +2583,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(S2_THREADS, 1)
         if (rank == 0) mbar_expect_tx(full_bar(s), 2 * (S2_HALF + b_bytes));   // both CTAs' copies
         const uint32_t dst = smem_u32(smem + s * S2_STAGE);
         const uint32_t fb = lead_bar0 + 8u * s;
-        const int kx = (split * p.kblocks + kb) * BK;
-        tma_load_2d_pair(dst, &tmA, kx, a_row, fb);
-        tma_load_2d_pair(dst + S2_HALF, &tmB, kx, b_row, fb);
+        tma_load_2d_pair(dst, &tmA, kb * BK, a_row, fb);
+        tma_load_2d_pair(dst + S2_HALF, &tmB, kb * BK, b_row, fb);
       }
     }
     if (ok) {
@@ -2600,7 +2601,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(S2_THREADS, 1)
     // ------------------------------------------------ MMA issuer (rank 0 for the pair)
     int it = 0, tc = 0;
     bool ok = true, issued = false;
-    for (int u = cid; u < p.num_units && ok; u += ncl) {
+    for (int x = x0; x < x1 && ok;) {
+      const int k0 = x % p.sp.kblocks, k1 = min(p.sp.kblocks, k0 + x1 - x);
+      x += k1 - k0;
       const int acc = tc & 1;
       const uint32_t ar = (uint32_t)(tc >> 1);
       ++tc;
@@ -2610,7 +2613,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(S2_THREADS, 1)
       }
       tc_fence_after();
       const uint32_t d_tmem = tmem_base + (uint32_t)(acc * 256);
-      for (int kb = 0; kb < p.kblocks; ++kb, ++it) {
+      for (int kb = k0; kb < k1; ++kb, ++it) {
         const int s = it % S2_STAGES;
         if (!mbar_wait(full_bar(s), (uint32_t)(it / S2_STAGES) & 1, abort_flag, p.status)) {
           ok = false;
@@ -2622,7 +2625,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(S2_THREADS, 1)
         const uint64_t bdesc = smem_desc(a_addr + S2_HALF);
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk)
-          mma_bf16_pair(d_tmem, adesc + (uint64_t)(kk * 2), bdesc + (uint64_t)(kk * 2), p.idesc, (kb | kk) != 0);
+          mma_bf16_pair(d_tmem, adesc + (uint64_t)(kk * 2), bdesc + (uint64_t)(kk * 2), p.idesc,
+                        ((kb - k0) | kk) != 0);
         issued = true;
         mma_commit_pair(empty_bar(s));
       }
@@ -2644,16 +2648,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(S2_THREADS, 1)
     const int row_in_tile = q * 32 + lane;
     const int nchunk = p.bn / 64;   // 32-column chunks per warp
     int tc = 0;
-    for (int u = cid; u < p.num_units; u += ncl) {
+    for (int x = x0; x < x1;) {
+      const int m = x / p.sp.kblocks, slot = cid - p.sp.cluster_of(m * p.sp.kblocks);
+      x = min((m + 1) * p.sp.kblocks, x1);
       const int acc = tc & 1;
       const uint32_t ar = (uint32_t)(tc >> 1);
       ++tc;
       if (!mbar_wait(tfull_bar(acc), ar & 1, abort_flag, p.status)) break;
       tc_fence_after();
-      const int m = u / p.splits, split = u % p.splits;
       const int r = m * 256 + (int)rank * 128 + row_in_tile;
       const uint32_t taddr = tmem_base + (uint32_t)(acc * 256) + ((uint32_t)(q * 32) << 16);
-      float* P = p.out + ((size_t)split * p.npad + r) * p.bn;
+      float* P = p.out + ((size_t)slot * p.npad + r) * p.bn;
       const bool in = r - lane < p.npad;   // the warp's 32 rows are all in or all past the padded order
       for (int c = half * nchunk; c < half * nchunk + nchunk; ++c) {
         float v[32];
@@ -3278,8 +3283,8 @@ int tc_square_grouped_pairs(cdl_ctx* ctx, const TcGroup* host_first, const TcGro
   return L.done();
 }
 
-// Residue products t[l] = (A_l B_l^T mod p_l) + 128 of `planes` planes. a_planes: planes x a_rows x K bf16 (a_rows a multiple of 256, K of
-// 64); b_planes: planes x b_rows x K, or null for B = A, of which only the
+// Residue products t[l] = (A_l B_l^T mod p_l) + 128 of `planes` planes.
+// a_planes: planes x a_rows x K bf16 (a_rows a multiple of 256, K of 64); b_planes: planes x b_rows x K, or null for B = A, of which only the
 // 256 x 256 blocks on and above the diagonal are formed. t: planes x a_rows x
 // (b_rows or a_rows) bytes, 32-byte aligned.
 bool crt_gemm_supported(cdl_ctx* ctx, int K) {
@@ -3895,25 +3900,54 @@ int score_tc(cdl_ctx* ctx, const void* uplanes, const void* vplanes, const long 
   return score_tc_tiles(ctx, uplanes, vplanes, dint, oscale, n, rows, k2p, A1, A2, 0, 0, -1, contrib);
 }
 
+// On CTA pairs (kp a multiple of 32): as many clusters as are resident, but at
+// least APPLY_MIN_KB k-blocks each (below that the pipeline's filling and the
+// partial products outweigh the parallelism). Else equal splits: the fewest (a
+// divisor of the K blocks, at most 16) whose tiles fill the last round of CTAs
+// to 95 %, or the best filling.
+constexpr int APPLY_MIN_KB = 8;
+ApplySplit apply_split(cdl_ctx* ctx, int np, int kp) {
+  ApplySplit a;
+  const int kblocks = np / BK, ncl = pair_clusters(ctx);
+  if (ncl > 0 && kp % 32 == 0 && np % 256 == 0) {
+    a.rowblocks = np / 256;
+    a.kblocks = kblocks;
+    a.clusters = (int)std::max(1ll, std::min((long long)ncl, (long long)a.rowblocks * kblocks / APPLY_MIN_KB));
+    for (int m = 0; m < a.rowblocks; ++m) a.slots = std::max(a.slots, a.slots_of(m));
+    return a;
+  }
+  const int mb = np / BM, sm = ctx->sm_count;
+  double best = 0.0;
+  for (int sp = 1; sp <= 16 && sp <= kblocks; ++sp) {
+    if (kblocks % sp) continue;
+    const long long tl = (long long)mb * sp;
+    const double fill = (double)tl / (double)(((tl + sm - 1) / sm) * sm);
+    if (fill > best + 1e-9) {
+      best = fill;
+      a.slots = sp;
+    }
+    if (fill >= 0.95) break;
+  }
+  return a;
+}
+
 int apply_tc(cdl_ctx* ctx, const cdl_chain* ch, int level, const void* xop, float* partial, int kp,
-             int splits) {
-  if (!ch->host_levels) return apply_tc_mat(ctx, ch->level16(level), (int)ch->npad, xop, partial, kp, splits);
+             const ApplySplit& sp) {
+  if (!ch->host_levels) return apply_tc_mat(ctx, ch->level16(level), (int)ch->npad, xop, partial, kp, sp);
   cdl_chain* mch = const_cast<cdl_chain*>(ch);   // slot bookkeeping only
   const void* lv = ooc_read(ctx, mch, level);
   if (!lv) return CDL_ERR_CUDA;
-  CDL_TRY(apply_tc_mat(ctx, lv, (int)ch->npad, xop, partial, kp, splits));
+  CDL_TRY(apply_tc_mat(ctx, lv, (int)ch->npad, xop, partial, kp, sp));
   CDL_TRY(ooc_read_done(ctx, mch, level));
   return ooc_prefetch(ctx, mch, (level + 1) % ch->d_eff);   // overlaps the next level's load with this update
 }
 
-int apply_tc_mat(cdl_ctx* ctx, const void* amat, int np, const void* xop, float* partial, int kp, int splits) {
+int apply_tc_mat(cdl_ctx* ctx, const void* amat, int np, const void* xop, float* partial, int kp,
+                 const ApplySplit& sp) {
   const int bn = 2 * kp;
   if (bn % 32 || bn < 32 || bn > MAX_BN) return CDL_ERR_UNSUPPORTED;
   const int mb = np / BM;
-  if ((np / BK) % splits) return CDL_ERR_INVALID_ARG;
-  const int ncl = pair_clusters(ctx);
-  if (ncl > 0 && bn % 64 == 0) {
-    // CTA pairs: 256-row blocks, each CTA staging half of the right-hand-side operand
+  if (sp.clusters > 0) {
     static bool attr = false;
     if (!attr) {
       CDL_CUDA_TRY(cudaFuncSetAttribute(k_tc_apply2, cudaFuncAttributeMaxDynamicSharedMemorySize, S2_SMEM_BYTES));
@@ -3923,19 +3957,18 @@ int apply_tc_mat(cdl_ctx* ctx, const void* amat, int np, const void* xop, float*
     CDL_TRY(make_map(&ma, amat, np, np, 128));
     CDL_TRY(make_map(&mbm, xop, bn, np, bn / 2));
     Apply2Params p{};
-    p.num_units = ((np + 255) / 256) * splits;
-    p.splits = splits;
-    p.kblocks = np / BK / splits;
+    p.sp = sp;
     p.npad = np;
     p.bn = bn;
     p.idesc = make_idesc_m256(bn);
     p.out = partial;
     p.status = ctx->dev_status;
-    const int clusters = std::min(p.num_units, ncl);
     Launch L(ctx, CDL_KC_APPLY, 2.0 * np * (double)np);
-    k_tc_apply2<<<2 * clusters, S2_THREADS, S2_SMEM_BYTES, ctx->stream>>>(ma, mbm, p);
+    k_tc_apply2<<<2 * sp.clusters, S2_THREADS, S2_SMEM_BYTES, ctx->stream>>>(ma, mbm, p);
     return L.done();
   }
+  const int splits = sp.slots;
+  if ((np / BK) % splits) return CDL_ERR_INVALID_ARG;
   const uint32_t* tiles;
   int count;
   CDL_TRY(get_tiles(ctx, "tc.apply." + std::to_string(mb) + "." + std::to_string(splits),
