@@ -146,22 +146,6 @@ __global__ void __launch_bounds__(256) k_split_a(const double* __restrict__ A, s
   }
 }
 
-// max |x_i| as float64 bits (for x >= 0 the bit patterns order like the values).
-__global__ void __launch_bounds__(256) k_abs_max_bits(const double* __restrict__ x, size_t count,
-                                                       unsigned long long* __restrict__ out) {
-  unsigned long long m = 0;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x[i]) & 0x7FFFFFFFFFFFFFFFull;
-    m = b > m ? b : m;
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long v = __shfl_xor_sync(0xffffffffu, m, o);
-    m = v > m ? v : m;
-  }
-  if ((threadIdx.x & 31) == 0 && m) atomicMax(out, m);
-}
-
 // A / 2^s on the grid 2^-48 as the integer N = round(A 2^(48 - s)), with 2^s
 // the least power of two (s >= 0) not below max A, so that A / 2^s lies in
 // [0, 1] (the kernel graphs have s = 0). The rounding uses the float64 bit
@@ -234,18 +218,19 @@ __device__ __forceinline__ void digits6_fbits(long long N, uint32_t (&f)[6]) {
   f[0] = __float_as_uint(__fmaf_rn(__uint_as_float(0x4B000000u | (uint32_t)hi), sc0, -8388608.0f * sc0));
 }
 
-// SL = false (the batched form's chains, which keep no slices): S and
-// a_scale are not touched (they may be null).
 // One group of 8 columns (index g over the npad x npad / 8 groups, row-major)
-// of k_chain_init_tc's outputs.
+// of k_chain_init_tc's outputs; the slices S (of A 2^-sexp) only if `slices`.
+// Returns the largest weight as a float (rounded to nearest: the digits hold
+// weights up to 1 + 2^-9 of the scale).
 template <bool SL>
-__device__ __forceinline__ void chain_init_tc_group(const double* __restrict__ A, int n, int npad,
+__device__ __forceinline__ float chain_init_tc_group(const double* __restrict__ A, int n, int npad,
                                                     const float* __restrict__ rsf, const float* __restrict__ uf,
                                                     __nv_bfloat16* __restrict__ L0, __nv_bfloat16* __restrict__ Ahi,
                                                     __nv_bfloat16* __restrict__ Alo, uint16_t* __restrict__ S, int sexp,
-                                                    size_t g) {
+                                                    bool slices, size_t g) {
   const size_t plane = (size_t)npad * npad;
   const int gpr = npad / 8;                               // groups of 8 columns per row
+  float mx = 0.f;
   {
     const int i = (int)(g / gpr), j0 = (int)(g % gpr) * 8;
     const size_t o = (size_t)i * npad + j0;
@@ -264,7 +249,10 @@ __device__ __forceinline__ void chain_init_tc_group(const double* __restrict__ A
             const double a = row[j];
             af[h] = d2f_rn_nonneg(a);
             v[h] = __fmaf_rn(af[h], __fmul_rn(ri, rsf[j]), -__fmul_rn(ui, uf[j]));
-            if constexpr (SL) digits6_fbits(grid48(a, sexp), dg[h]);
+            if constexpr (SL) {
+              digits6_fbits(grid48(a, sexp), dg[h]);
+              mx = fmaxf(mx, af[h]);
+            }
           }
         }
         const __nv_bfloat162 lv = __floats2bfloat162_rn(v[0], v[1]);
@@ -285,30 +273,62 @@ __device__ __forceinline__ void chain_init_tc_group(const double* __restrict__ A
     *reinterpret_cast<uint4*>(Ahi + o) = make_uint4(wh[0], wh[1], wh[2], wh[3]);
     *reinterpret_cast<uint4*>(Alo + o) = make_uint4(wo[0], wo[1], wo[2], wo[3]);
     if constexpr (SL) {
+      if (slices)
 #pragma unroll
-      for (int t = 0; t < 6; ++t)
-        *reinterpret_cast<uint4*>(S + (size_t)t * plane + o) = make_uint4(ws[t][0], ws[t][1], ws[t][2], ws[t][3]);
+        for (int t = 0; t < 6; ++t)
+          *reinterpret_cast<uint4*>(S + (size_t)t * plane + o) = make_uint4(ws[t][0], ws[t][1], ws[t][2], ws[t][3]);
     }
   }
+  return mx;
 }
 
+// The slices are formed with scale 2^0, right for kernel graphs (weights at most
+// 1): no pass over A for its largest weight. Where a weight above 1 turns up
+// (its float64 bits in *over, zeroed before) no further slices are written, and
+// k_a_slices forms them all with the scale that the finished maximum gives. SL =
+// false: no slices.
 template <bool SL>
 __global__ void __launch_bounds__(256) k_chain_init_tc(const double* __restrict__ A, int n, int npad,
                                                         const float* __restrict__ rsf, const float* __restrict__ uf,
                                                         __nv_bfloat16* __restrict__ L0, __nv_bfloat16* __restrict__ Ahi,
                                                         __nv_bfloat16* __restrict__ Alo, uint16_t* __restrict__ S,
-                                                        double* __restrict__ a_scale) {
-  int sexp = 0;
-  if constexpr (SL) {
-    sexp = pow2_exp_above((unsigned long long)__double_as_longlong(a_scale[1]));
-    if (blockIdx.x == 0 && threadIdx.x == 0) a_scale[0] = __longlong_as_double((long long)(1023 + sexp) << 52);
-  }
+                                                        unsigned long long* __restrict__ over) {
   const int gpr = npad / 8;                               // groups of 8 columns per row
+  float m = 1.f;
+  bool slices = true;
+  int it = 0;
   for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < (size_t)npad * gpr;
-       g += (size_t)gridDim.x * blockDim.x)
-    chain_init_tc_group<SL>(A, n, npad, rsf, uf, L0, Ahi, Alo, S, sexp, g);
+       g += (size_t)gridDim.x * blockDim.x, ++it) {
+    if (SL && slices && it % 8 == 0) slices = *reinterpret_cast<volatile unsigned long long*>(over) == 0;
+    const float x = chain_init_tc_group<SL>(A, n, npad, rsf, uf, L0, Ahi, Alo, S, 0, slices, g);
+    if (SL && x > m) {
+      if (m == 1.f) atomicMax(over, (unsigned long long)__double_as_longlong((double)x));   // tell the others at once
+      m = x;
+      slices = false;
+    }
+  }
+  if (SL && m > 1.f) atomicMax(over, (unsigned long long)__double_as_longlong((double)m));
 }
 
+// The slices of a graph with a weight above 1 (a_scale[1] its float64 bits; 0:
+// nothing to do), and their scale in a_scale[0].
+__global__ void __launch_bounds__(256) k_a_slices(const double* __restrict__ A, int n, int npad,
+                                                   uint16_t* __restrict__ S, double* __restrict__ a_scale) {
+  const int sexp = pow2_exp_above((unsigned long long)__double_as_longlong(a_scale[1]));
+  if (blockIdx.x == 0 && threadIdx.x == 0) a_scale[0] = __longlong_as_double((long long)(1023 + sexp) << 52);
+  if (sexp == 0) return;
+  const size_t plane = (size_t)npad * npad;
+  for (size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x; o < plane / 2; o += (size_t)gridDim.x * blockDim.x) {
+    const int i = (int)(2 * o / npad), j = (int)(2 * o % npad);
+    uint32_t dg[2][6] = {};
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (i < n && j + h < n) digits6_fbits(grid48(A[(size_t)i * n + j + h], sexp), dg[h]);
+#pragma unroll
+    for (int t = 0; t < 6; ++t)
+      reinterpret_cast<uint32_t*>(S + (size_t)t * plane)[o] = __byte_perm(dg[0][t], dg[1][t], 0x7632);
+  }
+}
 
 // C = P^T Q on CUDA cores: C[m][c] = sum_k P[k][m] Q[k][c]; P is K x M and Q
 // is K x N, both row-major, so both tiles are contiguous k-major slabs.
@@ -524,17 +544,9 @@ __global__ void __launch_bounds__(256) k_g_chain_init(const uint32_t* __restrict
   __nv_bfloat16* alo = ahi + (size_t)G.npad * G.npad;
   // the exact slices of A on the grids 2^-8s (kernel weights are at most 1: scale 2^0)
   for (size_t g = (size_t)(t >> 12) * 2048 + threadIdx.x; g < g1; g += 256)
-    chain_init_tc_group<true>(G.A, G.n, G.npad, G.rsf, G.uf, L0, ahi, alo, G.aslices, 0, g);
+    chain_init_tc_group<true>(G.A, G.n, G.npad, G.rsf, G.uf, L0, ahi, alo, G.aslices, 0, true, g);
 }
 }  // namespace
-
-int abs_max_bits(cdl_ctx* ctx, const double* x, size_t count, unsigned long long* out) {
-  CDL_CUDA_TRY(cudaMemsetAsync(out, 0, sizeof(unsigned long long), ctx->stream));
-  Launch L(ctx, CDL_KC_MISC, 8.0 * (double)count);
-  const size_t blocks = std::min<size_t>((count + 255) / 256, (size_t)ctx->sm_count * 8);
-  k_abs_max_bits<<<(unsigned)std::max<size_t>(blocks, 1), 256, 0, ctx->stream>>>(x, count, out);
-  return L.done();
-}
 
 int chain_split_a(cdl_ctx* ctx, const cdl_chain* ch, const double* A) {
   const size_t cnt = (size_t)ch->n * ch->n;
@@ -545,16 +557,6 @@ int chain_split_a(cdl_ctx* ctx, const cdl_chain* ch, const double* A) {
 
 int chain_init(cdl_ctx* ctx, cdl_chain* ch, const double* A) {
   const int n = (int)ch->n, np = (int)ch->npad;
-  if (ch->aslices) {   // the slices' scale: max A, known before level 0 is formed
-    unsigned long long* mb = reinterpret_cast<unsigned long long*>(ch->a_scale + 1);
-    if (ctx->amax_hint_A == A && ctx->amax_hint_bits)
-      CDL_CUDA_TRY(cudaMemcpyAsync(mb, ctx->amax_hint_bits, sizeof(unsigned long long), cudaMemcpyDeviceToDevice,
-                                   ctx->stream));
-    else
-      CDL_TRY(abs_max_bits(ctx, A, (size_t)n * n, mb));
-  }
-  ctx->amax_hint_A = nullptr;
-  ctx->amax_hint_bits = nullptr;
   void* wsu;
   CDL_TRY(ws_get(ctx, "chain.u", (size_t)np * (sizeof(double) + 2 * sizeof(float)), &wsu));
   double* u = static_cast<double*>(wsu);
@@ -572,32 +574,45 @@ int chain_init(cdl_ctx* ctx, cdl_chain* ch, const double* A) {
                        (ch->aop ? 4.0 * np * (double)np : 0.0) + (tensor ? 12.0 * np * (double)np : 0.0);
   const int blocks = std::min(np, ctx->sm_count * 8);
   // level 0 in bf16 with A hi/lo and the slices (tensor chains)
-  auto init16 = [&](void* L0) {
+  auto init16 = [&](void* L0) -> int {
     __nv_bfloat16* l0 = static_cast<__nv_bfloat16*>(L0);
     __nv_bfloat16* ahi = static_cast<__nv_bfloat16*>(ch->aop);
     __nv_bfloat16* alo = ahi + (size_t)np * np;
-    if (tensor)
-      k_chain_init_tc<true><<<ctx->sm_count * 8, 256, 0, ctx->stream>>>(
-          A, n, np, rsf, uf, l0, ahi, alo, static_cast<uint16_t*>(ch->aslices), ch->a_scale);
-    else
-      k_chain_init_tc<false><<<ctx->sm_count * 8, 256, 0, ctx->stream>>>(A, n, np, rsf, uf, l0, ahi, alo, nullptr,
-                                                                         nullptr);
+    uint16_t* sl = static_cast<uint16_t*>(ch->aslices);
+    {
+      Launch L(ctx, CDL_KC_CHAIN_INIT, bytes);
+      if (tensor) {
+        unsigned long long* over = reinterpret_cast<unsigned long long*>(ch->a_scale + 1);
+        CDL_CUDA_TRY(cudaMemsetAsync(over, 0, sizeof(unsigned long long), ctx->stream));
+        k_chain_init_tc<true><<<ctx->sm_count * 8, 256, 0, ctx->stream>>>(A, n, np, rsf, uf, l0, ahi, alo, sl, over);
+      } else {
+        k_chain_init_tc<false><<<ctx->sm_count * 8, 256, 0, ctx->stream>>>(A, n, np, rsf, uf, l0, ahi, alo, nullptr,
+                                                                           nullptr);
+      }
+      CDL_TRY(L.done());
+    }
+    if (!tensor) return CDL_OK;
+    Launch L(ctx, CDL_KC_CHAIN_INIT, 0);
+    k_a_slices<<<ctx->sm_count * 8, 256, 0, ctx->stream>>>(A, n, np, sl, ch->a_scale);
+    return L.done();
   };
-  Launch L(ctx, CDL_KC_CHAIN_INIT, bytes);
   switch (ch->dtype) {
-    case CDL_F64:
+    case CDL_F64: {
+      Launch L(ctx, CDL_KC_CHAIN_INIT, bytes);
       k_chain_init<double><<<blocks, 256, 0, ctx->stream>>>(A, n, np, ch->rsqrt_d, u,
                                                             static_cast<double*>(ch->level(0)));
-      break;
-    case CDL_F32:
+      return L.done();
+    }
+    case CDL_F32: {
+      Launch L(ctx, CDL_KC_CHAIN_INIT, bytes);
       k_chain_init<float><<<blocks, 256, 0, ctx->stream>>>(A, n, np, ch->rsqrt_d, u,
                                                            static_cast<float*>(ch->level(0)));
-      break;
+      return L.done();
+    }
     case CDL_FP8E4M3: {
       // bf16 level 0 (apply copy) and A_hi/A_lo, then the bound and the e4m3 level
       CDL_CUDA_TRY(cudaMemsetAsync(ch->amax, 0, ch->d * sizeof(unsigned), ctx->stream));
-      init16(ch->level16(0));
-      CDL_TRY(L.done());
+      CDL_TRY(init16(ch->level16(0)));
       const size_t cnt = (size_t)np * np;
       {
         Launch L2(ctx, CDL_KC_CHAIN_INIT, 2.0 * cnt);
@@ -611,19 +626,16 @@ int chain_init(cdl_ctx* ctx, cdl_chain* ch, const double* A) {
       return L3.done();
     }
     case CDL_FP8E4M3_T128:
-      init16(ch->level16(0));
-      CDL_TRY(L.done());
+      CDL_TRY(init16(ch->level16(0)));
       return fp8t_quantize_level0(ctx, ch);
     case CDL_BF16: {
       void* L0 = ch->host_levels ? ooc_write_begin(ctx, ch, 0) : ch->level(0);
-      init16(L0);
-      CDL_TRY(L.done());
+      CDL_TRY(init16(L0));
       return ch->host_levels ? ooc_write_end(ctx, ch, 0) : CDL_OK;
     }
     default:
       return CDL_ERR_UNSUPPORTED;
   }
-  return L.done();
 }
 
 // Max absolute row sum of an npad x npad level (rows of threads; atomicMax

@@ -81,11 +81,6 @@ struct cdl_ctx {
   std::map<std::string, int> tile_lists;
   int debug_flags = 0;   // CDL_DEBUG_* test hooks
   cdl::BatchPlan* batch = nullptr;   // plan of the last cdl_caddelag_batched call
-  // one-shot hint from the pair driver: the device float64 bits of max |A| of the
-  // graph at amax_hint_A (found while its kernel values were formed), taken and
-  // cleared by the next chain build of that graph instead of a pass over A
-  const double* amax_hint_A = nullptr;
-  const unsigned long long* amax_hint_bits = nullptr;
 };
 
 namespace cdl {
@@ -109,7 +104,7 @@ struct cdl_chain {
                               // (npad/128)^2 512-byte atoms, each the tile's e8m0 scale byte repeated
   void* aslices = nullptr;    // tensor chains: A / a_scale as 6 bf16 planes npad x npad on the grids 2^-8s
   double* a_scale = nullptr;  // tensor chains (device, 2 words): [0] the power of two >= max A that the
-                              // slices are taken of, [1] the float64 bits of max |A|
+                              // slices are taken of, [1] the float64 bits of the largest weight above 1 (0: none)
   double* rsqrt_d = nullptr;  // npad: D_i^{-1/2} (0 in padding)
   double* D = nullptr;        // npad: degrees (0 in padding)
   double* vol = nullptr;      // 1
@@ -152,10 +147,6 @@ int ws_get(cdl_ctx* ctx, const char* name, size_t bytes, void** out);
 bool ws_reclaim(cdl_ctx* ctx);
 cudaError_t malloc_reclaim(cdl_ctx* ctx, void** p, size_t bytes);
 
-// *out (device) = the float64 bit pattern of max |x_i| over count values
-// (asynchronous; out is zeroed first).
-int abs_max_bits(cdl_ctx* ctx, const double* x, size_t count, unsigned long long* out);
-
 // Folds src's pending timings and adds its launch counters into dst, then
 // zeroes src's counters.
 int ctx_absorb(cdl_ctx* dst, cdl_ctx* src);
@@ -187,10 +178,8 @@ inline int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 
 // ---- kernel launchers (one per translation unit family) ----
 // graph.cu
-// amax_bits (device, optional): receives the float64 bits of max A.
 int graph_build(cdl_ctx* ctx, const double* X, int64_t n, int T, double sigma, double* A,
-                double* D, double* vol, double* sigma_out, int kernel = 0,
-                unsigned long long* amax_bits = nullptr);
+                double* D, double* vol, double* sigma_out, int kernel = 0);
 int graph_degrees(cdl_ctx* ctx, const double* A, int64_t n, double* D, double* vol);
 int graph_add_edges(cdl_ctx* ctx, double* A, int64_t n, int64_t m, const int64_t* ij, const double* w,
                     int64_t* n_bad);
@@ -606,8 +595,7 @@ int chain_vectors_only(cdl_ctx* ctx, cdl_chain* ch);
 int chain_level0_panel(cdl_ctx* ctx, cdl_chain* ch, void* L0, const double* panel, int r0, int rows);
 int panel_slices_t(cdl_ctx* ctx, const double* panel, int n, int np, int r0, int rows, int Pw, void* slicesT);
 // project.cu: rows r0 .. r0 + rows - 1 of Y from a panel; column centring.
-int project_panel(cdl_ctx* ctx, const double* panel, int64_t n, int r0, int rows, int k, uint64_t seed, double* Y,
-                  const unsigned long long* amax_bits);
+int project_panel(cdl_ctx* ctx, const double* panel, int64_t n, int r0, int rows, int k, uint64_t seed, double* Y);
 int project_center(cdl_ctx* ctx, int64_t n, int k, double* Y);
 // score.cu: CAD scores (bf16 tensor-core Gram) with A1 and A2 supplied row
 // panel by row panel: fill(r0, rows, &A1, &A2) makes rows r0 .. r0 + rows - 1
@@ -627,10 +615,7 @@ int chain_create_regen(cdl_ctx* ctx, int64_t n, int d, int resident, cdl_chain**
 int chain_solve(cdl_ctx* ctx, const cdl_chain* ch, const double* A, const double* Y, int k,
                 const cdl_solve_opts* opts, double* Z, cdl_solve_stats* stats);
 // project.cu
-// amax_bits (device, optional): the float64 bits of max |A| if already known
-// (nullptr: found by a pass over A).
-int project(cdl_ctx* ctx, const double* A, int64_t n, int k, uint64_t seed, double* Y,
-            const unsigned long long* amax_bits = nullptr);
+int project(cdl_ctx* ctx, const double* A, int64_t n, int k, uint64_t seed, double* Y);
 // score.cu
 int cad_score(cdl_ctx* ctx, const double* A1, const double* A2, const double* Z1,
               const double* Z2, const double* vol1, const double* vol2, int64_t n, int k,

@@ -105,7 +105,6 @@ int pair_regen(cdl_ctx* ctx, const double* X1, const double* X2, int64_t n64, in
   cdl_chain* ch = ctx->regen_chain;
   if (ch->resident < 1) return CDL_ERR_UNSUPPORTED;   // level 0 is formed in place, panel by panel
 
-  unsigned long long* one_bits = reinterpret_cast<unsigned long long*>(ch->a_scale + 1);   // max A <= 1
   bool converged = true;
   for (int g = 0; g < 2; ++g) {
     G[g].id = g;
@@ -124,7 +123,7 @@ int pair_regen(cdl_ctx* ctx, const double* X1, const double* X2, int64_t n64, in
       const int rows = std::min(P, n - r0);
       CDL_TRY(regen_panel(ctx, G[g], panel[0], r0, rows, Dscr));
       CDL_TRY(chain_level0_panel(ctx, ch, L0, panel[0], r0, rows));
-      CDL_TRY(project_panel(ctx, panel[0], n64, r0, rows, k, o->seed, static_cast<double*>(dY), one_bits));
+      CDL_TRY(project_panel(ctx, panel[0], n64, r0, rows, k, o->seed, static_cast<double*>(dY)));
     }
     CDL_TRY(ooc_write_end(ctx, ch, 0));
     CDL_TRY(project_center(ctx, n64, k, static_cast<double*>(dY)));
