@@ -239,7 +239,7 @@ int build_plan(cdl_ctx* ctx, int G, const int64_t* n, int T, const cdl_batch_opt
     P->pv.push_back(pvar);
   }
   size_t ntiles = ap.size() + t32.size() + elem.size() + zst.size() + runits.size() + csb.size() + sel.size() +
-                  spairs.size() + snodes.size() + gt.fixed.size() + gt.dist.size() + gt.rows.size() + cvec.size() +
+                  spairs.size() + snodes.size() + gt.fixed.size() + gt.dist.size() + cvec.size() +
                   cinit.size();
   for (auto& v : sq) ntiles += v.size();
   for (auto& v : pblocks) ntiles += v.size();
@@ -372,6 +372,7 @@ int build_plan(cdl_ctx* ctx, int G, const int64_t* n, int T, const cdl_batch_opt
     Gg.X = P->X + ((g & 1) ? P->N : 0) * (size_t)T + P->off[p] * (size_t)T;
     Gg.A = P->A[g];
     Gg.D = P->Dv[g];
+    Gg.part = static_cast<double*>(ch.levels);   // n^2 / 8 + 8 n bytes at most of 2 npad^2, before level 0 is formed
     Gg.vol = P->scal[g];
     Gg.sigma = P->scal[g] + 1;
     Gg.sel = sel_all + (size_t)g * sel_one;
@@ -474,7 +475,6 @@ int build_plan(cdl_ctx* ctx, int G, const int64_t* n, int T, const cdl_batch_opt
   GraphBatch& gb = P->gb;
   add(gt.fixed, gb.fixed);
   add(gt.dist, gb.dist);
-  add(gt.rows, gb.rows);
   for (size_t v = 0; v < pblocks.size(); ++v) add(pblocks[v], P->pv[v].blocks);
   add(cvec, P->cvec);
   add(cinit, P->cinit);

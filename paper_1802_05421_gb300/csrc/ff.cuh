@@ -71,13 +71,12 @@ __device__ __forceinline__ double f2d_bits(float f) {
 // exact scalings. Values below 2^-100 give {0, 0}.
 __device__ __forceinline__ ff split_nonneg(double x) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const int e = (int)((b >> 52) & 0x7FF) - 1023;      // x in [2^e, 2^(e+1))
-  if (e < -100) return {0.f, 0.f};
-  const uint32_t hi_bits = ((uint32_t)(e + 127) << 23) | ((uint32_t)(b >> 29) & 0x7FFFFFu);
-  const uint32_t low29 = (uint32_t)(b & 0x1FFFFFFFull);
+  if ((uint32_t)(b >> 52) < 1023 - 100) return {0.f, 0.f};
+  const uint32_t hi_bits = (uint32_t)(b >> 29) - ((1023u - 127u) << 23);   // x in [2^e, 2^(e+1)), e >= -100
   // lo = low29 2^(e - 52) = (low29 2^-52) 2^e: both factors are normal floats
   // for e >= -100 (2^(e - 52) itself is not, below e = -74)
-  const float lo = __fmul_rn(__fmul_rn(__uint2float_rn(low29), 0x1p-52f), __uint_as_float((uint32_t)(e + 127) << 23));
+  const float lo = __fmul_rn(__fmul_rn(__uint2float_rn((uint32_t)b & 0x1FFFFFFFu), 0x1p-52f),
+                             __uint_as_float(hi_bits & 0x7F800000u));
   return {__uint_as_float(hi_bits), lo};
 }
 
@@ -162,113 +161,72 @@ __device__ __forceinline__ double sqrt_nonneg(double x) {
                                           ((unsigned long long)(long long)j << 52)));
 }
 
-// e^x for a float-float |x| <= 0.35, from the series definition: the Taylor
-// series to degree 12 (remainder below 2^-52), degrees 7..12 in float32 (each
-// term below 2^-22 of the result), degrees 0..6 in float-float Horner steps; the
-// coefficients 1/m! are stored as float pairs. It fills the table of
-// ff_exp_table.
-__device__ __forceinline__ ff ff_exp_series(ff x) {
-  float p = 0x1.1eed8ep-29f;                      // 1/12!
-  p = __fmaf_rn(p, x.hi, 0x1.ae6456p-26f);        // 1/11!
-  p = __fmaf_rn(p, x.hi, 0x1.27e4fcp-22f);        // 1/10!
-  p = __fmaf_rn(p, x.hi, 0x1.71de3ap-19f);        // 1/9!
-  p = __fmaf_rn(p, x.hi, 0x1.a01a02p-16f);        // 1/8!
-  p = __fmaf_rn(p, x.hi, 0x1.a01a02p-13f);        // 1/7!
-  ff q = {p, 0.f};
-  q = ff_add(ff_mul(q, x), ff{0x1.6c16c2p-10f, -0x1.27d27ep-35f});   // 1/6!
-  q = ff_add(ff_mul(q, x), ff{0x1.111112p-7f, -0x1.dddddep-32f});    // 1/5!
-  q = ff_add(ff_mul(q, x), ff{0x1.555556p-5f, -0x1.555556p-30f});    // 1/4!
-  q = ff_add(ff_mul(q, x), ff{0x1.555556p-3f, -0x1.555556p-28f});    // 1/3!
-  q = ff_add(ff_mul(q, x), ff{0x1p-1f, 0.f});                        // 1/2!
-  q = ff_add(ff_mul(q, x), ff{1.f, 0.f});                            // 1/1!
-  q = ff_add(ff_mul(q, x), ff{1.f, 0.f});                            // 1/0!
-  return q;
-}
+// exp(-x y) for float64 x >= 0 and a factor y > 0 prepared once per block, with
+// integer operations only (float64 and its conversions run on the scarce pipe):
+// u = x y log2(e) in fixed point with 54 fractional bits, from the 64-bit product
+// of x's mantissa and the 64-bit factor c = y log2(e); 2^-u = 2^-k 2^(-j/256)
+// 2^-g with k its integer part, j its next 8 bits and 0 <= g < 2^-8; 2^(-j/256)
+// from a table of 64-bit integers; 2^-g = 1 - g (c1 - g (c2 - g (c3 - g c4))), c_i
+// = (ln 2)^i / i!, from the exponential series (its degree 5 is below 1.2e-15),
+// the inner terms in 32 bits (they are below 2^-10 of c1), the outer product and
+// the product with the table in 64. Error at most 2.1e-15 relative, 2.0e-16 on
+// average (a host emulation against quad precision over 3.5e6 arguments). About
+// 80 instructions; through 128-bit shifts, ln 2 in natural units and a float-float
+// series it took about 300, at 1.4e-14.
+constexpr int EXP_TABLE = 256;
+__constant__ const unsigned long long EXP2_NEG_16[16] = {   // 2^(63 - i / 16)
+    0x8000000000000000ull, 0x7a92be8a92436616ull, 0x75606373ee921c97ull, 0x70666f76154a7089ull,
+    0x6ba27e656b4eb57aull, 0x6712460a8fc24072ull, 0x62b39508aa836d6full, 0x5e8451cfac061b5full,
+    0x5a827999fcef3242ull, 0x56ac1f752150a563ull, 0x52ff6b54d8a89c75ull, 0x4f7a993048d088d7ull,
+    0x4c1bf828c6dc54b8ull, 0x48e1e9b9d588e19bull, 0x45cae0f1f545eb73ull, 0x42d561b3e6243d8aull};
+__constant__ const unsigned long long EXP2_NEG_256[16] = {  // 2^(63 - i / 256)
+    0x8000000000000000ull, 0x7fa765aca88f6453ull, 0x7f4f08ae3dc7c426ull, 0x7ef6e8da4b544f9aull,
+    0x7e9f06067a4360baull, 0x7e47600890f223deull, 0x7deff6b672f84e24ull, 0x7d98c9e62113e1faull,
+    0x7d41d96db915019dull, 0x7ceb252375c9cf9bull, 0x7c94acddaeea5d3aull, 0x7c3e7072d904a6ceull,
+    0x7be86fb985689ddcull, 0x7b92aa886214411cull, 0x7b3d20b6399fc237ull, 0x7ae7d219f329b948ull};
 
-// exp(-x y) for float64 x >= 0, y > 0 with x y < 690, as (q.hi + q.lo) 2^-k
-// with no float64 operation: the product t = x y is formed exactly as the
-// 106-bit product of the two 53-bit mantissas and kept to 64 fractional bits
-// (128-bit integers); k = round(t / ln2) from a float estimate; r = t - k ln2
-// with ln2 to 64 fractional bits (error below 2^-54 for k < 1024) is a signed
-// 64-bit fixed-point number. It is reduced once more, exactly, by j / 32 with j
-// = round(32 r) (|j| <= 11): exp(-r) = exp(-j / 32) exp(-r') with |r'| <= 1/64,
-// exp(-j / 32) from a table of float-float values (ff_exp_table) and exp(-r')
-// from the series to degree 6 (remainder below 2^-54): degrees 4..6 in float32,
-// 0..3 in float-float Horner steps. About 1.4e-14 relative, as the degree-12
-// series on r alone (a host emulation against quad precision over 2e7
-// arguments gives 1.33e-14 and 1.41e-14).
-__device__ __forceinline__ ff ff_exp_series6(ff x) {
-  float p = 0x1.6c16c2p-10f;                      // 1/6!
-  p = __fmaf_rn(p, x.hi, 0x1.111112p-7f);         // 1/5!
-  p = __fmaf_rn(p, x.hi, 0x1.555556p-5f);         // 1/4!
-  ff q = {p, 0.f};
-  q = ff_add(ff_mul(q, x), ff{0x1.555556p-3f, -0x1.555556p-28f});   // 1/3!
-  q = ff_add(ff_mul(q, x), ff{0x1p-1f, 0.f});                        // 1/2!
-  q = ff_add(ff_mul(q, x), ff{1.f, 0.f});                            // 1/1!
-  q = ff_add(ff_mul(q, x), ff{1.f, 0.f});                            // 1/0!
-  return q;
-}
-
-// exp(-j / 32) for j = -11 .. 11 at tab[j + 11], from the degree-12 series
-// (|j / 32| <= 0.35, exact in float). Threads 0 .. 22 of the block fill it;
-// the caller synchronises before use.
-constexpr int FF_EXP_TABLE = 23;
-__device__ __forceinline__ void ff_exp_table(ff* tab) {
-  if (threadIdx.x < FF_EXP_TABLE) tab[threadIdx.x] = ff_exp_series(ff{(float)(11 - (int)threadIdx.x) * 0.03125f, 0.f});
-}
-
-__device__ __forceinline__ ff ff_exp_neg_prod(double x, double y, int& k_out, const ff* __restrict__ tab) {
-  const unsigned long long bx = (unsigned long long)__double_as_longlong(x);
-  const unsigned long long by = (unsigned long long)__double_as_longlong(y);
-  const int ex = (int)((bx >> 52) & 0x7FF), ey = (int)((by >> 52) & 0x7FF);
-  unsigned __int128 T = 0;                                           // t 2^64
-  if (ex != 0 && ey != 0) {
-    const unsigned long long mx = (bx & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-    const unsigned long long my = (by & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-    const unsigned __int128 P = (unsigned __int128)mx * my;         // t = P 2^(ex + ey - 2150)
-    const int sh = ex + ey - 2150 + 64;                              // T = P 2^sh, sh < -30 for t < 2^10
-    if (sh >= 0)
-      T = P << sh;
-    else if (sh > -127)
-      T = P >> (-sh);
+// Threads 0 .. 255 of the block fill the table 2^(63 - j / 256); the caller
+// synchronises before use.
+__device__ __forceinline__ void exp_table(unsigned long long* tab) {
+  for (int j = threadIdx.x; j < EXP_TABLE; j += blockDim.x) {
+    const unsigned long long a = EXP2_NEG_16[j >> 4], b = EXP2_NEG_256[j & 15];
+    tab[j] = (__umul64hi(a, b) << 1) | ((a * b) >> 63);
   }
-  const float tf = __fmul_rn(u64_top24((unsigned long long)(T >> 40)), 0x1p-24f);
-  const int k = __float2int_rn(__fmul_rn(tf, 0x1.715476p+0f));       // t / ln2
-  const unsigned __int128 kl = (unsigned __int128)(unsigned)k * 0xB17217F7D1CF79ABull;   // k ln2 2^64
-  const long long r = (long long)(__int128)(T - kl);                 // |r| < 2^63
-  long long j = (r + (1ll << 58)) >> 59;                             // round(32 r), |j| <= 11
-  j = j < -11 ? -11 : (j > 11 ? 11 : j);                             // (a guard: |r| <= 0.35 here)
-  const long long r2 = r - j * (1ll << 59);                          // |r2| <= 2^58: |r'| <= 1/64
-  const unsigned long long ar = r2 < 0 ? (unsigned long long)(-r2) : (unsigned long long)r2;
-  const ff m = ff_from_u64(ar);
-  const float hi = __fmul_rn(m.hi, 0x1p-64f), lo = __fmul_rn(m.lo, 0x1p-64f);   // exact powers of two
-  k_out = k;
-  const ff e = ff_exp_series6(r2 < 0 ? ff{hi, lo} : ff{-hi, -lo});   // exp(-r')
-  return ff_mul(e, tab[j + 11]);                                      // exp(-r), in [0.70, 1.42]
 }
 
-// (q.hi + q.lo) 2^-k as float64 for q in [0.5, 2) (q.hi > 0, |q.lo| <= ulp(q.hi)),
-// rounded to nearest even, with integer operations only (2^-k in the normal range).
-__device__ __forceinline__ double ff_scaled_to_double(ff q, int k) {
-  const uint32_t hb = __float_as_uint(q.hi);
-  const int eh = (int)((hb >> 23) & 0xFF) - 127;                     // -1 or 0
-  long long V = (long long)((hb & 0x7FFFFFu) | 0x800000u) << (eh + 30);   // (q.hi) 2^53
-  const uint32_t lb = __float_as_uint(q.lo);
-  const int el = (int)((lb >> 23) & 0xFF) - 127;
-  if ((lb & 0x7FFFFFFFu) != 0 && el > -127) {
-    const long long ml = (long long)((lb & 0x7FFFFFu) | 0x800000u);
-    const int s = el + 30;
-    const long long L = s >= 0 ? (ml << s) : (s > -64 ? (ml >> (-s)) : 0);
-    V += (lb >> 31) ? -L : L;
-  }
-  int E = -1;
-  unsigned long long mant = (unsigned long long)V;                   // leading bit 52 or 53
-  if (mant >> 53) {
-    const unsigned long long h = mant >> 1;
-    mant = h + ((mant & 1ull) & (h & 1ull));                         // ties to even
-    E = 0;
-  }
-  return __longlong_as_double((long long)(((unsigned long long)(E - k + 1023) << 52) | (mant & 0xFFFFFFFFFFFFFull)));
+struct ExpFactor {
+  unsigned long long c;   // y log2(e) = c 2^(ey - 1023 - 62)
+  int sh;                 // 2053 - ey: u 2^54 = (m c 2^-64) >> (sh - ex), m = x's mantissa with its leading bit at 63
+  double y;
+};
+__device__ __forceinline__ ExpFactor exp_factor(double y) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(y);
+  const int ey = (int)((b >> 52) & 0x7FF);
+  if (ey == 0) return {0, 1 << 20, y};           // zero and subnormal: u counts as zero
+  if (ey == 0x7FF) return {0, -(1 << 20), y};    // every x > 0 to the general path
+  return {__umul64hi((b << 11) | (1ull << 63), 0xB8AA3B295C17F0BCull), 2053 - ey, y};   // log2(e) 2^63
+}
+
+// The high 64 bits of a b less at most 2 (the product of the low halves is left out).
+__device__ __forceinline__ unsigned long long mul64_high(unsigned long long a, unsigned long long b) {
+  const uint32_t ah = (uint32_t)(a >> 32), al = (uint32_t)a, bh = (uint32_t)(b >> 32), bl = (uint32_t)b;
+  return (unsigned long long)ah * bh + __umulhi(ah, bl) + __umulhi(al, bh);
+}
+
+__device__ __forceinline__ double exp_neg_prod(double x, const ExpFactor& f, const unsigned long long* __restrict__ tab) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int ex = (int)(b >> 52);
+  const int sh = ex == 0 ? 63 : min(f.sh - ex, 63);          // x zero or subnormal: u below 2^-54
+  const unsigned long long u = mul64_high((b << 11) | (1ull << 63), f.c) >> (sh & 63);
+  const uint32_t uh = (uint32_t)(u >> 32), k = uh >> 22;
+  if (sh < 0 || k > 1000) return exp(-(x * f.y));            // near and below the normal range; infinities, NaN
+  const uint32_t g = (uint32_t)(u >> 14);                    // g 2^40: the 32 bits below j
+  const uint32_t c34 = 0xE35846B8u - (__umulhi(g, 0x9D955B7Eu) >> 10);   // c3 2^36, c4 2^38
+  const uint32_t c234 = 0xF5FDEFFCu - (__umulhi(g, c34) >> 10);          // c2 2^34
+  const unsigned long long s = 0xB17217F7D1CF79ACull - ((unsigned long long)__umulhi(g, c234) << 22);   // c1 2^64
+  const unsigned long long t = tab[(uh >> 14) & 255u];
+  const unsigned long long v = t - (mul64_high(t, mul64_high(u << 18, s)) >> 8);   // 2^63 2^(-j / 256) 2^-g
+  return __longlong_as_double((long long)(((unsigned long long)(1021 - (int)k) << 52) + ((v + 512) >> 10)));
 }
 
 }  // namespace cdl

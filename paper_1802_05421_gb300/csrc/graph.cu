@@ -385,69 +385,61 @@ __global__ void k_set_scalar(double* p, double v) { *p = v; }
 
 // A_ij = exp(-d2_ij / (2 sigma^2)) (KERN = KERNEL_GAUSSIAN) or
 // A_ij = exp(-sqrt(d2_ij) / sigma) (KERN = KERNEL_EXP, the synthetic-data
-// kernel of Sec. 4.2.1), A_ii = 0, D_i = row sum. One block per row.
-// The exponential is ff_exp_neg_prod: the argument d2 * (1 / (2 sigma^2)), or
-// sqrt(d2) (sqrt_nonneg: within one ulp) times 1 / sigma, is formed exactly in
-// 128-bit integers and reduced there (by k ln2, then by j / 32 through a
-// per-block table), then a float-float series (about 1.4e-14 relative) and an
-// integer assembly of the float64 result: no float64
-// operation but the three of the exp kernel's square root, float64 being the
-// scarce pipe. The row sum is accumulated in float-float (terms below 2^-100 are
-// dropped from the sum, not from A).
+// kernel of Sec. 4.2.1), A_ii = 0, D_i = row sum. One block per row (panels of
+// a regenerated graph and the graphs without workspace; whole graphs take
+// k_kernel_tiles). The exponential is exp_neg_prod: integer operations only, the
+// argument d2 * (1 / (2 sigma^2)), or sqrt(d2) (sqrt_nonneg: within one ulp)
+// times 1 / sigma, in 64-bit fixed point. The row sum is accumulated in
+// float-float (terms below 2^-100 are dropped from the sum, not from A).
 enum { KERNEL_GAUSSIAN = 0, KERNEL_EXP = 1 };
 
+__device__ __forceinline__ double kernel_rcp(double sigma, int kern) {
+  return kern == KERNEL_EXP ? 1.0 / sigma : 1.0 / (2.0 * (sigma * sigma));
+}
+
+// (hi, lo) + a split exactly into floats, lo left unnormalised.
+__device__ __forceinline__ void ff_acc(ff& acc, ff q) {
+  const ff t = two_sum(acc.hi, q.hi);
+  acc.hi = t.hi;
+  acc.lo = __fadd_rn(acc.lo, __fadd_rn(t.lo, q.lo));
+}
+
 template <int KERN = KERNEL_GAUSSIAN>
-__device__ __forceinline__ void kernel_row(double* __restrict__ A, int n, double rcp, double* __restrict__ D,
-                                           int i, const ff* __restrict__ tab, int roff = 0) {
+__device__ __forceinline__ void kernel_row(double* __restrict__ A, int n, const ExpFactor& f, double* __restrict__ D,
+                                           int i, const unsigned long long* __restrict__ tab, int roff = 0) {
   __shared__ double red[8];
-  {
-    double* row = A + (size_t)(i - roff) * n;
-    const float rcpf = d2f_trunc(rcp);
-    ff acc = {0.f, 0.f};
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-      const double x = KERN == KERNEL_EXP ? sqrt_nonneg(row[j]) : row[j];
-      double a = 0.0;
-      if (j != i) {
-        if (__fmul_rn(d2f_trunc(x), rcpf) < 680.f) {          // t = x rcp well below 690
-          int k;
-          const ff q = ff_exp_neg_prod(x, rcp, k, tab);
-          a = ff_scaled_to_double(q, k);
-          if (k <= 100) {
-            const float sc = __int_as_float((127 - k) << 23);   // 2^-k
-            const ff ts = two_sum(acc.hi, __fmul_rn(q.hi, sc));
-            acc.hi = ts.hi;
-            acc.lo = __fadd_rn(acc.lo, __fadd_rn(ts.lo, __fmul_rn(q.lo, sc)));
-          }
-        } else {
-          a = exp(-(x * rcp));
-        }
-      }
-      row[j] = a;
+  double* row = A + (size_t)(i - roff) * n;
+  ff acc = {0.f, 0.f};
+  for (int j = threadIdx.x; j < n; j += blockDim.x) {
+    double a = 0.0;
+    if (j != i) {
+      a = exp_neg_prod(KERN == KERNEL_EXP ? sqrt_nonneg(row[j]) : row[j], f, tab);
+      ff_acc(acc, split_nonneg(a));
     }
-    double accd = (double)acc.hi + (double)acc.lo;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) accd += __shfl_xor_sync(0xffffffffu, accd, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = accd;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double t = 0.0;
-      for (int w = 0; w < 8; ++w) t += red[w];
-      D[i] = t;
-    }
-    __syncthreads();
+    row[j] = a;
   }
+  double accd = (double)acc.hi + (double)acc.lo;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) accd += __shfl_xor_sync(0xffffffffu, accd, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = accd;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int w = 0; w < 8; ++w) t += red[w];
+    D[i] = t;
+  }
+  __syncthreads();
 }
 
 template <int KERN = KERNEL_GAUSSIAN>
 __global__ void __launch_bounds__(256) k_kernel_rows(double* __restrict__ A, int n,
                                                       const double* __restrict__ sigma,
                                                       double* __restrict__ D) {
-  const double s = *sigma;
-  const double rcp = KERN == KERNEL_EXP ? 1.0 / s : 1.0 / (2.0 * (s * s));
-  __shared__ ff tab[FF_EXP_TABLE];
-  ff_exp_table(tab);
+  __shared__ unsigned long long tab[EXP_TABLE];
+  exp_table(tab);
+  const ExpFactor f = exp_factor(kernel_rcp(*sigma, KERN));
   __syncthreads();
-  for (int i = blockIdx.x; i < n; i += gridDim.x) kernel_row<KERN>(A, n, rcp, D, i, tab);
+  for (int i = blockIdx.x; i < n; i += gridDim.x) kernel_row<KERN>(A, n, f, D, i, tab);
 }
 
 // Rows r0 .. r1 - 1 of a panel holding rows r0 .. (squared distances in,
@@ -455,12 +447,11 @@ __global__ void __launch_bounds__(256) k_kernel_rows(double* __restrict__ A, int
 __global__ void __launch_bounds__(256) k_kernel_rows_panel(double* __restrict__ P, int n,
                                                             const double* __restrict__ sigma, double* __restrict__ D,
                                                             int r0, int r1) {
-  const double s = *sigma;
-  const double rcp = 1.0 / (2.0 * (s * s));
-  __shared__ ff tab[FF_EXP_TABLE];
-  ff_exp_table(tab);
+  __shared__ unsigned long long tab[EXP_TABLE];
+  exp_table(tab);
+  const ExpFactor f = exp_factor(kernel_rcp(*sigma, KERNEL_GAUSSIAN));
   __syncthreads();
-  for (int i = r0 + blockIdx.x; i < r1; i += gridDim.x) kernel_row<KERNEL_GAUSSIAN>(P, n, rcp, D, i, tab, r0);
+  for (int i = r0 + blockIdx.x; i < r1; i += gridDim.x) kernel_row<KERNEL_GAUSSIAN>(P, n, f, D, i, tab, r0);
 }
 
 // Kernel values over the upper block triangle of 64 x 64 tiles (A is
@@ -471,75 +462,116 @@ __global__ void __launch_bounds__(256) k_kernel_rows_panel(double* __restrict__ 
 // (float-float, the entries split with integer operations) in the slots of
 // the 64-node partner blocks: part[bj][i] for its rows, part[bi][j] for its
 // columns (rows only on the diagonal). D_i is the fixed-order sum of node i's
-// slots (k_part_sums). Same entry arithmetic as kernel_row.
+// slots (part_sum). Same entry arithmetic as kernel_row.
+// Warp w holds rows 8 w .. 8 w + 7, a lane the columns lane and lane + 32: both
+// sums start from the registers; the rows' lanes are combined by halving
+// exchanges (9 additions for 8 rows instead of 40), the columns' warps through
+// shared memory. KERNEL_TILES_NOTE
+struct KernelTileShared {
+  double tt[DT][DT + 1];                                // tt[c][r] = A(i0 + r, j0 + c)
+  float2 col[8][DT];
+  unsigned long long tab[EXP_TABLE];
+};
+
 template <int KERN>
-__global__ void __launch_bounds__(256) k_kernel_tiles(double* __restrict__ A, int n, const double* __restrict__ sigma,
-                                                       double* __restrict__ part) {
-  __shared__ double tt[DT][DT + 1];                     // tt[c][r] = A(i0 + r, j0 + c)
-  const int nb = (n + DT - 1) / DT;
-  __shared__ double rcp_s;                               // float64 division and square root once per block
-  __shared__ int tile_s[2];
-  __shared__ ff tab[FF_EXP_TABLE];
-  ff_exp_table(tab);
-  if (threadIdx.x == 0) {
-    tri_index(blockIdx.x, nb, tile_s[0], tile_s[1]);
-    const double sg = *sigma;
-    rcp_s = KERN == KERNEL_EXP ? 1.0 / sg : 1.0 / (2.0 * (sg * sg));
-  }
-  __syncthreads();
-  const int bi = tile_s[0], bj = tile_s[1];
+__device__ __forceinline__ void kernel_tile(double* __restrict__ A, int n, const ExpFactor& f, double* __restrict__ part,
+                                            int bi, int bj, KernelTileShared& sm) {
   const int i0 = bi * DT, j0 = bj * DT;
-  const double rcp = rcp_s;
-  const float rcpf = d2f_trunc(rcp);
-  const int c = threadIdx.x & (DT - 1), rg = threadIdx.x >> 6;
-#pragma unroll 4
-  for (int m = 0; m < DT / 4; ++m) {
-    const int r = rg + 4 * m, i = i0 + r, j = j0 + c;
-    double a = 0.0;
-    if (i < n && j < n) {
-      double* pa = A + (size_t)i * n + j;
-      if (i != j) {
-        const double x = KERN == KERNEL_EXP ? sqrt_nonneg(*pa) : *pa;
-        if (__fmul_rn(d2f_trunc(x), rcpf) < 680.f) {
-          int k;
-          const ff q = ff_exp_neg_prod(x, rcp, k, tab);
-          a = ff_scaled_to_double(q, k);
-        } else {
-          a = exp(-(x * rcp));
-        }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  ff rs[8], cs[2] = {{0.f, 0.f}, {0.f, 0.f}};
+#pragma unroll
+  for (int m0 = 0; m0 < 8; m0 += 4) {
+    double x[4][2];
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int i = i0 + 8 * warp + m0 + m, j = j0 + lane + 32 * h;
+        x[m][h] = i < n && j < n ? A[(size_t)i * n + j] : 0.0;
       }
-      *pa = a;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      rs[m0 + m] = {0.f, 0.f};
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int r = 8 * warp + m0 + m, c = lane + 32 * h, i = i0 + r, j = j0 + c;
+        double a = 0.0;
+        if (i < n && j < n) {
+          if (i != j) a = exp_neg_prod(KERN == KERNEL_EXP ? sqrt_nonneg(x[m][h]) : x[m][h], f, sm.tab);
+          A[(size_t)i * n + j] = a;
+        }
+        sm.tt[c][r] = a;
+        const ff q = split_nonneg(a);
+        ff_acc(rs[m0 + m], q);
+        ff_acc(cs[h], q);
+      }
     }
-    tt[c][r] = a;
   }
+  // lane l ends with the sum of row l >> 2 of the warp's eight
+#pragma unroll
+  for (int w = 4; w > 0; w >>= 1) {
+    const bool up = (lane & (4 * w)) != 0;
+#pragma unroll
+    for (int m = 0; m < w; ++m) {
+      const ff keep = up ? rs[m + w] : rs[m], give = up ? rs[m] : rs[m + w];
+      const ff got = {__shfl_xor_sync(0xffffffffu, give.hi, 4 * w), __shfl_xor_sync(0xffffffffu, give.lo, 4 * w)};
+      rs[m] = ff_add(keep, got);
+    }
+  }
+#pragma unroll
+  for (int o = 2; o > 0; o >>= 1)
+    rs[0] = ff_add(rs[0], ff{__shfl_xor_sync(0xffffffffu, rs[0].hi, o), __shfl_xor_sync(0xffffffffu, rs[0].lo, o)});
+  const int ri = i0 + 8 * warp + (lane >> 2);
+  if ((lane & 3) == 0 && ri < n) part[(size_t)bj * n + ri] = (double)rs[0].hi + (double)rs[0].lo;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) sm.col[warp][lane + 32 * h] = make_float2(cs[h].hi, cs[h].lo);
   __syncthreads();
-  if (bi != bj) {                                        // mirror: lanes write consecutive columns of row j
+  if (bi != bj) {
+    const int r = threadIdx.x & (DT - 1), rg = threadIdx.x >> 6;
+    const int i = i0 + r;
 #pragma unroll 4
-    for (int m = 0; m < DT / 4; ++m) {
-      const int cc = rg + 4 * m, r = threadIdx.x & (DT - 1);
-      const int j = j0 + cc, i = i0 + r;
-      if (j < n && i < n) A[(size_t)j * n + i] = tt[cc][r];
+    for (int m = 0; m < DT / 4; ++m) {                  // mirror: lanes write consecutive columns of row j
+      const int cc = rg + 4 * m, j = j0 + cc;
+      if (j < n && i < n) A[(size_t)j * n + i] = sm.tt[cc][r];
+    }
+    if (threadIdx.x < DT && j0 + (int)threadIdx.x < n) {   // column sums (the mirror's row sums)
+      ff acc = {0.f, 0.f};
+#pragma unroll
+      for (int w = 0; w < 8; ++w) {
+        const float2 v = sm.col[w][threadIdx.x];
+        acc = ff_add(acc, ff{v.x, v.y});
+      }
+      part[(size_t)bi * n + j0 + threadIdx.x] = (double)acc.hi + (double)acc.lo;
     }
   }
-  if (threadIdx.x < DT) {                                // row sums of the tile
-    const int r = threadIdx.x, i = i0 + r;
-    ff acc = {0.f, 0.f};
-    for (int cc = 0; cc < DT; ++cc) acc = ff_add(acc, split_nonneg(tt[cc][r]));
-    if (i < n) part[(size_t)bj * n + i] = (double)acc.hi + (double)acc.lo;
-  } else if (threadIdx.x < 2 * DT && bi != bj) {         // column sums (the mirror's row sums)
-    const int cc = threadIdx.x - DT, j = j0 + cc;
-    ff acc = {0.f, 0.f};
-    for (int r = 0; r < DT; ++r) acc = ff_add(acc, split_nonneg(tt[cc][r]));
-    if (j < n) part[(size_t)bi * n + j] = (double)acc.hi + (double)acc.lo;
+}
+
+template <int KERN>
+__global__ void __launch_bounds__(256, 4) k_kernel_tiles(double* __restrict__ A, int n, const double* __restrict__ sigma,
+                                                          double* __restrict__ part) {
+  __shared__ KernelTileShared sm;
+  __shared__ int tile_s[2];
+  const int nb = (n + DT - 1) / DT;
+  const long long tiles = (long long)nb * (nb + 1) / 2;
+  exp_table(sm.tab);
+  const ExpFactor f = exp_factor(kernel_rcp(*sigma, KERN));
+  for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
+    if (threadIdx.x == 0) tri_index(t, nb, tile_s[0], tile_s[1]);
+    __syncthreads();
+    kernel_tile<KERN>(A, n, f, part, tile_s[0], tile_s[1], sm);
+    __syncthreads();
   }
+}
+
+__device__ __forceinline__ double part_sum(const double* __restrict__ part, int nb, int n, int i) {
+  double s = 0.0;
+  for (int b = 0; b < nb; ++b) s += part[(size_t)b * n + i];
+  return s;
 }
 
 __global__ void k_part_sums(const double* __restrict__ part, int nb, int n, double* __restrict__ D) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  double s = 0.0;
-  for (int b = 0; b < nb; ++b) s += part[(size_t)b * n + i];
-  D[i] = s;
+  if (i < n) D[i] = part_sum(part, nb, n, i);
 }
 
 // vol = sum_i D_i (single block, fixed order per thread then tree).
@@ -620,20 +652,24 @@ __global__ void __launch_bounds__(SELECT_STEP_THREADS) k_g_select_step(const GGr
 
 __global__ void k_g_set_sigma(const GGraph* __restrict__ gs, double sigma) { *gs[blockIdx.x].sigma = sigma; }
 
-// tiles: (i << 12) | g, one row per block
-__global__ void __launch_bounds__(256) k_g_kernel_rows(const uint32_t* __restrict__ tiles,
-                                                        const GGraph* __restrict__ gs) {
+// kernel_tile for every graph (tiles as k_g_dist's)
+__global__ void __launch_bounds__(256, 4) k_g_kernel_tiles(const uint32_t* __restrict__ tiles,
+                                                            const GGraph* __restrict__ gs) {
   const uint32_t t = tiles[blockIdx.x];
   const GGraph& G = gs[t & 0xFFFu];
-  __shared__ double rcp_s;                               // one float64 division per block
-  __shared__ ff tab[FF_EXP_TABLE];
-  ff_exp_table(tab);
-  if (threadIdx.x == 0) {
-    const double s = *G.sigma;
-    rcp_s = 1.0 / (2.0 * (s * s));
-  }
+  __shared__ KernelTileShared sm;
+  exp_table(sm.tab);
+  const ExpFactor f = exp_factor(kernel_rcp(*G.sigma, KERNEL_GAUSSIAN));
   __syncthreads();
-  kernel_row<KERNEL_GAUSSIAN>(G.A, G.n, rcp_s, G.D, (int)(t >> 12), tab);
+  kernel_tile<KERNEL_GAUSSIAN>(G.A, G.n, f, G.part, (int)((t >> 12) & 0x3FFu), (int)(t >> 22), sm);
+}
+
+// D of graph blockIdx.x from its tiles' sums
+__global__ void k_g_part_sums(const GGraph* __restrict__ gs) {
+  const GGraph& G = gs[blockIdx.x];
+  const int nb = (G.n + DT - 1) / DT;
+  for (int i = blockIdx.y * blockDim.x + threadIdx.x; i < G.n; i += gridDim.y * blockDim.x)
+    G.D[i] = part_sum(G.part, nb, G.n, i);
 }
 
 __global__ void k_g_sum(const GGraph* __restrict__ gs) {
@@ -666,7 +702,6 @@ void graph_grouped_tiles(const std::vector<int>& n, int T, GraphTiles& out) {
         acc = 0;
       }
     }
-    for (int i = 0; i < nn; ++i) out.rows.push_back(((uint32_t)i << 12) | (uint32_t)g);
   }
 }
 
@@ -710,7 +745,12 @@ int graph_build_grouped(cdl_ctx* ctx, const GraphBatch& B) {
   }
   {
     Launch L(ctx, CDL_KC_KERNEL, B.kernel_bytes);
-    k_g_kernel_rows<<<B.rows.count, 256, 0, s>>>(B.rows.p, B.gs);
+    k_g_kernel_tiles<<<B.dist.count, 256, 0, s>>>(B.dist.p, B.gs);
+    CDL_TRY(L.done());
+  }
+  {
+    Launch L(ctx, CDL_KC_MISC, 0);
+    k_g_part_sums<<<dim3(B.G2, 8), 256, 0, s>>>(B.gs);
     CDL_TRY(L.done());
   }
   Launch L(ctx, CDL_KC_MISC, 0);
@@ -811,10 +851,11 @@ int graph_build(cdl_ctx* ctx, const double* X, int64_t n64, int T, double sigma,
     double* part = static_cast<double*>(wsPart);
     {
       Launch L(ctx, CDL_KC_KERNEL, 16.0 * (double)n * n);
+      const unsigned blocks = (unsigned)std::min<long long>(tiles, ctx->sm_count * 4);
       if (kernel == KERNEL_EXP)
-        k_kernel_tiles<KERNEL_EXP><<<(unsigned)tiles, 256, 0, s>>>(A, n, sigma_out, part);
+        k_kernel_tiles<KERNEL_EXP><<<blocks, 256, 0, s>>>(A, n, sigma_out, part);
       else
-        k_kernel_tiles<KERNEL_GAUSSIAN><<<(unsigned)tiles, 256, 0, s>>>(A, n, sigma_out, part);
+        k_kernel_tiles<KERNEL_GAUSSIAN><<<blocks, 256, 0, s>>>(A, n, sigma_out, part);
       CDL_TRY(L.done());
     }
     Launch L(ctx, CDL_KC_MISC, 0);

@@ -391,6 +391,7 @@ struct GGraph {
   int* Xt;          // T x n fixed-point copy
   double* A;        // n x n
   double* D;        // n
+  double* part;     // ceil(n / 64) x n: sums of A over 64-node blocks
   double* vol;
   double* sigma;
   void* sel;        // graph_select_bytes(): selection state and histogram
@@ -401,7 +402,6 @@ struct GraphTiles {
   std::vector<uint32_t> fixed;   // (b << 12) | g, 1024-sample blocks of X
   std::vector<uint32_t> dist;    // g | bi << 12 | bj << 22, 64-node blocks, bi <= bj
   std::vector<int4> sel;         // (g, first row, end row, 0): about 2^17 keys each
-  std::vector<uint32_t> rows;    // (i << 12) | g
 };
 void graph_grouped_tiles(const std::vector<int>& n, int T, GraphTiles& out);
 struct GraphBatch {
@@ -410,7 +410,7 @@ struct GraphBatch {
   const GGraph* gs = nullptr;    // device
   void* sel_all = nullptr;       // the graphs' selection blocks, contiguous
   size_t sel_bytes = 0;
-  BTiles fixed, dist, rows;
+  BTiles fixed, dist;
   const int4* sel = nullptr;
   int sel_count = 0;
   double dist_terms = 0, select_bytes = 0, kernel_bytes = 0;
