@@ -31,16 +31,20 @@ struct SelectState {
   unsigned long long mask;      // which bits are selected
   long long rank;               // rank within the still-matching keys
   int flags;                    // bit 0: input off the 2^-16 grid
+  unsigned done;                // blocks of the running pass that have finished
+  unsigned long long ncomp;     // keys copied to the buffer
+  unsigned long long lo, hi;    // bracket of the wanted key, from a sample
+  unsigned long long below;     // keys below the bracket
+  int bracket;                  // BRACKET_TRY: lo, hi are set; BRACKET_HELD: the buffer holds the wanted key
   int pad;
-  unsigned long long ncomp;     // keys matching the prefix of the first two digits
 };
-// The third pass of the single-graph select also copies the keys that match
-// the first two digits (about 2^-12 of the value range around the median) to
-// a buffer of min(SELECT_CAP, max(m / 64, 1024)) keys (m keys in all); the
-// last three passes then read that buffer instead of the whole triangle,
-// unless more keys matched than it holds.
-constexpr long long SELECT_CAP = 1ll << 22;
-static_assert(sizeof(SelectState) <= 64, "the batched form keeps 64 bytes for the state");
+// Keys from which on a graph by itself takes the bracket form (n >= 4900; the
+// buffer then holds the samples): n = 4100 60 us by radix passes, 69 by a bracket;
+// n = 5003 85 and 77; n = 8192 160 and 109.
+constexpr long long SELECT_BRACKET_MIN = 12000000;
+enum { BRACKET_NONE = 0, BRACKET_HELD = 1, BRACKET_TRY = 2 };
+constexpr size_t SELECT_STATE_BYTES = 128;   // in front of the histogram in the batched form
+static_assert(sizeof(SelectState) <= SELECT_STATE_BYTES, "the batched form's room for the state");
 
 // X (float64, n x T) -> int32 fixed point a = x * 2^16, stored transposed
 // (T x n) for coalesced tile loads; flags input off the grid.
@@ -232,153 +236,453 @@ __global__ void __launch_bounds__(256) k_dist_f64(const double* __restrict__ X, 
   }
 }
 
-__global__ void k_select_init(SelectState* st, long long rank) {
+// The median of the m = n (n - 1) / 2 squared distances, exactly, over their
+// float64 bit patterns (for x >= 0 these order like the values).
+//
+// Radix form: six passes, digits from the top, each a histogram of the keys that
+// match the digits selected before; the pass's last block picks the bin with the
+// wanted rank. The third pass also copies the matching keys (about 2^-12 of the
+// value range around the median) to a buffer, which the later passes read
+// instead of A where they all fitted. Three passes over A, each bound by DRAM.
+//
+// Bracket form: one pass over A. SAMPLE keys, drawn at hashed positions, give two
+// of them SAMPLE_MARGIN ranks (4.5 standard deviations) to either side of the
+// wanted rank; a pass over A counts the keys below that bracket and copies those
+// inside (2.5 % of all) to the buffer; the radix passes then read the buffer
+// alone. Where the wanted rank is not inside, or the keys do not fit (many equal
+// distances: seen in the sample, then the pass over A is left out too), the radix
+// form runs instead. n = 20011 (2.0e8 keys, 1.6 GB): 1088 -> 400 us, of which the
+// pass over A 298 (5.4 TB/s); 128 batched graphs (2.2e8 keys): 2.53 -> 0.43 ms.
+constexpr int SELECT_THREADS = 512;
+constexpr int SELECT_WARPS = SELECT_THREADS / 32;
+constexpr int SELECT_STAGE = 256;                        // keys a warp gathers before it takes buffer space
+constexpr int SELECT_FINISH = 8192;                      // keys one block looks through for the rest
+constexpr int SAMPLE_THREADS = 1024;
+constexpr int SAMPLE = 32768;
+constexpr int SAMPLE_MARGIN = 407;                       // 4.5 sqrt(SAMPLE) / 2
+
+__device__ __forceinline__ void select_init(SelectState* st, long long rank) {
   st->prefix = 0;
   st->mask = 0;
   st->rank = rank;
   st->flags = 0;
+  st->done = 0;
   st->ncomp = 0;
+  st->below = 0;
+  st->bracket = BRACKET_NONE;
 }
 
-// Histogram of the `bits`-wide digit at `shift` over keys of the upper
-// triangle matching the current prefix.
-// rows r0, r0 + rstep, ... < r1 of the upper triangle
-// (A holds rows roff .. : row i at A + (i - roff) n)
-__device__ __forceinline__ void select_hist_rows(const double* __restrict__ A, int n, int shift, int bits,
-                                                 const SelectState* __restrict__ st,
-                                                 unsigned long long* __restrict__ hist, int r0, int r1, int rstep,
-                                                 int roff = 0) {
-  __shared__ unsigned int h[RADIX_BINS];
-  for (int b = threadIdx.x; b < RADIX_BINS; b += blockDim.x) h[b] = 0;
-  __syncthreads();
-  const unsigned long long prefix = st->prefix, mask = st->mask;
-  const unsigned long long dmask = (1ull << bits) - 1ull;
-  const unsigned long long* K = reinterpret_cast<const unsigned long long*>(A);
-  for (int i = r0; i < r1; i += rstep) {
-    const unsigned long long* row = K + (size_t)(i - roff) * n;
-    for (int j = i + 1 + threadIdx.x; j < n; j += blockDim.x) {
-      unsigned long long key = row[j];
-      if ((key & mask) == prefix) atomicAdd(&h[(key >> shift) & dmask], 1u);
-    }
-  }
-  __syncthreads();
-  for (int b = threadIdx.x; b < RADIX_BINS; b += blockDim.x)
-    if (h[b]) atomicAdd(&hist[b], (unsigned long long)h[b]);
-}
-
-__global__ void __launch_bounds__(512) k_select_hist(const double* __restrict__ A, int n, int shift,
-                                                      int bits, const SelectState* __restrict__ st,
+__global__ void __launch_bounds__(1024) k_select_init(SelectState* st, long long rank,
                                                       unsigned long long* __restrict__ hist) {
-  select_hist_rows(A, n, shift, bits, st, hist, blockIdx.x, n - 1, gridDim.x);
+  if (threadIdx.x == 0) select_init(st, rank);
+  for (int b = threadIdx.x; b < RADIX_BINS; b += blockDim.x) hist[b] = 0;
 }
 
-// The same histogram over rows r0 .. r1 - 1 of a panel holding rows r0 ..
-__global__ void __launch_bounds__(512) k_select_hist_panel(const double* __restrict__ P, int n, int shift, int bits,
-                                                            const SelectState* __restrict__ st,
-                                                            unsigned long long* __restrict__ hist, int r0, int r1) {
-  select_hist_rows(P, n, shift, bits, st, hist, r0 + blockIdx.x, r1, gridDim.x, r0);
+// f(key) for `len` consecutive keys by the lanes of a warp, eight loads in flight
+// each (one at a time left half of the DRAM bandwidth idle); every lane calls f
+// for every step, with ok = false past the end.
+template <class F>
+__device__ __forceinline__ void warp_keys(const unsigned long long* __restrict__ k, int len, F&& f) {
+  const int lane = threadIdx.x & 31;
+  for (int v0 = 0; v0 < len; v0 += 256) {
+    unsigned long long key[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int v = v0 + lane + 32 * e;
+      key[e] = v < len ? k[v] : 0;
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+      if (v0 + 32 * e < len) f(key[e], v0 + lane + 32 * e < len);
+  }
 }
 
-// The third pass: the histogram of select_hist_rows, and every key matching
-// the current prefix appended to buf (the first `cap`; st->ncomp counts all).
-__global__ void __launch_bounds__(512) k_select_hist_compact(const double* __restrict__ A, int n, int shift, int bits,
-                                                              SelectState* st, unsigned long long* __restrict__ hist,
-                                                              unsigned long long* __restrict__ buf, long long cap) {
-  __shared__ unsigned int h[RADIX_BINS];
-  for (int b = threadIdx.x; b < RADIX_BINS; b += blockDim.x) h[b] = 0;
-  __syncthreads();
-  const unsigned long long prefix = st->prefix, mask = st->mask;
-  const unsigned long long dmask = (1ull << bits) - 1ull;
+// The warps of a group of `warps` (this one `warp`) over the upper triangle of
+// rows r0 .. r1 - 1 (A holds rows roff ..: row i at A + (i - roff) n).
+template <class F>
+__device__ __forceinline__ void triangle_keys(const double* __restrict__ A, int n, int r0, int r1, int warp, int warps,
+                                              int roff, F&& f) {
   const unsigned long long* K = reinterpret_cast<const unsigned long long*>(A);
-  for (int i = blockIdx.x; i < n - 1; i += gridDim.x) {
-    const unsigned long long* row = K + (size_t)i * n;
-    for (int j = i + 1 + threadIdx.x; j < n; j += blockDim.x) {
-      const unsigned long long key = row[j];
-      if ((key & mask) == prefix) {
-        atomicAdd(&h[(key >> shift) & dmask], 1u);
-        const unsigned long long pos = atomicAdd(&st->ncomp, 1ull);
-        if (pos < (unsigned long long)cap) buf[pos] = key;
-      }
+  for (int i = r0 + warp; i < r1; i += warps) warp_keys(K + (size_t)(i - roff) * n + i + 1, n - 1 - i, f);
+}
+
+// The same over the whole triangle for an even load: rows i and n - 2 - i
+// together hold n keys; segments of 256 keys of such pairs of rows go around the
+// warps.
+template <class F>
+__device__ __forceinline__ void folded_keys(const double* __restrict__ A, int n, F&& f) {
+  const unsigned long long* K = reinterpret_cast<const unsigned long long*>(A);
+  const unsigned segs = (n + 255) / 256, items = (unsigned)(n / 2) * segs;   // n / 2 pairs of rows 0 .. n - 2
+  for (unsigned q = blockIdx.x * SELECT_WARPS + (threadIdx.x >> 5); q < items; q += gridDim.x * SELECT_WARPS) {
+    const int i = (int)(q / segs), v0 = (int)(q % segs) * 256, v1 = min(v0 + 256, n);
+    const int first = n - 1 - i, i2 = n - 2 - i;         // keys of row i; the partner row
+    if (v0 < first) warp_keys(K + (size_t)i * n + i + 1 + v0, min(v1, first) - v0, f);
+    if (v1 > first && i2 != i) {
+      const int w0 = max(v0, first) - first;
+      warp_keys(K + (size_t)i2 * n + i2 + 1 + w0, v1 - first - w0, f);
     }
   }
-  __syncthreads();
-  for (int b = threadIdx.x; b < RADIX_BINS; b += blockDim.x)
-    if (h[b]) atomicAdd(&hist[b], (unsigned long long)h[b]);
 }
 
-// The later passes: the histogram over the copied keys, or over the whole
-// triangle when they did not fit.
-__global__ void __launch_bounds__(512) k_select_hist_buf(const double* __restrict__ A, int n, int shift, int bits,
-                                                          const SelectState* __restrict__ st,
-                                                          unsigned long long* __restrict__ hist,
-                                                          const unsigned long long* __restrict__ buf, long long cap) {
-  const unsigned long long nc = st->ncomp;
-  if (nc > (unsigned long long)cap) {
-    select_hist_rows(A, n, shift, bits, st, hist, blockIdx.x, n - 1, gridDim.x);
-    return;
-  }
-  __shared__ unsigned int h[RADIX_BINS];
-  for (int b = threadIdx.x; b < RADIX_BINS; b += blockDim.x) h[b] = 0;
+struct SelectShared {
+  union {
+    unsigned int h[RADIX_BINS];
+    unsigned long long cnt[RADIX_BINS + SELECT_THREADS];   // one pad word per run: no bank conflicts
+    unsigned long long stage[SELECT_WARPS][SELECT_STAGE];
+  };
+  unsigned long long wsum[SELECT_WARPS];
+  unsigned long long bin;                                  // keys in the bin that the last step picked
+  int last;
+};
+
+// True in every thread of the last of `blocks` blocks to get here, after all
+// their writes before this are visible to it.
+__device__ __forceinline__ bool select_last_block(SelectState* st, unsigned blocks, int* flag) {
+  __threadfence();
   __syncthreads();
-  const unsigned long long prefix = st->prefix, mask = st->mask;
-  const unsigned long long dmask = (1ull << bits) - 1ull;
-  for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < nc; q += (size_t)gridDim.x * blockDim.x) {
-    const unsigned long long key = buf[q];
-    if ((key & mask) == prefix) atomicAdd(&h[(key >> shift) & dmask], 1u);
-  }
+  if (threadIdx.x == 0) *flag = atomicAdd(&st->done, 1u) == blocks - 1;
   __syncthreads();
-  for (int b = threadIdx.x; b < RADIX_BINS; b += blockDim.x)
-    if (h[b]) atomicAdd(&hist[b], (unsigned long long)h[b]);
+  if (!*flag) return false;
+  __threadfence();
+  return true;
 }
 
 // Pick the bin holding the remaining rank; extend the prefix; clear hist. One
-// block of SELECT_STEP_THREADS: every thread sums its run of up to 16 bins, a
-// block scan of the sums finds the run holding the rank, and its thread walks
-// the run. Bound by latency (32 KB of counts, one block): 3 us a step, where one
-// thread walking all 4096 bins took 56 us, six times per select.
-constexpr int SELECT_STEP_THREADS = 256;
-constexpr int SELECT_RUN = RADIX_BINS / SELECT_STEP_THREADS;
+// block: every thread sums its run of 8 bins, a block scan of the sums finds the
+// run holding the rank, and its thread walks the run. Bound by latency (32 KB of
+// counts, one block): 3 us, where one thread walking all 4096 bins took 56 us;
+// run by the last block of the histogram it costs no launch of its own.
 __device__ __forceinline__ void select_step(SelectState* st, unsigned long long* hist, int shift, int bits,
-                                            double* sigma_out, int last) {
-  __shared__ unsigned long long cnt[RADIX_BINS + SELECT_STEP_THREADS];   // one pad word per run: no bank conflicts
-  __shared__ unsigned long long wsum[SELECT_STEP_THREADS / 32];
+                                            double* sigma_out, int last, SelectShared& sm) {
+  constexpr int RUN = RADIX_BINS / SELECT_THREADS;
   const int nbins = 1 << bits, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 #pragma unroll
-  for (int e = 0; e < SELECT_RUN; ++e) {
-    const int b = tid + e * SELECT_STEP_THREADS;
-    cnt[b + b / SELECT_RUN] = b < nbins ? hist[b] : 0;
+  for (int e = 0; e < RUN; ++e) {
+    const int b = tid + e * SELECT_THREADS;
+    sm.cnt[b + b / RUN] = b < nbins ? __ldcg(hist + b) : 0;
     if (b < nbins) hist[b] = 0;
   }
   const unsigned long long r = (unsigned long long)st->rank;
   __syncthreads();
-  const unsigned long long* run = cnt + tid * (SELECT_RUN + 1);
+  const unsigned long long* run = sm.cnt + tid * (RUN + 1);
   unsigned long long own = 0;
 #pragma unroll
-  for (int e = 0; e < SELECT_RUN; ++e) own += run[e];
+  for (int e = 0; e < RUN; ++e) own += run[e];
   unsigned long long incl = own;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const unsigned long long v = __shfl_up_sync(0xffffffffu, incl, o);
     if (lane >= o) incl += v;
   }
-  if (lane == 31) wsum[warp] = incl;
+  if (lane == 31) sm.wsum[warp] = incl;
   __syncthreads();
-  for (int w = 0; w < warp; ++w) incl += wsum[w];
-  unsigned long long below = incl - own;
-  if (below <= r && r < incl) {   // exactly one thread: the histogram counts every key that still matches
+  for (int w = 0; w < warp; ++w) incl += sm.wsum[w];
+  const unsigned long long before = incl - own;
+  if (before <= r && r < incl) {   // exactly one thread: the histogram counts every key that still matches
+    unsigned long long below = before;
     int e = 0;
     while (r - below >= run[e]) below += run[e++];
-    st->prefix |= (unsigned long long)(tid * SELECT_RUN + e) << shift;
+    st->prefix |= (unsigned long long)(tid * RUN + e) << shift;
     st->mask |= (unsigned long long)(nbins - 1) << shift;
     st->rank = (long long)(r - below);
     if (last) *sigma_out = sqrt(__longlong_as_double((long long)st->prefix));
+    sm.bin = run[e];
+  }
+  if (tid == 0) st->done = 0;
+}
+
+// The rest of the selection in the block that made the step: of the nc keys in the
+// buffer the sm.bin (at most SELECT_THREADS) that match, each ranked among them by
+// counting. The later passes then find every digit selected and return: on small
+// graphs they took 8 us each.
+__device__ __forceinline__ void select_finish(SelectState* st, const unsigned long long* buf, unsigned long long nc,
+                                              double* sigma_out, SelectShared& sm) {
+  unsigned long long* list = &sm.stage[0][0];
+  const unsigned long long prefix = st->prefix, mask = st->mask;
+  const int r = (int)st->rank, c = (int)sm.bin;
+  __syncthreads();
+  if (threadIdx.x == 0) sm.last = 0;
+  __syncthreads();
+  for (unsigned long long q = threadIdx.x; q < nc; q += SELECT_THREADS) {
+    const unsigned long long key = __ldcg(buf + q);
+    if ((key & mask) == prefix) list[atomicAdd(&sm.last, 1)] = key;
+  }
+  __syncthreads();
+  if ((int)threadIdx.x >= c) return;
+  const unsigned long long key = list[threadIdx.x];
+  int less = 0, upto = 0;
+  for (int e = 0; e < c; ++e) {
+    less += list[e] < key;
+    upto += list[e] <= key;
+  }
+  if (less <= r && r < upto) {   // equal keys write the same
+    st->prefix = key;
+    st->mask = ~0ull;
+    *sigma_out = sqrt(__longlong_as_double((long long)key));
   }
 }
 
-__global__ void __launch_bounds__(SELECT_STEP_THREADS) k_select_step(SelectState* st, unsigned long long* hist,
-                                                                     int shift, int bits, double* sigma_out,
-                                                                     int last) {
-  select_step(st, hist, shift, bits, sigma_out, last);
+__global__ void __launch_bounds__(SELECT_THREADS, 2) k_select_step(SelectState* st, unsigned long long* hist, int shift,
+                                                                int bits, double* sigma_out, int last) {
+  __shared__ SelectShared sm;
+  select_step(st, hist, shift, bits, sigma_out, last, sm);
+}
+
+// Histogram of the digit at `shift` in shared memory around `keys`, a function
+// that calls its argument for this block's keys.
+template <class K>
+__device__ __forceinline__ void select_hist(const SelectState* st, int shift, int bits, unsigned long long* hist,
+                                            SelectShared& sm, K&& keys) {
+  for (int b = threadIdx.x; b < RADIX_BINS; b += blockDim.x) sm.h[b] = 0;
+  __syncthreads();
+  const unsigned long long prefix = st->prefix, mask = st->mask, dmask = (1ull << bits) - 1ull;
+  keys([&](unsigned long long key, bool ok) {
+    const bool hit = ok && (key & mask) == prefix;
+    if (hit) atomicAdd(&sm.h[(key >> shift) & dmask], 1u);
+    return hit;
+  });
+  __syncthreads();
+  for (int b = threadIdx.x; b < RADIX_BINS; b += blockDim.x)
+    if (sm.h[b]) atomicAdd(&hist[b], (unsigned long long)sm.h[b]);
+}
+
+// The digit at `shift` over rows r0 .. r1 - 1 of a panel holding rows r0 .. (the
+// regenerated graphs; the step is a launch of its own after the last panel)
+__global__ void __launch_bounds__(SELECT_THREADS, 2) k_select_hist_panel(const double* __restrict__ P, int n, int shift,
+                                                                      int bits, const SelectState* __restrict__ st,
+                                                                      unsigned long long* __restrict__ hist, int r0,
+                                                                      int r1) {
+  __shared__ SelectShared sm;
+  select_hist(st, shift, bits, hist, sm, [&](auto&& f) {
+    triangle_keys(P, n, r0, r1, blockIdx.x * SELECT_WARPS + (threadIdx.x >> 5), gridDim.x * SELECT_WARPS, r0, f);
+  });
+}
+
+// Digit p of the selection and its step. Block `block` of `blocks`; rows(f) calls
+// f for the block's share of the triangle.
+template <class R>
+__device__ __forceinline__ void select_pass(SelectState* st, unsigned long long* hist, int p, double* sigma_out,
+                                            unsigned long long* buf, unsigned long long cap, unsigned block,
+                                            unsigned blocks, SelectShared& sm, R&& rows) {
+  const int shift = p < 5 ? 52 - 12 * p : 0, bits = p < 5 ? 12 : 4;
+  const unsigned long long dmask = (1ull << bits) - 1ull;
+  if (((st->mask >> shift) & dmask) == dmask) return;    // the bracket's common leading digit
+  const unsigned long long nc = st->ncomp;
+  if (st->bracket == BRACKET_HELD || (p > 2 && cap && nc <= cap)) {
+    const size_t step = (size_t)blocks * SELECT_WARPS * 256;
+    const size_t w0 = ((size_t)block * SELECT_WARPS) * 256;
+    if (w0 < nc)
+      select_hist(st, shift, bits, hist, sm, [&](auto&& f) {
+        for (size_t q = w0 + (threadIdx.x >> 5) * 256; q < nc; q += step) warp_keys(buf + q, (int)min((size_t)256, (size_t)(nc - q)), f);
+      });
+  } else if (p == 2 && cap) {
+    bool full = false;
+    select_hist(st, shift, bits, hist, sm, [&](auto&& f) {
+      rows([&](unsigned long long key, bool ok) {
+        const bool hit = f(key, ok);
+        const unsigned m = __ballot_sync(0xffffffffu, hit);
+        if (m == 0 || full) return;
+        const int lane = threadIdx.x & 31;
+        unsigned long long pos = 0;
+        if (lane == 0) pos = atomicAdd(&st->ncomp, (unsigned long long)__popc(m));
+        pos = __shfl_sync(0xffffffffu, pos, 0);
+        full = pos > cap;                               // ncomp is above cap for good
+        pos += __popc(m & ((1u << lane) - 1u));
+        if (hit && pos < cap) buf[pos] = key;
+      });
+    });
+  } else {
+    select_hist(st, shift, bits, hist, sm, rows);
+  }
+  if (!select_last_block(st, blocks, &sm.last)) return;
+  select_step(st, hist, shift, bits, sigma_out, p == 5, sm);
+  if (p != 2 || cap == 0 || st->bracket == BRACKET_HELD) return;
+  __syncthreads();
+  const unsigned long long got = __ldcg(&st->ncomp);
+  if (got <= min(cap, (unsigned long long)SELECT_FINISH) && sm.bin <= SELECT_THREADS)
+    select_finish(st, buf, got, sigma_out, sm);
+}
+
+// One pass over A for the keys below the bracket and those inside.
+template <class R>
+__device__ __forceinline__ void select_bracket(SelectState* st, unsigned long long* buf, unsigned long long cap,
+                                               unsigned blocks, SelectShared& sm, R&& rows) {
+  if (st->bracket != BRACKET_TRY) return;
+  const unsigned long long lo = st->lo, hi = st->hi;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned long long* stage = sm.stage[warp];
+  unsigned below = 0;
+  int cnt = 0;
+  auto flush = [&]() {
+    __syncwarp();
+    unsigned long long pos = 0;
+    if (lane == 0) pos = atomicAdd(&st->ncomp, (unsigned long long)cnt);
+    pos = __shfl_sync(0xffffffffu, pos, 0);
+    for (int e = lane; e < cnt; e += 32)
+      if (pos + e < cap) buf[pos + e] = stage[e];
+    __syncwarp();
+    cnt = 0;
+  };
+  rows([&](unsigned long long key, bool ok) {
+    below += ok && key < lo;
+    const bool in = ok && key >= lo && key <= hi;
+    const unsigned m = __ballot_sync(0xffffffffu, in);
+    if (m) {
+      if (in) stage[cnt + __popc(m & ((1u << lane) - 1u))] = key;
+      cnt += __popc(m);
+      if (cnt > SELECT_STAGE - 32) flush();
+    }
+  });
+  if (cnt) flush();
+  below = __reduce_add_sync(0xffffffffu, below);
+  if (lane == 0 && below) atomicAdd(&st->below, (unsigned long long)below);
+  if (!select_last_block(st, blocks, &sm.last) || threadIdx.x != 0) return;
+  const unsigned long long nc = __ldcg(&st->ncomp), nb = __ldcg(&st->below);
+  const unsigned long long r = (unsigned long long)st->rank;
+  const bool held = nb <= r && r < nb + nc && nc <= cap;
+  if (held) {
+    st->rank = (long long)(r - nb);
+    if ((lo >> 52) == (hi >> 52)) {
+      st->prefix = lo >> 52 << 52;
+      st->mask = 0xFFFull << 52;
+    }
+  } else {
+    st->ncomp = 0;
+  }
+  st->bracket = held ? BRACKET_HELD : BRACKET_NONE;
+  st->done = 0;
+}
+
+// Sample q: the high word of the key at a hashed position.
+__device__ __forceinline__ uint32_t sample_key(const double* __restrict__ A, int n, uint32_t q) {
+  unsigned long long x = (q + 1) * 0x9E3779B97F4A7C15ull;   // two multiply-xorshift rounds
+  x = (x ^ (x >> 30)) * 0xBF58476D1CE4E5B9ull;
+  x = (x ^ (x >> 27)) * 0x94D049BB133111EBull;
+  x ^= x >> 31;
+  const uint32_t i = __umulhi((uint32_t)(x >> 32), (uint32_t)n);
+  uint32_t j = __umulhi((uint32_t)x, (uint32_t)(n - 1));
+  j += j >= i;
+  return reinterpret_cast<const uint32_t*>(A + (size_t)min(i, j) * n + max(i, j))[1];
+}
+
+__global__ void __launch_bounds__(256) k_sample_keys(const double* __restrict__ A, int n, uint32_t* __restrict__ out) {
+  const uint32_t q = blockIdx.x * 256 + threadIdx.x;
+  out[q] = sample_key(A, n, q);
+}
+
+// The bracket from SAMPLE keys (their high words; positions by a fixed hash, with
+// repetitions): two ranks found at once by three histograms in shared memory. One
+// block: 15 us, bound by the latency of its passes (with the scattered loads and one
+// histogram update per sample at the top digit, where most meet in one bin: 50).
+struct SampleShared {
+  uint32_t key[SAMPLE];
+  unsigned h[2][2048];
+  unsigned wsum[32];
+  uint32_t prefix[2];
+  int rank[2];
+  int open[2];                  // the bracket has no end on this side
+  int inside;
+};
+template <class K>
+__device__ __forceinline__ void select_sample(int n, SelectState* st, unsigned long long cap, SampleShared& sm,
+                                              K&& sample) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+#pragma unroll 16
+  for (int e = 0; e < SAMPLE / SAMPLE_THREADS; ++e)
+    sm.key[tid + e * SAMPLE_THREADS] = sample((uint32_t)(tid + e * SAMPLE_THREADS));
+  if (tid == 0) {
+    // where the wanted key falls among the samples
+    const int at = (int)(((double)st->rank + 0.5) / (0.5 * (double)n * (double)(n - 1)) * SAMPLE);
+    sm.rank[0] = at - SAMPLE_MARGIN;
+    sm.rank[1] = at + SAMPLE_MARGIN;
+    sm.open[0] = at < SAMPLE_MARGIN;
+    sm.open[1] = at + SAMPLE_MARGIN >= SAMPLE;
+    sm.prefix[0] = sm.prefix[1] = 0;
+    sm.inside = 0;
+  }
+  const int t = tid >> 9, u = tid & 511;                 // half of the block per rank, 4 bins a thread
+  uint32_t mask = 0;
+  for (int p = 0; p < 3; ++p) {
+    const int shift = p == 0 ? 21 : p == 1 ? 10 : 0, bits = p < 2 ? 11 : 10;
+    for (int b = tid; b < 4096; b += SAMPLE_THREADS) (&sm.h[0][0])[b] = 0;
+    __syncthreads();
+    const uint32_t p0 = sm.prefix[0], p1 = sm.prefix[1], dmask = (1u << bits) - 1u;
+    const bool same = p0 == p1;                        // one histogram serves both ranks
+#pragma unroll 4
+    for (int e = 0; e < SAMPLE / SAMPLE_THREADS; ++e) {
+      const uint32_t k = sm.key[tid + e * SAMPLE_THREADS], d = (k >> shift) & dmask;
+      if (p == 0) {                                      // exponents: most of a warp falls into one bin or two
+        const unsigned m = __match_any_sync(0xffffffffu, d);
+        if (lane == __ffs(m) - 1) atomicAdd(&sm.h[0][d], (unsigned)__popc(m));
+        continue;
+      }
+      if ((k & mask) == p0) atomicAdd(&sm.h[0][d], 1u);
+      if (!same && (k & mask) == p1) atomicAdd(&sm.h[1][d], 1u);
+    }
+    __syncthreads();
+    unsigned c[4], own = 0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) own += c[e] = sm.h[same ? 0 : t][4 * u + e];
+    unsigned incl = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
+    }
+    if (lane == 31) sm.wsum[warp] = incl;
+    const int r = sm.rank[t];
+    __syncthreads();
+    for (int w = t * 16; w < warp; ++w) incl += sm.wsum[w];
+    unsigned b0 = incl - own;
+    if (r >= 0 && b0 <= (unsigned)r && (unsigned)r < incl) {
+      int e = 0;
+      while ((unsigned)r - b0 >= c[e]) b0 += c[e++];
+      sm.prefix[t] |= (uint32_t)(4 * u + e) << shift;
+      sm.rank[t] = r - (int)b0;
+    }
+    mask |= dmask << shift;
+    __syncthreads();
+  }
+  const uint32_t lo = sm.open[0] ? 0u : sm.prefix[0], hi = sm.open[1] ? 0xFFFFFFFFu : sm.prefix[1];
+  int in = 0;
+#pragma unroll 4
+  for (int e = 0; e < SAMPLE / SAMPLE_THREADS; ++e) {
+    const uint32_t k = sm.key[tid + e * SAMPLE_THREADS];
+    in += k >= lo && k <= hi;
+  }
+  in = __reduce_add_sync(0xffffffffu, in);
+  if (lane == 0) atomicAdd(&sm.inside, in);
+  __syncthreads();
+  if (tid == 0) {
+    st->lo = (unsigned long long)lo << 32;
+    st->hi = (unsigned long long)hi << 32 | 0xFFFFFFFFull;
+    st->bracket = (double)sm.inside / SAMPLE * (0.5 * (double)n * (double)(n - 1)) < 0.95 * (double)cap + 4.0 ? BRACKET_TRY : BRACKET_NONE;
+  }
+}
+
+__global__ void __launch_bounds__(SAMPLE_THREADS) k_select_sample(const uint32_t* __restrict__ keys, int n,
+                                                                  SelectState* st, unsigned long long cap) {
+  extern __shared__ __align__(16) unsigned char sample_smem[];
+  select_sample(n, st, cap, *reinterpret_cast<SampleShared*>(sample_smem), [&](uint32_t q) { return keys[q]; });
+}
+
+__global__ void __launch_bounds__(SELECT_THREADS, 2) k_select_bracket(const double* __restrict__ A, int n, SelectState* st,
+                                                                   unsigned long long* __restrict__ buf,
+                                                                   unsigned long long cap) {
+  __shared__ SelectShared sm;
+  select_bracket(st, buf, cap, gridDim.x, sm, [&](auto&& f) {
+    folded_keys(A, n, f);
+  });
+}
+
+__global__ void __launch_bounds__(SELECT_THREADS, 2) k_select_pass(const double* __restrict__ A, int n, int p,
+                                                                SelectState* st, unsigned long long* __restrict__ hist,
+                                                                double* sigma_out, unsigned long long* __restrict__ buf,
+                                                                unsigned long long cap) {
+  __shared__ SelectShared sm;
+  select_pass(st, hist, p, sigma_out, buf, cap, blockIdx.x, gridDim.x, sm, [&](auto&& f) {
+    folded_keys(A, n, f);
+  });
 }
 
 __global__ void k_set_scalar(double* p, double v) { *p = v; }
@@ -466,7 +770,8 @@ __global__ void __launch_bounds__(256) k_kernel_rows_panel(double* __restrict__ 
 // Warp w holds rows 8 w .. 8 w + 7, a lane the columns lane and lane + 32: both
 // sums start from the registers; the rows' lanes are combined by halving
 // exchanges (9 additions for 8 rows instead of 40), the columns' warps through
-// shared memory. KERNEL_TILES_NOTE
+// shared memory. Bound by instruction issue (143 a weight): n = 20011 1314 us, 3.7 TB/s;
+// with 128-bit exponentials and sums read back from shared memory 2315.
 struct KernelTileShared {
   double tt[DT][DT + 1];                                // tt[c][r] = A(i0 + r, j0 + c)
   float2 col[8][DT];
@@ -597,13 +902,7 @@ __global__ void k_sum(const double* __restrict__ v, int n, double* __restrict__ 
 // finds its graph and work item in a tile table.
 __global__ void k_g_select_init(const GGraph* __restrict__ gs) {
   const GGraph& G = gs[blockIdx.x];
-  SelectState* st = static_cast<SelectState*>(G.sel);
-  const long long m = (long long)G.n * (G.n - 1) / 2;
-  st->prefix = 0;
-  st->mask = 0;
-  st->rank = (m - 1) / 2;
-  st->flags = 0;
-  st->ncomp = 0;
+  select_init(static_cast<SelectState*>(G.sel), ((long long)G.n * (G.n - 1) / 2 - 1) / 2);
 }
 
 __global__ void k_g_to_fixed(const uint32_t* __restrict__ tiles, const GGraph* __restrict__ gs) {
@@ -633,21 +932,39 @@ __global__ void __launch_bounds__(256) k_g_dist(const uint32_t* __restrict__ til
     dist_int_tile(G.Xt, G.n, G.T, G.A, bi, bj);
 }
 
-__global__ void __launch_bounds__(512) k_g_select_hist(const int4* __restrict__ tiles, const GGraph* __restrict__ gs,
-                                                        int shift, int bits) {
-  const int4 t = tiles[blockIdx.x];
-  const GGraph& G = gs[t.x];
-  SelectState* st = static_cast<SelectState*>(G.sel);
-  unsigned long long* hist = reinterpret_cast<unsigned long long*>(static_cast<char*>(G.sel) + 64);
-  select_hist_rows(G.A, G.n, shift, bits, st, hist, t.y, t.z, 1);
+// The buffer is the graph's `part` (as many keys), which is not formed yet.
+__device__ __forceinline__ unsigned long long g_select_cap(const GGraph& G) {
+  return (unsigned long long)((G.n + DT - 1) / DT) * G.n;
 }
 
-__global__ void __launch_bounds__(SELECT_STEP_THREADS) k_g_select_step(const GGraph* __restrict__ gs, int shift,
-                                                                       int bits, int last) {
+__global__ void __launch_bounds__(SAMPLE_THREADS) k_g_select_sample(const GGraph* __restrict__ gs) {
+  extern __shared__ __align__(16) unsigned char sample_smem[];
   const GGraph& G = gs[blockIdx.x];
-  SelectState* st = static_cast<SelectState*>(G.sel);
-  unsigned long long* hist = reinterpret_cast<unsigned long long*>(static_cast<char*>(G.sel) + 64);
-  select_step(st, hist, shift, bits, G.sigma, last);
+  select_sample(G.n, static_cast<SelectState*>(G.sel), g_select_cap(G), *reinterpret_cast<SampleShared*>(sample_smem),
+                [&](uint32_t q) { return sample_key(G.A, G.n, q); });
+}
+
+// tiles: (g, first row, end row, b | blocks << 16): block b of the graph's `blocks`
+__global__ void __launch_bounds__(SELECT_THREADS, 2) k_g_select_bracket(const int4* __restrict__ tiles,
+                                                                     const GGraph* __restrict__ gs) {
+  __shared__ SelectShared sm;
+  const int4 t = tiles[blockIdx.x];
+  const GGraph& G = gs[t.x];
+  select_bracket(static_cast<SelectState*>(G.sel), reinterpret_cast<unsigned long long*>(G.part), g_select_cap(G),
+                 (unsigned)t.w >> 16, sm,
+                 [&](auto&& f) { triangle_keys(G.A, G.n, t.y, t.z, threadIdx.x >> 5, SELECT_WARPS, 0, f); });
+}
+
+__global__ void __launch_bounds__(SELECT_THREADS, 2) k_g_select_pass(const int4* __restrict__ tiles,
+                                                                  const GGraph* __restrict__ gs, int p) {
+  __shared__ SelectShared sm;
+  const int4 t = tiles[blockIdx.x];
+  const GGraph& G = gs[t.x];
+  unsigned long long* hist =
+      reinterpret_cast<unsigned long long*>(static_cast<char*>(G.sel) + SELECT_STATE_BYTES);
+  select_pass(static_cast<SelectState*>(G.sel), hist, p, G.sigma, reinterpret_cast<unsigned long long*>(G.part),
+              g_select_cap(G), (unsigned)t.w & 0xFFFFu, (unsigned)t.w >> 16, sm,
+              [&](auto&& f) { triangle_keys(G.A, G.n, t.y, t.z, threadIdx.x >> 5, SELECT_WARPS, 0, f); });
 }
 
 __global__ void k_g_set_sigma(const GGraph* __restrict__ gs, double sigma) { *gs[blockIdx.x].sigma = sigma; }
@@ -679,7 +996,7 @@ __global__ void k_g_sum(const GGraph* __restrict__ gs) {
 
 }  // namespace
 
-size_t graph_select_bytes() { return 64 + RADIX_BINS * sizeof(unsigned long long); }
+size_t graph_select_bytes() { return SELECT_STATE_BYTES + RADIX_BINS * sizeof(unsigned long long); }
 
 void graph_grouped_tiles(const std::vector<int>& n, int T, GraphTiles& out) {
   std::vector<int> order(n.size());
@@ -694,15 +1011,22 @@ void graph_grouped_tiles(const std::vector<int>& n, int T, GraphTiles& out) {
     // selection: consecutive rows holding about 2^17 upper-triangle keys
     int r0 = 0;
     long long acc = 0;
+    const size_t sel0 = out.sel.size();
     for (int i = 0; i < nn - 1; ++i) {
       acc += nn - 1 - i;
       if (acc >= (1 << 17) || i == nn - 2) {
-        out.sel.push_back(make_int4(g, r0, i + 1, 0));
+        out.sel.push_back(make_int4(g, r0, i + 1, (int)(out.sel.size() - sel0)));
         r0 = i + 1;
         acc = 0;
       }
     }
+    for (size_t e = sel0; e < out.sel.size(); ++e) out.sel[e].w |= (int)((out.sel.size() - sel0) << 16);
   }
+}
+
+static int select_sample_smem(const void* kernel) {
+  CDL_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SampleShared)));
+  return CDL_OK;
 }
 
 int graph_build_grouped(cdl_ctx* ctx, const GraphBatch& B) {
@@ -728,19 +1052,21 @@ int graph_build_grouped(cdl_ctx* ctx, const GraphBatch& B) {
     k_g_set_sigma<<<B.G2, 1, 0, s>>>(B.gs, B.sigma);
     CDL_TRY(L.done());
   } else {
-    const int shifts[6] = {52, 40, 28, 16, 4, 0};
-    const int widths[6] = {12, 12, 12, 12, 12, 4};
+    CDL_TRY(select_sample_smem(reinterpret_cast<const void*>(k_g_select_sample)));
+    {
+      Launch L(ctx, CDL_KC_SELECT, 0);
+      k_g_select_sample<<<B.G2, SAMPLE_THREADS, sizeof(SampleShared), s>>>(B.gs);
+      CDL_TRY(L.done());
+    }
+    {
+      Launch L(ctx, CDL_KC_SELECT, B.select_bytes);
+      k_g_select_bracket<<<B.sel_count, SELECT_THREADS, 0, s>>>(B.sel, B.gs);
+      CDL_TRY(L.done());
+    }
     for (int p = 0; p < 6; ++p) {
-      {
-        Launch L(ctx, CDL_KC_SELECT, B.select_bytes);
-        k_g_select_hist<<<B.sel_count, 512, 0, s>>>(B.sel, B.gs, shifts[p], widths[p]);
-        CDL_TRY(L.done());
-      }
-      {
-        Launch L(ctx, CDL_KC_SELECT, 0);
-        k_g_select_step<<<B.G2, SELECT_STEP_THREADS, 0, s>>>(B.gs, shifts[p], widths[p], p == 5);
-        CDL_TRY(L.done());
-      }
+      Launch L(ctx, CDL_KC_SELECT, 0);
+      k_g_select_pass<<<B.sel_count, SELECT_THREADS, 0, s>>>(B.sel, B.gs, p);
+      CDL_TRY(L.done());
     }
   }
   {
@@ -770,10 +1096,9 @@ int graph_build(cdl_ctx* ctx, const double* X, int64_t n64, int T, double sigma,
   const long long m = (long long)n * (n - 1) / 2;
   {
     Launch L(ctx, CDL_KC_MISC, 0);
-    k_select_init<<<1, 1, 0, s>>>(st, (m - 1) / 2);
+    k_select_init<<<1, 1024, 0, s>>>(st, (m - 1) / 2, hist);
     CDL_TRY(L.done());
   }
-  CDL_CUDA_TRY(cudaMemsetAsync(hist, 0, RADIX_BINS * sizeof(unsigned long long), s));
   const int nb = (n + DT - 1) / DT;
   const long long tiles = (long long)nb * (nb + 1) / 2;
   if (tiles > 0x7fffffffLL) return CDL_ERR_INVALID_ARG;
@@ -813,42 +1138,44 @@ int graph_build(cdl_ctx* ctx, const double* X, int64_t n64, int T, double sigma,
     k_dist_f64<<<(unsigned)std::min<long long>(tiles, ctx->sm_count * 6), 256, 0, s>>>(X, n, T, A, st, bad, nb64);
     CDL_TRY(L.done());
   }
+  void* wsPart;
+  CDL_TRY(ws_get(ctx, "graph.dpart", (size_t)nb * n * sizeof(double), &wsPart));
+  double* part = static_cast<double*>(wsPart);
   if (sigma > 0) {
     Launch L(ctx, CDL_KC_MISC, 0);
     k_set_scalar<<<1, 1, 0, s>>>(sigma_out, sigma);
     CDL_TRY(L.done());
   } else {
-    // digits from the top: [52,64), [40,52), [28,40), [16,28), [4,16), [0,4)
-    const int shifts[6] = {52, 40, 28, 16, 4, 0};
-    const int widths[6] = {12, 12, 12, 12, 12, 4};
-    const int hblocks = std::min(n - 1, ctx->sm_count * 4);
-    const long long cap = std::min(SELECT_CAP, std::max(m / 64, 1024ll));
-    void* wsBuf;
-    CDL_TRY(ws_get(ctx, "graph.selbuf", (size_t)cap * sizeof(unsigned long long), &wsBuf));
-    unsigned long long* sbuf = static_cast<unsigned long long*>(wsBuf);
-    for (int p = 0; p < 6; ++p) {
+    // one buffer for the selection's keys and the kernel values' partial sums after it
+    unsigned long long* sbuf = reinterpret_cast<unsigned long long*>(part);
+    const unsigned long long cap = (unsigned long long)nb * n;
+    if (m >= SELECT_BRACKET_MIN) {
+      CDL_TRY(select_sample_smem(reinterpret_cast<const void*>(k_select_sample)));
       {
-        // work: bytes of the triangle for the full passes (the later ones read the copied keys)
-        Launch L(ctx, CDL_KC_SELECT, p < 3 ? 8.0 * (double)m : 0.0);
-        if (p < 2)
-          k_select_hist<<<hblocks, 512, 0, s>>>(A, n, shifts[p], widths[p], st, hist);
-        else if (p == 2)
-          k_select_hist_compact<<<hblocks, 512, 0, s>>>(A, n, shifts[p], widths[p], st, hist, sbuf, cap);
-        else
-          k_select_hist_buf<<<hblocks, 512, 0, s>>>(A, n, shifts[p], widths[p], st, hist, sbuf, cap);
+        // the samples into the buffer first: one block's scattered loads took 25 us
+        Launch L(ctx, CDL_KC_SELECT, 0);
+        k_sample_keys<<<SAMPLE / 256, 256, 0, s>>>(A, n, reinterpret_cast<uint32_t*>(sbuf));
         CDL_TRY(L.done());
       }
       {
         Launch L(ctx, CDL_KC_SELECT, 0);
-        k_select_step<<<1, SELECT_STEP_THREADS, 0, s>>>(st, hist, shifts[p], widths[p], sigma_out, p == 5);
+        k_select_sample<<<1, SAMPLE_THREADS, sizeof(SampleShared), s>>>(reinterpret_cast<const uint32_t*>(sbuf), n, st,
+                                                                        cap);
         CDL_TRY(L.done());
       }
+      Launch L(ctx, CDL_KC_SELECT, 8.0 * (double)m);
+      k_select_bracket<<<ctx->sm_count * 2, SELECT_THREADS, 0, s>>>(A, n, st, sbuf, cap);
+      CDL_TRY(L.done());
+    }
+    const unsigned hblocks = (unsigned)std::min<long long>((m + 4095) / 4096, ctx->sm_count * 2);
+    for (int p = 0; p < 6; ++p) {
+      // work: bytes of the triangle for the full passes (the later ones read the copied keys)
+      Launch L(ctx, CDL_KC_SELECT, p < 3 && m < SELECT_BRACKET_MIN ? 8.0 * (double)m : 0.0);
+      k_select_pass<<<hblocks, SELECT_THREADS, 0, s>>>(A, n, p, st, hist, sigma_out, sbuf, cap);
+      CDL_TRY(L.done());
     }
   }
   {
-    void* wsPart;
-    CDL_TRY(ws_get(ctx, "graph.dpart", (size_t)nb * n * sizeof(double), &wsPart));
-    double* part = static_cast<double*>(wsPart);
     {
       Launch L(ctx, CDL_KC_KERNEL, 16.0 * (double)n * n);
       const unsigned blocks = (unsigned)std::min<long long>(tiles, ctx->sm_count * 4);
@@ -904,10 +1231,9 @@ int graph_regen_init(cdl_ctx* ctx, RegenGraph& g, const double* X, int64_t n64, 
   const long long m = (long long)n * (n - 1) / 2;
   {
     Launch L(ctx, CDL_KC_MISC, 0);
-    k_select_init<<<1, 1, 0, s>>>(st, (m - 1) / 2);
+    k_select_init<<<1, 1024, 0, s>>>(st, (m - 1) / 2, hist);
     CDL_TRY(L.done());
   }
-  CDL_CUDA_TRY(cudaMemsetAsync(hist, 0, RADIX_BINS * sizeof(unsigned long long), s));
   {
     Launch L(ctx, CDL_KC_DISTANCE, 0);
     k_prepare_series<<<g.rows / 8, 256, 0, s>>>(X, n, T, g.rows, g.tp, static_cast<__nv_bfloat162*>(wsPl),
@@ -935,12 +1261,12 @@ int graph_regen_init(cdl_ctx* ctx, RegenGraph& g, const double* X, int64_t n64, 
         const int r1 = std::min(n - 1, r0 + pr);
         if (r1 <= r0) continue;
         Launch L(ctx, CDL_KC_SELECT, 8.0 * (double)pr * n);
-        k_select_hist_panel<<<std::min(r1 - r0, ctx->sm_count * 4), 512, 0, s>>>(panel, n, shifts[p], widths[p], st,
+        k_select_hist_panel<<<std::min((r1 - r0 + SELECT_WARPS - 1) / SELECT_WARPS, ctx->sm_count * 4), SELECT_THREADS, 0, s>>>(panel, n, shifts[p], widths[p], st,
                                                                                hist, r0, r1);
         CDL_TRY(L.done());
       }
       Launch L(ctx, CDL_KC_SELECT, 0);
-      k_select_step<<<1, SELECT_STEP_THREADS, 0, s>>>(st, hist, shifts[p], widths[p], g.sigma, p == 5);
+      k_select_step<<<1, SELECT_THREADS, 0, s>>>(st, hist, shifts[p], widths[p], g.sigma, p == 5);
       CDL_TRY(L.done());
     }
   }
@@ -1206,9 +1532,8 @@ int graph_build_static(const double* X, int64_t n64, int T, double sigma, double
   const long long m = (long long)n * (n - 1) / 2;
   // The array keeps the previous call's contents: the select state and the
   // histogram must start from zero, Xt is fully overwritten.
-  k_select_init<<<1, 1, 0, s>>>(st, (m - 1) / 2);
+  k_select_init<<<1, 1024, 0, s>>>(st, (m - 1) / 2, hist);
   CDL_TRY(launched());
-  CDL_CUDA_TRY(cudaMemsetAsync(hist, 0, RADIX_BINS * sizeof(unsigned long long), s));
   const size_t total = (size_t)n * T;
   k_to_fixed<<<(int)std::min<size_t>((total + 255) / 256, (size_t)sm_count * 8), 256, 0, s>>>(X, Xt, n, T, st);
   CDL_TRY(launched());
@@ -1222,13 +1547,9 @@ int graph_build_static(const double* X, int64_t n64, int T, double sigma, double
     k_set_scalar<<<1, 1, 0, s>>>(sigma_out, sigma);
     CDL_TRY(launched());
   } else {
-    const int shifts[6] = {52, 40, 28, 16, 4, 0};
-    const int widths[6] = {12, 12, 12, 12, 12, 4};
-    const int hblocks = std::min(n - 1, sm_count * 4);
-    for (int p = 0; p < 6; ++p) {
-      k_select_hist<<<hblocks, 512, 0, s>>>(A, n, shifts[p], widths[p], st, hist);
-      CDL_TRY(launched());
-      k_select_step<<<1, SELECT_STEP_THREADS, 0, s>>>(st, hist, shifts[p], widths[p], sigma_out, p == 5);
+    const unsigned hblocks = (unsigned)std::min<long long>((m + 4095) / 4096, sm_count * 2);
+    for (int p = 0; p < 6; ++p) {   // no buffer: every pass over A
+      k_select_pass<<<hblocks, SELECT_THREADS, 0, s>>>(A, n, p, st, hist, sigma_out, nullptr, 0);
       CDL_TRY(launched());
     }
   }
