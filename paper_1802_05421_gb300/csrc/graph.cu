@@ -30,7 +30,7 @@ struct SelectState {
   unsigned long long prefix;    // selected high bits so far
   unsigned long long mask;      // which bits are selected
   long long rank;               // rank within the still-matching keys
-  int flags;                    // bit 0: input off the 2^-16 grid
+  int flags;                    // bit 0: input off the 2^-16 grid; bit 1: a top digit above 64 in magnitude
   unsigned done;                // blocks of the running pass that have finished
   unsigned long long ncomp;     // keys copied to the buffer
   unsigned long long lo, hi;    // bracket of the wanted key, from a sample
@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(256) k_prepare_series(const double* __restrict
   const size_t plane = (size_t)rows * tp / 2;
   const double* x = X + (size_t)min(row, n - 1) * T;
   long long acc = 0;
-  bool off = false;
+  bool off = false, wide = false;
   for (int t2 = lane; t2 < tp / 2; t2 += 32) {
     int d[3][2];
 #pragma unroll
@@ -98,6 +98,7 @@ __global__ void __launch_bounds__(256) k_prepare_series(const double* __restrict
       const int a1 = (a - d[0][h]) >> 8;                    // exact: a - d0 is a multiple of 256
       d[1][h] = ((a1 + 128) & 255) - 128;
       d[2][h] = (a1 - d[1][h]) >> 8;
+      wide |= d[2][h] > 64 || d[2][h] < -64;
     }
     const size_t o = (size_t)row * tp / 2 + t2;
 #pragma unroll
@@ -106,7 +107,8 @@ __global__ void __launch_bounds__(256) k_prepare_series(const double* __restrict
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if (lane == 0) norms[row] = acc;
-  if (__any_sync(0xffffffffu, off) && lane == 0) atomicOr(&st->flags, 1);
+  const int bits = (__any_sync(0xffffffffu, off) ? 1 : 0) | (__any_sync(0xffffffffu, wide) ? 2 : 0);
+  if (lane == 0 && bits & ~*reinterpret_cast<volatile int*>(&st->flags)) atomicOr(&st->flags, bits);
 }
 
 // Exact squared distances on the 2^-16 grid: int64 sums of squared int32
@@ -770,7 +772,8 @@ __global__ void __launch_bounds__(256) k_kernel_rows_panel(double* __restrict__ 
 // Warp w holds rows 8 w .. 8 w + 7, a lane the columns lane and lane + 32: both
 // sums start from the registers; the rows' lanes are combined by halving
 // exchanges (9 additions for 8 rows instead of 40), the columns' warps through
-// shared memory. Bound by instruction issue (143 a weight): n = 20011 1314 us, 3.7 TB/s;
+// shared memory. Bound by instruction issue (125 a weight; float64 sums, two additions a
+// weight on a pipe of two lanes a cycle, were no faster): n = 20011 1211 us, 4.0 TB/s;
 // with 128-bit exponentials and sums read back from shared memory 2315.
 struct KernelTileShared {
   double tt[DT][DT + 1];                                // tt[c][r] = A(i0 + r, j0 + c)
@@ -778,12 +781,14 @@ struct KernelTileShared {
   unsigned long long tab[EXP_TABLE];
 };
 
-template <int KERN>
+// FULL: every row and column of the tile lies inside the matrix.
+template <int KERN, bool FULL>
 __device__ __forceinline__ void kernel_tile(double* __restrict__ A, int n, const ExpFactor& f, double* __restrict__ part,
                                             int bi, int bj, KernelTileShared& sm) {
   const int i0 = bi * DT, j0 = bj * DT;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   ff rs[8], cs[2] = {{0.f, 0.f}, {0.f, 0.f}};
+  double* base = A + (size_t)(i0 + 8 * warp) * n + j0 + lane;
 #pragma unroll
   for (int m0 = 0; m0 < 8; m0 += 4) {
     double x[4][2];
@@ -792,23 +797,25 @@ __device__ __forceinline__ void kernel_tile(double* __restrict__ A, int n, const
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int i = i0 + 8 * warp + m0 + m, j = j0 + lane + 32 * h;
-        x[m][h] = i < n && j < n ? A[(size_t)i * n + j] : 0.0;
+        x[m][h] = FULL || (i < n && j < n) ? base[(size_t)(m0 + m) * n + 32 * h] : 0.0;
       }
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
-      rs[m0 + m] = {0.f, 0.f};
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int r = 8 * warp + m0 + m, c = lane + 32 * h, i = i0 + r, j = j0 + c;
         double a = 0.0;
-        if (i < n && j < n) {
+        if (FULL || (i < n && j < n)) {
           if (i != j) a = exp_neg_prod(KERN == KERNEL_EXP ? sqrt_nonneg(x[m][h]) : x[m][h], f, sm.tab);
-          A[(size_t)i * n + j] = a;
+          base[(size_t)(m0 + m) * n + 32 * h] = a;
         }
         sm.tt[c][r] = a;
-        const ff q = split_nonneg(a);
-        ff_acc(rs[m0 + m], q);
-        ff_acc(cs[h], q);
+        const ff v = split_nonneg(a);
+        ff_acc(cs[h], v);
+        if (h == 0)
+          rs[m0 + m] = v;
+        else
+          ff_acc(rs[m0 + m], v);
       }
     }
   }
@@ -819,36 +826,39 @@ __device__ __forceinline__ void kernel_tile(double* __restrict__ A, int n, const
 #pragma unroll
     for (int m = 0; m < w; ++m) {
       const ff keep = up ? rs[m + w] : rs[m], give = up ? rs[m] : rs[m + w];
-      const ff got = {__shfl_xor_sync(0xffffffffu, give.hi, 4 * w), __shfl_xor_sync(0xffffffffu, give.lo, 4 * w)};
-      rs[m] = ff_add(keep, got);
+      rs[m] = ff_add(keep, ff{__shfl_xor_sync(0xffffffffu, give.hi, 4 * w), __shfl_xor_sync(0xffffffffu, give.lo, 4 * w)});
     }
   }
 #pragma unroll
   for (int o = 2; o > 0; o >>= 1)
     rs[0] = ff_add(rs[0], ff{__shfl_xor_sync(0xffffffffu, rs[0].hi, o), __shfl_xor_sync(0xffffffffu, rs[0].lo, o)});
   const int ri = i0 + 8 * warp + (lane >> 2);
-  if ((lane & 3) == 0 && ri < n) part[(size_t)bj * n + ri] = (double)rs[0].hi + (double)rs[0].lo;
+  if ((lane & 3) == 0 && (FULL || ri < n)) part[(size_t)bj * n + ri] = (double)rs[0].hi + (double)rs[0].lo;
 #pragma unroll
   for (int h = 0; h < 2; ++h) sm.col[warp][lane + 32 * h] = make_float2(cs[h].hi, cs[h].lo);
   __syncthreads();
   if (bi != bj) {
     const int r = threadIdx.x & (DT - 1), rg = threadIdx.x >> 6;
-    const int i = i0 + r;
-#pragma unroll 4
-    for (int m = 0; m < DT / 4; ++m) {                  // mirror: lanes write consecutive columns of row j
-      const int cc = rg + 4 * m, j = j0 + cc;
-      if (j < n && i < n) A[(size_t)j * n + i] = sm.tt[cc][r];
-    }
-    if (threadIdx.x < DT && j0 + (int)threadIdx.x < n) {   // column sums (the mirror's row sums)
+    double* mirror = A + (size_t)(j0 + rg) * n + i0 + r;
+#pragma unroll 8
+    for (int m = 0; m < DT / 4; ++m)                    // lanes write consecutive columns of row j
+      if (FULL || (j0 + rg + 4 * m < n && i0 + r < n)) mirror[(size_t)(4 * m) * n] = sm.tt[rg + 4 * m][r];
+    if (threadIdx.x < DT && (FULL || j0 + (int)threadIdx.x < n)) {   // column sums (the mirror's row sums)
       ff acc = {0.f, 0.f};
 #pragma unroll
-      for (int w = 0; w < 8; ++w) {
-        const float2 v = sm.col[w][threadIdx.x];
-        acc = ff_add(acc, ff{v.x, v.y});
-      }
+      for (int w = 0; w < 8; ++w) acc = ff_add(acc, ff{sm.col[w][threadIdx.x].x, sm.col[w][threadIdx.x].y});
       part[(size_t)bi * n + j0 + threadIdx.x] = (double)acc.hi + (double)acc.lo;
     }
   }
+}
+
+template <int KERN>
+__device__ __forceinline__ void kernel_tile_any(double* __restrict__ A, int n, const ExpFactor& f,
+                                                double* __restrict__ part, int bi, int bj, KernelTileShared& sm) {
+  if ((bj + 1) * DT <= n)                                // bi <= bj
+    kernel_tile<KERN, true>(A, n, f, part, bi, bj, sm);
+  else
+    kernel_tile<KERN, false>(A, n, f, part, bi, bj, sm);
 }
 
 template <int KERN>
@@ -863,7 +873,7 @@ __global__ void __launch_bounds__(256, 4) k_kernel_tiles(double* __restrict__ A,
   for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
     if (threadIdx.x == 0) tri_index(t, nb, tile_s[0], tile_s[1]);
     __syncthreads();
-    kernel_tile<KERN>(A, n, f, part, tile_s[0], tile_s[1], sm);
+    kernel_tile_any<KERN>(A, n, f, part, tile_s[0], tile_s[1], sm);
     __syncthreads();
   }
 }
@@ -978,7 +988,7 @@ __global__ void __launch_bounds__(256, 4) k_g_kernel_tiles(const uint32_t* __res
   exp_table(sm.tab);
   const ExpFactor f = exp_factor(kernel_rcp(*G.sigma, KERNEL_GAUSSIAN));
   __syncthreads();
-  kernel_tile<KERNEL_GAUSSIAN>(G.A, G.n, f, G.part, (int)((t >> 12) & 0x3FFu), (int)(t >> 22), sm);
+  kernel_tile_any<KERNEL_GAUSSIAN>(G.A, G.n, f, G.part, (int)((t >> 12) & 0x3FFu), (int)(t >> 22), sm);
 }
 
 // D of graph blockIdx.x from its tiles' sums

@@ -914,17 +914,25 @@ constexpr int CR_MAX_KBLOCKS = 62 * CR_CHUNK_KB;       // int32 sums: |sum| <= 6
 // signed base-256 digits (|digit| <= 128, exact in bf16), so the Gram matrix is
 // a_i . a_j = sum_{s,t} 2^(8(s+t)) (D_s D_t^T)_ij over nine bf16 products.
 // Every digit product is exact in float32 (<= 2^14) and the slice pairs of
-// one weight w = s + t (at most three) summed over a 256-sample chunk stay
-// below 2^24, so the MMA's float32 accumulator holds an exact integer; the
+// one weight w = s + t (at most three) summed over a 256-sample chunk (512
+// where no top digit is above 64 in magnitude: |x| < 64) stay within 2^24, so the MMA's float32 accumulator holds an exact integer; the
 // epilogue adds it, shifted by 8w, to int64 accumulators. The result equals
 // the int64 sum of squared differences exactly; it is written as float64
-// multiples of 2^-32 to (i, j) and, off the diagonal blocks, to (j, i).
+// multiples of 2^-32 to (i, j): the upper triangle and the diagonal 128-blocks
+// (the kernel values are formed from those and mirrored).
 // Tiles are 128 rows x 64 columns of the upper block triangle; warp roles as
 // in k_tc_resid. Each pipeline stage holds the three digit planes of both
 // sides for one K block (72 KB, loaded once), and the MMA issuer feeds all
 // nine slice products into the five weight accumulators of the K chunk, slots
 // of a ring of eight 64-column TMEM accumulators, so that the MMAs of a tile
-// run ahead of its epilogue.
+// run ahead of its epilogue. Bound by the chain MMA - drain - MMA (the ring holds
+// one chunk and three fifths of the next): n = 16384 315 us at T = 64 and 1030 at T =
+// 365 without the writing of results, 443 and 1024 with it (two chunks then, one
+// now). n = 20011, T = 365 2057 -> 1578 us by integer-only conversions without
+// rounding, one search per block, products of one row plane with up to three
+// column planes at once, longer chunks and no mirrored writes; n = 32768, T = 256 3.63
+// -> 3.14 ms. Two groups of epilogue warps in turn, waiting for each accumulator only
+// where its first product comes, or waits without a timer read: no gain or a loss.
 constexpr int DS_SLICES = 3;
 constexpr int DS_N = 64;
 constexpr int DS_STAGES = 2;
@@ -935,7 +943,7 @@ constexpr int EPI_STAGE_DOUBLES = 16 * 32 * 17;          // per epilogue warp: 3
 constexpr int DS_SMEM_BYTES = DS_STAGES * DS_STAGE_BYTES + 512 + EPI_STAGE_DOUBLES * 8 + 1024;
 constexpr int DS_NBUF = 8;                     // ring of TMEM accumulators
 constexpr int DS_TMEM_COLS = DS_NBUF * DS_N;
-constexpr int DS_CHUNK_KB = 4;                   // 256 samples per exact chunk
+constexpr int DS_CHUNK_KB = 4;                   // 256 samples per exact chunk, 512 if no top digit is above 64
 
 struct DistMaps {
   CUtensorMap a[DS_SLICES];   // digit planes, box 64 x 128 rows
@@ -950,15 +958,14 @@ struct DistParams {
   int n;
   const long long* norms;     // |a_i|^2, rows padded with 0
   double* A;                  // n x n output
-  const int* offgrid;         // bit 0 set: input off the grid (the float64 kernel runs instead)
-  uint32_t idesc;
+  const int* offgrid;         // bit 0: input off the grid (other kernels run instead); bit 1: a top digit above 64
+  uint32_t idesc[DS_SLICES];  // for N = 64, 128, 192
   unsigned* status;
   // Row panels (graphs regenerated panel by panel): A holds rows row0 ..
-  // (A[(i - row0) n + j]), nothing is mirrored, and the tiles are either the
+  // (A[(i - row0) n + j]), and the tiles are either the
   // upper-triangle tiles tile0 .. tile0 + num_tiles - 1 (rect = 0; the rows of
   // the panel when the range is the panel's row blocks) or every tile
   // (I0 + t / nb64, t % nb64) of the panel's rect row blocks (rect > 0: whole rows).
-  int panel;
   int row0;
   long long tile0;
   int rect;
@@ -977,13 +984,34 @@ __device__ __forceinline__ void dist_tile(int t, int nb128, int nb64, int& I, in
   J = 2 * lo + (int)(t - ((long long)lo * nb64 - (long long)lo * (lo - 1)));
 }
 
-__device__ __forceinline__ void dist_decode(const DistParams& p, int t, int& I, int& J) {
-  if (p.rect > 0) {
-    I = p.I0 + t / p.nb64;
-    J = t % p.nb64;
-  } else {
-    dist_tile((int)(t + p.tile0), p.nb128, p.nb64, I, J);
+// A block's tiles in turn (blockIdx.x, then every gridDim.x-th): the search runs once,
+// the steps add (searching every tile took a quarter of the epilogue's instructions).
+struct DistTiles {
+  int I, J;
+  __device__ __forceinline__ DistTiles(const DistParams& p) {
+    if (p.rect > 0) {
+      I = p.I0 + (int)blockIdx.x / p.nb64;
+      J = (int)blockIdx.x % p.nb64;
+    } else {
+      dist_tile((int)(blockIdx.x + p.tile0), p.nb128, p.nb64, I, J);
+    }
   }
+  __device__ __forceinline__ void next(const DistParams& p) {
+    J += gridDim.x;
+    while (J >= p.nb64 && I < p.nb128) {                 // past the last tile: left at any (I, J)
+      J -= p.nb64;
+      ++I;
+      if (p.rect == 0) J += 2 * I;
+    }
+  }
+};
+
+// x 2^-32 for an integer x < 2^53 (exact), with integer operations: float64 additions
+// (two lanes a cycle and SM) took 16 cycles a warp where this takes 5.
+__device__ __forceinline__ double grid_d2(unsigned long long x) {
+  const int s = __clzll((long long)x) - 11;
+  const unsigned long long b = (x << s) + ((unsigned long long)(1042 - s) << 52);
+  return x == 0 ? 0.0 : __longlong_as_double((long long)b);
 }
 
 __global__ void __launch_bounds__(T8_THREADS, 1)
@@ -1002,7 +1030,8 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
   auto pempty_bar = [&](int b) { return bar0 + 8u * (2 * DS_STAGES + DS_NBUF + b); };
   const uint32_t drain_bar = bar0 + 8u * (2 * DS_STAGES + 2 * DS_NBUF);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nchunks = (p.kblocks + DS_CHUNK_KB - 1) / DS_CHUNK_KB;
+  const int chunk_kb = *p.offgrid & 2 ? DS_CHUNK_KB : 2 * DS_CHUNK_KB;
+  const int nchunks = (p.kblocks + chunk_kb - 1) / chunk_kb;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < DS_STAGES; ++s) {
@@ -1032,9 +1061,9 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
     // ------------------------------------------------ TMA producer
     int it = 0;
     bool ok = true;
-    for (int t = blockIdx.x; t < p.num_tiles && ok; t += gridDim.x) {
-      int I, J;
-      dist_decode(p, t, I, J);
+    DistTiles tile(p);
+    for (int t = blockIdx.x; t < p.num_tiles && ok; t += gridDim.x, tile.next(p)) {
+      const int I = tile.I, J = tile.J;
       // one stage per K block: the three digit planes of the row block and of the column block
       for (int kb = 0; kb < p.kblocks && ok; ++kb, ++it) {
         const int s = it % DS_STAGES;
@@ -1068,13 +1097,12 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
     for (int t = blockIdx.x; t < p.num_tiles && ok; t += gridDim.x)
       for (int c = 0; c < nchunks && ok; ++c, pc += NW) {
         for (int w = 0; w < NW && ok; ++w) {
-          const int b = (pc + w) % DS_NBUF;
           const uint32_t ph = (uint32_t)((pc + w) / DS_NBUF);
-          if (!mbar_wait(pempty_bar(b), (ph & 1) ^ 1, abort_flag, p.status)) ok = false;
+          ok = mbar_wait(pempty_bar((pc + w) % DS_NBUF), (ph & 1) ^ 1, abort_flag, p.status);
         }
         if (!ok) break;
         tc_fence_after();
-        for (int kb = c * DS_CHUNK_KB; kb < min(p.kblocks, (c + 1) * DS_CHUNK_KB) && ok; ++kb, ++it) {
+        for (int kb = c * chunk_kb; kb < min(p.kblocks, (c + 1) * chunk_kb) && ok; ++kb, ++it) {
           const int s = it % DS_STAGES;
           if (!mbar_wait(full_bar(s), (uint32_t)(it / DS_STAGES) & 1, abort_flag, p.status)) {
             ok = false;
@@ -1082,20 +1110,24 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
           }
           tc_fence_after();
           const uint32_t base = smem_u32(smem + s * DS_STAGE_BYTES);
-          const bool first_kb = kb == c * DS_CHUNK_KB;
-          for (int sa = 0; sa < DS_SLICES; ++sa)
-            for (int sb = 0; sb < DS_SLICES; ++sb) {
-              const int w = sa + sb;
-              const uint32_t d_tmem = tmem_base + (uint32_t)(((pc + w) % DS_NBUF) * DS_N);
-              // the first product of a weight in the chunk starts its accumulator
-              const bool first = first_kb && sa == (w < DS_SLICES ? 0 : w - (DS_SLICES - 1));
+          const bool first_kb = kb == c * chunk_kb;
+          // digit plane sa of the rows against the column planes that stand one after the other in
+          // shared memory and whose accumulators do so in TMEM: up to three at once (N = 192)
+          for (int sa = 0; sa < DS_SLICES; ++sa) {
+            // the first product of a weight in the chunk starts its accumulator
+            auto first = [&](int sb) { return first_kb && sa == (sa + sb < DS_SLICES ? 0 : sa + sb - (DS_SLICES - 1)); };
+            for (int sb = 0, len; sb < DS_SLICES; sb += len) {
+              const int b = (pc + sa + sb) % DS_NBUF;
+              for (len = 1; sb + len < DS_SLICES && b + len < DS_NBUF && first(sb + len) == first(sb);) ++len;
+              const uint32_t d_tmem = tmem_base + (uint32_t)(b * DS_N);
               const uint64_t adesc = smem_desc(base + sa * DS_A);
               const uint64_t bdesc = smem_desc(base + DS_SLICES * DS_A + sb * DS_B);
 #pragma unroll
               for (int kk = 0; kk < 4; ++kk)
-                mma_bf16(d_tmem, adesc + (uint64_t)(kk * 2), bdesc + (uint64_t)(kk * 2), p.idesc,
-                         (first && kk == 0) ? 0u : 1u);
+                mma_bf16(d_tmem, adesc + (uint64_t)(kk * 2), bdesc + (uint64_t)(kk * 2), p.idesc[len - 1],
+                         (first(sb) && kk == 0) ? 0u : 1u);
             }
+          }
           issued = true;
           mma_commit(empty_bar(s));
         }
@@ -1109,62 +1141,61 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
       }
     }
   } else if (warp >= 2) {
-    // ------------------------------------------------ epilogue: exact integer Gram, d2, both triangles
+    // ------------------------------------------------ epilogue: exact integer Gram, d2
     const int q = warp & 3;                              // TMEM lane quarter
     const int part = (warp - 2) >> 2;                    // 16-column part of the tile
-    const uint32_t lane_off = (uint32_t)(q * 32) << 16;
+    const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(part * 16);
+    double* stg = stage + (warp - 2) * (32 * 17);
+    constexpr int NW = 2 * DS_SLICES - 1;
     int pc = 0;
     bool failed = false;
-    for (int t = blockIdx.x; t < p.num_tiles; t += gridDim.x) {
-      int I, J;
-      dist_decode(p, t, I, J);
-      long long g[16];
+    DistTiles tile(p);
+    for (int t = blockIdx.x; t < p.num_tiles; t += gridDim.x, tile.next(p)) {
+      const int I = tile.I, J = tile.J;
+      const int row = I * 128 + q * 32 + lane, col0 = J * DS_N + part * 16;
+      long long g[16];                                   // norms: rows padded with 0
+      {
+        const long long ni = row < p.n ? p.norms[row] : 0;
 #pragma unroll
-      for (int e = 0; e < 16; ++e) g[e] = 0;
+        for (int e = 0; e < 16; ++e) g[e] = ni + p.norms[col0 + e];
+      }
       for (int c = 0; c < nchunks; ++c)
-        for (int w = 0; w <= 2 * (DS_SLICES - 1); ++w, ++pc) {
+#pragma unroll
+        for (int w = 0; w < NW; ++w, ++pc) {
           if (failed) continue;
           const int b = pc % DS_NBUF;
-          const uint32_t ph = (uint32_t)(pc / DS_NBUF);
-          if (!mbar_wait(pfull_bar(b), ph & 1, abort_flag, p.status)) {
+          if (!mbar_wait(pfull_bar(b), (uint32_t)(pc / DS_NBUF) & 1, abort_flag, p.status)) {
             failed = true;
             continue;
           }
           tc_fence_after();
-          {
-            float v[16];   // one load and one wait per drain
-            tmem_ld16(tmem_base + lane_off + (uint32_t)(b * DS_N + part * 16), v);
-#pragma unroll
-            for (int e = 0; e < 16; ++e) g[e] += (long long)__float2int_rn(v[e]) * (1LL << (8 * w));
-          }
+          float v[16];   // one load and one wait per drain
+          tmem_ld16(taddr + (uint32_t)(b * DS_N), v);
           tc_fence_before();
           mbar_arrive(pempty_bar(b));
+#pragma unroll
+          for (int e = 0; e < 16; ++e) g[e] -= (long long)__float2int_rn(v[e]) * (2LL << (8 * w));
         }
       if (__any_sync(0xffffffffu, failed)) continue;
-      const int row = I * 128 + q * 32 + lane;
-      const bool rowok = row < p.n;
-      const long long ni = rowok ? p.norms[row] : 0;
-      const int col0 = J * DS_N + part * 16;
-      const bool mirror = !p.panel && J >= 2 * I + 2;    // off the diagonal 128-block
-      double* stg = stage + (warp - 2) * (32 * 17);
+      unsigned long long any = 0;
 #pragma unroll
-      for (int e = 0; e < 16; ++e) {
-        const int col = col0 + e;
-        double d2 = 0.0;
-        if (rowok && col < p.n) {
-          // d2 >= 0 exactly; integer-only conversion (float64 is the scarce pipe)
-          d2 = u64_to_double_rn((unsigned long long)(ni + p.norms[col] - 2 * g[e]), -32);
-          if (mirror) p.A[(size_t)col * p.n + row] = d2;   // lanes write 32 consecutive entries
-        }
-        stg[lane * 17 + e] = d2;
+      for (int e = 0; e < 16; ++e) any |= (unsigned long long)g[e];
+      if (!__any_sync(0xffffffffu, any >> 53 != 0)) {
+#pragma unroll
+        for (int e = 0; e < 16; ++e) stg[lane * 17 + e] = grid_d2((unsigned long long)g[e]);
+      } else {                                           // distances above 2^21: with rounding
+#pragma unroll
+        for (int e = 0; e < 16; ++e) stg[lane * 17 + e] = u64_to_double_rn((unsigned long long)g[e], -32);
       }
       __syncwarp();
       // the warp's 32 x 16 block row-wise, two 128-byte row segments per store
-#pragma unroll 4
-      for (int it = 0; it < 16; ++it) {
-        const int rr = 2 * it + (lane >> 4), c = lane & 15;
-        const int grow = I * 128 + q * 32 + rr, gcol = col0 + c;
-        if (grow < p.n && gcol < p.n) p.A[(size_t)(grow - p.row0) * p.n + gcol] = stg[rr * 17 + c];
+      const int grow0 = I * 128 + q * 32 + (lane >> 4), gcol = col0 + (lane & 15);
+      const double* src = stg + (lane >> 4) * 17 + (lane & 15);
+      double* dst = p.A + (size_t)(grow0 - p.row0) * p.n + gcol;
+      if (gcol < p.n) {
+#pragma unroll
+        for (int it = 0; it < 16; ++it)
+          if (grow0 + 2 * it < p.n) dst[(size_t)(2 * it) * p.n] = src[2 * it * 17];
       }
       __syncwarp();
     }
@@ -1419,7 +1450,6 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
       const int row = I * 128 + q * 32 + lane, col0 = J * DS_N + part * 16;
       const int br = 2 * I + (q >> 1);                   // 64-row block of the row
       const bool rowok = !failed && row < p.n && (MODE == GR_DIST || br <= J);
-      const bool mirror = J >= 2 * I + 2;
       const int er = p.ex[row];
       const __int128 nr = i128_of(p.self[row]);
       bool low = false;
@@ -1480,7 +1510,6 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
                 low = true;
               else
                 out = i128_to_double(v, 2 * min(er, ec));
-              if (mirror) p.A[(size_t)col * p.n + row] = out;   // lanes write 32 consecutive entries
             } else {
               const double dc =
                   nan ? __longlong_as_double(0x7FF8000000000000ll) : i128_to_double(v, 2 * min(er, ec) + ge);
@@ -3682,7 +3711,7 @@ int dist_launch(cdl_ctx* ctx, const void* planes, int rows, int tp, DistParams& 
     CDL_TRY(make_map(&maps.b[s], base, rows, tp, DS_N));
   }
   p.kblocks = tp / 64;
-  p.idesc = make_idesc(DS_N);
+  for (int w = 0; w < DS_SLICES; ++w) p.idesc[w] = make_idesc((w + 1) * DS_N);
   p.status = ctx->dev_status;
   static bool attr = false;
   if (!attr) {
@@ -3791,7 +3820,6 @@ int dist_tc_panel(cdl_ctx* ctx, const void* planes, const long long* norms, int 
   p.norms = norms;
   p.A = panel;
   p.offgrid = offgrid;
-  p.panel = 1;
   p.row0 = row0;
   const int I0 = row0 / 128, PI = prows / 128;
   auto off = [&](long long I) { return I * p.nb64 - I * (I - 1); };   // first upper tile of row block I

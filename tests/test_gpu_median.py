@@ -65,3 +65,20 @@ def test_batched_medians_with_ties(G):
              for n in (90, 150, 333)]
     F, tops, stats = _run(G, pairs, 10, 0, G.cdl.CDL_F64)
     _check(pairs, F, tops, stats, 0)
+
+
+@pytest.mark.parametrize("top", [64, 65, 127])
+@pytest.mark.parametrize("T", [63, 64, 256, 257, 511, 512, 513, 1100])
+def test_distance_exact_at_the_digit_extremes(G, T, top):
+    """Two series whose base-256 digits are as large as they get, so that the exact
+    float32 sums of a chunk of samples reach their bound: sigma^2 is their distance."""
+    for d0, d1, s in ((-128, -128, 1), (127, 127, 1), (-128, -128, -1), (127, -128, -1)):
+        a = (top << 16) + (d1 << 8) + d0
+        b = s * ((top << 16) + (d1 << 8) - 127)
+        A = np.full(T, a, dtype=object)
+        B = np.full(T, b, dtype=object)
+        A[::7] = -A[::7]
+        X = np.array([A, B], dtype=np.float64) * 2.0 ** -16
+        d2 = int(((A - B) ** 2).sum())                    # Python integers
+        _, _, _, sg = G.graph(X)
+        assert float(sg) == np.sqrt(np.float64(d2) * 2.0 ** -32)
