@@ -222,10 +222,15 @@ int build_plan(cdl_ctx* ctx, int G, const int64_t* n, int T, const cdl_batch_opt
     for (int b = 0; b < (nn + 255) / 256; ++b) snodes.push_back(((uint32_t)b << 12) | (uint32_t)p);
   }
   GraphTiles gt;
+  const int tp = (int)round_up(T, 64);
+  std::vector<char> tc_dist(G2);
   {
     std::vector<int> gns(G2);
     for (int g = 0; g < G2; ++g) gns[g] = gn(g);
-    graph_grouped_tiles(gns, T, gt);
+    // The digit planes of the tensor-core distances (6 npad tp bytes) lie where the slices of A
+    // (12 npad^2) come later: every series but the longest on the smallest graphs.
+    for (int g = 0; g < G2; ++g) tc_dist[g] = tp <= 2 * gnp(g);
+    graph_grouped_tiles(gns, tc_dist, T, gt);
   }
   // projection variants: node rows per block
   std::vector<std::vector<uint32_t>> pblocks;
@@ -239,11 +244,14 @@ int build_plan(cdl_ctx* ctx, int G, const int64_t* n, int T, const cdl_batch_opt
     P->pv.push_back(pvar);
   }
   size_t ntiles = ap.size() + t32.size() + elem.size() + zst.size() + runits.size() + csb.size() + sel.size() +
-                  spairs.size() + snodes.size() + gt.fixed.size() + gt.dist.size() + cvec.size() +
+                  spairs.size() + snodes.size() + gt.fixed.size() + gt.dist.size() + gt.prep.size() + gt.tc.size() + cvec.size() +
                   cinit.size();
   for (auto& v : sq) ntiles += v.size();
   for (auto& v : pblocks) ntiles += v.size();
   std::vector<GGraph> ggs(G2);
+  std::vector<DistGroup> dgs(G2);
+  std::memset(dgs.data(), 0, G2 * sizeof(DistGroup));
+  DistGroup* d_dgs = nullptr;
   std::vector<PGraph> pgs(G2);
   std::vector<CGraph> cgs(G2);
   GGraph* d_ggs = nullptr;
@@ -271,6 +279,7 @@ int build_plan(cdl_ctx* ctx, int G, const int64_t* n, int T, const cdl_batch_opt
     res_groups = c.take<TcGroup>(2 * G2);
     d_tiles = c.take<uint32_t>(ntiles);
     d_ggs = c.take<GGraph>(G2);
+    d_dgs = c.take<DistGroup>(G2);
     d_pgs = c.take<PGraph>(G2);
     d_cgs = c.take<CGraph>(G2);
     d_sel = c.take<int4>(gt.sel.size());
@@ -378,6 +387,12 @@ int build_plan(cdl_ctx* ctx, int G, const int64_t* n, int T, const cdl_batch_opt
     Gg.sel = sel_all + (size_t)g * sel_one;
     Gg.n = nn;
     Gg.T = T;
+    Gg.npad = np;
+    Gg.tp = tp;
+    Gg.planes = tc_dist[g] ? cgs[g].aslices : nullptr;
+    Gg.norms = reinterpret_cast<long long*>(P->Dv[g]);     // npad, until D is formed
+    if (tc_dist[g] && (st = dist_group(&dgs[g], Gg.planes, np, tp, Gg.norms, Gg.A, graph_select_flags(Gg.sel), nn)) != CDL_OK)
+      return fail(st);
     CGraph& Cg = cgs[g];
     Cg.A = P->A[g];
     Cg.D = ch.D;
@@ -475,6 +490,8 @@ int build_plan(cdl_ctx* ctx, int G, const int64_t* n, int T, const cdl_batch_opt
   GraphBatch& gb = P->gb;
   add(gt.fixed, gb.fixed);
   add(gt.dist, gb.dist);
+  add(gt.prep, gb.prep);
+  add(gt.tc, gb.tc);
   for (size_t v = 0; v < pblocks.size(); ++v) add(pblocks[v], P->pv[v].blocks);
   add(cvec, P->cvec);
   add(cinit, P->cinit);
@@ -483,6 +500,7 @@ int build_plan(cdl_ctx* ctx, int G, const int64_t* n, int T, const cdl_batch_opt
   P->pv_choice = 0;
   if ((st = upload(P->stream, d_tiles, all)) != CDL_OK || (st = upload(P->stream, d_gs, gs)) != CDL_OK ||
       (st = upload(P->stream, P->jobs, jobs)) != CDL_OK || (st = upload(P->stream, d_ggs, ggs)) != CDL_OK ||
+      (st = upload(P->stream, d_dgs, dgs)) != CDL_OK ||
       (st = upload(P->stream, d_pgs, pgs)) != CDL_OK || (st = upload(P->stream, d_sel, gt.sel)) != CDL_OK ||
       (st = upload(P->stream, d_cgs, cgs)) != CDL_OK)
     return fail(st);
@@ -490,6 +508,8 @@ int build_plan(cdl_ctx* ctx, int G, const int64_t* n, int T, const cdl_batch_opt
   gb.G2 = G2;
   gb.sigma = o->sigma;
   gb.gs = d_ggs;
+  gb.dist_groups = d_dgs;
+  gb.tp = tp;
   gb.sel_all = sel_all;
   gb.sel_bytes = (size_t)G2 * sel_one;
   gb.sel = d_sel;

@@ -71,11 +71,10 @@ __global__ void k_to_fixed(const double* __restrict__ X, int* __restrict__ Xt, i
 // other kernels handle it). Bound by memory: 8 bytes read and 6 written per
 // sample; three kernels with a pass each (one an int32 copy that nothing
 // read) took 238 us at n = 20011, T = 365.
-__global__ void __launch_bounds__(256) k_prepare_series(const double* __restrict__ X, int n, int T, int rows, int tp,
-                                                         __nv_bfloat162* __restrict__ planes,
-                                                         long long* __restrict__ norms, SelectState* st) {
-  const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (row >= rows) return;
+__device__ __forceinline__ void prepare_series_row(const double* __restrict__ X, int n, int T, int row, int rows, int tp,
+                                                   __nv_bfloat162* __restrict__ planes, long long* __restrict__ norms,
+                                                   SelectState* st) {
+  const int lane = threadIdx.x & 31;
   const size_t plane = (size_t)rows * tp / 2;
   const double* x = X + (size_t)min(row, n - 1) * T;
   long long acc = 0;
@@ -109,6 +108,13 @@ __global__ void __launch_bounds__(256) k_prepare_series(const double* __restrict
   if (lane == 0) norms[row] = acc;
   const int bits = (__any_sync(0xffffffffu, off) ? 1 : 0) | (__any_sync(0xffffffffu, wide) ? 2 : 0);
   if (lane == 0 && bits & ~*reinterpret_cast<volatile int*>(&st->flags)) atomicOr(&st->flags, bits);
+}
+
+__global__ void __launch_bounds__(256) k_prepare_series(const double* __restrict__ X, int n, int T, int rows, int tp,
+                                                         __nv_bfloat162* __restrict__ planes,
+                                                         long long* __restrict__ norms, SelectState* st) {
+  const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (row < rows) prepare_series_row(X, n, T, row, rows, tp, planes, norms, st);
 }
 
 // Exact squared distances on the 2^-16 grid: int64 sums of squared int32
@@ -931,14 +937,25 @@ __global__ void k_g_to_fixed(const uint32_t* __restrict__ tiles, const GGraph* _
   if (__syncthreads_or(off) && threadIdx.x == 0) atomicOr(&static_cast<SelectState*>(G.sel)->flags, 1);
 }
 
-// tiles: g | bi << 12 | bj << 22 (64-node blocks, bi <= bj)
+// tiles: (b << 12) | g, rows 8 b .. of the graph's digit planes
+__global__ void __launch_bounds__(256) k_g_prepare_series(const uint32_t* __restrict__ tiles,
+                                                           const GGraph* __restrict__ gs) {
+  const uint32_t t = tiles[blockIdx.x];
+  const GGraph& G = gs[t & 0xFFFu];
+  prepare_series_row(G.X, G.n, G.T, (int)(t >> 12) * 8 + (threadIdx.x >> 5), G.npad, G.tp,
+                     static_cast<__nv_bfloat162*>(G.planes), G.norms, static_cast<SelectState*>(G.sel));
+}
+
+// tiles: g | bi << 12 | bj << 22 (64-node blocks, bi <= bj); what the tensor-core
+// distances leave over (128 graphs, T = 64: all by int64 tiles 2.44 ms, through the
+// digit planes 0.59 and 0.19 for the planes and the blocks that return here)
 __global__ void __launch_bounds__(256) k_g_dist(const uint32_t* __restrict__ tiles, const GGraph* __restrict__ gs) {
   const uint32_t t = tiles[blockIdx.x];
   const GGraph& G = gs[t & 0xFFFu];
   const int bi = (int)((t >> 12) & 0x3FFu), bj = (int)(t >> 22);
   if (static_cast<const SelectState*>(G.sel)->flags & 1)
     dist_f64_tile(G.X, G.n, G.T, G.A, bi, bj);
-  else
+  else if (!G.planes)
     dist_int_tile(G.Xt, G.n, G.T, G.A, bi, bj);
 }
 
@@ -1006,16 +1023,25 @@ __global__ void k_g_sum(const GGraph* __restrict__ gs) {
 
 }  // namespace
 
+const int* graph_select_flags(const void* sel) { return &static_cast<const SelectState*>(sel)->flags; }
+
 size_t graph_select_bytes() { return SELECT_STATE_BYTES + RADIX_BINS * sizeof(unsigned long long); }
 
-void graph_grouped_tiles(const std::vector<int>& n, int T, GraphTiles& out) {
+void graph_grouped_tiles(const std::vector<int>& n, const std::vector<char>& tc, int T, GraphTiles& out) {
   std::vector<int> order(n.size());
   for (size_t g = 0; g < n.size(); ++g) order[g] = (int)g;
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return n[a] > n[b]; });
   for (int g : order) {
     const int nn = n[g], nb = (nn + DT - 1) / DT;
     const size_t total = (size_t)nn * T;
-    for (size_t b = 0; b * 1024 < total; ++b) out.fixed.push_back(((uint32_t)b << 12) | (uint32_t)g);
+    if (tc[g]) {
+      const int nb128 = (nn + 127) / 128;
+      for (int b = 0; b < nb128 * 16; ++b) out.prep.push_back(((uint32_t)b << 12) | (uint32_t)g);
+      for (int I = 0; I < nb128; ++I)
+        for (int J = 2 * I; J < 2 * nb128; ++J) out.tc.push_back((uint32_t)g | ((uint32_t)I << 12) | ((uint32_t)J << 22));
+    } else {
+      for (size_t b = 0; b * 1024 < total; ++b) out.fixed.push_back(((uint32_t)b << 12) | (uint32_t)g);
+    }
     for (int bi = 0; bi < nb; ++bi)
       for (int bj = bi; bj < nb; ++bj) out.dist.push_back((uint32_t)g | ((uint32_t)bi << 12) | ((uint32_t)bj << 22));
     // selection: consecutive rows holding about 2^17 upper-triangle keys
@@ -1047,13 +1073,19 @@ int graph_build_grouped(cdl_ctx* ctx, const GraphBatch& B) {
     k_g_select_init<<<B.G2, 1, 0, s>>>(B.gs);
     CDL_TRY(L.done());
   }
-  {
+  if (B.prep.count > 0) {
+    Launch L(ctx, CDL_KC_DISTANCE, 0);
+    k_g_prepare_series<<<B.prep.count, 256, 0, s>>>(B.prep.p, B.gs);
+    CDL_TRY(L.done());
+  }
+  if (B.fixed.count > 0) {
     Launch L(ctx, CDL_KC_DISTANCE, 0);
     k_g_to_fixed<<<B.fixed.count, 256, 0, s>>>(B.fixed.p, B.gs);
     CDL_TRY(L.done());
   }
+  if (B.tc.count > 0) CDL_TRY(dist_tc_grouped(ctx, B.dist_groups, B.tc.p, B.tc.count, B.tp, B.dist_terms));
   {
-    Launch L(ctx, CDL_KC_DISTANCE, B.dist_terms);
+    Launch L(ctx, CDL_KC_DISTANCE, B.tc.count > 0 ? 0 : B.dist_terms);
     k_g_dist<<<B.dist.count, 256, 0, s>>>(B.dist.p, B.gs);
     CDL_TRY(L.done());
   }

@@ -388,29 +388,55 @@ struct BTiles {
 // Graph build of one graph of a batch (device pointers).
 struct GGraph {
   const double* X;  // n x T
-  int* Xt;          // T x n fixed-point copy
+  int* Xt;          // T x n fixed-point copy (planes null)
+  void* planes;     // 3 x npad x tp digit planes (bf16) for the tensor-core distances, or null
+  long long* norms; // npad
   double* A;        // n x n
   double* D;        // n
   double* part;     // ceil(n / 64) x n: sums of A over 64-node blocks
   double* vol;
   double* sigma;
   void* sel;        // graph_select_bytes(): selection state and histogram
-  int n, T;
+  int n, T, npad, tp;
 };
 size_t graph_select_bytes();
+const int* graph_select_flags(const void* sel);   // bit 0: input off the grid
+// A graph of the grouped tensor-core distances: three 128-row and three 64-row
+// maps of its digit planes, and where its results go.
+struct DistMaps {
+  CUtensorMap a[3];   // digit planes, box 64 x 128 rows
+  CUtensorMap b[3];   // digit planes, box 64 x 64 rows
+};
+struct DistGroup {
+  DistMaps maps;
+  const long long* norms;   // |a_i|^2, rows padded with 0
+  double* A;
+  const int* offgrid;       // bit 0: other kernels form this graph's distances
+  int n;
+  int pad[9];
+};
+static_assert(sizeof(DistGroup) % 64 == 0, "DistGroup keeps its tensor maps 64-byte aligned in arrays");
+int dist_group(DistGroup* d, const void* planes, int rows, int tp, const long long* norms, double* A, const int* offgrid,
+               int n);
+// tiles: g | I << 12 | J << 22 (128 x 64 tiles, J >= 2 I), all of one padded length tp
+int dist_tc_grouped(cdl_ctx* ctx, const DistGroup* groups, const uint32_t* tiles, int ntiles, int tp, double terms);
 struct GraphTiles {
   std::vector<uint32_t> fixed;   // (b << 12) | g, 1024-sample blocks of X
   std::vector<uint32_t> dist;    // g | bi << 12 | bj << 22, 64-node blocks, bi <= bj
+  std::vector<uint32_t> prep;    // (b << 12) | g, 8 rows of the digit planes
+  std::vector<uint32_t> tc;      // g | I << 12 | J << 22, 128 x 64 tiles of the tensor-core distances
   std::vector<int4> sel;         // (g, first row, end row, 0): about 2^17 keys each
 };
-void graph_grouped_tiles(const std::vector<int>& n, int T, GraphTiles& out);
+void graph_grouped_tiles(const std::vector<int>& n, const std::vector<char>& tc, int T, GraphTiles& out);
 struct GraphBatch {
   int G2 = 0;
   double sigma = 0;              // <= 0: median rule per graph
   const GGraph* gs = nullptr;    // device
   void* sel_all = nullptr;       // the graphs' selection blocks, contiguous
   size_t sel_bytes = 0;
-  BTiles fixed, dist;
+  BTiles fixed, dist, prep, tc;
+  const DistGroup* dist_groups = nullptr;   // device
+  int tp = 0;
   const int4* sel = nullptr;
   int sel_count = 0;
   double dist_terms = 0, select_bytes = 0, kernel_bytes = 0;

@@ -945,11 +945,6 @@ constexpr int DS_NBUF = 8;                     // ring of TMEM accumulators
 constexpr int DS_TMEM_COLS = DS_NBUF * DS_N;
 constexpr int DS_CHUNK_KB = 4;                   // 256 samples per exact chunk, 512 if no top digit is above 64
 
-struct DistMaps {
-  CUtensorMap a[DS_SLICES];   // digit planes, box 64 x 128 rows
-  CUtensorMap b[DS_SLICES];   // digit planes, box 64 x 64 rows
-};
-
 struct DistParams {
   int nb128;                  // row blocks of 128
   int nb64;                   // column blocks of 64 (2 nb128)
@@ -970,6 +965,9 @@ struct DistParams {
   long long tile0;
   int rect;
   int I0;
+  // Grouped launches: tile table and graphs (dist_tc_grouped)
+  const uint32_t* tiles;
+  const DistGroup* groups;
 };
 
 // tile t -> (I, J): row block I holds nb64 - 2 I tiles J = 2 I .. nb64 - 1
@@ -986,17 +984,32 @@ __device__ __forceinline__ void dist_tile(int t, int nb128, int nb64, int& I, in
 
 // A block's tiles in turn (blockIdx.x, then every gridDim.x-th): the search runs once,
 // the steps add (searching every tile took a quarter of the epilogue's instructions).
+template <bool GRP>
 struct DistTiles {
-  int I, J;
-  __device__ __forceinline__ DistTiles(const DistParams& p) {
-    if (p.rect > 0) {
-      I = p.I0 + (int)blockIdx.x / p.nb64;
-      J = (int)blockIdx.x % p.nb64;
+  int t, I, J;
+  const DistGroup* G;
+  __device__ __forceinline__ void entry(const DistParams& p) {
+    const uint32_t e = t < p.num_tiles ? p.tiles[t] : 0;
+    G = p.groups + (e & 0xFFFu);
+    I = (int)((e >> 12) & 0x3FFu);
+    J = (int)(e >> 22);
+  }
+  __device__ __forceinline__ DistTiles(const DistParams& p) : t(blockIdx.x), G(nullptr) {
+    if (GRP) {
+      entry(p);
+    } else if (p.rect > 0) {
+      I = p.I0 + t / p.nb64;
+      J = t % p.nb64;
     } else {
-      dist_tile((int)(blockIdx.x + p.tile0), p.nb128, p.nb64, I, J);
+      dist_tile((int)(t + p.tile0), p.nb128, p.nb64, I, J);
     }
   }
   __device__ __forceinline__ void next(const DistParams& p) {
+    t += gridDim.x;
+    if (GRP) {
+      entry(p);
+      return;
+    }
     J += gridDim.x;
     while (J >= p.nb64 && I < p.nb128) {                 // past the last tile: left at any (I, J)
       J -= p.nb64;
@@ -1004,6 +1017,8 @@ struct DistTiles {
       if (p.rect == 0) J += 2 * I;
     }
   }
+  // a graph of a grouped launch whose series is off the grid
+  __device__ __forceinline__ bool skip() const { return GRP && (*G->offgrid & 1); }
 };
 
 // x 2^-32 for an integer x < 2^53 (exact), with integer operations: float64 additions
@@ -1014,9 +1029,10 @@ __device__ __forceinline__ double grid_d2(unsigned long long x) {
   return x == 0 ? 0.0 : __longlong_as_double((long long)b);
 }
 
+template <bool GRP>
 __global__ void __launch_bounds__(T8_THREADS, 1)
     k_tc_dist(const __grid_constant__ DistMaps maps, const DistParams p) {
-  if (*p.offgrid & 1) return;                            // uniform: before any barrier or allocation
+  if (!GRP && *p.offgrid & 1) return;                            // uniform: before any barrier or allocation
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + DS_STAGES * DS_STAGE_BYTES);
@@ -1030,7 +1046,7 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
   auto pempty_bar = [&](int b) { return bar0 + 8u * (2 * DS_STAGES + DS_NBUF + b); };
   const uint32_t drain_bar = bar0 + 8u * (2 * DS_STAGES + 2 * DS_NBUF);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int chunk_kb = *p.offgrid & 2 ? DS_CHUNK_KB : 2 * DS_CHUNK_KB;
+  const int chunk_kb = GRP || *p.offgrid & 2 ? DS_CHUNK_KB : 2 * DS_CHUNK_KB;
   const int nchunks = (p.kblocks + chunk_kb - 1) / chunk_kb;
 
   if (threadIdx.x == 0) {
@@ -1061,9 +1077,10 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
     // ------------------------------------------------ TMA producer
     int it = 0;
     bool ok = true;
-    DistTiles tile(p);
-    for (int t = blockIdx.x; t < p.num_tiles && ok; t += gridDim.x, tile.next(p)) {
+    for (DistTiles<GRP> tile(p); tile.t < p.num_tiles && ok; tile.next(p)) {
+      if (tile.skip()) continue;
       const int I = tile.I, J = tile.J;
+      const DistMaps* m = GRP ? &tile.G->maps : &maps;
       // one stage per K block: the three digit planes of the row block and of the column block
       for (int kb = 0; kb < p.kblocks && ok; ++kb, ++it) {
         const int s = it % DS_STAGES;
@@ -1075,8 +1092,8 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
         const uint32_t dst = smem_u32(smem + s * DS_STAGE_BYTES);
         mbar_expect_tx(full_bar(s), DS_STAGE_BYTES);
         for (int pl = 0; pl < DS_SLICES; ++pl) {
-          tma_load_2d(dst + pl * DS_A, &maps.a[pl], kb * 64, I * 128, full_bar(s));
-          tma_load_2d(dst + DS_SLICES * DS_A + pl * DS_B, &maps.b[pl], kb * 64, J * DS_N, full_bar(s));
+          tma_load_2d(dst + pl * DS_A, &m->a[pl], kb * 64, I * 128, full_bar(s));
+          tma_load_2d(dst + DS_SLICES * DS_A + pl * DS_B, &m->b[pl], kb * 64, J * DS_N, full_bar(s));
         }
       }
     }
@@ -1094,7 +1111,8 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
     constexpr int NW = 2 * DS_SLICES - 1;
     int it = 0, pc = 0;
     bool ok = true, issued = false;
-    for (int t = blockIdx.x; t < p.num_tiles && ok; t += gridDim.x)
+    for (DistTiles<GRP> tile(p); tile.t < p.num_tiles && ok; tile.next(p)) {
+      if (tile.skip()) continue;
       for (int c = 0; c < nchunks && ok; ++c, pc += NW) {
         for (int w = 0; w < NW && ok; ++w) {
           const uint32_t ph = (uint32_t)((pc + w) / DS_NBUF);
@@ -1134,6 +1152,7 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
         if (!ok) break;
         for (int w = 0; w < NW; ++w) mma_commit(pfull_bar((pc + w) % DS_NBUF));
       }
+    }
     if (!ok && issued) {
       mma_commit(drain_bar);
       const unsigned long long t0 = globaltimer();
@@ -1149,15 +1168,17 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
     constexpr int NW = 2 * DS_SLICES - 1;
     int pc = 0;
     bool failed = false;
-    DistTiles tile(p);
-    for (int t = blockIdx.x; t < p.num_tiles; t += gridDim.x, tile.next(p)) {
+    for (DistTiles<GRP> tile(p); tile.t < p.num_tiles; tile.next(p)) {
+      if (tile.skip()) continue;
       const int I = tile.I, J = tile.J;
+      const int n = GRP ? tile.G->n : p.n;
+      const long long* norms = GRP ? tile.G->norms : p.norms;
       const int row = I * 128 + q * 32 + lane, col0 = J * DS_N + part * 16;
       long long g[16];                                   // norms: rows padded with 0
       {
-        const long long ni = row < p.n ? p.norms[row] : 0;
+        const long long ni = norms[row];
 #pragma unroll
-        for (int e = 0; e < 16; ++e) g[e] = ni + p.norms[col0 + e];
+        for (int e = 0; e < 16; ++e) g[e] = ni + norms[col0 + e];
       }
       for (int c = 0; c < nchunks; ++c)
 #pragma unroll
@@ -1191,11 +1212,11 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
       // the warp's 32 x 16 block row-wise, two 128-byte row segments per store
       const int grow0 = I * 128 + q * 32 + (lane >> 4), gcol = col0 + (lane & 15);
       const double* src = stg + (lane >> 4) * 17 + (lane & 15);
-      double* dst = p.A + (size_t)(grow0 - p.row0) * p.n + gcol;
-      if (gcol < p.n) {
+      double* dst = (GRP ? tile.G->A : p.A) + (size_t)(grow0 - (GRP ? 0 : p.row0)) * n + gcol;
+      if (gcol < n) {
 #pragma unroll
         for (int it = 0; it < 16; ++it)
-          if (grow0 + 2 * it < p.n) dst[(size_t)(2 * it) * p.n] = src[2 * it * 17];
+          if (grow0 + 2 * it < n) dst[(size_t)(2 * it) * n] = src[2 * it * 17];
       }
       __syncwarp();
     }
@@ -3702,29 +3723,60 @@ int resid_tc_grouped(cdl_ctx* ctx, const ResidGroup* dgroups, const uint32_t* un
 }
 
 namespace {
-int dist_launch(cdl_ctx* ctx, const void* planes, int rows, int tp, DistParams& p, double terms) {
-  DistMaps maps;
-  std::memset(&maps, 0, sizeof(maps));
+int dist_maps(DistMaps* maps, const void* planes, int rows, int tp) {
   for (int s = 0; s < DS_SLICES; ++s) {
     const char* base = static_cast<const char*>(planes) + (size_t)s * rows * tp * 2;
-    CDL_TRY(make_map(&maps.a[s], base, rows, tp, 128));
-    CDL_TRY(make_map(&maps.b[s], base, rows, tp, DS_N));
+    CDL_TRY(make_map(&maps->a[s], base, rows, tp, 128));
+    CDL_TRY(make_map(&maps->b[s], base, rows, tp, DS_N));
   }
+  return CDL_OK;
+}
+
+template <bool GRP>
+int dist_run(cdl_ctx* ctx, const DistMaps& maps, int tp, DistParams& p, double terms) {
   p.kblocks = tp / 64;
   for (int w = 0; w < DS_SLICES; ++w) p.idesc[w] = make_idesc((w + 1) * DS_N);
   p.status = ctx->dev_status;
   static bool attr = false;
   if (!attr) {
-    CDL_CUDA_TRY(cudaFuncSetAttribute(k_tc_dist, cudaFuncAttributeMaxDynamicSharedMemorySize, DS_SMEM_BYTES));
+    CDL_CUDA_TRY(cudaFuncSetAttribute(k_tc_dist<GRP>, cudaFuncAttributeMaxDynamicSharedMemorySize, DS_SMEM_BYTES));
     attr = true;
   }
   if (p.num_tiles <= 0) return CDL_OK;
   const int grid = std::min(p.num_tiles, ctx->sm_count);
   Launch L(ctx, CDL_KC_DISTANCE, terms);
-  k_tc_dist<<<grid, T8_THREADS, DS_SMEM_BYTES, ctx->stream>>>(maps, p);
+  k_tc_dist<GRP><<<grid, T8_THREADS, DS_SMEM_BYTES, ctx->stream>>>(maps, p);
   return L.done();
 }
+
+int dist_launch(cdl_ctx* ctx, const void* planes, int rows, int tp, DistParams& p, double terms) {
+  DistMaps maps;
+  std::memset(&maps, 0, sizeof(maps));
+  CDL_TRY(dist_maps(&maps, planes, rows, tp));
+  return dist_run<false>(ctx, maps, tp, p, terms);
+}
 }  // namespace
+
+int dist_group(DistGroup* d, const void* planes, int rows, int tp, const long long* norms, double* A, const int* offgrid,
+               int n) {
+  if (rows % 128 || tp % 64 || rows < n) return CDL_ERR_INVALID_ARG;
+  d->norms = norms;
+  d->A = A;
+  d->offgrid = offgrid;
+  d->n = n;
+  return dist_maps(&d->maps, planes, rows, tp);
+}
+
+int dist_tc_grouped(cdl_ctx* ctx, const DistGroup* groups, const uint32_t* tiles, int ntiles, int tp, double terms) {
+  DistMaps maps;
+  std::memset(&maps, 0, sizeof(maps));   // unused
+  DistParams p;
+  std::memset(&p, 0, sizeof(p));
+  p.num_tiles = ntiles;
+  p.tiles = tiles;
+  p.groups = groups;
+  return dist_run<true>(ctx, maps, tp, p, terms);
+}
 
 int dist_tc(cdl_ctx* ctx, const void* planes, const long long* norms, int n, int rows, int tp, double* A,
             const int* offgrid, double terms) {

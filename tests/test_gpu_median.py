@@ -82,3 +82,19 @@ def test_distance_exact_at_the_digit_extremes(G, T, top):
         d2 = int(((A - B) ** 2).sum())                    # Python integers
         _, _, _, sg = G.graph(X)
         assert float(sg) == np.sqrt(np.float64(d2) * 2.0 ** -32)
+
+
+@pytest.mark.parametrize("T", [64, 257, 300])
+def test_batched_distances_on_every_route(G, T):
+    """One batch with graphs on the grid (through the tensor cores; long series on small
+    orders, whose digit planes have no room, through int64) and off it (float64)."""
+    from test_gpu_batched import _check, _run
+    from workloads import iid_pair
+    pairs = []
+    for p, n in enumerate((90, 127, 129, 200, 333)):
+        X1, X2 = (np.array(x) for x in iid_pair(n, T, 3, 40 + p).X)
+        if p % 2:
+            X1 = X1 + 1e-7                                # X2 stays on the grid
+        pairs.append(SimpleNamespace(X=(X1, X2)))
+    F, tops, stats = _run(G, pairs, 10, 3, G.cdl.CDL_F64)
+    _check(pairs, F, tops, stats, 3)
