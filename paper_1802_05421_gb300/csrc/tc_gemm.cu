@@ -982,8 +982,20 @@ __device__ __forceinline__ void dist_tile(int t, int nb128, int nb64, int& I, in
   J = 2 * lo + (int)(t - ((long long)lo * nb64 - (long long)lo * (lo - 1)));
 }
 
-// A block's tiles in turn (blockIdx.x, then every gridDim.x-th): the search runs once,
-// the steps add (searching every tile took a quarter of the epilogue's instructions).
+// A block's tiles in turn (the first, then every gridDim.x-th): the search runs once,
+// the steps add (searching every tile took a quarter of the distances' epilogue).
+struct TriTiles {
+  int I, J;
+  __device__ __forceinline__ TriTiles(long long t, int nb128, int nb64) { dist_tile((int)t, nb128, nb64, I, J); }
+  __device__ __forceinline__ void next(int nb128, int nb64) {
+    J += gridDim.x;
+    while (J >= nb64 && I < nb128) {                     // past the last tile: left at any (I, J)
+      ++I;
+      J += 2 * I - nb64;
+    }
+  }
+};
+
 template <bool GRP>
 struct DistTiles {
   int t, I, J;
@@ -1011,7 +1023,7 @@ struct DistTiles {
       return;
     }
     J += gridDim.x;
-    while (J >= p.nb64 && I < p.nb128) {                 // past the last tile: left at any (I, J)
+    while (J >= p.nb64 && I < p.nb128) {                 // as TriTiles
       J -= p.nb64;
       ++I;
       if (p.rect == 0) J += 2 * I;
@@ -1356,9 +1368,9 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
     // ------------------------------------------------ TMA producer
     int it = 0;
     bool ok = true;
-    for (int t = blockIdx.x; t < p.num_tiles && ok; t += gridDim.x) {
-      int I, J;
-      dist_tile(t, p.nb128, p.nb64, I, J);
+    TriTiles tile(blockIdx.x, p.nb128, p.nb64);
+    for (int t = blockIdx.x; t < p.num_tiles && ok; t += gridDim.x, tile.next(p.nb128, p.nb64)) {
+      const int I = tile.I, J = tile.J;
       for (int l = 0; l < NP && ok; ++l)
         for (int kb = 0; kb < p.kblocks; ++kb, ++it) {
           const int s = it % GR_STAGES;
@@ -1429,9 +1441,9 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
     const int ge = MODE == GR_SCORE ? *p.gexp : 0;
     int pc = 0, tpar = 0;
     bool failed = false;
-    for (int t = blockIdx.x; t < p.num_tiles; t += gridDim.x) {
-      int I, J;
-      dist_tile(t, p.nb128, p.nb64, I, J);
+    TriTiles tile(blockIdx.x, p.nb128, p.nb64);
+    for (int t = blockIdx.x; t < p.num_tiles; t += gridDim.x, tile.next(p.nb128, p.nb64)) {
+      const int I = tile.I, J = tile.J;
 #pragma unroll 1
       for (int l = 0; l < NP; ++l) {
         const float mod = p.mod[l], rmod = p.rmod[l];
@@ -1712,9 +1724,9 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
     // 1-3 with v slices 1-6, then u slices 4-6 with v slices 1-3
     int it = 0;
     bool ok = true;
-    for (int t = blockIdx.x; t < p.num_tiles && ok; t += gridDim.x) {
-      int I, J;
-      dist_tile((int)(t + p.tile0), p.nb128, p.nb64, I, J);
+    TriTiles tile(blockIdx.x + p.tile0, p.nb128, p.nb64);
+    for (int t = blockIdx.x; t < p.num_tiles && ok; t += gridDim.x, tile.next(p.nb128, p.nb64)) {
+      const int I = tile.I, J = tile.J;
       for (int kb = 0; kb < p.kblocks && ok; ++kb)
         for (int h = 0; h < 2 && ok; ++h, ++it) {
           const int s = it % SC_STAGES;
@@ -1806,9 +1818,9 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
     const double osc = *p.oscale;
     int pc = 0;
     bool failed = false;
-    for (int t = blockIdx.x; t < p.num_tiles; t += gridDim.x) {
-      int I, J;
-      dist_tile((int)(t + p.tile0), p.nb128, p.nb64, I, J);
+    TriTiles tile(blockIdx.x + p.tile0, p.nb128, p.nb64);
+    for (int t = blockIdx.x; t < p.num_tiles; t += gridDim.x, tile.next(p.nb128, p.nb64)) {
+      const int I = tile.I, J = tile.J;
       {
         // bring this thread's A1 and A2 row segments into L2 while the MMAs run
         const int prow = I * 128 + q * 32 + lane, pc0 = J * SC_N + part * 16;
