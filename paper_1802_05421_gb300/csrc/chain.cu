@@ -40,6 +40,7 @@ __device__ __forceinline__ void chain_vector(const double* __restrict__ D, const
 __global__ void k_chain_vectors(const double* __restrict__ D, const double* __restrict__ vol,
                                 int n, int npad, double* __restrict__ rsd, double* __restrict__ u,
                                 float* __restrict__ rsf, float* __restrict__ uf) {
+  follow();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < npad) chain_vector(D, vol, n, rsd, u, rsf, uf, i);
 }
@@ -57,6 +58,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_chain_init(const double* __restrict__ A, int n, int npad,
                                                      const double* __restrict__ rsd,
                                                      const double* __restrict__ u, T* __restrict__ L0) {
+  follow();
   for (int i = blockIdx.x; i < npad; i += gridDim.x) {
     T* out = L0 + (size_t)i * npad;
     if (i >= n) {
@@ -84,6 +86,7 @@ __device__ __forceinline__ float fp8_scale_of(unsigned amax_bits) {
 // amax_0 = max |level 0| over the bf16 level.
 __global__ void __launch_bounds__(256) k_absmax_bf16(const __nv_bfloat16* __restrict__ L, size_t count,
                                                       unsigned* __restrict__ amax) {
+  follow();
   float m = 0.f;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x)
     m = fmaxf(m, fabsf(__bfloat162float(L[i])));
@@ -95,6 +98,7 @@ __global__ void __launch_bounds__(256) k_absmax_bf16(const __nv_bfloat16* __rest
 // level 0 in e4m3 from its bf16 copy.
 __global__ void __launch_bounds__(256) k_quant_fp8(const __nv_bfloat16* __restrict__ L, size_t count,
                                                     const unsigned* __restrict__ amax, uint8_t* __restrict__ Q) {
+  follow();
   const float inv = 1.0f / fp8_scale_of(*amax);
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x)
     Q[i] = (uint8_t)__nv_cvt_float_to_fp8(__bfloat162float(L[i]) * inv, __NV_SATFINITE, __NV_E4M3);
@@ -106,6 +110,7 @@ __global__ void __launch_bounds__(256) k_quant_fp8(const __nv_bfloat16* __restri
 __global__ void __launch_bounds__(256) k_rownorm_fp8(const uint8_t* __restrict__ Q, int npad,
                                                       const unsigned* __restrict__ amax_in,
                                                       unsigned* __restrict__ amax_out) {
+  follow();
   __shared__ float red[8];
   const float s = fp8_scale_of(*amax_in);
   float m = 0.f;
@@ -139,6 +144,7 @@ __global__ void __launch_bounds__(256) k_rownorm_fp8(const uint8_t* __restrict__
 // A as float hi + lo planes for the float-float residual (integer split).
 __global__ void __launch_bounds__(256) k_split_a(const double* __restrict__ A, size_t count,
                                                   float* __restrict__ hi, float* __restrict__ lo) {
+  follow();
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x) {
     const ff v = split_nonneg(A[i]);
     hi[i] = v.hi;
@@ -293,6 +299,7 @@ __global__ void __launch_bounds__(256) k_chain_init_tc(const double* __restrict_
                                                         __nv_bfloat16* __restrict__ L0, __nv_bfloat16* __restrict__ Ahi,
                                                         __nv_bfloat16* __restrict__ Alo, uint16_t* __restrict__ S,
                                                         unsigned long long* __restrict__ over) {
+  follow();
   const int gpr = npad / 8;                               // groups of 8 columns per row
   float m = 1.f;
   bool slices = true;
@@ -314,6 +321,7 @@ __global__ void __launch_bounds__(256) k_chain_init_tc(const double* __restrict_
 // nothing to do), and their scale in a_scale[0].
 __global__ void __launch_bounds__(256) k_a_slices(const double* __restrict__ A, int n, int npad,
                                                    uint16_t* __restrict__ S, double* __restrict__ a_scale) {
+  follow();
   const int sexp = pow2_exp_above((unsigned long long)__double_as_longlong(a_scale[1]));
   if (blockIdx.x == 0 && threadIdx.x == 0) a_scale[0] = __longlong_as_double((long long)(1023 + sexp) << 52);
   if (sexp == 0) return;
@@ -339,6 +347,7 @@ template <typename T, int BM, int BN, int BK, int TM, int TN, bool SYM>
 __global__ void __launch_bounds__(256) k_gemm_tn(const T* __restrict__ P, int ldp,
                                                   const T* __restrict__ Q, int ldq, T* __restrict__ C,
                                                   int ldc, int M, int N, int kchunk) {
+  follow();
   static_assert((BM / TM) * (BN / TN) == 256, "256 threads");
   __shared__ __align__(16) T As[2][BK][BM];
   __shared__ __align__(16) T Bs[2][BK][BN];
@@ -451,13 +460,13 @@ int square_impl(cdl_ctx* ctx, cdl_chain* ch, int level) {
     constexpr int B = 128;
     const int nb = np / B;
     Launch L(ctx, CDL_KC_SQUARE, flops);
-    k_gemm_tn<T, B, B, 8, 8, 8, true><<<nb * (nb + 1) / 2, 256, 0, ctx->stream>>>(S, np, S, np, C, np, np, np, np);
+    launch_next(k_gemm_tn<T, B, B, 8, 8, 8, true>, nb * (nb + 1) / 2, 256, 0, ctx->stream, S, np, S, np, C, np, np, np, np);
     return L.done();
   } else {
     constexpr int B = 64;
     const int nb = np / B;
     Launch L(ctx, CDL_KC_SQUARE, flops);
-    k_gemm_tn<T, B, B, 8, 4, 4, true><<<nb * (nb + 1) / 2, 256, 0, ctx->stream>>>(S, np, S, np, C, np, np, np, np);
+    launch_next(k_gemm_tn<T, B, B, 8, 4, 4, true>, nb * (nb + 1) / 2, 256, 0, ctx->stream, S, np, S, np, C, np, np, np, np);
     return L.done();
   }
 }
@@ -470,6 +479,7 @@ int square_impl(cdl_ctx* ctx, cdl_chain* ch, int level) {
 __global__ void __launch_bounds__(256) k_panel_level0(const double* __restrict__ P, int n, int npad, int r0,
                                                        int rows, const float* __restrict__ rsf,
                                                        const float* __restrict__ uf, __nv_bfloat16* __restrict__ L0) {
+  follow();
   const int gpr = npad / 8;
   for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < (size_t)rows * gpr;
        g += (size_t)gridDim.x * blockDim.x) {
@@ -502,6 +512,7 @@ __global__ void __launch_bounds__(256) k_panel_level0(const double* __restrict__
 // tiles through shared memory: read along i, written along c.
 __global__ void __launch_bounds__(256) k_panel_slices_t(const double* __restrict__ P, int n, int npad, int r0,
                                                          int rows, int Pw, uint16_t* __restrict__ S) {
+  follow();
   __shared__ double tile[32][33];
   const int ntc = Pw / 32, nti = npad / 32;
   const size_t plane = (size_t)npad * Pw;
@@ -551,7 +562,7 @@ __global__ void __launch_bounds__(256) k_g_chain_init(const uint32_t* __restrict
 int chain_split_a(cdl_ctx* ctx, const cdl_chain* ch, const double* A) {
   const size_t cnt = (size_t)ch->n * ch->n;
   Launch L(ctx, CDL_KC_RESIDUAL, 0);
-  k_split_a<<<ctx->sm_count * 8, 256, 0, ctx->stream>>>(A, cnt, ch->ahl, ch->ahl + cnt);
+  launch_next(k_split_a, ctx->sm_count * 8, 256, 0, ctx->stream, A, cnt, ch->ahl, ch->ahl + cnt);
   return L.done();
 }
 
@@ -564,7 +575,7 @@ int chain_init(cdl_ctx* ctx, cdl_chain* ch, const double* A) {
   float* uf = rsf + np;
   {
     Launch L(ctx, CDL_KC_MISC, 0);
-    k_chain_vectors<<<(np + 255) / 256, 256, 0, ctx->stream>>>(ch->D, ch->vol, n, np, ch->rsqrt_d, u, rsf, uf);
+    launch_next(k_chain_vectors, (np + 255) / 256, 256, 0, ctx->stream, ch->D, ch->vol, n, np, ch->rsqrt_d, u, rsf, uf);
     CDL_TRY(L.done());
   }
   const bool tensor = ch->aslices != nullptr;
@@ -584,28 +595,28 @@ int chain_init(cdl_ctx* ctx, cdl_chain* ch, const double* A) {
       if (tensor) {
         unsigned long long* over = reinterpret_cast<unsigned long long*>(ch->a_scale + 1);
         CDL_CUDA_TRY(cudaMemsetAsync(over, 0, sizeof(unsigned long long), ctx->stream));
-        k_chain_init_tc<true><<<ctx->sm_count * 8, 256, 0, ctx->stream>>>(A, n, np, rsf, uf, l0, ahi, alo, sl, over);
+        launch_next(k_chain_init_tc<true>, ctx->sm_count * 8, 256, 0, ctx->stream, A, n, np, rsf, uf, l0, ahi, alo, sl, over);
       } else {
-        k_chain_init_tc<false><<<ctx->sm_count * 8, 256, 0, ctx->stream>>>(A, n, np, rsf, uf, l0, ahi, alo, nullptr,
+        launch_next(k_chain_init_tc<false>, ctx->sm_count * 8, 256, 0, ctx->stream, A, n, np, rsf, uf, l0, ahi, alo, nullptr,
                                                                            nullptr);
       }
       CDL_TRY(L.done());
     }
     if (!tensor) return CDL_OK;
     Launch L(ctx, CDL_KC_CHAIN_INIT, 0);
-    k_a_slices<<<ctx->sm_count * 8, 256, 0, ctx->stream>>>(A, n, np, sl, ch->a_scale);
+    launch_next(k_a_slices, ctx->sm_count * 8, 256, 0, ctx->stream, A, n, np, sl, ch->a_scale);
     return L.done();
   };
   switch (ch->dtype) {
     case CDL_F64: {
       Launch L(ctx, CDL_KC_CHAIN_INIT, bytes);
-      k_chain_init<double><<<blocks, 256, 0, ctx->stream>>>(A, n, np, ch->rsqrt_d, u,
+      launch_next(k_chain_init<double>, blocks, 256, 0, ctx->stream, A, n, np, ch->rsqrt_d, u,
                                                             static_cast<double*>(ch->level(0)));
       return L.done();
     }
     case CDL_F32: {
       Launch L(ctx, CDL_KC_CHAIN_INIT, bytes);
-      k_chain_init<float><<<blocks, 256, 0, ctx->stream>>>(A, n, np, ch->rsqrt_d, u,
+      launch_next(k_chain_init<float>, blocks, 256, 0, ctx->stream, A, n, np, ch->rsqrt_d, u,
                                                            static_cast<float*>(ch->level(0)));
       return L.done();
     }
@@ -616,12 +627,12 @@ int chain_init(cdl_ctx* ctx, cdl_chain* ch, const double* A) {
       const size_t cnt = (size_t)np * np;
       {
         Launch L2(ctx, CDL_KC_CHAIN_INIT, 2.0 * cnt);
-        k_absmax_bf16<<<ctx->sm_count * 4, 256, 0, ctx->stream>>>(
+        launch_next(k_absmax_bf16, ctx->sm_count * 4, 256, 0, ctx->stream, 
             static_cast<const __nv_bfloat16*>(ch->level16(0)), cnt, ch->amax);
         CDL_TRY(L2.done());
       }
       Launch L3(ctx, CDL_KC_CHAIN_INIT, 3.0 * cnt);
-      k_quant_fp8<<<ctx->sm_count * 4, 256, 0, ctx->stream>>>(static_cast<const __nv_bfloat16*>(ch->level16(0)),
+      launch_next(k_quant_fp8, ctx->sm_count * 4, 256, 0, ctx->stream, static_cast<const __nv_bfloat16*>(ch->level16(0)),
                                                               cnt, ch->amax, static_cast<uint8_t*>(ch->level(0)));
       return L3.done();
     }
@@ -642,6 +653,7 @@ int chain_init(cdl_ctx* ctx, cdl_chain* ch, const double* A) {
 // on the bits of non-negative floats orders them like their values).
 template <typename T>
 __global__ void __launch_bounds__(256) k_level_inf_norm(const T* __restrict__ L, int np, unsigned* __restrict__ out) {
+  follow();
   __shared__ float red[8];
   for (int i = blockIdx.x; i < np; i += gridDim.x) {
     float s = 0.f;
@@ -667,16 +679,16 @@ int level_inf_norm(cdl_ctx* ctx, const cdl_chain* ch, int level, unsigned* out_b
   Launch L(ctx, CDL_KC_MISC, 2.0 * np * (double)np);
   switch (ch->dtype) {
     case CDL_F64:
-      k_level_inf_norm<double><<<blocks, 256, 0, ctx->stream>>>(static_cast<const double*>(ch->level(level)), np,
+      launch_next(k_level_inf_norm<double>, blocks, 256, 0, ctx->stream, static_cast<const double*>(ch->level(level)), np,
                                                                 out_bits);
       break;
     case CDL_F32:
-      k_level_inf_norm<float><<<blocks, 256, 0, ctx->stream>>>(static_cast<const float*>(ch->level(level)), np,
+      launch_next(k_level_inf_norm<float>, blocks, 256, 0, ctx->stream, static_cast<const float*>(ch->level(level)), np,
                                                                out_bits);
       break;
     default:   // bf16 levels, or the bf16 copies of e4m3 levels
       if (ch->host_levels) return CDL_ERR_UNSUPPORTED;
-      k_level_inf_norm<__nv_bfloat16><<<blocks, 256, 0, ctx->stream>>>(
+      launch_next(k_level_inf_norm<__nv_bfloat16>, blocks, 256, 0, ctx->stream, 
           static_cast<const __nv_bfloat16*>(ch->level16(level)), np, out_bits);
       break;
   }
@@ -686,7 +698,7 @@ int level_inf_norm(cdl_ctx* ctx, const cdl_chain* ch, int level, unsigned* out_b
 int fp8_level_bound(cdl_ctx* ctx, cdl_chain* ch, int level) {
   const int np = (int)ch->npad;
   Launch L(ctx, CDL_KC_MISC, (double)np * np);
-  k_rownorm_fp8<<<std::min(np, ctx->sm_count * 8), 256, 0, ctx->stream>>>(
+  launch_next(k_rownorm_fp8, std::min(np, ctx->sm_count * 8), 256, 0, ctx->stream, 
       static_cast<const uint8_t*>(ch->level(level)), np, ch->amax + level, ch->amax + level + 1);
   return L.done();
 }
@@ -708,7 +720,7 @@ int apply_simt(cdl_ctx* ctx, const cdl_chain* ch, int level, const void* x, void
     constexpr int BM = 128, BN = 64;
     dim3 grid(np / BM, (kp + BN - 1) / BN, splits);
     Launch L(ctx, CDL_KC_APPLY, bytes);
-    k_gemm_tn<float, BM, BN, 8, 8, 4, false><<<grid, 256, 0, ctx->stream>>>(
+    launch_next(k_gemm_tn<float, BM, BN, 8, 8, 4, false>, grid, 256, 0, ctx->stream, 
         static_cast<const float*>(ch->level(level)), np, static_cast<const float*>(x), kp,
         static_cast<float*>(partial), kp, np, kp, kchunk);
     return L.done();
@@ -717,7 +729,7 @@ int apply_simt(cdl_ctx* ctx, const cdl_chain* ch, int level, const void* x, void
     constexpr int BM = 64, BN = 64;
     dim3 grid(np / BM, (kp + BN - 1) / BN, splits);
     Launch L(ctx, CDL_KC_APPLY, bytes);
-    k_gemm_tn<double, BM, BN, 8, 4, 4, false><<<grid, 256, 0, ctx->stream>>>(
+    launch_next(k_gemm_tn<double, BM, BN, 8, 4, 4, false>, grid, 256, 0, ctx->stream, 
         static_cast<const double*>(ch->level(level)), np, static_cast<const double*>(x), kp,
         static_cast<double*>(partial), kp, np, kp, kchunk);
     return L.done();
@@ -736,7 +748,7 @@ int chain_vectors_only(cdl_ctx* ctx, cdl_chain* ch) {
   float* rsf = reinterpret_cast<float*>(u + np);
   float* uf = rsf + np;
   Launch L(ctx, CDL_KC_MISC, 0);
-  k_chain_vectors<<<(np + 255) / 256, 256, 0, ctx->stream>>>(ch->D, ch->vol, n, np, ch->rsqrt_d, u, rsf, uf);
+  launch_next(k_chain_vectors, (np + 255) / 256, 256, 0, ctx->stream, ch->D, ch->vol, n, np, ch->rsqrt_d, u, rsf, uf);
   return L.done();
 }
 
@@ -748,7 +760,7 @@ int chain_level0_panel(cdl_ctx* ctx, cdl_chain* ch, void* L0, const double* pane
   const float* rsf = reinterpret_cast<const float*>(static_cast<double*>(wsu) + np);
   const float* uf = rsf + np;
   Launch L(ctx, CDL_KC_CHAIN_INIT, 8.0 * rows * (double)n + 2.0 * rows * (double)np);
-  k_panel_level0<<<ctx->sm_count * 8, 256, 0, ctx->stream>>>(panel, n, np, r0, rows, rsf, uf,
+  launch_next(k_panel_level0, ctx->sm_count * 8, 256, 0, ctx->stream, panel, n, np, r0, rows, rsf, uf,
                                                              static_cast<__nv_bfloat16*>(L0));
   return L.done();
 }
@@ -756,7 +768,7 @@ int chain_level0_panel(cdl_ctx* ctx, cdl_chain* ch, void* L0, const double* pane
 int panel_slices_t(cdl_ctx* ctx, const double* panel, int n, int np, int r0, int rows, int Pw, void* slicesT) {
   if (Pw % 32 || np % 32) return CDL_ERR_INVALID_ARG;
   Launch L(ctx, CDL_KC_RESIDUAL, 0);
-  k_panel_slices_t<<<ctx->sm_count * 8, 256, 0, ctx->stream>>>(panel, n, np, r0, rows, Pw,
+  launch_next(k_panel_slices_t, ctx->sm_count * 8, 256, 0, ctx->stream, panel, n, np, r0, rows, Pw,
                                                                static_cast<uint16_t*>(slicesT));
   return L.done();
 }

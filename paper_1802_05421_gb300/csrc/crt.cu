@@ -146,6 +146,7 @@ __device__ __forceinline__ uint32_t residue_bits(const float (&d)[ND], int l) {
 template <typename T>
 __global__ void __launch_bounds__(256) k_crt_residues(const T* __restrict__ X, int rows, int cols, int ldx, int np,
                                                        int* __restrict__ ex, uint32_t* __restrict__ planes) {
+  follow();
   typedef LevelType<T> LT;
   __shared__ unsigned long long wmax[8];
   __shared__ float wsum[8];
@@ -232,6 +233,7 @@ struct Combine<float> {
 template <typename T>
 __global__ void __launch_bounds__(256) k_crt_combine(const uint8_t* __restrict__ t, int np,
                                                       const int* __restrict__ ex, T* __restrict__ C) {
+  follow();
   constexpr int NP = Combine<T>::NP;
   __shared__ T tile[64][65];
   int bi, bj;
@@ -280,6 +282,7 @@ __global__ void __launch_bounds__(128) k_series_residues(const double* __restric
                                                           ulonglong2* __restrict__ norms,
                                                           uint32_t* __restrict__ planes, uint32_t* __restrict__ bad,
                                                           int bad_words) {
+  follow();
   if (!(*offgrid & 1)) return;
   typedef LevelType<double> LT;
   __shared__ unsigned long long wmax[2][4];
@@ -376,6 +379,7 @@ __global__ void __launch_bounds__(256) k_score_maxima(const double* __restrict__
                                                        const double* __restrict__ vol1,
                                                        const double* __restrict__ vol2, size_t cnt,
                                                        int* __restrict__ mx) {
+  follow();
   const double s1 = sqrt(*vol1), s2 = sqrt(*vol2);
   int ea = 0, eb = 0;
   for (size_t o = blockIdx.x * (size_t)256 + threadIdx.x; o < cnt; o += (size_t)gridDim.x * 256) {
@@ -408,6 +412,7 @@ __global__ void __launch_bounds__(128) k_score_residues(const double* __restrict
                                                          ulonglong2* __restrict__ dself,
                                                          __nv_bfloat16* __restrict__ up,
                                                          __nv_bfloat16* __restrict__ vp) {
+  follow();
   typedef LevelType<double> LT;
   __shared__ unsigned long long wmax[4];
   __shared__ float wsum[4];
@@ -496,6 +501,7 @@ __global__ void __launch_bounds__(128) k_score_residues(const double* __restrict
 // np), zero beyond; 32 x 32 tiles.
 __global__ void __launch_bounds__(256) k_transpose_pad(const double* __restrict__ X, int rows, int cols, int ldx,
                                                         int np, double* __restrict__ out) {
+  follow();
   __shared__ double tile[32][33];
   const int i0 = blockIdx.x * 32, c0 = blockIdx.y * 32, tx = threadIdx.x & 31;
   for (int a = threadIdx.x >> 5; a < 32; a += 8)
@@ -524,6 +530,7 @@ __device__ __forceinline__ void product4(const uint8_t* __restrict__ t, int np, 
 __global__ void __launch_bounds__(128) k_crt_add(const uint8_t* __restrict__ t, int np, int kpb, int kp,
                                                   const int* __restrict__ erow, const int* __restrict__ ecol,
                                                   double* __restrict__ x) {
+  follow();
   const int q = kp / 4;
   const size_t idx = blockIdx.x * (size_t)128 + threadIdx.x;
   if (idx >= (size_t)np * q) return;
@@ -540,6 +547,7 @@ __global__ void __launch_bounds__(128) k_crt_residual(const uint8_t* __restrict_
                                                        const double* __restrict__ Y, const double* __restrict__ Z,
                                                        const double* __restrict__ D, int n, int k,
                                                        double* __restrict__ R, double* __restrict__ part) {
+  follow();
   __shared__ double red[4];
   const int q = (k + 3) / 4;
   double sq = 0.0;
@@ -570,14 +578,14 @@ int square_impl(cdl_ctx* ctx, cdl_chain* ch, int level, void* planes, uint8_t* t
   const int np = (int)ch->npad;
   {
     Launch L(ctx, CDL_KC_SQUARE, 0);
-    k_crt_residues<T><<<np, 256, 0, ctx->stream>>>(static_cast<const T*>(ch->level(level)), np, np, np, np, ex,
+    launch_next(k_crt_residues<T>, np, 256, 0, ctx->stream, static_cast<const T*>(ch->level(level)), np, np, np, np, ex,
                                                    static_cast<uint32_t*>(planes));
     CDL_TRY(L.done());
   }
   CDL_TRY(crt_gemm(ctx, planes, np, nullptr, 0, np, NP, t, CDL_KC_SQUARE, (double)ch->n * ch->n * (ch->n + 1.0)));
   const int nb = np / 64;
   Launch L(ctx, CDL_KC_SQUARE, 0);
-  k_crt_combine<T><<<nb * (nb + 1) / 2, 256, 0, ctx->stream>>>(t, np, ex, static_cast<T*>(ch->level(level + 1)));
+  launch_next(k_crt_combine<T>, nb * (nb + 1) / 2, 256, 0, ctx->stream, t, np, ex, static_cast<T*>(ch->level(level + 1)));
   return L.done();
 }
 
@@ -635,7 +643,7 @@ int crt_apply_begin(cdl_ctx* ctx, int np, int k, CrtApply* a) {
 
 int crt_apply_matrix(cdl_ctx* ctx, const CrtApply& a, const double* M, int n, int kc) {
   Launch L(ctx, kc, 0);
-  k_crt_residues<double><<<a.np, 256, 0, ctx->stream>>>(M, n, n, n, a.np, a.erow, a.planes);
+  launch_next(k_crt_residues<double>, a.np, 256, 0, ctx->stream, M, n, n, n, a.np, a.erow, a.planes);
   return L.done();
 }
 
@@ -643,12 +651,12 @@ int crt_apply_product(cdl_ctx* ctx, const CrtApply& a, const double* x, int rows
                       double work) {
   {
     Launch L(ctx, CDL_KC_MISC, 0);
-    k_transpose_pad<<<dim3(a.np / 32, a.kpb / 32), 256, 0, ctx->stream>>>(x, rows, cols, ldx, a.np, a.xt);
+    launch_next(k_transpose_pad, dim3(a.np / 32, a.kpb / 32), 256, 0, ctx->stream, x, rows, cols, ldx, a.np, a.xt);
     CDL_TRY(L.done());
   }
   {
     Launch L(ctx, CDL_KC_MISC, 0);
-    k_crt_residues<double><<<a.kpb, 256, 0, ctx->stream>>>(a.xt, a.kpb, a.np, a.np, a.np, a.ecol, a.xplanes);
+    launch_next(k_crt_residues<double>, a.kpb, 256, 0, ctx->stream, a.xt, a.kpb, a.np, a.np, a.np, a.ecol, a.xplanes);
     CDL_TRY(L.done());
   }
   return crt_gemm(ctx, a.planes, a.np, a.xplanes, a.kpb, a.np, 16, a.t, kc, work);
@@ -656,7 +664,7 @@ int crt_apply_product(cdl_ctx* ctx, const CrtApply& a, const double* x, int rows
 
 int crt_apply_add(cdl_ctx* ctx, const CrtApply& a, double* x, int kp) {
   Launch L(ctx, CDL_KC_MISC, 0);
-  k_crt_add<<<(unsigned)(((size_t)a.np * (kp / 4) + 127) / 128), 128, 0, ctx->stream>>>(a.t, a.np, a.kpb, kp, a.erow,
+  launch_next(k_crt_add, (unsigned)(((size_t)a.np * (kp / 4) + 127) / 128), 128, 0, ctx->stream, a.t, a.np, a.kpb, kp, a.erow,
                                                                                          a.ecol, x);
   return L.done();
 }
@@ -664,14 +672,14 @@ int crt_apply_add(cdl_ctx* ctx, const CrtApply& a, double* x, int kp) {
 int crt_apply_residual(cdl_ctx* ctx, const CrtApply& a, const double* Y, const double* Z, const double* D, int n, int k,
                        double* R, double* part, int nblocks) {
   Launch L(ctx, CDL_KC_RESIDUAL, 0);
-  k_crt_residual<<<nblocks, 128, 0, ctx->stream>>>(a.t, a.np, a.kpb, a.erow, a.ecol, Y, Z, D, n, k, R, part);
+  launch_next(k_crt_residual, nblocks, 128, 0, ctx->stream, a.t, a.np, a.kpb, a.erow, a.ecol, Y, Z, D, n, k, R, part);
   return L.done();
 }
 
 int series_residues(cdl_ctx* ctx, const double* X, int n, int T, int rows, int kp, const int* offgrid, int* ex,
                     void* norms, void* planes, void* bad, int bad_words) {
   Launch L(ctx, CDL_KC_DISTANCE, 0);
-  k_series_residues<<<rows, 128, 0, ctx->stream>>>(X, n, T, rows, kp, offgrid, ex, static_cast<ulonglong2*>(norms),
+  launch_next(k_series_residues, rows, 128, 0, ctx->stream, X, n, T, rows, kp, offgrid, ex, static_cast<ulonglong2*>(norms),
                                                    static_cast<uint32_t*>(planes), static_cast<uint32_t*>(bad),
                                                    bad_words);
   return L.done();
@@ -696,19 +704,19 @@ int score_pairs_residues(cdl_ctx* ctx, const double* Z1, const double* Z2, const
   {
     Launch L(ctx, CDL_KC_MISC, 0);
     const size_t nk = (size_t)n * k;
-    k_score_maxima<<<(unsigned)std::min<size_t>((nk + 255) / 256, (size_t)ctx->sm_count * 8), 256, 0, ctx->stream>>>(
+    launch_next(k_score_maxima, (unsigned)std::min<size_t>((nk + 255) / 256, (size_t)ctx->sm_count * 8), 256, 0, ctx->stream, 
         Z1, Z2, vol1, vol2, nk, mx);
     CDL_TRY(L.done());
   }
   {
     Launch L(ctx, CDL_KC_MISC, 0);
     if (fp64)
-      k_score_residues<16><<<rows, 128, 0, ctx->stream>>>(Z1, Z2, vol1, vol2, n, k, rows, kp, mx, ex,
+      launch_next(k_score_residues<16>, rows, 128, 0, ctx->stream, Z1, Z2, vol1, vol2, n, k, rows, kp, mx, ex,
                                                           static_cast<ulonglong2*>(vd),
                                                           static_cast<__nv_bfloat16*>(vu),
                                                           static_cast<__nv_bfloat16*>(vv));
     else
-      k_score_residues<13><<<rows, 128, 0, ctx->stream>>>(Z1, Z2, vol1, vol2, n, k, rows, kp, mx, ex,
+      launch_next(k_score_residues<13>, rows, 128, 0, ctx->stream, Z1, Z2, vol1, vol2, n, k, rows, kp, mx, ex,
                                                           static_cast<ulonglong2*>(vd),
                                                           static_cast<__nv_bfloat16*>(vu),
                                                           static_cast<__nv_bfloat16*>(vv));

@@ -50,6 +50,7 @@ static_assert(sizeof(SelectState) <= SELECT_STATE_BYTES, "the batched form's roo
 // (T x n) for coalesced tile loads; flags input off the grid.
 __global__ void k_to_fixed(const double* __restrict__ X, int* __restrict__ Xt, int n, int T,
                            SelectState* st) {
+  follow();
   const size_t total = (size_t)n * T;
   size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   size_t stride = (size_t)gridDim.x * blockDim.x;
@@ -113,6 +114,7 @@ __device__ __forceinline__ void prepare_series_row(const double* __restrict__ X,
 __global__ void __launch_bounds__(256) k_prepare_series(const double* __restrict__ X, int n, int T, int rows, int tp,
                                                          __nv_bfloat162* __restrict__ planes,
                                                          long long* __restrict__ norms, SelectState* st) {
+  follow();
   const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (row < rows) prepare_series_row(X, n, T, row, rows, tp, planes, norms, st);
 }
@@ -173,6 +175,7 @@ __device__ __forceinline__ void dist_int_tile(const int* __restrict__ Xt, int n,
 
 __global__ void __launch_bounds__(256) k_dist_int(const int* __restrict__ Xt, int n, int T,
                                                    double* __restrict__ A, const SelectState* st) {
+  follow();
   if (st->flags & 1) return;   // off-grid input: the float64 kernel handles it
   const int nb = (n + DT - 1) / DT;
   int bi, bj;
@@ -231,6 +234,7 @@ __device__ __forceinline__ void dist_f64_tile(const double* __restrict__ X, int 
 __global__ void __launch_bounds__(256) k_dist_f64(const double* __restrict__ X, int n, int T,
                                                    double* __restrict__ A, const SelectState* st,
                                                    const unsigned char* __restrict__ bad, int bad_stride) {
+  follow();
   if (!(st->flags & 1)) return;
   __shared__ int tile[2];
   const int nb = (n + DT - 1) / DT;
@@ -282,6 +286,7 @@ __device__ __forceinline__ void select_init(SelectState* st, long long rank) {
 
 __global__ void __launch_bounds__(1024) k_select_init(SelectState* st, long long rank,
                                                       unsigned long long* __restrict__ hist) {
+  follow();
   if (threadIdx.x == 0) select_init(st, rank);
   for (int b = threadIdx.x; b < RADIX_BINS; b += blockDim.x) hist[b] = 0;
 }
@@ -432,6 +437,7 @@ __device__ __forceinline__ void select_finish(SelectState* st, const unsigned lo
 
 __global__ void __launch_bounds__(SELECT_THREADS, 2) k_select_step(SelectState* st, unsigned long long* hist, int shift,
                                                                 int bits, double* sigma_out, int last) {
+  follow();
   __shared__ SelectShared sm;
   select_step(st, hist, shift, bits, sigma_out, last, sm);
 }
@@ -460,6 +466,7 @@ __global__ void __launch_bounds__(SELECT_THREADS, 2) k_select_hist_panel(const d
                                                                       int bits, const SelectState* __restrict__ st,
                                                                       unsigned long long* __restrict__ hist, int r0,
                                                                       int r1) {
+  follow();
   __shared__ SelectShared sm;
   select_hist(st, shift, bits, hist, sm, [&](auto&& f) {
     triangle_keys(P, n, r0, r1, blockIdx.x * SELECT_WARPS + (threadIdx.x >> 5), gridDim.x * SELECT_WARPS, r0, f);
@@ -574,6 +581,7 @@ __device__ __forceinline__ uint32_t sample_key(const double* __restrict__ A, int
 }
 
 __global__ void __launch_bounds__(256) k_sample_keys(const double* __restrict__ A, int n, uint32_t* __restrict__ out) {
+  follow();
   const uint32_t q = blockIdx.x * 256 + threadIdx.x;
   out[q] = sample_key(A, n, q);
 }
@@ -670,6 +678,7 @@ __device__ __forceinline__ void select_sample(int n, SelectState* st, unsigned l
 
 __global__ void __launch_bounds__(SAMPLE_THREADS) k_select_sample(const uint32_t* __restrict__ keys, int n,
                                                                   SelectState* st, unsigned long long cap) {
+  follow();
   extern __shared__ __align__(16) unsigned char sample_smem[];
   select_sample(n, st, cap, *reinterpret_cast<SampleShared*>(sample_smem), [&](uint32_t q) { return keys[q]; });
 }
@@ -677,6 +686,7 @@ __global__ void __launch_bounds__(SAMPLE_THREADS) k_select_sample(const uint32_t
 __global__ void __launch_bounds__(SELECT_THREADS, 2) k_select_bracket(const double* __restrict__ A, int n, SelectState* st,
                                                                    unsigned long long* __restrict__ buf,
                                                                    unsigned long long cap) {
+  follow();
   __shared__ SelectShared sm;
   select_bracket(st, buf, cap, gridDim.x, sm, [&](auto&& f) {
     folded_keys(A, n, f);
@@ -687,13 +697,15 @@ __global__ void __launch_bounds__(SELECT_THREADS, 2) k_select_pass(const double*
                                                                 SelectState* st, unsigned long long* __restrict__ hist,
                                                                 double* sigma_out, unsigned long long* __restrict__ buf,
                                                                 unsigned long long cap) {
+  follow();
   __shared__ SelectShared sm;
   select_pass(st, hist, p, sigma_out, buf, cap, blockIdx.x, gridDim.x, sm, [&](auto&& f) {
     folded_keys(A, n, f);
   });
 }
 
-__global__ void k_set_scalar(double* p, double v) { *p = v; }
+__global__ void k_set_scalar(double* p, double v) {
+  follow(); *p = v; }
 
 // A_ij = exp(-d2_ij / (2 sigma^2)) (KERN = KERNEL_GAUSSIAN) or
 // A_ij = exp(-sqrt(d2_ij) / sigma) (KERN = KERNEL_EXP, the synthetic-data
@@ -747,6 +759,7 @@ template <int KERN = KERNEL_GAUSSIAN>
 __global__ void __launch_bounds__(256) k_kernel_rows(double* __restrict__ A, int n,
                                                       const double* __restrict__ sigma,
                                                       double* __restrict__ D) {
+  follow();
   __shared__ unsigned long long tab[EXP_TABLE];
   exp_table(tab);
   const ExpFactor f = exp_factor(kernel_rcp(*sigma, KERN));
@@ -759,6 +772,7 @@ __global__ void __launch_bounds__(256) k_kernel_rows(double* __restrict__ A, int
 __global__ void __launch_bounds__(256) k_kernel_rows_panel(double* __restrict__ P, int n,
                                                             const double* __restrict__ sigma, double* __restrict__ D,
                                                             int r0, int r1) {
+  follow();
   __shared__ unsigned long long tab[EXP_TABLE];
   exp_table(tab);
   const ExpFactor f = exp_factor(kernel_rcp(*sigma, KERNEL_GAUSSIAN));
@@ -870,6 +884,7 @@ __device__ __forceinline__ void kernel_tile_any(double* __restrict__ A, int n, c
 template <int KERN>
 __global__ void __launch_bounds__(256, 4) k_kernel_tiles(double* __restrict__ A, int n, const double* __restrict__ sigma,
                                                           double* __restrict__ part) {
+  follow();
   __shared__ KernelTileShared sm;
   __shared__ int tile_s[2];
   const int nb = (n + DT - 1) / DT;
@@ -891,6 +906,7 @@ __device__ __forceinline__ double part_sum(const double* __restrict__ part, int 
 }
 
 __global__ void k_part_sums(const double* __restrict__ part, int nb, int n, double* __restrict__ D) {
+  follow();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) D[i] = part_sum(part, nb, n, i);
 }
@@ -911,7 +927,8 @@ __device__ __forceinline__ void block_sum_to(const double* __restrict__ v, int n
   }
 }
 
-__global__ void k_sum(const double* __restrict__ v, int n, double* __restrict__ out) { block_sum_to(v, n, out); }
+__global__ void k_sum(const double* __restrict__ v, int n, double* __restrict__ out) {
+  follow(); block_sum_to(v, n, out); }
 
 // ---------------------------------------------------------------- batched form
 // The same steps for every graph of a batch, one launch per step; a block
@@ -1138,7 +1155,7 @@ int graph_build(cdl_ctx* ctx, const double* X, int64_t n64, int T, double sigma,
   const long long m = (long long)n * (n - 1) / 2;
   {
     Launch L(ctx, CDL_KC_MISC, 0);
-    k_select_init<<<1, 1024, 0, s>>>(st, (m - 1) / 2, hist);
+    launch_next(k_select_init, 1, 1024, 0, s, st, (m - 1) / 2, hist);
     CDL_TRY(L.done());
   }
   const int nb = (n + DT - 1) / DT;
@@ -1152,7 +1169,7 @@ int graph_build(cdl_ctx* ctx, const double* X, int64_t n64, int T, double sigma,
     CDL_TRY(ws_get(ctx, "graph.norms", (size_t)rows * sizeof(long long), &wsNo));
     {
       Launch L(ctx, CDL_KC_DISTANCE, 0);
-      k_prepare_series<<<rows / 8, 256, 0, s>>>(X, n, T, rows, tp, static_cast<__nv_bfloat162*>(wsPl),
+      launch_next(k_prepare_series, rows / 8, 256, 0, s, X, n, T, rows, tp, static_cast<__nv_bfloat162*>(wsPl),
                                                 static_cast<long long*>(wsNo), st);
       CDL_TRY(L.done());
     }
@@ -1177,7 +1194,7 @@ int graph_build(cdl_ctx* ctx, const double* X, int64_t n64, int T, double sigma,
   }
   {
     Launch L(ctx, CDL_KC_DISTANCE, 0);
-    k_dist_f64<<<(unsigned)std::min<long long>(tiles, ctx->sm_count * 6), 256, 0, s>>>(X, n, T, A, st, bad, nb64);
+    launch_next(k_dist_f64, (unsigned)std::min<long long>(tiles, ctx->sm_count * 6), 256, 0, s, X, n, T, A, st, bad, nb64);
     CDL_TRY(L.done());
   }
   void* wsPart;
@@ -1185,7 +1202,7 @@ int graph_build(cdl_ctx* ctx, const double* X, int64_t n64, int T, double sigma,
   double* part = static_cast<double*>(wsPart);
   if (sigma > 0) {
     Launch L(ctx, CDL_KC_MISC, 0);
-    k_set_scalar<<<1, 1, 0, s>>>(sigma_out, sigma);
+    launch_next(k_set_scalar, 1, 1, 0, s, sigma_out, sigma);
     CDL_TRY(L.done());
   } else {
     // one buffer for the selection's keys and the kernel values' partial sums after it
@@ -1196,24 +1213,24 @@ int graph_build(cdl_ctx* ctx, const double* X, int64_t n64, int T, double sigma,
       {
         // the samples into the buffer first: one block's scattered loads took 25 us
         Launch L(ctx, CDL_KC_SELECT, 0);
-        k_sample_keys<<<SAMPLE / 256, 256, 0, s>>>(A, n, reinterpret_cast<uint32_t*>(sbuf));
+        launch_next(k_sample_keys, SAMPLE / 256, 256, 0, s, A, n, reinterpret_cast<uint32_t*>(sbuf));
         CDL_TRY(L.done());
       }
       {
         Launch L(ctx, CDL_KC_SELECT, 0);
-        k_select_sample<<<1, SAMPLE_THREADS, sizeof(SampleShared), s>>>(reinterpret_cast<const uint32_t*>(sbuf), n, st,
+        launch_next(k_select_sample, 1, SAMPLE_THREADS, sizeof(SampleShared), s, reinterpret_cast<const uint32_t*>(sbuf), n, st,
                                                                         cap);
         CDL_TRY(L.done());
       }
       Launch L(ctx, CDL_KC_SELECT, 8.0 * (double)m);
-      k_select_bracket<<<ctx->sm_count * 2, SELECT_THREADS, 0, s>>>(A, n, st, sbuf, cap);
+      launch_next(k_select_bracket, ctx->sm_count * 2, SELECT_THREADS, 0, s, A, n, st, sbuf, cap);
       CDL_TRY(L.done());
     }
     const unsigned hblocks = (unsigned)std::min<long long>((m + 4095) / 4096, ctx->sm_count * 2);
     for (int p = 0; p < 6; ++p) {
       // work: bytes of the triangle for the full passes (the later ones read the copied keys)
       Launch L(ctx, CDL_KC_SELECT, p < 3 && m < SELECT_BRACKET_MIN ? 8.0 * (double)m : 0.0);
-      k_select_pass<<<hblocks, SELECT_THREADS, 0, s>>>(A, n, p, st, hist, sigma_out, sbuf, cap);
+      launch_next(k_select_pass, hblocks, SELECT_THREADS, 0, s, A, n, p, st, hist, sigma_out, sbuf, cap);
       CDL_TRY(L.done());
     }
   }
@@ -1222,18 +1239,18 @@ int graph_build(cdl_ctx* ctx, const double* X, int64_t n64, int T, double sigma,
       Launch L(ctx, CDL_KC_KERNEL, 16.0 * (double)n * n);
       const unsigned blocks = (unsigned)std::min<long long>(tiles, ctx->sm_count * 4);
       if (kernel == KERNEL_EXP)
-        k_kernel_tiles<KERNEL_EXP><<<blocks, 256, 0, s>>>(A, n, sigma_out, part);
+        launch_next(k_kernel_tiles<KERNEL_EXP>, blocks, 256, 0, s, A, n, sigma_out, part);
       else
-        k_kernel_tiles<KERNEL_GAUSSIAN><<<blocks, 256, 0, s>>>(A, n, sigma_out, part);
+        launch_next(k_kernel_tiles<KERNEL_GAUSSIAN>, blocks, 256, 0, s, A, n, sigma_out, part);
       CDL_TRY(L.done());
     }
     Launch L(ctx, CDL_KC_MISC, 0);
-    k_part_sums<<<(n + 255) / 256, 256, 0, s>>>(part, nb, n, D);
+    launch_next(k_part_sums, (n + 255) / 256, 256, 0, s, part, nb, n, D);
     CDL_TRY(L.done());
   }
   {
     Launch L(ctx, CDL_KC_MISC, 0);
-    k_sum<<<1, 1024, 0, s>>>(D, n, vol);
+    launch_next(k_sum, 1, 1024, 0, s, D, n, vol);
     CDL_TRY(L.done());
   }
   return CDL_OK;
@@ -1273,12 +1290,12 @@ int graph_regen_init(cdl_ctx* ctx, RegenGraph& g, const double* X, int64_t n64, 
   const long long m = (long long)n * (n - 1) / 2;
   {
     Launch L(ctx, CDL_KC_MISC, 0);
-    k_select_init<<<1, 1024, 0, s>>>(st, (m - 1) / 2, hist);
+    launch_next(k_select_init, 1, 1024, 0, s, st, (m - 1) / 2, hist);
     CDL_TRY(L.done());
   }
   {
     Launch L(ctx, CDL_KC_DISTANCE, 0);
-    k_prepare_series<<<g.rows / 8, 256, 0, s>>>(X, n, T, g.rows, g.tp, static_cast<__nv_bfloat162*>(wsPl),
+    launch_next(k_prepare_series, g.rows / 8, 256, 0, s, X, n, T, g.rows, g.tp, static_cast<__nv_bfloat162*>(wsPl),
                                                 static_cast<long long*>(wsNo), st);
     CDL_TRY(L.done());
   }
@@ -1291,7 +1308,7 @@ int graph_regen_init(cdl_ctx* ctx, RegenGraph& g, const double* X, int64_t n64, 
   }
   if (sigma > 0) {
     Launch L(ctx, CDL_KC_MISC, 0);
-    k_set_scalar<<<1, 1, 0, s>>>(g.sigma, sigma);
+    launch_next(k_set_scalar, 1, 1, 0, s, g.sigma, sigma);
     CDL_TRY(L.done());
   } else {
     const int shifts[6] = {52, 40, 28, 16, 4, 0};
@@ -1303,12 +1320,12 @@ int graph_regen_init(cdl_ctx* ctx, RegenGraph& g, const double* X, int64_t n64, 
         const int r1 = std::min(n - 1, r0 + pr);
         if (r1 <= r0) continue;
         Launch L(ctx, CDL_KC_SELECT, 8.0 * (double)pr * n);
-        k_select_hist_panel<<<std::min((r1 - r0 + SELECT_WARPS - 1) / SELECT_WARPS, ctx->sm_count * 4), SELECT_THREADS, 0, s>>>(panel, n, shifts[p], widths[p], st,
+        launch_next(k_select_hist_panel, std::min((r1 - r0 + SELECT_WARPS - 1) / SELECT_WARPS, ctx->sm_count * 4), SELECT_THREADS, 0, s, panel, n, shifts[p], widths[p], st,
                                                                                hist, r0, r1);
         CDL_TRY(L.done());
       }
       Launch L(ctx, CDL_KC_SELECT, 0);
-      k_select_step<<<1, SELECT_THREADS, 0, s>>>(st, hist, shifts[p], widths[p], g.sigma, p == 5);
+      launch_next(k_select_step, 1, SELECT_THREADS, 0, s, st, hist, shifts[p], widths[p], g.sigma, p == 5);
       CDL_TRY(L.done());
     }
   }
@@ -1318,7 +1335,7 @@ int graph_regen_init(cdl_ctx* ctx, RegenGraph& g, const double* X, int64_t n64, 
     CDL_TRY(regen_panel(ctx, g, panel, r0, pr, g.D));
   }
   Launch L(ctx, CDL_KC_MISC, 0);
-  k_sum<<<1, 1024, 0, s>>>(g.D, n, g.vol);
+  launch_next(k_sum, 1, 1024, 0, s, g.D, n, g.vol);
   return L.done();
 }
 
@@ -1327,7 +1344,7 @@ int regen_panel(cdl_ctx* ctx, const RegenGraph& g, double* panel, int r0, int ro
   CDL_TRY(dist_tc_panel(ctx, g.planes, g.norms, g.n, g.rows, g.tp, panel, r0, pr, false, g.offgrid));
   const int r1 = std::min(g.n, r0 + rows);
   Launch L(ctx, CDL_KC_KERNEL, 16.0 * (double)(r1 - r0) * g.n);
-  k_kernel_rows_panel<<<std::min(r1 - r0, ctx->sm_count * 8), 256, 0, ctx->stream>>>(panel, g.n, g.sigma, D, r0, r1);
+  launch_next(k_kernel_rows_panel, std::min(r1 - r0, ctx->sm_count * 8), 256, 0, ctx->stream, panel, g.n, g.sigma, D, r0, r1);
   return L.done();
 }
 
@@ -1348,6 +1365,7 @@ __device__ __forceinline__ void neumaier_add(double& s, double& c, double a) {
 }
 
 __global__ void __launch_bounds__(256) k_degrees(const double* __restrict__ A, int n, double* __restrict__ D) {
+  follow();
   __shared__ double red_s[8], red_c[8];
   for (int i = blockIdx.x; i < n; i += gridDim.x) {
     const double* row = A + (size_t)i * n;
@@ -1383,6 +1401,7 @@ __global__ void __launch_bounds__(256) k_degrees(const double* __restrict__ A, i
 // two entries once, so distinct pairs give exact, order-free results.
 __global__ void k_add_edges(double* __restrict__ A, int n, long long m, const long long* __restrict__ ij,
                             const double* __restrict__ w, unsigned long long* __restrict__ bad) {
+  follow();
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += stride) {
     const long long i = ij[2 * e], j = ij[2 * e + 1];
@@ -1401,11 +1420,11 @@ int graph_degrees(cdl_ctx* ctx, const double* A, int64_t n64, double* D, double*
   cudaStream_t s = ctx->stream;
   {
     Launch L(ctx, CDL_KC_KERNEL, 8.0 * (double)n * n);
-    k_degrees<<<std::min(n, ctx->sm_count * 8), 256, 0, s>>>(A, n, D);
+    launch_next(k_degrees, std::min(n, ctx->sm_count * 8), 256, 0, s, A, n, D);
     CDL_TRY(L.done());
   }
   Launch L(ctx, CDL_KC_MISC, 0);
-  k_sum<<<1, 1024, 0, s>>>(D, n, vol);
+  launch_next(k_sum, 1, 1024, 0, s, D, n, vol);
   return L.done();
 }
 
@@ -1419,7 +1438,7 @@ int graph_add_edges(cdl_ctx* ctx, double* A, int64_t n, int64_t m, const int64_t
   if (m > 0) {
     const long long blocks = std::min<long long>((m + 255) / 256, (long long)ctx->sm_count * 16);
     Launch L(ctx, CDL_KC_MISC, 0);
-    k_add_edges<<<(unsigned)blocks, 256, 0, s>>>(A, (int)n, (long long)m, reinterpret_cast<const long long*>(ij),
+    launch_next(k_add_edges, (unsigned)blocks, 256, 0, s, A, (int)n, (long long)m, reinterpret_cast<const long long*>(ij),
                                                  w, bad);
     CDL_TRY(L.done());
   }
@@ -1574,30 +1593,30 @@ int graph_build_static(const double* X, int64_t n64, int T, double sigma, double
   const long long m = (long long)n * (n - 1) / 2;
   // The array keeps the previous call's contents: the select state and the
   // histogram must start from zero, Xt is fully overwritten.
-  k_select_init<<<1, 1024, 0, s>>>(st, (m - 1) / 2, hist);
+  launch_next(k_select_init, 1, 1024, 0, s, st, (m - 1) / 2, hist);
   CDL_TRY(launched());
   const size_t total = (size_t)n * T;
-  k_to_fixed<<<(int)std::min<size_t>((total + 255) / 256, (size_t)sm_count * 8), 256, 0, s>>>(X, Xt, n, T, st);
+  launch_next(k_to_fixed, (int)std::min<size_t>((total + 255) / 256, (size_t)sm_count * 8), 256, 0, s, X, Xt, n, T, st);
   CDL_TRY(launched());
   const int nb = (n + DT - 1) / DT;
   const long long tiles = (long long)nb * (nb + 1) / 2;
-  k_dist_int<<<(unsigned)tiles, 256, 0, s>>>(Xt, n, T, A, st);
+  launch_next(k_dist_int, (unsigned)tiles, 256, 0, s, Xt, n, T, A, st);
   CDL_TRY(launched());
-  k_dist_f64<<<(unsigned)std::min<long long>(tiles, sm_count * 6), 256, 0, s>>>(X, n, T, A, st, nullptr, 0);
+  launch_next(k_dist_f64, (unsigned)std::min<long long>(tiles, sm_count * 6), 256, 0, s, X, n, T, A, st, nullptr, 0);
   CDL_TRY(launched());
   if (sigma > 0) {
-    k_set_scalar<<<1, 1, 0, s>>>(sigma_out, sigma);
+    launch_next(k_set_scalar, 1, 1, 0, s, sigma_out, sigma);
     CDL_TRY(launched());
   } else {
     const unsigned hblocks = (unsigned)std::min<long long>((m + 4095) / 4096, sm_count * 2);
     for (int p = 0; p < 6; ++p) {   // no buffer: every pass over A
-      k_select_pass<<<hblocks, SELECT_THREADS, 0, s>>>(A, n, p, st, hist, sigma_out, nullptr, 0);
+      launch_next(k_select_pass, hblocks, SELECT_THREADS, 0, s, A, n, p, st, hist, sigma_out, nullptr, 0);
       CDL_TRY(launched());
     }
   }
-  k_kernel_rows<KERNEL_GAUSSIAN><<<std::min(n, sm_count * 8), 256, 0, s>>>(A, n, sigma_out, D);
+  launch_next(k_kernel_rows<KERNEL_GAUSSIAN>, std::min(n, sm_count * 8), 256, 0, s, A, n, sigma_out, D);
   CDL_TRY(launched());
-  k_sum<<<1, 1024, 0, s>>>(D, n, vol);
+  launch_next(k_sum, 1, 1024, 0, s, D, n, vol);
   return launched();
 }
 

@@ -41,6 +41,7 @@ constexpr int RED_THREADS = 256;
 // per-block partial sums of squares (deterministic order)
 __global__ void __launch_bounds__(RED_THREADS) k_sumsq(const double* __restrict__ v, size_t count,
                                                         double* __restrict__ part) {
+  follow();
   __shared__ double red[RED_THREADS / 32];
   double acc = 0.0;
   for (size_t i = blockIdx.x * (size_t)RED_THREADS + threadIdx.x; i < count;
@@ -60,6 +61,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_sumsq(const double* __restrict_
 }
 
 __global__ void k_reduce(const double* __restrict__ part, int count, double* __restrict__ out) {
+  follow();
   __shared__ double red[32];
   double acc = 0.0;
   for (int i = threadIdx.x; i < count; i += blockDim.x) acc += part[i];
@@ -77,6 +79,7 @@ __global__ void k_reduce(const double* __restrict__ part, int count, double* __r
 template <typename T>
 __global__ void k_precond_in(const double* __restrict__ R, const double* __restrict__ rsd, int n,
                              int k, int np, int kp, T* __restrict__ x) {
+  follow();
   size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   if (idx >= (size_t)np * kp) return;
   int i = (int)(idx / kp), r = (int)(idx % kp);
@@ -93,6 +96,7 @@ __global__ void __launch_bounds__(256) k_precond_out(const T* __restrict__ x, co
                                                       const double* __restrict__ D, int n, int k, int kp,
                                                       double* __restrict__ Z, float* __restrict__ dZ,
                                                       double* __restrict__ part) {
+  follow();
   __shared__ double red[8][33];
   const int i0 = blockIdx.x * 32, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   for (int c0 = 0; c0 < kp; c0 += 32) {
@@ -126,6 +130,7 @@ __global__ void __launch_bounds__(256) k_precond_out(const T* __restrict__ x, co
 // x[i][r] += sum_s part[s][i][r] (CUDA-core chains)
 template <typename T>
 __global__ void k_update_simt(T* __restrict__ x, const T* __restrict__ part, int splits, size_t elems) {
+  follow();
   size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   if (idx >= elems) return;
   T acc = x[idx];
@@ -139,6 +144,7 @@ __global__ void k_update_simt(T* __restrict__ x, const T* __restrict__ part, int
 __global__ void __launch_bounds__(256) k_update_bf16(float* __restrict__ x, const float* __restrict__ part,
                                                       ApplySplit sp, int np, int kp,
                                                       __nv_bfloat16* __restrict__ xop, int accumulate) {
+  follow();
   __shared__ float tile[32][33];
   const int i0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
   const int splits = accumulate ? sp.slots_of(i0 / 256) : 0;
@@ -177,6 +183,7 @@ __global__ void __launch_bounds__(256) k_update_bf16(float* __restrict__ x, cons
 __global__ void __launch_bounds__(256) k_center_shift(const double* __restrict__ part, int nparts, int k,
                                                        const double* __restrict__ vol, double* __restrict__ shift,
                                                        unsigned long long* __restrict__ mbits) {
+  follow();
   __shared__ double red[8][33];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, r = blockIdx.x * 32 + lane;
   double s = 0.0;
@@ -196,6 +203,7 @@ __global__ void __launch_bounds__(256) k_center_shift(const double* __restrict__
 // per block and column.
 __global__ void __launch_bounds__(256) k_center(double* __restrict__ Z, const double* __restrict__ shift, int n, int k,
                                                  unsigned long long* __restrict__ mbits) {
+  follow();
   __shared__ unsigned long long red[8][32];
   const int i0 = blockIdx.x * 64, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   for (int c0 = 0; c0 < k; c0 += 32) {
@@ -227,6 +235,7 @@ __global__ void __launch_bounds__(256) k_center(double* __restrict__ Z, const do
 // Z (float64) -> float hi + lo pair for the float-float residual.
 __global__ void k_split(const double* __restrict__ Z, size_t count, float* __restrict__ hi,
                         float* __restrict__ lo) {
+  follow();
   size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   if (idx >= count) return;
   const double z = Z[idx];
@@ -349,6 +358,7 @@ __global__ void __launch_bounds__(256) k_residual(const float* __restrict__ Ahi,
                                                    const double* __restrict__ Z, const double* __restrict__ Y,
                                                    const double* __restrict__ D, int n, int k,
                                                    double* __restrict__ R, double* __restrict__ part) {
+  follow();
   const double t = residual_tile<RB_M, RB_N>(Ahi, Alo, Zh, Zl, Z, Y, D, n, k, R, blockIdx.x * RB_M,
                                              blockIdx.y * RB_N);
   if (threadIdx.x == 0) part[blockIdx.y * gridDim.x + blockIdx.x] = t;
@@ -363,6 +373,7 @@ constexpr int RU_M = 128, RU_N = 128, RU_K = 16;
 __global__ void __launch_bounds__(256) k_residual_update(const double* __restrict__ A, const float* __restrict__ dZ,
                                                           const double* __restrict__ D, int n, int k, int kp,
                                                           double* __restrict__ R, double* __restrict__ part) {
+  follow();
   __shared__ __align__(16) float As[RU_K][RU_M + 4];
   __shared__ __align__(16) float Bs[RU_K][RU_N];
   __shared__ double red[8];
@@ -451,6 +462,7 @@ __global__ void __launch_bounds__(256) k_residual_update_tc(const float* __restr
                                                              ApplySplit sp, int np, const float* __restrict__ dZ,
                                                              const double* __restrict__ D, int n, int k, int kp,
                                                              double* __restrict__ R, double* __restrict__ part) {
+  follow();
   __shared__ double red[8];
   double sq = 0.0;
   const size_t total = (size_t)n * k;
@@ -498,6 +510,7 @@ __device__ __forceinline__ double pow2_above(unsigned long long bits) {
 __global__ void __launch_bounds__(256) k_zslice(const double* __restrict__ Z, int n, int k, int np, int c0, int kg,
                                                  const unsigned long long* __restrict__ mbits,
                                                  __nv_bfloat16* __restrict__ S, double* __restrict__ cs) {
+  follow();
   const size_t plane = (size_t)kg * np;
   for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < plane; idx += (size_t)gridDim.x * blockDim.x) {
     const int rl = (int)(idx / np), j = (int)(idx % np);
@@ -527,6 +540,7 @@ __global__ void __launch_bounds__(256) k_resid_combine(const double* __restrict_
                                                         const double* __restrict__ G, const double* __restrict__ cs,
                                                         const double* __restrict__ a_scale,
                                                         double* __restrict__ R, double* __restrict__ part) {
+  follow();
   __shared__ double red[8];
   const double as = a_scale[0];
   double sq = 0.0;
@@ -983,12 +997,12 @@ struct SolveBlock {
       const int nb = (int)std::min<size_t>(1024, (nk + RED_THREADS - 1) / RED_THREADS);
       {
         Launch L(ctx, CDL_KC_MISC, 0);
-        k_sumsq<<<nb, RED_THREADS, 0, st>>>(Y, nk, red);
+        launch_next(k_sumsq, nb, RED_THREADS, 0, st, Y, nk, red);
         CDL_TRY(L.done());
       }
       {
         Launch L(ctx, CDL_KC_MISC, 0);
-        k_reduce<<<1, 1024, 0, st>>>(red, nb, scal);
+        launch_next(k_reduce, 1, 1024, 0, st, red, nb, scal);
         CDL_TRY(L.done());
       }
       CDL_CUDA_TRY(cudaMemcpyAsync(&yy, scal, 8, cudaMemcpyDeviceToHost, st));
@@ -1023,7 +1037,7 @@ struct SolveBlock {
         double* Gg = static_cast<double*>(vG) + (size_t)g * RESID_PAIRS * np * 128;
         {
           Launch L(ctx, CDL_KC_MISC, 0);
-          k_zslice<<<ctx->sm_count * 4, 256, 0, st>>>(Z, n, k, np, c0, kg,
+          launch_next(k_zslice, ctx->sm_count * 4, 256, 0, st, Z, n, k, np, c0, kg,
                                                        static_cast<const unsigned long long*>(vzmax),
                                                        static_cast<__nv_bfloat16*>(vzs), static_cast<double*>(vcz));
           CDL_TRY(L.done());
@@ -1038,7 +1052,7 @@ struct SolveBlock {
       }
       const int nb = std::min(1024, (int)blocks_for(nk, 256));
       Launch L(ctx, CDL_KC_RESIDUAL, 0);
-      k_resid_combine<<<nb, 256, 0, st>>>(Y, Z, ch->D, n, k, np, static_cast<const double*>(vG),
+      launch_next(k_resid_combine, nb, 256, 0, st, Y, Z, ch->D, n, k, np, static_cast<const double*>(vG),
                                           static_cast<const double*>(vcz), ch->a_scale, R, red);
       CDL_TRY(L.done());
       nparts = nb;
@@ -1056,7 +1070,7 @@ struct SolveBlock {
         const int kg = std::min(128, (k - c0 + 31) / 32 * 32);
         {
           Launch L(ctx, CDL_KC_MISC, 0);
-          k_zslice<<<ctx->sm_count * 4, 256, 0, st>>>(Z, n, k, np, c0, kg,
+          launch_next(k_zslice, ctx->sm_count * 4, 256, 0, st, Z, n, k, np, c0, kg,
                                                        static_cast<const unsigned long long*>(vzmax),
                                                        static_cast<__nv_bfloat16*>(vzs), static_cast<double*>(vcz));
           CDL_TRY(L.done());
@@ -1065,7 +1079,7 @@ struct SolveBlock {
       }
       const int nb = std::min(1024, (int)blocks_for(nk, 256));
       Launch L(ctx, CDL_KC_RESIDUAL, 0);
-      k_resid_combine<<<nb, 256, 0, st>>>(Y, Z, ch->D, n, k, np, static_cast<const double*>(vG),
+      launch_next(k_resid_combine, nb, 256, 0, st, Y, Z, ch->D, n, k, np, static_cast<const double*>(vG),
                                           static_cast<const double*>(vcz), ch->a_scale, R, red);
       CDL_TRY(L.done());
       nparts = nb;
@@ -1083,13 +1097,13 @@ struct SolveBlock {
     a_ready = true;
     {
       Launch L(ctx, CDL_KC_MISC, 0);
-      k_split<<<blocks_for(nk, 256), 256, 0, st>>>(Z, nk, static_cast<float*>(vzh), static_cast<float*>(vzl));
+      launch_next(k_split, blocks_for(nk, 256), 256, 0, st, Z, nk, static_cast<float*>(vzh), static_cast<float*>(vzl));
       CDL_TRY(L.done());
     }
     {
       dim3 g(res_gx, res_gy);
       Launch L(ctx, CDL_KC_RESIDUAL, (double)n * n * k);
-      k_residual<<<g, 256, 0, st>>>(ch->ahl, ch->ahl + (size_t)n * n, static_cast<const float*>(vzh),
+      launch_next(k_residual, g, 256, 0, st, ch->ahl, ch->ahl + (size_t)n * n, static_cast<const float*>(vzh),
                                      static_cast<const float*>(vzl), Z, Y, ch->D, n, k, R, red);
       CDL_TRY(L.done());
     }
@@ -1104,7 +1118,7 @@ struct SolveBlock {
       {
         dim3 g((np + 31) / 32, (kp + 31) / 32);
         Launch L(ctx, CDL_KC_MISC, 0);
-        k_update_bf16<<<g, 256, 0, st>>>(static_cast<float*>(vdz), nullptr, sp, np, kp,
+        launch_next(k_update_bf16, g, 256, 0, st, static_cast<float*>(vdz), nullptr, sp, np, kp,
                                          static_cast<__nv_bfloat16*>(vdzop), 0);
         CDL_TRY(L.done());
       }
@@ -1113,14 +1127,14 @@ struct SolveBlock {
       CDL_TRY(apply_tc_mat(ctx, ahi + (size_t)np * np, np, vdzop, static_cast<float*>(vpart2), kp, sp));
       const int nb = (int)std::min<size_t>((nk + 255) / 256, (size_t)ctx->sm_count * 4);
       Launch L(ctx, CDL_KC_RESIDUAL, 0);
-      k_residual_update_tc<<<nb, 256, 0, st>>>(static_cast<const float*>(vpart), static_cast<const float*>(vpart2),
+      launch_next(k_residual_update_tc, nb, 256, 0, st, static_cast<const float*>(vpart), static_cast<const float*>(vpart2),
                                                sp, np, static_cast<const float*>(vdz), ch->D, n, k, kp, R, red);
       nparts = nb;
       return L.done();
     }
     dim3 g(upd_gx, upd_gy);
     Launch L(ctx, CDL_KC_RESIDUAL, (double)n * n * k);
-    k_residual_update<<<g, 256, 0, st>>>(A, static_cast<const float*>(vdz), ch->D, n, k, kp, R, red);
+    launch_next(k_residual_update, g, 256, 0, st, A, static_cast<const float*>(vdz), ch->D, n, k, kp, R, red);
     nparts = upd_gx * upd_gy;
     return L.done();
   }
@@ -1129,7 +1143,7 @@ struct SolveBlock {
     double rr = 0.0;
     {
       Launch L(ctx, CDL_KC_MISC, 0);
-      k_reduce<<<1, 1024, 0, st>>>(red, nparts, scal + 1);
+      launch_next(k_reduce, 1, 1024, 0, st, red, nparts, scal + 1);
       CDL_TRY(L.done());
     }
     CDL_CUDA_TRY(cudaMemcpyAsync(&rr, scal + 1, 8, cudaMemcpyDeviceToHost, st));
@@ -1166,17 +1180,17 @@ struct SolveBlock {
       const size_t cnt = (size_t)np * kp;
       Launch L(ctx, CDL_KC_MISC, 0);
       if (ch->dtype == CDL_F64)
-        k_precond_in<double><<<blocks_for(cnt, 256), 256, 0, st>>>(R, ch->rsqrt_d, n, k, np, kp,
+        launch_next(k_precond_in<double>, blocks_for(cnt, 256), 256, 0, st, R, ch->rsqrt_d, n, k, np, kp,
                                                                     static_cast<double*>(vx));
       else
-        k_precond_in<float><<<blocks_for(cnt, 256), 256, 0, st>>>(R, ch->rsqrt_d, n, k, np, kp,
+        launch_next(k_precond_in<float>, blocks_for(cnt, 256), 256, 0, st, R, ch->rsqrt_d, n, k, np, kp,
                                                                    static_cast<float*>(vx));
       CDL_TRY(L.done());
     }
     if (bf16) {
       dim3 g((np + 31) / 32, (kp + 31) / 32);
       Launch L(ctx, CDL_KC_MISC, 0);
-      k_update_bf16<<<g, 256, 0, st>>>(static_cast<float*>(vx), nullptr, sp, np, kp,
+      launch_next(k_update_bf16, g, 256, 0, st, static_cast<float*>(vx), nullptr, sp, np, kp,
                                        static_cast<__nv_bfloat16*>(vxop), 0);
       CDL_TRY(L.done());
     }
@@ -1189,7 +1203,7 @@ struct SolveBlock {
       CDL_TRY(apply_tc(ctx, ch, lvl, vxop, static_cast<float*>(vpart), kp, sp));
       dim3 g((np + 31) / 32, (kp + 31) / 32);
       Launch L(ctx, CDL_KC_MISC, 0);
-      k_update_bf16<<<g, 256, 0, st>>>(static_cast<float*>(vx), static_cast<const float*>(vpart), sp, np, kp,
+      launch_next(k_update_bf16, g, 256, 0, st, static_cast<float*>(vx), static_cast<const float*>(vpart), sp, np, kp,
                                        static_cast<__nv_bfloat16*>(vxop), 1);
       return L.done();
     }
@@ -1203,10 +1217,10 @@ struct SolveBlock {
     const size_t cnt = (size_t)np * kp;
     Launch L(ctx, CDL_KC_MISC, 0);
     if (ch->dtype == CDL_F64)
-      k_update_simt<double><<<blocks_for(cnt, 256), 256, 0, st>>>(
+      launch_next(k_update_simt<double>, blocks_for(cnt, 256), 256, 0, st, 
           static_cast<double*>(vx), static_cast<const double*>(vpart), splits, cnt);
     else
-      k_update_simt<float><<<blocks_for(cnt, 256), 256, 0, st>>>(
+      launch_next(k_update_simt<float>, blocks_for(cnt, 256), 256, 0, st, 
           static_cast<float*>(vx), static_cast<const float*>(vpart), splits, cnt);
     return L.done();
   }
@@ -1218,10 +1232,10 @@ struct SolveBlock {
       Launch L(ctx, CDL_KC_MISC, 0);
       double* cs = static_cast<double*>(vcs);
       if (ch->dtype == CDL_F64)
-        k_precond_out<double><<<cs_parts, 256, 0, st>>>(static_cast<const double*>(vx), ch->rsqrt_d, ch->D, n, k, kp, Z,
+        launch_next(k_precond_out<double>, cs_parts, 256, 0, st, static_cast<const double*>(vx), ch->rsqrt_d, ch->D, n, k, kp, Z,
                                                         static_cast<float*>(vdz), cs);
       else
-        k_precond_out<float><<<cs_parts, 256, 0, st>>>(static_cast<const float*>(vx), ch->rsqrt_d, ch->D, n, k, kp, Z,
+        launch_next(k_precond_out<float>, cs_parts, 256, 0, st, static_cast<const float*>(vx), ch->rsqrt_d, ch->D, n, k, kp, Z,
                                                        static_cast<float*>(vdz), cs);
       CDL_TRY(L.done());
     }
@@ -1230,12 +1244,12 @@ struct SolveBlock {
       unsigned long long* zmax = static_cast<unsigned long long*>(vzmax);
       {
         Launch L(ctx, CDL_KC_MISC, 0);
-        k_center_shift<<<(k + 31) / 32, 256, 0, st>>>(static_cast<const double*>(vcs), cs_parts, k, ch->vol, shift,
+        launch_next(k_center_shift, (k + 31) / 32, 256, 0, st, static_cast<const double*>(vcs), cs_parts, k, ch->vol, shift,
                                                       zmax);
         CDL_TRY(L.done());
       }
       Launch L(ctx, CDL_KC_MISC, 0);
-      k_center<<<(n + 63) / 64, 256, 0, st>>>(Z, shift, n, k, zmax);
+      launch_next(k_center, (n + 63) / 64, 256, 0, st, Z, shift, n, k, zmax);
       CDL_TRY(L.done());
     }
     ++iters;
@@ -1270,6 +1284,7 @@ struct SolveBlock {
 
 // columns c0 .. c0 + kb - 1 of the n x k matrix Y into the n x kb matrix Yb, and back
 __global__ void k_gather_cols(const double* __restrict__ Y, int n, int k, int c0, int kb, double* __restrict__ Yb) {
+  follow();
   const size_t cnt = (size_t)n * kb;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < cnt; e += (size_t)gridDim.x * blockDim.x) {
     const size_t i = e / kb;
@@ -1278,6 +1293,7 @@ __global__ void k_gather_cols(const double* __restrict__ Y, int n, int k, int c0
 }
 
 __global__ void k_scatter_cols(const double* __restrict__ Zb, int n, int kb, int c0, int k, double* __restrict__ Z) {
+  follow();
   const size_t cnt = (size_t)n * kb;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < cnt; e += (size_t)gridDim.x * blockDim.x) {
     const size_t i = e / kb;
@@ -1327,7 +1343,7 @@ int chain_solve(cdl_ctx* ctx, const cdl_chain* ch, const double* A, const double
       s.Z = static_cast<double*>(vzb);
       s.stats = &bst[b];
       Launch L(ctx, CDL_KC_MISC, 0);
-      k_gather_cols<<<gb, 256, 0, st>>>(Y, n, k, c0, s.k, static_cast<double*>(vyb));
+      launch_next(k_gather_cols, gb, 256, 0, st, Y, n, k, c0, s.k, static_cast<double*>(vyb));
       CDL_TRY(L.done());
     }
     CDL_TRY(s.init(b));
@@ -1363,7 +1379,7 @@ int chain_solve(cdl_ctx* ctx, const cdl_chain* ch, const double* A, const double
     if (s.status(opts) != CDL_OK) status = CDL_ERR_NOT_CONVERGED;
     {
       Launch L(ctx, CDL_KC_MISC, 0);
-      k_scatter_cols<<<gb, 256, 0, st>>>(s.Z, n, s.k, b * kb_max, k, Z);
+      launch_next(k_scatter_cols, gb, 256, 0, st, s.Z, n, s.k, b * kb_max, k, Z);
       CDL_TRY(L.done());
     }
     yy_all += s.yy;

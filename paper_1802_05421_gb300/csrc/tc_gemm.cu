@@ -707,6 +707,7 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
 // per thread fit.
 __global__ void __launch_bounds__(T8_THREADS, 1)
     k_tc_resid(const __grid_constant__ ResidMaps maps, const ResidParams p) {
+  follow();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + RS_STAGES * RS_STAGE_BYTES);
@@ -1044,6 +1045,7 @@ __device__ __forceinline__ double grid_d2(unsigned long long x) {
 template <bool GRP>
 __global__ void __launch_bounds__(T8_THREADS, 1)
     k_tc_dist(const __grid_constant__ DistMaps maps, const DistParams p) {
+  follow();
   if (!GRP && *p.offgrid & 1) return;                            // uniform: before any barrier or allocation
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -1322,6 +1324,7 @@ __device__ __forceinline__ __int128 i128_of(ulonglong2 v) { return (__int128)(((
 template <int MODE, int NP>
 __global__ void __launch_bounds__(T8_THREADS, 1)
     k_tc_gramr(const __grid_constant__ CUtensorMap tmU, const __grid_constant__ CUtensorMap tmV, const GramParams p) {
+  follow();
   // uniform: before any barrier or allocation
   if (MODE == GR_DIST && (!(*p.offgrid & 1) || p.kblocks == 0)) return;
   extern __shared__ uint8_t smem_raw[];
@@ -2377,6 +2380,7 @@ __device__ __forceinline__ uint32_t crt_byte_of_sum(int sum, uint32_t p, uint32_
 template <int NCH>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(S2_THREADS, 1)
     k_tc_crt(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const CrtGemmParams p) {
+  follow();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S2_STAGES * S2_STAGE);
@@ -2586,6 +2590,7 @@ struct Apply2Params {
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(S2_THREADS, 1)
     k_tc_apply2(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                 const Apply2Params p) {
+  follow();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S2_STAGES * S2_STAGE);
@@ -3363,7 +3368,7 @@ int crt_launch(cdl_ctx* ctx, const CUtensorMap& ma, const CUtensorMap& mb, const
     attr = true;
   }
   Launch L(ctx, kc, work);
-  k_tc_crt<NCH><<<2 * clusters, S2_THREADS, S2_SMEM_BYTES, ctx->stream>>>(ma, mb, p);
+  launch_next(k_tc_crt<NCH>, 2 * clusters, S2_THREADS, S2_SMEM_BYTES, ctx->stream, ma, mb, p);
   return L.done();
 }
 }  // namespace
@@ -3639,8 +3644,7 @@ int fp8t_quantize_level0(cdl_ctx* ctx, cdl_chain* ch) {
   const int np = (int)ch->npad;
   const int nt = np / 128;
   Launch L(ctx, CDL_KC_CHAIN_INIT, 3.0 * np * (double)np);
-  k_quant_fp8_tiles<<<nt * nt, 256, 0, ctx->stream>>>(static_cast<const __nv_bfloat16*>(ch->level16(0)), np,
-                                                      static_cast<uint8_t*>(ch->level(0)), ch->tscale, ch->tatoms);
+  k_quant_fp8_tiles<<<nt * nt, 256, 0, ctx->stream>>>(static_cast<const __nv_bfloat16*>(ch->level16(0)), np, static_cast<uint8_t*>(ch->level(0)), ch->tscale, ch->tatoms);
   return L.done();
 }
 
@@ -3680,7 +3684,7 @@ int resid_tc(cdl_ctx* ctx, const cdl_chain* ch, const void* zslices, int kp, dou
   }
   const int grid = std::min(p.num_tiles * p.npairs, ctx->sm_count);
   Launch L(ctx, CDL_KC_RESIDUAL, 2.0 * p.npairs * (double)np * np * kp);
-  k_tc_resid<<<grid, T8_THREADS, RS_SMEM_BYTES, ctx->stream>>>(maps, p);
+  launch_next(k_tc_resid, grid, T8_THREADS, RS_SMEM_BYTES, ctx->stream, maps, p);
   return L.done();
 }
 
@@ -3757,7 +3761,10 @@ int dist_run(cdl_ctx* ctx, const DistMaps& maps, int tp, DistParams& p, double t
   if (p.num_tiles <= 0) return CDL_OK;
   const int grid = std::min(p.num_tiles, ctx->sm_count);
   Launch L(ctx, CDL_KC_DISTANCE, terms);
-  k_tc_dist<GRP><<<grid, T8_THREADS, DS_SMEM_BYTES, ctx->stream>>>(maps, p);
+  if (GRP)
+    k_tc_dist<GRP><<<grid, T8_THREADS, DS_SMEM_BYTES, ctx->stream>>>(maps, p);
+  else
+    launch_next(k_tc_dist<GRP>, grid, T8_THREADS, DS_SMEM_BYTES, ctx->stream, maps, p);
   return L.done();
 }
 
@@ -3837,8 +3844,7 @@ int gram_launch(cdl_ctx* ctx, const void* u, const void* v, int n, int rows, int
     attr = true;
   }
   Launch L(ctx, kc, work);
-  k_tc_gramr<MODE, NP>
-      <<<std::min(p.num_tiles, ctx->sm_count), T8_THREADS, GR_SMEM_BYTES, ctx->stream>>>(mu, mv, p);
+  launch_next(k_tc_gramr<MODE, NP>, std::min(p.num_tiles, ctx->sm_count), T8_THREADS, GR_SMEM_BYTES, ctx->stream, mu, mv, p);
   return L.done();
 }
 }  // namespace
@@ -3939,7 +3945,7 @@ int resid_tc_panel(cdl_ctx* ctx, const void* slicesT, int np, int Pw, int Pk, in
   }
   const int grid = std::min(p.num_tiles * p.npairs, ctx->sm_count);
   Launch L(ctx, CDL_KC_RESIDUAL, 2.0 * p.npairs * (double)np * Pk * kp);
-  k_tc_resid<<<grid, T8_THREADS, RS_SMEM_BYTES, ctx->stream>>>(maps, p);
+  launch_next(k_tc_resid, grid, T8_THREADS, RS_SMEM_BYTES, ctx->stream, maps, p);
   return L.done();
 }
 
@@ -4056,7 +4062,7 @@ int apply_tc_mat(cdl_ctx* ctx, const void* amat, int np, const void* xop, float*
     p.out = partial;
     p.status = ctx->dev_status;
     Launch L(ctx, CDL_KC_APPLY, 2.0 * np * (double)np);
-    k_tc_apply2<<<2 * sp.clusters, S2_THREADS, S2_SMEM_BYTES, ctx->stream>>>(ma, mbm, p);
+    launch_next(k_tc_apply2, 2 * sp.clusters, S2_THREADS, S2_SMEM_BYTES, ctx->stream, ma, mbm, p);
     return L.done();
   }
   const int splits = sp.slots;
