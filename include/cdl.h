@@ -262,8 +262,9 @@ int cdl_graph_add_edges(cdl_ctx* ctx, void* A, cdl_dtype a_dtype, int64_t n, int
  * chains (bf16, e4m3) also keep A as two bf16 matrices (A_hi + A_lo,
  * 4 npad^2 bytes), the operand of the solve's tensor-core residual update,
  * and A / 2^q as six exact bf16 slices (12 npad^2 bytes; 2^q, q >= 0, the
- * least power of two not below max A, found by one pass over A), the operand
- * of its full residual.
+ * least power of two not below max A: 0 for weights up to 1, else found while
+ * level 0 is formed and the slices formed again), the operand of its full
+ * residual.
  * CDL_CHAIN_HOST_LEVELS (bf16 chains): the levels live in pinned host memory
  * (d * npad^2 * 2 bytes, allocated by the library) and two device slots of
  * npad^2 bf16 hold the ones in use: each squaring writes level i + 1 to a
@@ -325,8 +326,8 @@ int cdl_chain_level_scale(const cdl_chain* chain, int32_t i, double* scale);
  * (a component in the null space of L that no solve could match).
  * A: device n x n (a_dtype = CDL_F64), weights finite, non-negative and
  * below 2^200 (any graph, not only kernel graphs: the terms are split on
- * grids scaled to sqrt(max A), found by one pass over A). Y: device n x k
- * float64 output. Requires 1 <= k <= 1024. */
+ * grids scaled, for every chunk of a row, to the square root of its largest
+ * weight). Y: device n x k float64 output. Requires 1 <= k <= 1024. */
 int cdl_project(cdl_ctx* ctx, const void* A, cdl_dtype a_dtype, int64_t n, int32_t k,
                 uint64_t seed, double* Y);
 
@@ -338,8 +339,8 @@ typedef struct {
                          exactly max_iter applications                       */
   int32_t flags;      /* CDL_SOLVE_* bits                                    */
 } cdl_solve_opts;
-/* Form the float-float residual after every application (default: after the
- * first one, then update it recursively, R -= L dZ, in float32). */
+/* Form the full residual after every application (default on tensor-core
+ * chains: after the first one, then update it recursively, R -= L dZ). */
 enum { CDL_SOLVE_FULL_RESIDUAL = 1 };
 
 typedef struct {
@@ -361,13 +362,17 @@ typedef struct {
  * per column, each as six signed base-256 digits on the grids 2^-8s; every
  * slice product and every 256-term chunk sum is exact in float32; chunk sums
  * are added as integers and scaled into float64), leaving about 2^-50 of
- * |A||Z|; for CUDA-core chains in float-float arithmetic (about 48
- * significant bits). Later steps update it recursively, R -= D dZ - A dZ,
- * with A dZ in float32 (error about 1e-7 of ||L dZ||, i.e. of the previous
- * residual). A bound on the accumulated error of these updates is kept; when
- * the stopping test passes with that bound above rel_tol / 10, the residual
- * is formed in float-float again before stopping. flags =
- * CDL_SOLVE_FULL_RESIDUAL forms it in float-float after every application.
+ * |A||Z|; for CUDA-core chains A Z through integer residues on the tensor
+ * cores (rows of A and columns of Z to 2^-60 of their norms), after every
+ * application. Tensor-core chains update it recursively in later steps,
+ * R -= D dZ - A dZ, with A dZ in bf16 hi + lo products (error about 1e-7 of
+ * ||L dZ||, i.e. of the previous residual). A bound on the accumulated error
+ * of these updates is kept; when the stopping test passes with that bound
+ * above rel_tol / 10, the residual is formed in full again before stopping.
+ * flags = CDL_SOLVE_FULL_RESIDUAL forms it in full after every application.
+ * Where the workspace limit leaves no room for the residue planes, CUDA-core
+ * chains take the float-float form (about 48 significant bits) with float32
+ * recursive updates.
  * Synchronises once per application to read the residual norm.
  * chain: from cdl_chain_build on the same graph. A: device n x n (CDL_F64).
  * Y: device n x k float64. Z: device n x k float64 output; 1 <= k <= 1024.

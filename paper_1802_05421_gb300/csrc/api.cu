@@ -213,7 +213,7 @@ int chain_create_regen(cdl_ctx* ctx, int64_t n, int d, int resident, cdl_chain**
     return CDL_ERR_OOM;
   }
   // Gaussian-kernel graphs: A <= 1, so the exact slices are taken of A itself
-  // (a_scale[0] = 1) and 1 bounds max A (a_scale[1], the projection's grids)
+  // (a_scale[0] = 1)
   if (cudaMemcpy(ch->a_scale, &one, sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(ch->a_scale + 1, &one, sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess) {
     cdl_chain_free(ch);

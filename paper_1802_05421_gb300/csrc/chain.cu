@@ -175,8 +175,8 @@ __device__ __forceinline__ long long grid48(double a, int s) {
 // A as two bf16 matrices A_hi + A_lo (the operand of the solve's recursive
 // residual update); and A / 2^s as six exact bf16 digit planes (N of grid48
 // split into signed base-256 digits d_t, plane t holding d_t 2^-8t), the
-// operand of its full residual; all in one pass over A; padding rows
-// and columns zero. Conversions avoid the float64 pipe (the scarce one): the
+// operand of its full residual (s = 0; k_a_slices forms them again where a weight
+// is above 1); all in one pass over A; padding rows and columns zero. Conversions avoid the float64 pipe (the scarce one): the
 // float of A_ij rounded to nearest by integer operations, the digits bottom-up
 // (balanced base 256 on two 24-bit halves of N = A_ij 2^(48-s)) and their bf16
 // bit patterns by exact float32 arithmetic (digits6_fbits).

@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(256) k_crt_combine(const uint8_t* __restrict__
   for (int e = threadIdx.x; e < 64 * 64; e += 256) C[(size_t)(c0 + e / 64) * np + r0 + e % 64] = tile[e / 64][e % 64];
 }
 
-// Node series for the residue distances (k_tc_distr): row i less the series of
+// Node series for the residue distances (k_tc_gramr): row i less the series of
 // node 0 (distances do not change, and the common part of all nodes costs no
 // bits), scaled by the power of two 2^{e_i} that brings its 2-norm to 2^60.96
 // at most and keeps both series below 2^61, rounded to integers (each entry

@@ -12,10 +12,12 @@
 // Residual. The first step forms R = Y - D Z + A Z in full, to float64-class
 // accuracy: on tensor-core chains A Z comes from exact bf16 slices of A and
 // Z on the tensor cores with integer accumulation (k_tc_resid), on the
-// CUDA-core chains from float-float products and sums on the float32 pipes
-// (float64 runs at about 1/72 of the float32 rate on this GPU). Later steps
-// update it recursively, R -= D dZ - A dZ, on the tensor cores (bf16 hi + lo
-// operands) or in float32; each such update adds a bounded error (1e-5 of
+// CUDA-core chains from integer residues of A's rows and Z's columns on the
+// tensor cores (crt.cu), in full on every step; where the workspace limit leaves
+// no room for the residues, from float-float products and sums on the float32
+// pipes (float64 runs at about 1/72 of the float32 rate on this GPU). Later steps
+// of the other forms update it recursively, R -= D dZ - A dZ, on the tensor cores
+// (bf16 hi + lo operands) or in float32; each such update adds a bounded error (1e-5 of
 // the residual before it), summed as a drift bound. A recursive residual
 // that stops falling (less than halved) is formed again in full, and one
 // that meets the tolerance is certified by a full residual before the solve
