@@ -291,7 +291,7 @@ int build_plan(cdl_ctx* ctx, int G, const int64_t* n, int T, const cdl_batch_opt
       const size_t nk = (size_t)nn * k;
       BGraph& B = gs[g];
       cdl_chain& ch = P->chains[g];
-      ggs[g].Xt = c.take<int>((size_t)nn * T);
+      ggs[g].Xt = tc_dist[g] ? nullptr : c.take<int>((size_t)nn * T);
       P->A[g] = c.take<double>((size_t)nn * nn);
       P->Dv[g] = c.take<double>(np);
       P->scal[g] = c.take<double>(2);   // vol, sigma

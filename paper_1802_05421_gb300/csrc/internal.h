@@ -420,7 +420,7 @@ struct BTiles {
 // Graph build of one graph of a batch (device pointers).
 struct GGraph {
   const double* X;  // n x T
-  int* Xt;          // T x n fixed-point copy (planes null)
+  int* Xt;          // T x n fixed-point copy, where planes is null
   void* planes;     // 3 x npad x tp digit planes (bf16) for the tensor-core distances, or null
   long long* norms; // npad
   double* A;        // n x n
