@@ -68,10 +68,11 @@ __device__ __forceinline__ double f2d_bits(float f) {
 // and lo the remaining 29 mantissa bits rounded to 24 (|x - hi - lo| <=
 // 2^-48 x; below 2^-74, where lo falls under the float normal range, lo is
 // subnormal and the bound is 2^-149 absolute), by integer operations and two
-// exact scalings. Values below 2^-100 give {0, 0}.
+// exact scalings. Values below 2^-100 give {0, 0}, and so does -0.0 (the sign is
+// shifted out).
 __device__ __forceinline__ ff split_nonneg(double x) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  if ((uint32_t)(b >> 52) < 1023 - 100) return {0.f, 0.f};
+  if ((uint32_t)(b >> 32) << 1 < (1023u - 100u) << 21) return {0.f, 0.f};
   const uint32_t hi_bits = (uint32_t)(b >> 29) - ((1023u - 127u) << 23);   // x in [2^e, 2^(e+1)), e >= -100
   // lo = low29 2^(e - 52) = (low29 2^-52) 2^e: both factors are normal floats
   // for e >= -100 (2^(e - 52) itself is not, below e = -74)
