@@ -363,8 +363,8 @@ typedef struct {
  * slice product and every 256-term chunk sum is exact in float32; chunk sums
  * are added as integers and scaled into float64), leaving about 2^-50 of
  * |A||Z|; for CUDA-core chains A Z through integer residues on the tensor
- * cores (rows of A and columns of Z to 2^-60 of their norms), after every
- * application. Tensor-core chains update it recursively in later steps,
+ * cores (rows of A D^{-1/2} and columns of D^{1/2} Z, the roots as powers of
+ * two, to 2^-60 of their norms), after every application. Tensor-core chains update it recursively in later steps,
  * R -= D dZ - A dZ, with A dZ in bf16 hi + lo products (error about 1e-7 of
  * ||L dZ||, i.e. of the previous residual). A bound on the accumulated error
  * of these updates is kept; when the stopping test passes with that bound

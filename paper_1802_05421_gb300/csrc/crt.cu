@@ -139,33 +139,47 @@ __device__ __forceinline__ uint32_t residue_bits(const float (&d)[ND], int l) {
   return __float_as_uint(__fmaf_rn(-q, c_res.mod[l], r));
 }
 
+// The power of two next to sqrt(d) as its exponent (0 for zero and non-finite d)
+__device__ __forceinline__ int sqrt_exponent(double d) {
+  const int e = (int)(LevelType<double>::mag(d) >> 52);
+  return e == 0 || e == 0x7FF ? 0 : (e - 1023) >> 1;
+}
+
 // One block per row of a rows x cols matrix (zero beyond, to gridDim.x x np):
-// the row's largest magnitude, then its 2-norm relative to it (float32, a
+// the row's largest exponent, then its 2-norm relative to it (float32, a
 // margin covers its rounding), e_i, and the residues. Columns in pairs; np a
-// multiple of 64.
-template <typename T>
+// multiple of 64. W: column j is first scaled by the power of two next to
+// w_j^{-1/2}.
+template <typename T, bool W = false>
 __global__ void __launch_bounds__(256) k_crt_residues(const T* __restrict__ X, int rows, int cols, int ldx, int np,
-                                                       int* __restrict__ ex, uint32_t* __restrict__ planes) {
+                                                       const double* __restrict__ w, int* __restrict__ ex,
+                                                       uint32_t* __restrict__ planes) {
   follow();
   typedef LevelType<T> LT;
-  __shared__ unsigned long long wmax[8];
+  constexpr unsigned BIG = ~0u;                           // key of a non-finite entry
+  constexpr int OFF = 4096;                               // keys of the others: exponent + OFF; of zeros: 0
+  __shared__ unsigned wmax[8];
   __shared__ float wsum[8];
   const int row = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const T* x = X + (size_t)row * ldx;
   if (row >= rows) cols = 0;
-  unsigned long long mx = 0;
-  for (int j = tid; j < cols; j += 256) mx = max(mx, LT::mag(x[j]));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  auto shift = [&](int j) { return W ? sqrt_exponent(w[j]) : 0; };
+  unsigned mx = 0;
+  for (int j = tid; j < cols; j += 256) {
+    const unsigned long long m = LT::mag(x[j]);
+    mx = max(mx, m == 0 ? 0u : LT::finite(m) ? (unsigned)(LT::exponent(m) - shift(j) + OFF) : BIG);
+  }
+  mx = __reduce_max_sync(0xffffffffu, mx);
   if (lane == 0) wmax[warp] = mx;
   __syncthreads();
 #pragma unroll
-  for (int w = 0; w < 8; ++w) mx = max(mx, wmax[w]);
+  for (int q = 0; q < 8; ++q) mx = max(mx, wmax[q]);
+  const bool fin = mx != BIG;
   // |x| 2^-emax in [0, 2): emax = exponent of the largest
-  const int emax = LT::exponent(mx) - LT::BIAS + (sizeof(T) == 8 ? 52 : 23);
+  const int emax = fin ? (int)mx - OFF - LT::BIAS + (sizeof(T) == 8 ? 52 : 23) : 0;
   float s = 0.f;
   for (int j = tid; j < cols; j += 256) {
-    const float v = (float)(int)scaled_int(x[j], 22 - emax);   // magnitude up to 2^23, exact in float32
+    const float v = (float)(int)scaled_int(x[j], 22 - emax - shift(j));   // magnitude up to 2^23, exact in float32
     s = __fmaf_rn(v, v, s);
   }
 #pragma unroll
@@ -174,9 +188,8 @@ __global__ void __launch_bounds__(256) k_crt_residues(const T* __restrict__ X, i
   __syncthreads();
   s = 0.f;
 #pragma unroll
-  for (int w = 0; w < 8; ++w) s += wsum[w];
+  for (int q = 0; q < 8; ++q) s += wsum[q];
   // norm 2^(e + 22 - emax) = sqrt(s); rounding and truncation within the 0.02 bits of margin
-  const bool fin = LT::finite(mx);
   // (s < 1: zero, or so far below the smallest normal number that every square underflows)
   const int e = s >= 1.f ? (int)floorf(crt_norm_bits(LT::NP) - 0.02f - 0.5f * log2f(s)) + 22 - emax : 0;
   if (tid == 0) ex[row] = fin ? e : CRT_ROW_NAN;
@@ -186,7 +199,8 @@ __global__ void __launch_bounds__(256) k_crt_residues(const T* __restrict__ X, i
     constexpr int ND = sizeof(T) == 8 ? 4 : 2;
     float d[2][ND];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) digits16<ND>(fin && 2 * j + h < cols ? scaled_int(x[2 * j + h], e) : 0, d[h]);
+    for (int h = 0; h < 2; ++h)
+      digits16<ND>(fin && 2 * j + h < cols ? scaled_int(x[2 * j + h], e - shift(2 * j + h)) : 0, d[h]);
 #pragma unroll
     for (int l = 0; l < LT::NP; ++l)
       out[l * plane + j] = __byte_perm(residue_bits<ND>(d[0], l), residue_bits<ND>(d[1], l), 0x7632);
@@ -498,14 +512,20 @@ __global__ void __launch_bounds__(128) k_score_residues(const double* __restrict
 }
 
 // X (rows x cols, leading dimension ldx) transposed to out (gridDim.y 32 rows x
-// np), zero beyond; 32 x 32 tiles.
+// np), zero beyond; 32 x 32 tiles. With w (may be null) row i is scaled by the
+// power of two next to w_i^{1/2} (exactly).
 __global__ void __launch_bounds__(256) k_transpose_pad(const double* __restrict__ X, int rows, int cols, int ldx,
-                                                        int np, double* __restrict__ out) {
+                                                        int np, const double* __restrict__ w,
+                                                        double* __restrict__ out) {
   follow();
   __shared__ double tile[32][33];
   const int i0 = blockIdx.x * 32, c0 = blockIdx.y * 32, tx = threadIdx.x & 31;
-  for (int a = threadIdx.x >> 5; a < 32; a += 8)
-    tile[a][tx] = (i0 + a < rows && c0 + tx < cols) ? X[(size_t)(i0 + a) * ldx + c0 + tx] : 0.0;
+  for (int a = threadIdx.x >> 5; a < 32; a += 8) {
+    const int i = i0 + a;
+    double v = (i < rows && c0 + tx < cols) ? X[(size_t)i * ldx + c0 + tx] : 0.0;
+    if (w && i < rows) v *= __longlong_as_double((long long)(1023 + sqrt_exponent(w[i])) << 52);
+    tile[a][tx] = v;
+  }
   __syncthreads();
   for (int a = threadIdx.x >> 5; a < 32; a += 8) out[(size_t)(c0 + a) * np + i0 + tx] = tile[tx][a];
 }
@@ -578,8 +598,8 @@ int square_impl(cdl_ctx* ctx, cdl_chain* ch, int level, void* planes, uint8_t* t
   const int np = (int)ch->npad;
   {
     Launch L(ctx, CDL_KC_SQUARE, 0);
-    launch_next(k_crt_residues<T>, np, 256, 0, ctx->stream, static_cast<const T*>(ch->level(level)), np, np, np, np, ex,
-                                                   static_cast<uint32_t*>(planes));
+    launch_next(k_crt_residues<T>, np, 256, 0, ctx->stream, static_cast<const T*>(ch->level(level)), np, np, np, np,
+                nullptr, ex, static_cast<uint32_t*>(planes));
     CDL_TRY(L.done());
   }
   CDL_TRY(crt_gemm(ctx, planes, np, nullptr, 0, np, NP, t, CDL_KC_SQUARE, (double)ch->n * ch->n * (ch->n + 1.0)));
@@ -615,7 +635,12 @@ int chain_square_crt(cdl_ctx* ctx, cdl_chain* ch, int level) {
 // M x for a float64 matrix M (a chain level, or the graph in the residual) and
 // k right-hand sides, through 16 residues as the squaring: the rows of M and
 // the columns of x are scaled by their 2-norms, the product is exact, one
-// rounding per entry. The float64 pipe's dot products took 0.52 ms per level
+// rounding per entry. With weights w (the residual's degrees D) it is formed as
+// (M w^{-1/2}) (w^{1/2} x), the roots as powers of two, so exactly the same: A
+// D^{-1/2} and D^{1/2} Z have entries of one size also where degrees span many
+// orders of magnitude (Z is about D^{-1/2}), and no bits go to a few huge entries
+// of Z. Without, one node of degree 5e-18 of the others' left a relative residual of
+// 3e-12 that no further step made smaller (n = 600, float64 chain). The float64 pipe's dot products took 0.52 ms per level
 // at n = 2000, k = 32 (its FMA rate); here the residues of M take most of the
 // time (8 n^2 bytes read, 32 n^2 written).
 int crt_apply_begin(cdl_ctx* ctx, int np, int k, CrtApply* a) {
@@ -641,22 +666,26 @@ int crt_apply_begin(cdl_ctx* ctx, int np, int k, CrtApply* a) {
   return CDL_OK;
 }
 
-int crt_apply_matrix(cdl_ctx* ctx, const CrtApply& a, const double* M, int n, int kc) {
+int crt_apply_matrix(cdl_ctx* ctx, const CrtApply& a, const double* M, int n, const double* w, int kc) {
   Launch L(ctx, kc, 0);
-  launch_next(k_crt_residues<double>, a.np, 256, 0, ctx->stream, M, n, n, n, a.np, a.erow, a.planes);
+  if (w)
+    launch_next(k_crt_residues<double, true>, a.np, 256, 0, ctx->stream, M, n, n, n, a.np, w, a.erow, a.planes);
+  else
+    launch_next(k_crt_residues<double>, a.np, 256, 0, ctx->stream, M, n, n, n, a.np, nullptr, a.erow, a.planes);
   return L.done();
 }
 
-int crt_apply_product(cdl_ctx* ctx, const CrtApply& a, const double* x, int rows, int cols, int ldx, int kc,
-                      double work) {
+int crt_apply_product(cdl_ctx* ctx, const CrtApply& a, const double* x, int rows, int cols, int ldx, const double* w,
+                      int kc, double work) {
   {
     Launch L(ctx, CDL_KC_MISC, 0);
-    launch_next(k_transpose_pad, dim3(a.np / 32, a.kpb / 32), 256, 0, ctx->stream, x, rows, cols, ldx, a.np, a.xt);
+    launch_next(k_transpose_pad, dim3(a.np / 32, a.kpb / 32), 256, 0, ctx->stream, x, rows, cols, ldx, a.np, w, a.xt);
     CDL_TRY(L.done());
   }
   {
     Launch L(ctx, CDL_KC_MISC, 0);
-    launch_next(k_crt_residues<double>, a.kpb, 256, 0, ctx->stream, a.xt, a.kpb, a.np, a.np, a.np, a.ecol, a.xplanes);
+    launch_next(k_crt_residues<double>, a.kpb, 256, 0, ctx->stream, a.xt, a.kpb, a.np, a.np, a.np, nullptr, a.ecol,
+                a.xplanes);
     CDL_TRY(L.done());
   }
   return crt_gemm(ctx, a.planes, a.np, a.xplanes, a.kpb, a.np, 16, a.t, kc, work);

@@ -228,7 +228,8 @@ int chain_square_crt(cdl_ctx* ctx, cdl_chain* ch, int level);
 // other ws_get of the operation, which could reclaim it; CDL_ERR_UNSUPPORTED
 // where it is not to be had), matrix forms the residues of M (kept until the
 // next matrix call on the context), product those of x (rows x cols) and of
-// M x; add and residual put M x together: x += M x (x np x kp), R = Y - D o Z
+// M x, both with the same weights w (device, n; may be null: see the
+// definition); add and residual put M x together: x += M x (x np x kp), R = Y - D o Z
 // + M Z with `nblocks` partial sums of R^2.
 struct CrtApply {
   int np = 0, kpb = 0;
@@ -238,9 +239,9 @@ struct CrtApply {
   int *erow = nullptr, *ecol = nullptr;
 };
 int crt_apply_begin(cdl_ctx* ctx, int np, int k, CrtApply* a);
-int crt_apply_matrix(cdl_ctx* ctx, const CrtApply& a, const double* M, int n, int kc);
-int crt_apply_product(cdl_ctx* ctx, const CrtApply& a, const double* x, int rows, int cols, int ldx, int kc,
-                      double work);
+int crt_apply_matrix(cdl_ctx* ctx, const CrtApply& a, const double* M, int n, const double* w, int kc);
+int crt_apply_product(cdl_ctx* ctx, const CrtApply& a, const double* x, int rows, int cols, int ldx, const double* w,
+                      int kc, double work);
 int crt_apply_add(cdl_ctx* ctx, const CrtApply& a, double* x, int kp);
 int crt_apply_residual(cdl_ctx* ctx, const CrtApply& a, const double* Y, const double* Z, const double* D, int n, int k,
                        double* R, double* part, int nblocks);

@@ -1089,9 +1089,9 @@ struct SolveBlock {
     }
     if (crt) {
       // the level products of a float64 chain use the same residue planes
-      if (!a_ready || ch->dtype == CDL_F64) CDL_TRY(crt_apply_matrix(ctx, ca, A, n, CDL_KC_RESIDUAL));
+      if (!a_ready || ch->dtype == CDL_F64) CDL_TRY(crt_apply_matrix(ctx, ca, A, n, ch->D, CDL_KC_RESIDUAL));
       a_ready = true;
-      CDL_TRY(crt_apply_product(ctx, ca, Z, n, k, k, CDL_KC_RESIDUAL, (double)n * n * k));
+      CDL_TRY(crt_apply_product(ctx, ca, Z, n, k, k, ch->D, CDL_KC_RESIDUAL, (double)n * n * k));
       nparts = std::min(1024, (int)blocks_for((size_t)n * ((k + 3) / 4), 128));
       return crt_apply_residual(ctx, ca, Y, Z, ch->D, n, k, R, red, nparts);
     }
@@ -1211,8 +1211,9 @@ struct SolveBlock {
     }
     if (crt && ch->dtype == CDL_F64) {
       double* x = static_cast<double*>(vx);
-      CDL_TRY(crt_apply_matrix(ctx, ca, static_cast<const double*>(ch->level(lvl)), np, CDL_KC_APPLY));
-      CDL_TRY(crt_apply_product(ctx, ca, x, np, kp, kp, CDL_KC_APPLY, 8.0 * np * (double)np));
+      CDL_TRY(crt_apply_matrix(ctx, ca, static_cast<const double*>(ch->level(lvl)), np, nullptr,
+                               CDL_KC_APPLY));
+      CDL_TRY(crt_apply_product(ctx, ca, x, np, kp, kp, nullptr, CDL_KC_APPLY, 8.0 * np * (double)np));
       return crt_apply_add(ctx, ca, x, kp);
     }
     CDL_TRY(apply_simt(ctx, ch, lvl, vx, vpart, kp, splits));
