@@ -388,41 +388,86 @@ __device__ __forceinline__ void score_ab(const double* __restrict__ Z1, const do
   b = w + v;
 }
 
-// Largest |a| and |b| (exponents of their float64 bit patterns): mx[0], mx[1].
+// What g is chosen from (zeroed before): the largest |a| and |b| as exponent
+// fields, and over the rows' largest |a| and |b| the sums of the exponents and
+// the rows that have one. A warp per row, one set of global atomics per block
+// (per warp they took 20 us at n = 8192).
+struct ScoreScale {
+  int amax, bmax;
+  int gexp;               // log2 g, left by k_score_residues
+  int asum, acnt, bsum, bcnt;
+  int pad;
+};
+
 __global__ void __launch_bounds__(256) k_score_maxima(const double* __restrict__ Z1, const double* __restrict__ Z2,
                                                        const double* __restrict__ vol1,
-                                                       const double* __restrict__ vol2, size_t cnt,
-                                                       int* __restrict__ mx) {
+                                                       const double* __restrict__ vol2, int n, int k,
+                                                       ScoreScale* __restrict__ sc) {
   follow();
+  __shared__ ScoreScale bl;
   const double s1 = sqrt(*vol1), s2 = sqrt(*vol2);
-  int ea = 0, eb = 0;
-  for (size_t o = blockIdx.x * (size_t)256 + threadIdx.x; o < cnt; o += (size_t)gridDim.x * 256) {
-    double a, b;
-    score_ab(Z1, Z2, s1, s2, o, a, b);
-    ea = max(ea, (int)(LevelType<double>::mag(a) >> 52));
-    eb = max(eb, (int)(LevelType<double>::mag(b) >> 52));
+  const int lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) bl = ScoreScale{};
+  __syncthreads();
+  int ma = 0, mb = 0, asum = 0, acnt = 0, bsum = 0, bcnt = 0;
+  for (int i = blockIdx.x * 8 + (threadIdx.x >> 5); i < n; i += gridDim.x * 8) {
+    int ea = 0, eb = 0;
+    for (int r = lane; r < k; r += 32) {
+      double a, b;
+      score_ab(Z1, Z2, s1, s2, (size_t)i * k + r, a, b);
+      ea = max(ea, (int)(LevelType<double>::mag(a) >> 52));
+      eb = max(eb, (int)(LevelType<double>::mag(b) >> 52));
+    }
+    ea = __reduce_max_sync(0xffffffffu, ea);
+    eb = __reduce_max_sync(0xffffffffu, eb);
+    ma = max(ma, ea);
+    mb = max(mb, eb);
+    if (ea > 0 && ea < 0x7FF) {
+      asum += ea - 1023;
+      ++acnt;
+    }
+    if (eb > 0 && eb < 0x7FF) {
+      bsum += eb - 1023;
+      ++bcnt;
+    }
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    ea = max(ea, __shfl_xor_sync(0xffffffffu, ea, o));
-    eb = max(eb, __shfl_xor_sync(0xffffffffu, eb, o));
-  }
-  if ((threadIdx.x & 31) == 0) {
-    atomicMax(mx, ea);
-    atomicMax(mx + 1, eb);
-  }
+  auto add = [](ScoreScale* t, int a, int b, int as, int ac, int bs, int bc) {
+    atomicMax(&t->amax, a);
+    atomicMax(&t->bmax, b);
+    atomicAdd(&t->asum, as);
+    atomicAdd(&t->acnt, ac);
+    atomicAdd(&t->bsum, bs);
+    atomicAdd(&t->bcnt, bc);
+  };
+  if (lane == 0) add(&bl, ma, mb, asum, acnt, bsum, bcnt);
+  __syncthreads();
+  if (threadIdx.x == 0) add(sc, bl.amax, bl.bmax, bl.asum, bl.acnt, bl.bsum, bl.bcnt);
+}
+
+// log2 g: g brings the largest |a| to the binade of the largest |b|, or of three
+// binades above the rows' mean exponent of |b| where that is less (g > 1; for g <
+// 1 the halves change places): a few rows far above the others (nodes of tiny
+// degree) must not scale the other rows' a up until their b has no bits left. With
+// g = 1 every row keeps both halves to 2^-B of its own size, which is within the
+// rounding of a and b themselves. One node of 200 with |Z| 1e9 times the others',
+// equal volumes, float64 scores: 5e-10 relative by the largest alone, 8e-16 so.
+__device__ __forceinline__ int score_gexp(const ScoreScale& s) {
+  auto mean = [](int sum, int cnt) { return cnt > 0 ? sum / cnt + (sum % cnt > 0) : 0; };   // rounded up
+  const int ea = s.amax, eb = s.bmax;
+  if (ea == 0 || eb == 0 || ea >= 0x7FF || eb >= 0x7FF) return 0;   // zero or non-finite maxima: no balancing
+  if (eb > ea) return min(eb - ea, max(0, mean(s.bsum, s.bcnt) + 3 - (ea - 1023)));
+  return max(eb - ea, min(0, (eb - 1023) - mean(s.asum, s.acnt) - 3));
 }
 
 // Row i: u_i = [g a_i | b_i] of 2-norm 2^B at most (B = crt_norm_bits) after the
 // power of two 2^{e_i}, rounded to integers, as NP residue planes of u and of v
 // = [b_i | g a_i] (rows x kp, zero padded), and d'_i = (g a_i) . b_i of the
-// integers, exact. g = 2^gexp brings the largest |a| to the binade of the
-// largest |b| (gexp = mx[1] - mx[0] is left in mx[2]). A block of 128 per row.
+// integers, exact; g from score_gexp. A block of 128 per row.
 template <int NP>
 __global__ void __launch_bounds__(128) k_score_residues(const double* __restrict__ Z1, const double* __restrict__ Z2,
                                                          const double* __restrict__ vol1,
                                                          const double* __restrict__ vol2, int n, int k, int rows,
-                                                         int kp, int* __restrict__ mx, int* __restrict__ ex,
+                                                         int kp, ScoreScale* __restrict__ sc, int* __restrict__ ex,
                                                          ulonglong2* __restrict__ dself,
                                                          __nv_bfloat16* __restrict__ up,
                                                          __nv_bfloat16* __restrict__ vp) {
@@ -433,9 +478,8 @@ __global__ void __launch_bounds__(128) k_score_residues(const double* __restrict
   __shared__ ulonglong2 wn[4];
   const int row = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const double s1 = sqrt(*vol1), s2 = sqrt(*vol2);
-  // zero or non-finite maxima: no balancing
-  const int ea = mx[0], eb = mx[1], ge = ea > 0 && eb > 0 && ea < 0x7FF && eb < 0x7FF ? eb - ea : 0;
-  if (row == 0 && tid == 0) mx[2] = ge;
+  const int ge = score_gexp(*sc);
+  if (row == 0 && tid == 0) sc->gexp = ge;
   const int cols = row < n ? k : 0;
   // magnitudes as exponents relative to g: |g a| is compared through the exponent field
   unsigned long long m = 0;
@@ -724,34 +768,30 @@ int score_pairs_residues(cdl_ctx* ctx, const double* Z1, const double* Z2, const
   if (ws_get(ctx, "crt.score.u", cnt * 2, &vu) != CDL_OK || ws_get(ctx, "crt.score.v", cnt * 2, &vv) != CDL_OK ||
       ws_get(ctx, "crt.score.d", (size_t)rows * 16, &vd) != CDL_OK ||
       ws_get(ctx, "crt.score.e", (size_t)rows * sizeof(int), &ve) != CDL_OK ||
-      ws_get(ctx, "crt.score.max", 16, &vm) != CDL_OK) {
+      ws_get(ctx, "crt.score.max", sizeof(ScoreScale), &vm) != CDL_OK) {
     ws_reclaim(ctx);
     return CDL_ERR_UNSUPPORTED;
   }
-  int *mx = static_cast<int*>(vm), *ex = static_cast<int*>(ve);
-  CDL_CUDA_TRY(cudaMemsetAsync(mx, 0, 16, ctx->stream));
+  ScoreScale* sc = static_cast<ScoreScale*>(vm);
+  int* ex = static_cast<int*>(ve);
+  CDL_CUDA_TRY(cudaMemsetAsync(sc, 0, sizeof(ScoreScale), ctx->stream));
   {
     Launch L(ctx, CDL_KC_MISC, 0);
-    const size_t nk = (size_t)n * k;
-    launch_next(k_score_maxima, (unsigned)std::min<size_t>((nk + 255) / 256, (size_t)ctx->sm_count * 8), 256, 0, ctx->stream, 
-        Z1, Z2, vol1, vol2, nk, mx);
+    launch_next(k_score_maxima, std::min((n + 7) / 8, ctx->sm_count * 4), 256, 0, ctx->stream, Z1, Z2, vol1, vol2, n, k,
+                sc);
     CDL_TRY(L.done());
   }
   {
     Launch L(ctx, CDL_KC_MISC, 0);
     if (fp64)
-      launch_next(k_score_residues<16>, rows, 128, 0, ctx->stream, Z1, Z2, vol1, vol2, n, k, rows, kp, mx, ex,
-                                                          static_cast<ulonglong2*>(vd),
-                                                          static_cast<__nv_bfloat16*>(vu),
-                                                          static_cast<__nv_bfloat16*>(vv));
+      launch_next(k_score_residues<16>, rows, 128, 0, ctx->stream, Z1, Z2, vol1, vol2, n, k, rows, kp, sc, ex,
+                  static_cast<ulonglong2*>(vd), static_cast<__nv_bfloat16*>(vu), static_cast<__nv_bfloat16*>(vv));
     else
-      launch_next(k_score_residues<13>, rows, 128, 0, ctx->stream, Z1, Z2, vol1, vol2, n, k, rows, kp, mx, ex,
-                                                          static_cast<ulonglong2*>(vd),
-                                                          static_cast<__nv_bfloat16*>(vu),
-                                                          static_cast<__nv_bfloat16*>(vv));
+      launch_next(k_score_residues<13>, rows, 128, 0, ctx->stream, Z1, Z2, vol1, vol2, n, k, rows, kp, sc, ex,
+                  static_cast<ulonglong2*>(vd), static_cast<__nv_bfloat16*>(vu), static_cast<__nv_bfloat16*>(vv));
     CDL_TRY(L.done());
   }
-  return score_residues_tc(ctx, vu, vv, planes, ex, vd, mx + 2, n, rows, kp, A1, A2, contrib, E,
+  return score_residues_tc(ctx, vu, vv, planes, ex, vd, &sc->gexp, n, rows, kp, A1, A2, contrib, E,
                            8.0 * (double)n * (n - 1));
 }
 
