@@ -555,14 +555,15 @@ __global__ void __launch_bounds__(256) k_edge_maxkey(const double* __restrict__ 
 // State of the cut search. The cut's key lies in [lo, lo + 16 2^sh): 16 bins
 // of 2^sh keys each, next to be summed (sh = 52: a window of binades from the
 // largest key down; sh < 0: found, lo alone); `above` = the sum of all entries
-// with larger keys.
+// with larger keys. The lowest window reaches down to key 0 and may overlap the
+// one before it: keys from `hi` on (a whole binade) are in `above` already.
 struct U128 {
   unsigned long long lo, hi;
 };
 struct EdgeCut {
   unsigned long long kmax;
   U128 total, above;
-  unsigned long long lo;
+  unsigned long long lo, hi;
   unsigned long long cnt;     // entries in the range
   int sh;
   int have_total;
@@ -666,6 +667,7 @@ __global__ void __launch_bounds__(256) k_edge_bins(const double* __restrict__ E,
 __global__ void k_edge_cut_init(EdgeCut* c) {
   const unsigned long long binade = c->kmax >> 52;
   c->lo = binade > 15 ? (binade - 15) << 52 : 0;
+  c->hi = (binade + 1) << 52;
   c->sh = 52;
 }
 
@@ -708,7 +710,7 @@ __global__ void __launch_bounds__(32 * EC_BINS) k_edge_step(const U128* __restri
   }
   const unsigned __int128 total = u128_of(c->total);
   unsigned __int128 above = u128_of(c->above);
-  int d = 15;
+  int d = c->sh == 52 ? (int)((c->hi - c->lo) >> 52) - 1 : 15;
   for (; d >= 0; --d) {
     const unsigned __int128 ge = above + u128_of(bs[d]);
     if (total - ge < need) break;   // taking everything from this bin on suffices
@@ -717,6 +719,7 @@ __global__ void __launch_bounds__(32 * EC_BINS) k_edge_step(const U128* __restri
   c->above = u128_to(above);
   if (d < 0) {                       // below this window of binades (only the first passes)
     const unsigned long long step = 16ull << 52;
+    c->hi = c->lo;
     c->lo = c->lo > step ? c->lo - step : 0;
     return;
   }
