@@ -71,6 +71,14 @@ int ws_get(cdl_ctx* ctx, const char* name, size_t bytes, void** out) {
   return CDL_OK;
 }
 
+int allow_smem_of(cdl_ctx* ctx, const void* kernel, int bytes) {
+  for (const void* k : ctx->smem_kernels)
+    if (k == kernel) return CDL_OK;
+  CDL_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  ctx->smem_kernels.push_back(kernel);
+  return CDL_OK;
+}
+
 static cudaEvent_t take_event(cdl_ctx* ctx) {
   if (!ctx->free_events.empty()) {
     cudaEvent_t e = ctx->free_events.back();

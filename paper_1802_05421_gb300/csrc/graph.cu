@@ -1077,11 +1077,6 @@ void graph_grouped_tiles(const std::vector<int>& n, const std::vector<char>& tc,
   }
 }
 
-static int select_sample_smem(const void* kernel) {
-  CDL_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SampleShared)));
-  return CDL_OK;
-}
-
 int graph_build_grouped(cdl_ctx* ctx, const GraphBatch& B) {
   cudaStream_t s = ctx->stream;
   CDL_CUDA_TRY(cudaMemsetAsync(B.sel_all, 0, B.sel_bytes, s));
@@ -1111,7 +1106,7 @@ int graph_build_grouped(cdl_ctx* ctx, const GraphBatch& B) {
     k_g_set_sigma<<<B.G2, 1, 0, s>>>(B.gs, B.sigma);
     CDL_TRY(L.done());
   } else {
-    CDL_TRY(select_sample_smem(reinterpret_cast<const void*>(k_g_select_sample)));
+    CDL_TRY(allow_smem(ctx, k_g_select_sample, (int)sizeof(SampleShared)));
     {
       Launch L(ctx, CDL_KC_SELECT, 0);
       k_g_select_sample<<<B.G2, SAMPLE_THREADS, sizeof(SampleShared), s>>>(B.gs);
@@ -1209,7 +1204,7 @@ int graph_build(cdl_ctx* ctx, const double* X, int64_t n64, int T, double sigma,
     unsigned long long* sbuf = reinterpret_cast<unsigned long long*>(part);
     const unsigned long long cap = (unsigned long long)nb * n;
     if (m >= SELECT_BRACKET_MIN) {
-      CDL_TRY(select_sample_smem(reinterpret_cast<const void*>(k_select_sample)));
+      CDL_TRY(allow_smem(ctx, k_select_sample, (int)sizeof(SampleShared)));
       {
         // the samples into the buffer first: one block's scattered loads took 25 us
         Launch L(ctx, CDL_KC_SELECT, 0);

@@ -80,6 +80,8 @@ struct cdl_ctx {
   } last_pair;
   // tile schedules uploaded to the workspace, by workspace name -> tile count
   std::map<std::string, int> tile_lists;
+  std::vector<const void*> smem_kernels;   // allow_smem
+  int pair_clusters = -1;                  // CTA pairs that can be resident at once (-1: not asked yet)
   int debug_flags = 0;   // CDL_DEBUG_* test hooks
   cdl::BatchPlan* batch = nullptr;   // plan of the last cdl_caddelag_batched call
 };
@@ -194,6 +196,15 @@ __device__ __forceinline__ void follow() {
 #endif
 }
 #endif
+
+// Lets `kernel` be launched with `bytes` (always the same for one kernel) of dynamic
+// shared memory, above the 48 KB that need no leave. The leave holds for one device,
+// so it is asked for once per context.
+int allow_smem_of(cdl_ctx* ctx, const void* kernel, int bytes);
+template <typename F>
+inline int allow_smem(cdl_ctx* ctx, F* kernel, int bytes) {
+  return allow_smem_of(ctx, reinterpret_cast<const void*>(kernel), bytes);
+}
 
 // Timing of one host-link copy on stream `s` (class CDL_KC_HOST_LINK): events
 // around it when timing is on; counted as a copy, not as a kernel launch.

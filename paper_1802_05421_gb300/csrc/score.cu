@@ -1348,11 +1348,7 @@ int cad_edges(cdl_ctx* ctx, const double* A1, const double* A2, const double* Z1
     k_edge_cut_init<<<1, 1, 0, st>>>(cut);
     CDL_TRY(L.done());
   }
-  static bool attr = false;
-  if (!attr) {
-    CDL_CUDA_TRY(cudaFuncSetAttribute(k_edge_bins, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)EC_SMEM));
-    attr = true;
-  }
+  CDL_TRY(allow_smem(ctx, k_edge_bins, (int)EC_SMEM));
   auto pass = [&]() -> int {
     {
       Launch L(ctx, CDL_KC_MISC, 0);

@@ -3235,12 +3235,8 @@ int get_tiles(cdl_ctx* ctx, const std::string& name, Builder build, const uint32
 
 int launch(cdl_ctx* ctx, const CUtensorMap& a, const CUtensorMap& b, const TcParams& p, int kc,
            double work, bool fp8 = false) {
-  static bool attr = false;
-  if (!attr) {
-    CDL_CUDA_TRY(cudaFuncSetAttribute(k_tc_gemm<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
-    CDL_CUDA_TRY(cudaFuncSetAttribute(k_tc_gemm<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
-    attr = true;
-  }
+  CDL_TRY(allow_smem(ctx, k_tc_gemm<false>, SMEM_BYTES));
+  CDL_TRY(allow_smem(ctx, k_tc_gemm<true>, SMEM_BYTES));
   const int grid = std::min(p.num_tiles, ctx->sm_count);
   Launch L(ctx, kc, work);
   if (fp8)
@@ -3281,13 +3277,9 @@ uint32_t make_idesc_m256(int n) {
 
 // Clusters of two that can be resident at once (0: cluster launch unavailable).
 int pair_clusters(cdl_ctx* ctx) {
-  static int max_clusters = -1;
-  if (max_clusters < 0) {
-    if (cudaFuncSetAttribute(k_tc_sq2, cudaFuncAttributeMaxDynamicSharedMemorySize, S2_SMEM_BYTES) != cudaSuccess) {
-      cudaGetLastError();
-      max_clusters = 0;
-      return 0;
-    }
+  if (ctx->pair_clusters < 0) {
+    ctx->pair_clusters = 0;
+    if (allow_smem(ctx, k_tc_sq2, S2_SMEM_BYTES) != CDL_OK) return 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * (ctx->sm_count / 2), 1, 1);
     cfg.blockDim = dim3(S2_THREADS, 1, 1);
@@ -3297,9 +3289,9 @@ int pair_clusters(cdl_ctx* ctx) {
       cudaGetLastError();
       mc = 0;
     }
-    max_clusters = std::max(mc, 0);
+    ctx->pair_clusters = std::max(mc, 0);
   }
-  return max_clusters;
+  return ctx->pair_clusters;
 }
 
 // bf16 squaring of a level on CTA pairs (k_tc_sq2)
@@ -3362,11 +3354,7 @@ namespace {
 template <int NCH>
 int crt_launch(cdl_ctx* ctx, const CUtensorMap& ma, const CUtensorMap& mb, const CrtGemmParams& p, int clusters, int kc,
                double work) {
-  static bool attr = false;
-  if (!attr) {
-    CDL_CUDA_TRY(cudaFuncSetAttribute(k_tc_crt<NCH>, cudaFuncAttributeMaxDynamicSharedMemorySize, S2_SMEM_BYTES));
-    attr = true;
-  }
+  CDL_TRY(allow_smem(ctx, k_tc_crt<NCH>, S2_SMEM_BYTES));
   Launch L(ctx, kc, work);
   launch_next(k_tc_crt<NCH>, 2 * clusters, S2_THREADS, S2_SMEM_BYTES, ctx->stream, ma, mb, p);
   return L.done();
@@ -3613,11 +3601,7 @@ int chain_square_fp8t(cdl_ctx* ctx, cdl_chain* ch, int level) {
   CDL_TRY(make_map(&mb, ch->level(level), np, np, 256, 1));
   if (!ch->tatoms) return CDL_ERR_INVALID_ARG;
   {
-    static bool mattr = false;
-    if (!mattr) {
-      CDL_CUDA_TRY(cudaFuncSetAttribute(k_tc_mx8, cudaFuncAttributeMaxDynamicSharedMemorySize, M8_SMEM_BYTES));
-      mattr = true;
-    }
+    CDL_TRY(allow_smem(ctx, k_tc_mx8, M8_SMEM_BYTES));
     const size_t atoms = (size_t)nt * nt * M8_SF;
     Mx8Params p;
     std::memset(&p, 0, sizeof(p));
@@ -3677,11 +3661,7 @@ int resid_tc(cdl_ctx* ctx, const cdl_chain* ch, const void* zslices, int kp, dou
   p.idesc = make_idesc(kp);
   p.status = ctx->dev_status;
   p.assign = 1;   // every element of every plane belongs to one unit: its first flush stores it
-  static bool attr = false;
-  if (!attr) {
-    CDL_CUDA_TRY(cudaFuncSetAttribute(k_tc_resid, cudaFuncAttributeMaxDynamicSharedMemorySize, RS_SMEM_BYTES));
-    attr = true;
-  }
+  CDL_TRY(allow_smem(ctx, k_tc_resid, RS_SMEM_BYTES));
   const int grid = std::min(p.num_tiles * p.npairs, ctx->sm_count);
   Launch L(ctx, CDL_KC_RESIDUAL, 2.0 * p.npairs * (double)np * np * kp);
   launch_next(k_tc_resid, grid, T8_THREADS, RS_SMEM_BYTES, ctx->stream, maps, p);
@@ -3727,11 +3707,7 @@ int resid_tc_grouped(cdl_ctx* ctx, const ResidGroup* dgroups, const uint32_t* un
   p.units = units;
   p.gate_mask = gate_mask;
   p.assign = 1;
-  static bool attr = false;
-  if (!attr) {
-    CDL_CUDA_TRY(cudaFuncSetAttribute(k_tc_resid, cudaFuncAttributeMaxDynamicSharedMemorySize, RS_SMEM_BYTES));
-    attr = true;
-  }
+  CDL_TRY(allow_smem(ctx, k_tc_resid, RS_SMEM_BYTES));
   const int grid = std::min(nunits * p.npairs, ctx->sm_count);
   Launch L(ctx, CDL_KC_RESIDUAL, work);
   k_tc_resid<<<grid, T8_THREADS, RS_SMEM_BYTES, ctx->stream>>>(maps, p);
@@ -3753,11 +3729,7 @@ int dist_run(cdl_ctx* ctx, const DistMaps& maps, int tp, DistParams& p, double t
   p.kblocks = tp / 64;
   for (int w = 0; w < DS_SLICES; ++w) p.idesc[w] = make_idesc((w + 1) * DS_N);
   p.status = ctx->dev_status;
-  static bool attr = false;
-  if (!attr) {
-    CDL_CUDA_TRY(cudaFuncSetAttribute(k_tc_dist<GRP>, cudaFuncAttributeMaxDynamicSharedMemorySize, DS_SMEM_BYTES));
-    attr = true;
-  }
+  CDL_TRY(allow_smem(ctx, k_tc_dist<GRP>, DS_SMEM_BYTES));
   if (p.num_tiles <= 0) return CDL_OK;
   const int grid = std::min(p.num_tiles, ctx->sm_count);
   Launch L(ctx, CDL_KC_DISTANCE, terms);
@@ -3837,12 +3809,7 @@ int gram_launch(cdl_ctx* ctx, const void* u, const void* v, int n, int rows, int
   CUtensorMap mu, mv;
   CDL_TRY(make_map(&mu, u, (int64_t)NP * rows, kp, 128));
   CDL_TRY(make_map(&mv, v, (int64_t)NP * rows, kp, DS_N));
-  static bool attr = false;
-  if (!attr) {
-    CDL_CUDA_TRY(
-        cudaFuncSetAttribute(k_tc_gramr<MODE, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, GR_SMEM_BYTES));
-    attr = true;
-  }
+  CDL_TRY(allow_smem(ctx, k_tc_gramr<MODE, NP>, GR_SMEM_BYTES));
   Launch L(ctx, kc, work);
   launch_next(k_tc_gramr<MODE, NP>, std::min(p.num_tiles, ctx->sm_count), T8_THREADS, GR_SMEM_BYTES, ctx->stream, mu, mv, p);
   return L.done();
@@ -3938,11 +3905,7 @@ int resid_tc_panel(cdl_ctx* ctx, const void* slicesT, int np, int Pw, int Pk, in
   p.gstride = (size_t)np * kp;
   p.idesc = make_idesc(kp);
   p.status = ctx->dev_status;
-  static bool attr = false;
-  if (!attr) {
-    CDL_CUDA_TRY(cudaFuncSetAttribute(k_tc_resid, cudaFuncAttributeMaxDynamicSharedMemorySize, RS_SMEM_BYTES));
-    attr = true;
-  }
+  CDL_TRY(allow_smem(ctx, k_tc_resid, RS_SMEM_BYTES));
   const int grid = std::min(p.num_tiles * p.npairs, ctx->sm_count);
   Launch L(ctx, CDL_KC_RESIDUAL, 2.0 * p.npairs * (double)np * Pk * kp);
   launch_next(k_tc_resid, grid, T8_THREADS, RS_SMEM_BYTES, ctx->stream, maps, p);
@@ -3981,11 +3944,7 @@ int score_tc_tiles(cdl_ctx* ctx, const void* uplanes, const void* vplanes, const
   p.contrib = contrib;
   p.idesc = make_idesc(SC_N);
   p.status = ctx->dev_status;
-  static bool attr = false;
-  if (!attr) {
-    CDL_CUDA_TRY(cudaFuncSetAttribute(k_tc_score, cudaFuncAttributeMaxDynamicSharedMemorySize, SC_SMEM_BYTES));
-    attr = true;
-  }
+  CDL_TRY(allow_smem(ctx, k_tc_score, SC_SMEM_BYTES));
   const int grid = (int)std::min<long long>(tiles, ctx->sm_count);
   // 21 slice products over the computed tiles
   Launch L(ctx, CDL_KC_SCORE, 2.0 * 21 * (double)tiles * 128 * SC_N * k2p);
@@ -4046,11 +4005,7 @@ int apply_tc_mat(cdl_ctx* ctx, const void* amat, int np, const void* xop, float*
   if (bn % 32 || bn < 32 || bn > MAX_BN) return CDL_ERR_UNSUPPORTED;
   const int mb = np / BM;
   if (sp.clusters > 0) {
-    static bool attr = false;
-    if (!attr) {
-      CDL_CUDA_TRY(cudaFuncSetAttribute(k_tc_apply2, cudaFuncAttributeMaxDynamicSharedMemorySize, S2_SMEM_BYTES));
-      attr = true;
-    }
+    CDL_TRY(allow_smem(ctx, k_tc_apply2, S2_SMEM_BYTES));
     CUtensorMap ma, mbm;
     CDL_TRY(make_map(&ma, amat, np, np, 128));
     CDL_TRY(make_map(&mbm, xop, bn, np, bn / 2));
