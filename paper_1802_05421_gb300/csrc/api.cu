@@ -13,9 +13,11 @@ void set_last_error(const char* msg, const char* file, int line) {
   snprintf(g_last_error, sizeof(g_last_error), "%s (%s:%d)", msg, file, line);
 }
 
-// Buffers named crt.* only make a kernel faster (their users have a form
+// Buffers named crt.* and opt.* only make a call faster (their users have a form
 // without them): they are given up before any other request is refused.
-static bool reclaimable(const std::string& name) { return name.compare(0, 4, "crt.") == 0; }
+static bool reclaimable(const std::string& name) {
+  return name.compare(0, 4, "crt.") == 0 || name.compare(0, 4, "opt.") == 0;
+}
 
 bool ws_reclaim(cdl_ctx* ctx) {
   bool any = false;
@@ -69,6 +71,30 @@ int ws_get(cdl_ctx* ctx, const char* name, size_t bytes, void** out) {
   ctx->ws[name] = {p, bytes};
   *out = p;
   return CDL_OK;
+}
+
+int ws_get_opt(cdl_ctx* ctx, std::initializer_list<WsOpt> list) {
+  bool reclaimed = false;
+  if (ctx->ws_cap) {
+    size_t needed = 0, want = 0, grow = 0;   // what calls cannot do without; this request; what it adds to what is held
+    for (const auto& b : ctx->ws)
+      if (!reclaimable(b.first)) needed += b.second.second;
+    for (const WsOpt& o : list) {
+      const auto it = ctx->ws.find(o.name);
+      const size_t old = it == ctx->ws.end() ? 0 : it->second.second;
+      want += o.bytes;
+      grow += o.bytes > old ? o.bytes - old : 0;
+    }
+    if (needed + want > ctx->ws_cap) return CDL_ERR_OOM;
+    if (ctx->ws_used + grow > ctx->ws_cap) reclaimed = ws_reclaim(ctx);
+  }
+  for (int attempt = 0;; ++attempt) {
+    int st = CDL_OK;
+    for (const WsOpt& o : list)
+      if (st == CDL_OK) st = ws_get(ctx, o.name, o.bytes, o.out);
+    if (st == CDL_OK) return CDL_OK;
+    if (!ws_reclaim(ctx) || reclaimed || attempt > 0) return st;   // what was got of the list goes too
+  }
 }
 
 int allow_smem_of(cdl_ctx* ctx, const void* kernel, int bytes) {

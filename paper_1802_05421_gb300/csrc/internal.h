@@ -6,6 +6,7 @@
 #include <cstdint>
 #include <cstdio>
 #include <functional>
+#include <initializer_list>
 #include <map>
 #include <string>
 #include <utility>
@@ -144,10 +145,20 @@ namespace cdl {
 // reusing or growing it (respecting ctx->ws_cap).
 int ws_get(cdl_ctx* ctx, const char* name, size_t bytes, void** out);
 // Frees the buffers of faster forms that a slower one can do without (names
-// crt.*; synchronises the stream); true if there were any. ws_get does so by
+// crt.* and opt.*; synchronises the stream); true if there were any. ws_get does so by
 // itself before it refuses another buffer, and malloc_reclaim is a cudaMalloc
 // that does.
 bool ws_reclaim(cdl_ctx* ctx);
+// All of a list of such buffers, or none (CDL_ERR_OOM). Others of their kind are
+// given up for them, so that under a cap the answer depends on the buffers that
+// calls cannot do without alone, not on what ran before; where it is no, nothing is
+// allocated or freed. Take them after every other buffer of the call.
+struct WsOpt {
+  const char* name;
+  size_t bytes;
+  void** out;
+};
+int ws_get_opt(cdl_ctx* ctx, std::initializer_list<WsOpt> list);
 cudaError_t malloc_reclaim(cdl_ctx* ctx, void** p, size_t bytes);
 
 // Folds src's pending timings and adds its launch counters into dst, then
