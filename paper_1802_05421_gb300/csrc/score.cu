@@ -730,8 +730,8 @@ __global__ void __launch_bounds__(32 * EC_BINS) k_edge_step(const U128* __restri
 
 // The entries of the cut's range, in any order.
 __global__ void __launch_bounds__(256) k_edge_collect(const double* __restrict__ E, int n, EdgeCut* __restrict__ c,
-                                                       unsigned long long* __restrict__ buf) {
-  if (c->sh < 0 || c->sh == 52 || c->none || c->cnt > EC_BUF) return;
+                                                       unsigned long long* __restrict__ buf, unsigned bufcap) {
+  if (c->sh < 0 || c->sh == 52 || c->none || c->cnt > bufcap) return;
   const unsigned long long lo = c->lo;
   const int sh = c->sh + 4;
   for (int i = blockIdx.x; i < n - 1; i += gridDim.x) {
@@ -741,7 +741,7 @@ __global__ void __launch_bounds__(256) k_edge_collect(const double* __restrict__
       const unsigned long long key = dkey(row[j]);
       if (key >= lo && ((key - lo) >> sh) == 0) {
         const unsigned p = atomicAdd(&c->nbuf, 1u);
-        if (p < EC_BUF) buf[p] = key;
+        if (p < bufcap) buf[p] = key;
       }
     }
   }
@@ -749,10 +749,10 @@ __global__ void __launch_bounds__(256) k_edge_collect(const double* __restrict__
 
 // The cut among the collected entries: a bitonic sort of their keys, then the
 // distinct ones from the largest down.
-__global__ void __launch_bounds__(1024) k_edge_cut(const unsigned long long* __restrict__ buf, double delta,
-                                                    EdgeCut* __restrict__ c) {
+__global__ void __launch_bounds__(1024) k_edge_cut(const unsigned long long* __restrict__ buf, unsigned bufcap,
+                                                    double delta, EdgeCut* __restrict__ c) {
   __shared__ unsigned long long key[EC_BUF];
-  if (c->sh < 0 || c->sh == 52 || c->none || c->cnt > EC_BUF) return;
+  if (c->sh < 0 || c->sh == 52 || c->none || c->cnt > bufcap) return;
   const int m = (int)c->cnt;
   for (int e = threadIdx.x; e < EC_BUF; e += 1024) key[e] = e < m ? buf[e] : 0ull;
   for (int w = 2; w <= EC_BUF; w <<= 1)
@@ -1307,20 +1307,25 @@ int cad_edges(cdl_ctx* ctx, const double* A1, const double* A2, const double* Z1
   const int n = (int)n64;
   cudaStream_t st = ctx->stream;
   const int nb = (n + ST - 1) / ST;
-  void *vab, *vc, *vE, *vF, *vp, *vs, *vbuf, *vcnt, *voff;
-  CDL_TRY(ws_get(ctx, "score.contrib", (size_t)nb * n * sizeof(double), &vc));
+  void *vab, *vc, *vE, *vF, *vs, *vcnt, *voff;
+  // The node scores' partial sums; once these are reduced, the same room holds the
+  // block sums of a pass of the cut search (fewer blocks where it is small) and, after
+  // the passes, the entries that are left.
+  constexpr size_t block_bytes = EC_BINS * (sizeof(U128) + sizeof(unsigned long long));
+  const size_t room = std::max((size_t)nb * n * sizeof(double), block_bytes);
+  CDL_TRY(ws_get(ctx, "score.contrib", room, &vc));
   CDL_TRY(ws_get(ctx, "edges.E", (size_t)n * n * sizeof(double), &vE));
   CDL_TRY(ws_get(ctx, "edges.F", (size_t)n * sizeof(double), &vF));
   const int mb = std::min(n, ctx->sm_count * 8);
-  const int eb = std::min(n, ctx->sm_count * EC_BLOCKS_PER_SM);
-  CDL_TRY(ws_get(ctx, "edges.part", (size_t)eb * EC_BINS * 24, &vp));
+  const int eb = (int)std::min<size_t>(std::min(n, ctx->sm_count * EC_BLOCKS_PER_SM), room / block_bytes);
+  const unsigned bufcap = (unsigned)std::min<size_t>(EC_BUF, room / sizeof(unsigned long long));
   CDL_TRY(ws_get(ctx, "edges.cut", sizeof(EdgeCut), &vs));
-  CDL_TRY(ws_get(ctx, "edges.buf", EC_BUF * sizeof(unsigned long long), &vbuf));
   CDL_TRY(ws_get(ctx, "edges.rowcnt", 2 * (size_t)n * sizeof(int), &vcnt));
   CDL_TRY(ws_get(ctx, "edges.rowoff", 2 * (size_t)n * sizeof(long long) + 16, &voff));
   double* E = static_cast<double*>(vE);
   double* Fw = F ? F : static_cast<double*>(vF);
-  U128* psum = static_cast<U128*>(vp);
+  U128* psum = static_cast<U128*>(vc);
+  unsigned long long* buf = static_cast<unsigned long long*>(vc);
   unsigned long long* pcnt = reinterpret_cast<unsigned long long*>(psum + (size_t)eb * EC_BINS);
   const int rc = score_pairs_residues(ctx, Z1, Z2, vol1, vol2, n, k, fp64, A1, A2, static_cast<double*>(vc), E);
   if (rc != CDL_ERR_UNSUPPORTED) CDL_TRY(rc);
@@ -1367,18 +1372,17 @@ int cad_edges(cdl_ctx* ctx, const double* A1, const double* A2, const double* Z1
   while (true) {
     {
       Launch L(ctx, CDL_KC_MISC, 0);
-      k_edge_collect<<<mb, 256, 0, st>>>(E, n, cut, static_cast<unsigned long long*>(vbuf));
+      k_edge_collect<<<mb, 256, 0, st>>>(E, n, cut, buf, bufcap);
       CDL_TRY(L.done());
     }
     {
       Launch L(ctx, CDL_KC_MISC, 0);
-      k_edge_cut<<<1, 1024, 0, st>>>(static_cast<const unsigned long long*>(vbuf), delta, cut);
+      k_edge_cut<<<1, 1024, 0, st>>>(buf, bufcap, delta, cut);
       CDL_TRY(L.done());
     }
     CDL_CUDA_TRY(cudaMemcpyAsync(&h, cut, sizeof(h), cudaMemcpyDeviceToHost, st));
     CDL_CUDA_TRY(cudaStreamSynchronize(st));
-    if (h.none || h.sh < 0 || (h.sh < 52 && h.cnt <= EC_BUF) || (h.kmax >> 52) >= 0x7FF)
-      break;
+    if (h.none || h.sh < 0 || (h.sh < 52 && h.cnt <= bufcap) || (h.kmax >> 52) >= 0x7FF) break;
     CDL_TRY(pass());
   }
   typedef unsigned __int128 u128;

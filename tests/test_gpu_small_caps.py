@@ -54,3 +54,36 @@ def test_projection(G, n, k, splits, more):
         assert cdl.cdl_sync(h) == 0
     # exact digit sums, one float64 rounding per split or chunk of 4096 edges
     np.testing.assert_allclose(Y.cpu().numpy(), ref.cpu().numpy(), rtol=0, atol=64 * 2.0 ** -53 * float(ref.abs().max()))
+
+
+@pytest.mark.parametrize("name", ["f64", "f32"])
+@pytest.mark.parametrize("n,k", [(20, 3), (130, 8), (700, 8)])
+def test_edges(G, name, n, k):
+    """The edge scores (8 n^2), the partial sums and the operand copies of the CUDA-core scores, counts and offsets
+    per row, and 512 bytes; the cut search has no room of its own. Sums over as few as one block, and entries left
+    over that take further passes, give the same set."""
+    cdl = G.cdl
+    g = [G.graph(iid_pair(n, 8, 2, seed=n).X[i]) for i in range(2)]
+    rng = np.random.default_rng(n)
+    Z = [torch.from_numpy(rng.standard_normal((n, k))).cuda() for _ in range(2)]
+    nb = (n + 63) // 64
+    cap = max(8 * nb * n, 17 * 24) + 8 * n * n + 8 * n + 8 * n + 16 * n + 16 + 16 * n * k + 16 * k + 512
+    out = []
+    for frac in (0.9, 0.2):
+        for c in (0, cap):
+            with Capped(G, c) as h:
+                m = n * (n - 1) // 2
+                F = torch.empty(n, dtype=torch.float64, device="cuda")
+                v = (torch.ones(1, dtype=torch.float64, device="cuda"), torch.full((1,), 2.0, dtype=torch.float64,
+                                                                                   device="cuda"))
+                sd = cdl.CDL_F64 if name == "f64" else cdl.CDL_F32
+                assert cdl.cdl_cad_score(G.h, g[0][0], g[1][0], cdl.CDL_F64, *Z, *v, n, k, sd, 0, F, None) == 0
+                delta = frac * 0.5 * float(F.sum())
+                ij = torch.full((m, 2), -1, dtype=torch.int64, device="cuda")
+                de = torch.zeros(m, dtype=torch.float64, device="cuda")
+                st, r = cdl.cdl_cad_edges(h, g[0][0], g[1][0], cdl.CDL_F64, *Z, *v, n, k, sd, delta, m, ij, de, None, 0,
+                                          0, None, None, None)
+                assert st == 0 and cdl.cdl_sync(h) == 0
+                out.append((r.n_edges, ij.cpu().numpy()))
+    for a, b in (out[:2], out[2:]):
+        assert a[0] == b[0] > 0 and np.array_equal(a[1], b[1])
