@@ -279,7 +279,7 @@ int build_plan(cdl_ctx* ctx, int G, const int64_t* n, int T, const cdl_batch_opt
     res_groups = c.take<TcGroup>(2 * G2);
     d_tiles = c.take<uint32_t>(ntiles);
     d_ggs = c.take<GGraph>(G2);
-    d_dgs = c.take<DistGroup>(G2);
+    if (!gt.tc.empty()) d_dgs = c.take<DistGroup>(G2);
     d_pgs = c.take<PGraph>(G2);
     d_cgs = c.take<CGraph>(G2);
     d_sel = c.take<int4>(gt.sel.size());
@@ -500,7 +500,7 @@ int build_plan(cdl_ctx* ctx, int G, const int64_t* n, int T, const cdl_batch_opt
   P->pv_choice = 0;
   if ((st = upload(P->stream, d_tiles, all)) != CDL_OK || (st = upload(P->stream, d_gs, gs)) != CDL_OK ||
       (st = upload(P->stream, P->jobs, jobs)) != CDL_OK || (st = upload(P->stream, d_ggs, ggs)) != CDL_OK ||
-      (st = upload(P->stream, d_dgs, dgs)) != CDL_OK ||
+      (d_dgs && (st = upload(P->stream, d_dgs, dgs)) != CDL_OK) ||
       (st = upload(P->stream, d_pgs, pgs)) != CDL_OK || (st = upload(P->stream, d_sel, gt.sel)) != CDL_OK ||
       (st = upload(P->stream, d_cgs, cgs)) != CDL_OK)
     return fail(st);

@@ -33,8 +33,8 @@ struct SelectState {
   int flags;                    // bit 0: input off the 2^-16 grid; bit 1: a top digit above 64 in magnitude
   unsigned done;                // blocks of the running pass that have finished
   unsigned long long ncomp;     // keys copied to the buffer
-  unsigned long long lo, hi;    // bracket of the wanted key, from a sample
   unsigned long long below;     // keys below the bracket
+  uint32_t lo, hi;              // bracket of the wanted key, from a sample: the ends' high words
   int bracket;                  // BRACKET_TRY: lo, hi are set; BRACKET_HELD: the buffer holds the wanted key
   int pad;
 };
@@ -43,7 +43,7 @@ struct SelectState {
 // n = 5003 85 and 77; n = 8192 160 and 109.
 constexpr long long SELECT_BRACKET_MIN = 12000000;
 enum { BRACKET_NONE = 0, BRACKET_HELD = 1, BRACKET_TRY = 2 };
-constexpr size_t SELECT_STATE_BYTES = 128;   // in front of the histogram in the batched form
+constexpr size_t SELECT_STATE_BYTES = 64;    // in front of the histogram in the batched form
 static_assert(sizeof(SelectState) <= SELECT_STATE_BYTES, "the batched form's room for the state");
 
 // X (float64, n x T) -> int32 fixed point a = x * 2^16, stored transposed
@@ -523,7 +523,7 @@ template <class R>
 __device__ __forceinline__ void select_bracket(SelectState* st, unsigned long long* buf, unsigned long long cap,
                                                unsigned blocks, SelectShared& sm, R&& rows) {
   if (st->bracket != BRACKET_TRY) return;
-  const unsigned long long lo = st->lo, hi = st->hi;
+  const unsigned long long lo = (unsigned long long)st->lo << 32, hi = (unsigned long long)st->hi << 32 | 0xFFFFFFFFull;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   unsigned long long* stage = sm.stage[warp];
   unsigned below = 0;
@@ -670,8 +670,8 @@ __device__ __forceinline__ void select_sample(int n, SelectState* st, unsigned l
   if (lane == 0) atomicAdd(&sm.inside, in);
   __syncthreads();
   if (tid == 0) {
-    st->lo = (unsigned long long)lo << 32;
-    st->hi = (unsigned long long)hi << 32 | 0xFFFFFFFFull;
+    st->lo = lo;
+    st->hi = hi;
     st->bracket = (double)sm.inside / SAMPLE * (0.5 * (double)n * (double)(n - 1)) < 0.95 * (double)cap + 4.0 ? BRACKET_TRY : BRACKET_NONE;
   }
 }

@@ -87,3 +87,33 @@ def test_edges(G, name, n, k):
                 out.append((r.n_edges, ij.cpu().numpy()))
     for a, b in (out[:2], out[2:]):
         assert a[0] == b[0] > 0 and np.array_equal(a[1], b[1])
+
+
+def _smallest_cap(cdl, call):
+    """The smallest cap, to 256 bytes, under which call(ctx) returns CDL_OK."""
+    lo, hi = 0, 1 << 30
+    while hi - lo > 256:
+        mid = (lo + hi) // 2
+        st, h = cdl.cdl_ctx_create(0, torch.cuda.current_stream().cuda_stream, mid)
+        assert st == 0
+        lo, hi = (lo, mid) if call(h) == 0 else (mid, hi)
+        assert cdl.cdl_ctx_destroy(h) == 0
+    return hi
+
+
+@pytest.mark.parametrize("n,T", [([20] * 6, 300), ([100, 130, 90], 600)])
+def test_batch_of_series_too_long_for_digit_planes(G, n, T):
+    """A plan without the tensor-core distances holds nothing for them: no tensor maps, and 64 bytes of selection
+    state per graph, as the 32 KB histogram beside it, so every graph's share is a whole number of 64 bytes. The
+    bound is the plan's size with none of it, counted for these two (measured before those distances came)."""
+    cdl = G.cdl
+    k, d = (4, 2) if len(n) == 6 else (16, 4)
+    N = sum(n)
+    rng = np.random.default_rng(N)
+    X = [torch.from_numpy(np.round(rng.standard_normal((N, T)) * 65536) / 65536).cuda() for _ in range(2)]
+    F = torch.empty(N, dtype=torch.float64, device="cuda")
+    top = torch.empty((len(n), 2), dtype=torch.int64, device="cuda")
+    o = cdl.cdl_batch_opts(k, d, cdl.CDL_BF16, cdl.CDL_F32, 3, 0.0, cdl.cdl_solve_opts(20, 1e-10, 0), 2, 0, 0)
+    nn = np.array(n, dtype=np.int64)
+    cap = _smallest_cap(cdl, lambda h: cdl.cdl_caddelag_batched(h, len(n), nn, T, X[0], X[1], o, F, top, None))
+    assert cap <= {6: 15028224, 3: 16943104}[len(n)]
