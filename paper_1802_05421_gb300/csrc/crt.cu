@@ -665,11 +665,10 @@ int chain_square_crt(cdl_ctx* ctx, cdl_chain* ch, int level) {
     return CDL_ERR_UNSUPPORTED;
   CDL_TRY(crt_gemm_prepare(ctx, (int)ch->npad, 0));
   void *vp, *vt, *ve;
-  if (ws_get(ctx, "crt.planes", planes * cnt * 2, &vp) != CDL_OK || ws_get(ctx, "crt.t", planes * cnt, &vt) != CDL_OK ||
-      ws_get(ctx, "crt.e", (size_t)ch->npad * sizeof(int), &ve) != CDL_OK) {
-    ws_reclaim(ctx);
+  if (ws_get_opt(ctx, {{"crt.planes", planes * cnt * 2, &vp},
+                       {"crt.t", planes * cnt, &vt},
+                       {"crt.e", (size_t)ch->npad * sizeof(int), &ve}}) != CDL_OK)
     return CDL_ERR_UNSUPPORTED;
-  }
   if (ch->dtype == CDL_F64)
     return square_impl<double>(ctx, ch, level, vp, static_cast<uint8_t*>(vt), static_cast<int*>(ve));
   return square_impl<float>(ctx, ch, level, vp, static_cast<uint8_t*>(vt), static_cast<int*>(ve));
@@ -694,13 +693,12 @@ int crt_apply_begin(cdl_ctx* ctx, int np, int k, CrtApply* a) {
   CDL_TRY(crt_gemm_prepare(ctx, np, a->kpb));
   const size_t kx = (size_t)a->kpb * np;
   void *vp, *vx, *vxp, *vt, *ve;
-  if (ws_get(ctx, "crt.planes", (size_t)16 * np * np * 2, &vp) != CDL_OK ||
-      ws_get(ctx, "crt.xt", kx * sizeof(double), &vx) != CDL_OK ||
-      ws_get(ctx, "crt.xplanes", 16 * kx * 2, &vxp) != CDL_OK || ws_get(ctx, "crt.xprod", 16 * kx, &vt) != CDL_OK ||
-      ws_get(ctx, "crt.xe", (size_t)(np + a->kpb) * sizeof(int), &ve) != CDL_OK) {
-    ws_reclaim(ctx);
+  if (ws_get_opt(ctx, {{"crt.planes", (size_t)16 * np * np * 2, &vp},
+                       {"crt.xt", kx * sizeof(double), &vx},
+                       {"crt.xplanes", 16 * kx * 2, &vxp},
+                       {"crt.xprod", 16 * kx, &vt},
+                       {"crt.xe", (size_t)(np + a->kpb) * sizeof(int), &ve}}) != CDL_OK)
     return CDL_ERR_UNSUPPORTED;
-  }
   a->planes = static_cast<uint32_t*>(vp);
   a->xt = static_cast<double*>(vx);
   a->xplanes = static_cast<uint32_t*>(vxp);
@@ -765,13 +763,13 @@ int score_pairs_residues(cdl_ctx* ctx, const double* Z1, const double* Z2, const
   if (!tc_supported(ctx)) return CDL_ERR_UNSUPPORTED;
   const size_t cnt = (size_t)planes * rows * kp;
   void *vu, *vv, *vd, *ve, *vm;
-  if (ws_get(ctx, "crt.score.u", cnt * 2, &vu) != CDL_OK || ws_get(ctx, "crt.score.v", cnt * 2, &vv) != CDL_OK ||
-      ws_get(ctx, "crt.score.d", (size_t)rows * 16, &vd) != CDL_OK ||
-      ws_get(ctx, "crt.score.e", (size_t)rows * sizeof(int), &ve) != CDL_OK ||
-      ws_get(ctx, "crt.score.max", sizeof(ScoreScale), &vm) != CDL_OK) {
-    ws_reclaim(ctx);
+  // the planes lie where the squarings and the solve of this context put theirs
+  if (ws_get_opt(ctx, {{"crt.planes", cnt * 2, &vu},
+                       {"crt.t", cnt * 2, &vv},
+                       {"crt.score.d", (size_t)rows * 16, &vd},
+                       {"crt.score.e", (size_t)rows * sizeof(int), &ve},
+                       {"crt.score.max", sizeof(ScoreScale), &vm}}) != CDL_OK)
     return CDL_ERR_UNSUPPORTED;
-  }
   ScoreScale* sc = static_cast<ScoreScale*>(vm);
   int* ex = static_cast<int*>(ve);
   CDL_CUDA_TRY(cudaMemsetAsync(sc, 0, sizeof(ScoreScale), ctx->stream));

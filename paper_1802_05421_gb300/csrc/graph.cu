@@ -1171,30 +1171,28 @@ int graph_build(cdl_ctx* ctx, const double* X, int64_t n64, int T, double sigma,
     CDL_TRY(dist_tc(ctx, wsPl, static_cast<const long long*>(wsNo), n, rows, tp, A, &st->flags,
                     0.5 * (double)n * (double)(n - 1) * T));
   }
+  void* wsPart;
+  CDL_TRY(ws_get(ctx, "graph.dpart", (size_t)nb * n * sizeof(double), &wsPart));
+  double* part = static_cast<double*>(wsPart);
   // off the grid: through residues on the tensor cores, and what that leaves over in float64
   const unsigned char* bad = nullptr;
   const int rows = (n + 127) / 128 * 128, kp = (T + 63) / 64 * 64, nb64 = rows / 64;
   const size_t bad_bytes = ((size_t)nb64 * nb64 + 3) / 4 * 4;
   void *wsRp, *wsRn, *wsRe, *wsBad;
-  if (ws_get(ctx, "crt.dist.planes", T < DIST_RES_MIN_T ? 0 : (size_t)16 * rows * kp * 2, &wsRp) == CDL_OK &&
-      ws_get(ctx, "crt.dist.norms", (size_t)rows * 16, &wsRn) == CDL_OK &&
-      ws_get(ctx, "crt.dist.e", (size_t)rows * sizeof(int), &wsRe) == CDL_OK &&
-      ws_get(ctx, "crt.dist.bad", bad_bytes, &wsBad) == CDL_OK) {
+  if (ws_get_opt(ctx, {{"crt.planes", T < DIST_RES_MIN_T ? 256 : (size_t)16 * rows * kp * 2, &wsRp},
+                       {"crt.dist.norms", (size_t)rows * 16, &wsRn},
+                       {"crt.dist.e", (size_t)rows * sizeof(int), &wsRe},
+                       {"crt.dist.bad", bad_bytes, &wsBad}}) == CDL_OK) {
     CDL_TRY(series_residues(ctx, X, n, T, rows, kp, &st->flags, static_cast<int*>(wsRe), wsRn, wsRp, wsBad,
                             (int)(bad_bytes / 4)));
     CDL_TRY(dist_residues_tc(ctx, wsRp, static_cast<const int*>(wsRe), wsRn, n, T, rows, kp, A, &st->flags, wsBad));
     bad = static_cast<const unsigned char*>(wsBad);
-  } else {
-    ws_reclaim(ctx);
   }
   {
     Launch L(ctx, CDL_KC_DISTANCE, 0);
     launch_next(k_dist_f64, (unsigned)std::min<long long>(tiles, ctx->sm_count * 6), 256, 0, s, X, n, T, A, st, bad, nb64);
     CDL_TRY(L.done());
   }
-  void* wsPart;
-  CDL_TRY(ws_get(ctx, "graph.dpart", (size_t)nb * n * sizeof(double), &wsPart));
-  double* part = static_cast<double*>(wsPart);
   if (sigma > 0) {
     Launch L(ctx, CDL_KC_MISC, 0);
     launch_next(k_set_scalar, 1, 1, 0, s, sigma_out, sigma);

@@ -117,3 +117,38 @@ def test_batch_of_series_too_long_for_digit_planes(G, n, T):
     nn = np.array(n, dtype=np.int64)
     cap = _smallest_cap(cdl, lambda h: cdl.cdl_caddelag_batched(h, len(n), nn, T, X[0], X[1], o, F, top, None))
     assert cap <= {6: 15028224, 3: 16943104}[len(n)]
+
+
+@pytest.mark.parametrize("name", ["f64", "f32"])
+def test_the_same_call_gives_the_same_bits_whatever_ran_before(G, name):
+    """Residue planes of an earlier solve stand in the room that the scores' planes need under this cap: they are
+    given up for them at once, so the first call and the second take the same form and give the same bits, those
+    of a context of their own."""
+    cdl = G.cdl
+    n, npad, k, ks = 300, 512, 8, 1024
+    dtype = cdl.CDL_F64 if name == "f64" else cdl.CDL_F32
+    A, D, vol, _ = G.graph(iid_pair(n, 8, 1, seed=4).X[0])
+    A2 = G.graph(iid_pair(n, 8, 1, seed=5).X[0])[0]
+    Y = G.project(A, k, 3)
+    rng = np.random.default_rng(1)
+    Z = [torch.from_numpy(rng.standard_normal((n, ks))).cuda() for _ in range(2)]
+    planes = 16 if name == "f64" else 13
+    # the scores' planes (rows padded to 128, 2 ks columns), their small buffers, and half of the solve's planes
+    cap = 2 * planes * 384 * 2 * ks * 2 + 2 * 8 * 5 * n + (1 << 20) + 16 * npad * npad
+
+    def score(h):
+        F = torch.empty(n, dtype=torch.float64, device="cuda")
+        assert cdl.cdl_cad_score(h, A, A2, cdl.CDL_F64, Z[0], Z[1], vol, vol, n, ks, dtype, 0, F, None) == 0
+        assert cdl.cdl_sync(h) == 0
+        return F
+
+    with Capped(G, cap) as h:
+        alone = score(h)
+    with Capped(G, cap) as h:
+        st, ch = cdl.cdl_chain_build(h, A, cdl.CDL_F64, D, vol, n, 2, cdl.CDL_F64)
+        assert st == 0
+        Zs = torch.empty((n, k), dtype=torch.float64, device="cuda")
+        assert cdl.cdl_chain_solve(h, ch, A, cdl.CDL_F64, Y, k, cdl.cdl_solve_opts(40, 1e-10, 0), Zs, None) == 0
+        first, second = score(h), score(h)
+        cdl.cdl_chain_free(ch)
+    assert torch.equal(first, second) and torch.equal(first, alone)
