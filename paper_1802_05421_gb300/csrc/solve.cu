@@ -982,7 +982,7 @@ struct SolveBlock {
     CDL_TRY(ws("solve.scal", idx, 64, &vscal));
     CDL_TRY(ws("solve.zh", idx, (size_t)n * k * 4, &vzh));
     CDL_TRY(ws("solve.zl", idx, (size_t)n * k * 4, &vzl));
-    CDL_TRY(ws("solve.colsum", idx, (size_t)(cs_parts + 1) * k * 8, &vcs));   // partial sums, then the shift
+    vcs = vpart;   // column sums of the centring, then the shift: less than 1/3 of one partial product, free by then
     CDL_TRY(ws("solve.dz", idx, (size_t)np * kp * 4, &vdz));
     CDL_TRY(ws("solve.zmax", idx, (size_t)k * 8, &vzmax));   // of the current Z, left by k_center
     if (bf16) {

@@ -152,3 +152,30 @@ def test_the_same_call_gives_the_same_bits_whatever_ran_before(G, name):
         first, second = score(h), score(h)
         cdl.cdl_chain_free(ch)
     assert torch.equal(first, second) and torch.equal(first, alone)
+
+
+@pytest.mark.parametrize("name,elem", [("f64", 8), ("f32", 4)])
+def test_solve_of_many_columns(G, name, elem):
+    """One level and k far above n: the solve's buffers are what the cap has to hold. Residual, iterate and its
+    partial products, Z as float pairs and dZ, and 64 KB for the rest; no room of its own for the centring (17 rows
+    of 1024 column sums, 139 KB)."""
+    cdl = G.cdl
+    n, npad, k = 300, 512, 1024
+    A, D, vol, _ = G.graph(iid_pair(n, 8, 1, seed=6).X[0])
+    Y = G.project(A, k, 3)
+    dtype = cdl.CDL_F64 if name == "f64" else cdl.CDL_F32
+
+    def call(h):
+        st, ch = cdl.cdl_chain_build(h, A, cdl.CDL_F64, D, vol, n, 1, dtype)
+        if st == 0:
+            Z = torch.empty((n, k), dtype=torch.float64, device="cuda")
+            st = cdl.cdl_chain_solve(h, ch, A, cdl.CDL_F64, Y, k, cdl.cdl_solve_opts(60, 1e-9, 0), Z, None)
+            cdl.cdl_sync(h)
+            cdl.cdl_chain_free(ch)
+        return st
+
+    # the partial products: with 152 SMs (npad / 64 or / 128) x 16 tiles leave room for 9 or 16 splits, 8 or 16 of
+    # the 64 blocks of K each
+    splits = {"f64": 8, "f32": 16}[name]
+    bound = n * k * 8 + npad * k * elem * (1 + splits) + 2 * n * k * 4 + npad * k * 4 + (1 << 16)
+    assert _smallest_cap(cdl, call) <= bound
