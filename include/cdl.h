@@ -149,9 +149,9 @@ int cdl_ctx_set_debug(cdl_ctx* ctx, int flags);
  * vol, sigma_out: device, one float64 each (sigma_out receives the sigma used).
  * Squared distances are exact when every x is a multiple of 2^-16 below 2^7
  * in magnitude (int64 arithmetic). Otherwise, for T >= 16 each is the exact
- * squared distance of the two series rounded to 2^-60 of their distances to
- * node 0 (or to 2^-60 of the largest sample, if that is more), correctly
- * rounded, where that leaves it within about 2^-53 relative; the others, and
+ * squared distance of the two series rounded to 2^-60 of their distances to one
+ * common series, the median sample by sample of five nodes' (or to 2^-60 of the
+ * largest sample, if that is more), correctly rounded, where that leaves it within about 2^-53 relative; the others, and
  * all for T < 16, are computed in float64 with one rounding per subtraction,
  * product and sum, samples in order.
  * Requires 2 <= n <= 2^20, 1 <= T <= 4096. */

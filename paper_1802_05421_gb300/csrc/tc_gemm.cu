@@ -1252,15 +1252,15 @@ __global__ void __launch_bounds__(T8_THREADS, 1)
 // (crt.cuh), and what is made of them in the epilogue:
 //
 // GR_DIST  squared distances of float64 series off the 2^-16 grid. Row i of the
-//   series less the series of node 0 is 2^-e_i times integers x'_i of norm
+//   series less one common series is 2^-e_i times integers x'_i of norm
 //   2^60.96 at most, rounded to one unit (k_series_residues); d2' = |x'_i|^2 +
 //   |x'_j|^2 - 2 x'_i . x'_j in 128-bit integers, in units of the coarser of the
 //   two rows, rounded once to float64. With d2' >= 2^109 the rounding of the
 //   series is below 2^-54 of d2 (rms 0.6 units per sample and pair, so 1.2 /
 //   sqrt(d2') relative), where a float64 sum of rounded squares has about
 //   sqrt(T) 2^-54: tiles with a smaller entry (a distance below 2^-6 of the
-//   nodes' distances to node 0, duplicates, non-finite series) are flagged and
-//   formed by the float64 kernel.
+//   nodes' distances to the common series, duplicates, non-finite series) are
+//   flagged and formed by the float64 kernel.
 //
 // GR_SCORE  CAD edge scores and their sums. With a and b as in k_tc_score, u_i =
 //   [g a_i | b_i] and v_i = [b_i | g a_i] (g one power of two that balances the
