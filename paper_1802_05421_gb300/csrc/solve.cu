@@ -91,8 +91,10 @@ __global__ void k_precond_in(const double* __restrict__ R, const double* __restr
 
 // Z += dZ with dZ = D^{-1/2} x (dZ is also kept in float32, npad x kp, zero
 // padded, for the recursive residual update), and the column sums of D o Z over
-// the block's 32 rows for the centring (part[block][r], fixed order). Lanes along
-// the columns, a warp every eighth row.
+// the block's 32 rows for the centring (part[block][r], fixed order). 32 x 32 tiles:
+// lanes along the columns, a warp every eighth row (a block for all columns left
+// small orders with many columns to a few blocks: float32 solve at n = 64, k = 1024
+// 531 us, 329 before the sums came into this kernel).
 template <typename T>
 __global__ void __launch_bounds__(256) k_precond_out(const T* __restrict__ x, const double* __restrict__ rsd,
                                                       const double* __restrict__ D, int n, int k, int kp,
@@ -100,32 +102,28 @@ __global__ void __launch_bounds__(256) k_precond_out(const T* __restrict__ x, co
                                                       double* __restrict__ part) {
   follow();
   __shared__ double red[8][33];
-  const int i0 = blockIdx.x * 32, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int c0 = 0; c0 < kp; c0 += 32) {
-    const int r = c0 + lane;
-    double acc = 0.0;
+  const int i0 = blockIdx.x * 32, lane = threadIdx.x & 31, w = threadIdx.x >> 5, r = blockIdx.y * 32 + lane;
+  double acc = 0.0;
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      const int i = i0 + w + 8 * a;
-      float dzf = 0.f;
-      if (i < n && r < k) {
-        const double dz = (double)x[(size_t)i * kp + r] * rsd[i];
-        const double z = Z[(size_t)i * k + r] + dz;
-        Z[(size_t)i * k + r] = z;
-        acc = fma(D[i], z, acc);
-        dzf = (float)dz;
-      }
-      if (r < kp) dZ[(size_t)i * kp + r] = dzf;
+  for (int a = 0; a < 4; ++a) {
+    const int i = i0 + w + 8 * a;
+    float dzf = 0.f;
+    if (i < n && r < k) {
+      const double dz = (double)x[(size_t)i * kp + r] * rsd[i];
+      const double z = Z[(size_t)i * k + r] + dz;
+      Z[(size_t)i * k + r] = z;
+      acc = fma(D[i], z, acc);
+      dzf = (float)dz;
     }
-    red[w][lane] = acc;
-    __syncthreads();
-    if (w == 0 && r < k) {
-      double t = red[0][lane];
+    if (r < kp) dZ[(size_t)i * kp + r] = dzf;
+  }
+  red[w][lane] = acc;
+  __syncthreads();
+  if (w == 0 && r < k) {
+    double t = red[0][lane];
 #pragma unroll
-      for (int q = 1; q < 8; ++q) t += red[q][lane];
-      part[(size_t)blockIdx.x * k + r] = t;
-    }
-    __syncthreads();
+    for (int q = 1; q < 8; ++q) t += red[q][lane];
+    part[(size_t)blockIdx.x * k + r] = t;
   }
 }
 
@@ -201,36 +199,32 @@ __global__ void __launch_bounds__(256) k_center_shift(const double* __restrict__
 }
 
 // Z -= shift, and each column's largest |Z| as float64 bits (for the slices of
-// the exact residual): 64 rows per block, lanes along the columns, one atomic
-// per block and column.
+// the exact residual): 64 rows x 32 columns per block, lanes along the columns, one
+// atomic per block and column.
 __global__ void __launch_bounds__(256) k_center(double* __restrict__ Z, const double* __restrict__ shift, int n, int k,
                                                  unsigned long long* __restrict__ mbits) {
   follow();
   __shared__ unsigned long long red[8][32];
-  const int i0 = blockIdx.x * 64, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int c0 = 0; c0 < k; c0 += 32) {
-    const int r = c0 + lane;
-    unsigned long long m = 0;
-    if (r < k) {
-      const double s = shift[r];
+  const int i0 = blockIdx.x * 64, lane = threadIdx.x & 31, w = threadIdx.x >> 5, r = blockIdx.y * 32 + lane;
+  unsigned long long m = 0;
+  if (r < k) {
+    const double s = shift[r];
 #pragma unroll
-      for (int a = 0; a < 8; ++a) {
-        const int i = i0 + w + 8 * a;
-        if (i < n) {
-          const double z = Z[(size_t)i * k + r] - s;
-          Z[(size_t)i * k + r] = z;
-          m = max(m, (unsigned long long)__double_as_longlong(z) & 0x7FFFFFFFFFFFFFFFull);
-        }
+    for (int a = 0; a < 8; ++a) {
+      const int i = i0 + w + 8 * a;
+      if (i < n) {
+        const double z = Z[(size_t)i * k + r] - s;
+        Z[(size_t)i * k + r] = z;
+        m = max(m, (unsigned long long)__double_as_longlong(z) & 0x7FFFFFFFFFFFFFFFull);
       }
     }
-    red[w][lane] = m;
-    __syncthreads();
-    if (w == 0 && r < k) {
+  }
+  red[w][lane] = m;
+  __syncthreads();
+  if (w == 0 && r < k) {
 #pragma unroll
-      for (int q = 1; q < 8; ++q) m = max(m, red[q][lane]);
-      atomicMax(mbits + r, m);
-    }
-    __syncthreads();
+    for (int q = 1; q < 8; ++q) m = max(m, red[q][lane]);
+    atomicMax(mbits + r, m);
   }
 }
 
@@ -1235,11 +1229,11 @@ struct SolveBlock {
       Launch L(ctx, CDL_KC_MISC, 0);
       double* cs = static_cast<double*>(vcs);
       if (ch->dtype == CDL_F64)
-        launch_next(k_precond_out<double>, cs_parts, 256, 0, st, static_cast<const double*>(vx), ch->rsqrt_d, ch->D, n, k, kp, Z,
-                                                        static_cast<float*>(vdz), cs);
+        launch_next(k_precond_out<double>, dim3(cs_parts, (kp + 31) / 32), 256, 0, st, static_cast<const double*>(vx),
+                    ch->rsqrt_d, ch->D, n, k, kp, Z, static_cast<float*>(vdz), cs);
       else
-        launch_next(k_precond_out<float>, cs_parts, 256, 0, st, static_cast<const float*>(vx), ch->rsqrt_d, ch->D, n, k, kp, Z,
-                                                       static_cast<float*>(vdz), cs);
+        launch_next(k_precond_out<float>, dim3(cs_parts, (kp + 31) / 32), 256, 0, st, static_cast<const float*>(vx),
+                    ch->rsqrt_d, ch->D, n, k, kp, Z, static_cast<float*>(vdz), cs);
       CDL_TRY(L.done());
     }
     {
@@ -1252,7 +1246,7 @@ struct SolveBlock {
         CDL_TRY(L.done());
       }
       Launch L(ctx, CDL_KC_MISC, 0);
-      launch_next(k_center, (n + 63) / 64, 256, 0, st, Z, shift, n, k, zmax);
+      launch_next(k_center, dim3((n + 63) / 64, (k + 31) / 32), 256, 0, st, Z, shift, n, k, zmax);
       CDL_TRY(L.done());
     }
     ++iters;
