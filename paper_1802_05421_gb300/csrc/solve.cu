@@ -536,7 +536,6 @@ __global__ void __launch_bounds__(256) k_resid_combine(const double* __restrict_
                                                         const double* __restrict__ G, const double* __restrict__ cs,
                                                         const double* __restrict__ a_scale,
                                                         double* __restrict__ R, double* __restrict__ part) {
-  follow();
   __shared__ double red[8];
   const double as = a_scale[0];
   double sq = 0.0;
@@ -1016,6 +1015,17 @@ struct SolveBlock {
     return CDL_OK;
   }
 
+  // R and its partial sums of squares from the slice products G. Launched plainly: its blocks, set up
+  // while the products' kernel fills every SM, would come to lie together on few of them (one application
+  // at n = 4000: k = 1, 16 blocks, 341 us so and 224 plainly; k = 8, 125 blocks, 228 and 217; n = 9000, k = 50,
+  // where they fill the chip, 715 and 711).
+  int resid_combine(const double* G, const double* cs) {
+    nparts = std::min(1024, (int)blocks_for(nk, 256));
+    Launch L(ctx, CDL_KC_RESIDUAL, 0);
+    k_resid_combine<<<nparts, 256, 0, st>>>(Y, Z, ch->D, n, k, np, G, cs, ch->a_scale, R, red);
+    return L.done();
+  }
+
   // Full residual R = Y - L Z (float64-class).
   int full_residual() {
     if (ch->regen) {
@@ -1046,13 +1056,7 @@ struct SolveBlock {
           CDL_TRY(resid_tc_panel(ctx, rs.slicesT, np, rs.P, std::min(rs.P, np - r0), r0, vzs, kg, Gg));
         }
       }
-      const int nb = std::min(1024, (int)blocks_for(nk, 256));
-      Launch L(ctx, CDL_KC_RESIDUAL, 0);
-      launch_next(k_resid_combine, nb, 256, 0, st, Y, Z, ch->D, n, k, np, static_cast<const double*>(vG),
-                                          static_cast<const double*>(vcz), ch->a_scale, R, red);
-      CDL_TRY(L.done());
-      nparts = nb;
-      return CDL_OK;
+      return resid_combine(static_cast<const double*>(vG), static_cast<const double*>(vcz));
     }
     if (ch->aslices) {
       // A Z from exact bf16 slices on the tensor cores, in column groups of <= 128
@@ -1073,13 +1077,7 @@ struct SolveBlock {
         }
         CDL_TRY(resid_tc(ctx, ch, vzs, kg, static_cast<double*>(vG) + (size_t)g * RESID_PAIRS * np * 128));
       }
-      const int nb = std::min(1024, (int)blocks_for(nk, 256));
-      Launch L(ctx, CDL_KC_RESIDUAL, 0);
-      launch_next(k_resid_combine, nb, 256, 0, st, Y, Z, ch->D, n, k, np, static_cast<const double*>(vG),
-                                          static_cast<const double*>(vcz), ch->a_scale, R, red);
-      CDL_TRY(L.done());
-      nparts = nb;
-      return CDL_OK;
+      return resid_combine(static_cast<const double*>(vG), static_cast<const double*>(vcz));
     }
     if (crt) {
       // the level products of a float64 chain use the same residue planes
