@@ -27,7 +27,9 @@
  *  - Work is enqueued asynchronously on the context's stream unless the
  *    entry point says it synchronises. cdl_sync() waits and reports deferred
  *    device errors. A call that fails validation launches nothing.
- *  - There is no CPU fallback and no silent change of precision.
+ *  - There is no CPU fallback, and no form has less than the stated precision.
+ *    Where an entry point names two forms, the one that runs follows from the
+ *    workspace that is to be had (the cap, or the device's free memory).
  */
 #ifndef CDL_H
 #define CDL_H
@@ -67,7 +69,16 @@ typedef struct cdl_chain cdl_chain;
  * cudaStream_t (NULL = the legacy default stream); every kernel of every call
  * on this context is launched on it. `ws_cap_bytes` caps the device workspace
  * the context may allocate (0 = no cap); a call that would exceed it returns
- * CDL_ERR_OOM without launching. *out receives the context. */
+ * CDL_ERR_OOM without launching. *out receives the context.
+ * Workspace is kept from call to call and freed with the context. Part of it only
+ * makes calls faster: the residue planes of float64 and float32 chains (up to
+ * 48 npad^2 bytes), of CDL_F64 and CDL_F32 scores (128 and 104 n k) and of
+ * distances off the grid (32 n T, taken by every build of 16 samples and more), in
+ * one room for all of them, and the partial sums of the projection (up to 2 GB).
+ * The library gives that part up before it refuses anything else, but a caller's
+ * own allocator cannot reach it: a program that needs the memory itself sets a cap,
+ * under which such calls take the other forms described at each entry point
+ * (slower, with the stated errors), or destroys the context. */
 int cdl_ctx_create(cdl_ctx** out, int device, void* cuda_stream, size_t ws_cap_bytes);
 
 /* Synchronise the stream, free all workspace and the context. NULL is a no-op. */
@@ -151,9 +162,10 @@ int cdl_ctx_set_debug(cdl_ctx* ctx, int flags);
  * in magnitude (int64 arithmetic). Otherwise, for T >= 16 each is the exact
  * squared distance of the two series rounded to 2^-60 of their distances to one
  * common series, the median sample by sample of five nodes' (or to 2^-60 of the
- * largest sample, if that is more), correctly rounded, where that leaves it within about 2^-53 relative; the others, and
- * all for T < 16, are computed in float64 with one rounding per subtraction,
- * product and sum, samples in order.
+ * largest sample, if that is more), correctly rounded, where that leaves it within
+ * about 2^-53 relative; the others, all for T < 16 and where the workspace is not
+ * to be had, are computed in float64 with one rounding per subtraction, product
+ * and sum, samples in order.
  * Requires 2 <= n <= 2^20, 1 <= T <= 4096. */
 int cdl_build_graph(cdl_ctx* ctx, const double* X, int64_t n, int32_t T, double sigma,
                     cdl_dtype a_dtype, void* A, double* D, double* vol, double* sigma_out);
@@ -364,9 +376,10 @@ typedef struct {
  * are added as integers and scaled into float64), leaving about 2^-50 of
  * |A||Z|; for CUDA-core chains A Z through integer residues on the tensor
  * cores (rows of A D^{-1/2} and columns of D^{1/2} Z, the roots as powers of
- * two, to 2^-60 of their norms), after every application. Tensor-core chains update it recursively in later steps,
- * R -= D dZ - A dZ, with A dZ in bf16 hi + lo products (error about 1e-7 of
- * ||L dZ||, i.e. of the previous residual). A bound on the accumulated error
+ * two, to 2^-60 of their norms), after every application. Tensor-core chains
+ * update it recursively in later steps, R -= D dZ - A dZ, with A dZ in bf16 hi +
+ * lo products (error about 1e-7 of ||L dZ||, i.e. of the previous residual). A
+ * bound on the accumulated error
  * of these updates is kept; when the stopping test passes with that bound
  * above rel_tol / 10, the residual is formed in full again before stopping.
  * flags = CDL_SOLVE_FULL_RESIDUAL forms it in full after every application.
@@ -469,7 +482,9 @@ int cdl_changed_nodes(cdl_ctx* ctx, const double* X1, const double* X2, int64_t 
  * graphs share sigma (cdl_build_graph with the same sigma > 0), A1 and A2
  * differ only in the rows and columns of the nodes whose series changed, so
  * every edge with Delta A != 0 has an endpoint in `changed` and the scores
- * equal cdl_cad_score's (same per-edge arithmetic, sums in another order).
+ * are cdl_cad_score's up to rounding: the per-edge arithmetic is that of
+ * cdl_cad_score without workspace for the residues (see there), and the sums
+ * run in another order.
  * Work is n_changed x n edges instead of n^2 / 2. Precondition (not
  * checked): A1_ij == A2_ij whenever neither i nor j is in `changed`.
  * changed: device, n_changed node indices (distinct), 0 <= n_changed <=
@@ -567,8 +582,9 @@ typedef struct {
  * pair), run together: per step, one launch covers every graph of the batch
  * (one grouped tcgen05 launch per chain level, one grouped launch per
  * refinement kernel, one grouped launch per scoring kernel). Each pair's
- * results equal what cdl_caddelag_pair computes for it up to the rounding
- * order of the chain apply (no split-K here).
+ * results equal what cdl_caddelag_pair computes for it up to rounding: the order
+ * of the chain apply (no split-K here), distances off the 2^-16 grid in float64 for
+ * every T, and the scores' k-term products as in cdl_cad_score without workspace.
  * n: host array of G orders, 2 <= n[p] <= 32768, sum <= 2^26.
  * X1, X2: (sum n) x T float64, row-major; pair p's nodes are rows
  *   off_p .. off_p + n[p] - 1 with off_p = n[0] + ... + n[p-1].

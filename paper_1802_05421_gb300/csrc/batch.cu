@@ -244,8 +244,8 @@ int build_plan(cdl_ctx* ctx, int G, const int64_t* n, int T, const cdl_batch_opt
     P->pv.push_back(pvar);
   }
   size_t ntiles = ap.size() + t32.size() + elem.size() + zst.size() + runits.size() + csb.size() + sel.size() +
-                  spairs.size() + snodes.size() + gt.fixed.size() + gt.dist.size() + gt.prep.size() + gt.tc.size() + cvec.size() +
-                  cinit.size();
+                  spairs.size() + snodes.size() + gt.fixed.size() + gt.dist.size() + gt.prep.size() + gt.tc.size() +
+                  cvec.size() + cinit.size();
   for (auto& v : sq) ntiles += v.size();
   for (auto& v : pblocks) ntiles += v.size();
   std::vector<GGraph> ggs(G2);
@@ -391,8 +391,10 @@ int build_plan(cdl_ctx* ctx, int G, const int64_t* n, int T, const cdl_batch_opt
     Gg.tp = tp;
     Gg.planes = tc_dist[g] ? cgs[g].aslices : nullptr;
     Gg.norms = reinterpret_cast<long long*>(P->Dv[g]);     // npad, until D is formed
-    if (tc_dist[g] && (st = dist_group(&dgs[g], Gg.planes, np, tp, Gg.norms, Gg.A, graph_select_flags(Gg.sel), nn)) != CDL_OK)
-      return fail(st);
+    if (tc_dist[g]) {
+      st = dist_group(&dgs[g], Gg.planes, np, tp, Gg.norms, Gg.A, graph_select_flags(Gg.sel), nn);
+      if (st != CDL_OK) return fail(st);
+    }
     CGraph& Cg = cgs[g];
     Cg.A = P->A[g];
     Cg.D = ch.D;

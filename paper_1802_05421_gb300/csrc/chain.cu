@@ -176,8 +176,9 @@ __device__ __forceinline__ long long grid48(double a, int s) {
 // residual update); and A / 2^s as six exact bf16 digit planes (N of grid48
 // split into signed base-256 digits d_t, plane t holding d_t 2^-8t), the
 // operand of its full residual (s = 0; k_a_slices forms them again where a weight
-// is above 1); all in one pass over A; padding rows and columns zero. Conversions avoid the float64 pipe (the scarce one): the
-// float of A_ij rounded to nearest by integer operations, the digits bottom-up
+// is above 1); all in one pass over A; padding rows and columns zero.
+// Conversions avoid the float64 pipe (the scarce one): the float of A_ij
+// rounded to nearest by integer operations, the digits bottom-up
 // (balanced base 256 on two 24-bit halves of N = A_ij 2^(48-s)) and their bf16
 // bit patterns by exact float32 arithmetic (digits6_fbits).
 __device__ __forceinline__ float d2f_rn_nonneg(double x) {
@@ -460,13 +461,15 @@ int square_impl(cdl_ctx* ctx, cdl_chain* ch, int level) {
     constexpr int B = 128;
     const int nb = np / B;
     Launch L(ctx, CDL_KC_SQUARE, flops);
-    launch_next(k_gemm_tn<T, B, B, 8, 8, 8, true>, nb * (nb + 1) / 2, 256, 0, ctx->stream, S, np, S, np, C, np, np, np, np);
+    launch_next(k_gemm_tn<T, B, B, 8, 8, 8, true>, nb * (nb + 1) / 2, 256, 0, ctx->stream, S, np, S, np, C, np, np, np,
+                np);
     return L.done();
   } else {
     constexpr int B = 64;
     const int nb = np / B;
     Launch L(ctx, CDL_KC_SQUARE, flops);
-    launch_next(k_gemm_tn<T, B, B, 8, 4, 4, true>, nb * (nb + 1) / 2, 256, 0, ctx->stream, S, np, S, np, C, np, np, np, np);
+    launch_next(k_gemm_tn<T, B, B, 8, 4, 4, true>, nb * (nb + 1) / 2, 256, 0, ctx->stream, S, np, S, np, C, np, np, np,
+                np);
     return L.done();
   }
 }
@@ -595,10 +598,11 @@ int chain_init(cdl_ctx* ctx, cdl_chain* ch, const double* A) {
       if (tensor) {
         unsigned long long* over = reinterpret_cast<unsigned long long*>(ch->a_scale + 1);
         CDL_CUDA_TRY(cudaMemsetAsync(over, 0, sizeof(unsigned long long), ctx->stream));
-        launch_next(k_chain_init_tc<true>, ctx->sm_count * 8, 256, 0, ctx->stream, A, n, np, rsf, uf, l0, ahi, alo, sl, over);
+        launch_next(k_chain_init_tc<true>, ctx->sm_count * 8, 256, 0, ctx->stream, A, n, np, rsf, uf, l0, ahi, alo, sl,
+                    over);
       } else {
-        launch_next(k_chain_init_tc<false>, ctx->sm_count * 8, 256, 0, ctx->stream, A, n, np, rsf, uf, l0, ahi, alo, nullptr,
-                                                                           nullptr);
+        launch_next(k_chain_init_tc<false>, ctx->sm_count * 8, 256, 0, ctx->stream, A, n, np, rsf, uf, l0, ahi, alo,
+                    nullptr, nullptr);
       }
       CDL_TRY(L.done());
     }
@@ -611,13 +615,13 @@ int chain_init(cdl_ctx* ctx, cdl_chain* ch, const double* A) {
     case CDL_F64: {
       Launch L(ctx, CDL_KC_CHAIN_INIT, bytes);
       launch_next(k_chain_init<double>, blocks, 256, 0, ctx->stream, A, n, np, ch->rsqrt_d, u,
-                                                            static_cast<double*>(ch->level(0)));
+                  static_cast<double*>(ch->level(0)));
       return L.done();
     }
     case CDL_F32: {
       Launch L(ctx, CDL_KC_CHAIN_INIT, bytes);
       launch_next(k_chain_init<float>, blocks, 256, 0, ctx->stream, A, n, np, ch->rsqrt_d, u,
-                                                           static_cast<float*>(ch->level(0)));
+                  static_cast<float*>(ch->level(0)));
       return L.done();
     }
     case CDL_FP8E4M3: {
@@ -627,13 +631,14 @@ int chain_init(cdl_ctx* ctx, cdl_chain* ch, const double* A) {
       const size_t cnt = (size_t)np * np;
       {
         Launch L2(ctx, CDL_KC_CHAIN_INIT, 2.0 * cnt);
-        launch_next(k_absmax_bf16, ctx->sm_count * 4, 256, 0, ctx->stream, 
-            static_cast<const __nv_bfloat16*>(ch->level16(0)), cnt, ch->amax);
+        launch_next(k_absmax_bf16, ctx->sm_count * 4, 256, 0, ctx->stream,
+                    static_cast<const __nv_bfloat16*>(ch->level16(0)), cnt, ch->amax);
         CDL_TRY(L2.done());
       }
       Launch L3(ctx, CDL_KC_CHAIN_INIT, 3.0 * cnt);
-      launch_next(k_quant_fp8, ctx->sm_count * 4, 256, 0, ctx->stream, static_cast<const __nv_bfloat16*>(ch->level16(0)),
-                                                              cnt, ch->amax, static_cast<uint8_t*>(ch->level(0)));
+      launch_next(k_quant_fp8, ctx->sm_count * 4, 256, 0, ctx->stream,
+                  static_cast<const __nv_bfloat16*>(ch->level16(0)), cnt, ch->amax,
+                  static_cast<uint8_t*>(ch->level(0)));
       return L3.done();
     }
     case CDL_FP8E4M3_T128:
@@ -679,17 +684,17 @@ int level_inf_norm(cdl_ctx* ctx, const cdl_chain* ch, int level, unsigned* out_b
   Launch L(ctx, CDL_KC_MISC, 2.0 * np * (double)np);
   switch (ch->dtype) {
     case CDL_F64:
-      launch_next(k_level_inf_norm<double>, blocks, 256, 0, ctx->stream, static_cast<const double*>(ch->level(level)), np,
-                                                                out_bits);
+      launch_next(k_level_inf_norm<double>, blocks, 256, 0, ctx->stream, static_cast<const double*>(ch->level(level)),
+                  np, out_bits);
       break;
     case CDL_F32:
       launch_next(k_level_inf_norm<float>, blocks, 256, 0, ctx->stream, static_cast<const float*>(ch->level(level)), np,
-                                                               out_bits);
+                  out_bits);
       break;
     default:   // bf16 levels, or the bf16 copies of e4m3 levels
       if (ch->host_levels) return CDL_ERR_UNSUPPORTED;
-      launch_next(k_level_inf_norm<__nv_bfloat16>, blocks, 256, 0, ctx->stream, 
-          static_cast<const __nv_bfloat16*>(ch->level16(level)), np, out_bits);
+      launch_next(k_level_inf_norm<__nv_bfloat16>, blocks, 256, 0, ctx->stream,
+                  static_cast<const __nv_bfloat16*>(ch->level16(level)), np, out_bits);
       break;
   }
   return L.done();
@@ -698,8 +703,8 @@ int level_inf_norm(cdl_ctx* ctx, const cdl_chain* ch, int level, unsigned* out_b
 int fp8_level_bound(cdl_ctx* ctx, cdl_chain* ch, int level) {
   const int np = (int)ch->npad;
   Launch L(ctx, CDL_KC_MISC, (double)np * np);
-  launch_next(k_rownorm_fp8, std::min(np, ctx->sm_count * 8), 256, 0, ctx->stream, 
-      static_cast<const uint8_t*>(ch->level(level)), np, ch->amax + level, ch->amax + level + 1);
+  launch_next(k_rownorm_fp8, std::min(np, ctx->sm_count * 8), 256, 0, ctx->stream,
+              static_cast<const uint8_t*>(ch->level(level)), np, ch->amax + level, ch->amax + level + 1);
   return L.done();
 }
 
@@ -720,18 +725,18 @@ int apply_simt(cdl_ctx* ctx, const cdl_chain* ch, int level, const void* x, void
     constexpr int BM = 128, BN = 64;
     dim3 grid(np / BM, (kp + BN - 1) / BN, splits);
     Launch L(ctx, CDL_KC_APPLY, bytes);
-    launch_next(k_gemm_tn<float, BM, BN, 8, 8, 4, false>, grid, 256, 0, ctx->stream, 
-        static_cast<const float*>(ch->level(level)), np, static_cast<const float*>(x), kp,
-        static_cast<float*>(partial), kp, np, kp, kchunk);
+    launch_next(k_gemm_tn<float, BM, BN, 8, 8, 4, false>, grid, 256, 0, ctx->stream,
+                static_cast<const float*>(ch->level(level)), np, static_cast<const float*>(x), kp,
+                static_cast<float*>(partial), kp, np, kp, kchunk);
     return L.done();
   }
   if (ch->dtype == CDL_F64) {
     constexpr int BM = 64, BN = 64;
     dim3 grid(np / BM, (kp + BN - 1) / BN, splits);
     Launch L(ctx, CDL_KC_APPLY, bytes);
-    launch_next(k_gemm_tn<double, BM, BN, 8, 4, 4, false>, grid, 256, 0, ctx->stream, 
-        static_cast<const double*>(ch->level(level)), np, static_cast<const double*>(x), kp,
-        static_cast<double*>(partial), kp, np, kp, kchunk);
+    launch_next(k_gemm_tn<double, BM, BN, 8, 4, 4, false>, grid, 256, 0, ctx->stream,
+                static_cast<const double*>(ch->level(level)), np, static_cast<const double*>(x), kp,
+                static_cast<double*>(partial), kp, np, kp, kchunk);
     return L.done();
   }
   return CDL_ERR_UNSUPPORTED;
@@ -761,7 +766,7 @@ int chain_level0_panel(cdl_ctx* ctx, cdl_chain* ch, void* L0, const double* pane
   const float* uf = rsf + np;
   Launch L(ctx, CDL_KC_CHAIN_INIT, 8.0 * rows * (double)n + 2.0 * rows * (double)np);
   launch_next(k_panel_level0, ctx->sm_count * 8, 256, 0, ctx->stream, panel, n, np, r0, rows, rsf, uf,
-                                                             static_cast<__nv_bfloat16*>(L0));
+              static_cast<__nv_bfloat16*>(L0));
   return L.done();
 }
 
@@ -769,7 +774,7 @@ int panel_slices_t(cdl_ctx* ctx, const double* panel, int n, int np, int r0, int
   if (Pw % 32 || np % 32) return CDL_ERR_INVALID_ARG;
   Launch L(ctx, CDL_KC_RESIDUAL, 0);
   launch_next(k_panel_slices_t, ctx->sm_count * 8, 256, 0, ctx->stream, panel, n, np, r0, rows, Pw,
-                                                               static_cast<uint16_t*>(slicesT));
+              static_cast<uint16_t*>(slicesT));
   return L.done();
 }
 

@@ -675,7 +675,8 @@ int square_impl(cdl_ctx* ctx, cdl_chain* ch, int level, void* planes, uint8_t* t
   CDL_TRY(crt_gemm(ctx, planes, np, nullptr, 0, np, NP, t, CDL_KC_SQUARE, (double)ch->n * ch->n * (ch->n + 1.0)));
   const int nb = np / 64;
   Launch L(ctx, CDL_KC_SQUARE, 0);
-  launch_next(k_crt_combine<T>, nb * (nb + 1) / 2, 256, 0, ctx->stream, t, np, ex, static_cast<T*>(ch->level(level + 1)));
+  launch_next(k_crt_combine<T>, nb * (nb + 1) / 2, 256, 0, ctx->stream, t, np, ex,
+              static_cast<T*>(ch->level(level + 1)));
   return L.done();
 }
 
@@ -709,9 +710,9 @@ int chain_square_crt(cdl_ctx* ctx, cdl_chain* ch, int level) {
 // D^{-1/2} and D^{1/2} Z have entries of one size also where degrees span many
 // orders of magnitude (Z is about D^{-1/2}), and no bits go to a few huge entries
 // of Z. Without, one node of degree 5e-18 of the others' left a relative residual of
-// 3e-12 that no further step made smaller (n = 600, float64 chain). The float64 pipe's dot products took 0.52 ms per level
-// at n = 2000, k = 32 (its FMA rate); here the residues of M take most of the
-// time (8 n^2 bytes read, 32 n^2 written).
+// 3e-12 that no further step made smaller (n = 600, float64 chain). The float64
+// pipe's dot products took 0.52 ms per level at n = 2000, k = 32 (its FMA rate);
+// here the residues of M take most of the time (8 n^2 bytes read, 32 n^2 written).
 int crt_apply_begin(cdl_ctx* ctx, int np, int k, CrtApply* a) {
   if (!crt_gemm_supported(ctx, np)) return CDL_ERR_UNSUPPORTED;
   a->np = np;
@@ -761,8 +762,8 @@ int crt_apply_product(cdl_ctx* ctx, const CrtApply& a, const double* x, int rows
 
 int crt_apply_add(cdl_ctx* ctx, const CrtApply& a, double* x, int kp) {
   Launch L(ctx, CDL_KC_MISC, 0);
-  launch_next(k_crt_add, (unsigned)(((size_t)a.np * (kp / 4) + 127) / 128), 128, 0, ctx->stream, a.t, a.np, a.kpb, kp, a.erow,
-                                                                                         a.ecol, x);
+  launch_next(k_crt_add, (unsigned)(((size_t)a.np * (kp / 4) + 127) / 128), 128, 0, ctx->stream, a.t, a.np, a.kpb, kp,
+              a.erow, a.ecol, x);
   return L.done();
 }
 

@@ -488,7 +488,8 @@ __device__ __forceinline__ void select_pass(SelectState* st, unsigned long long*
     const size_t w0 = ((size_t)block * SELECT_WARPS) * 256;
     if (w0 < nc)
       select_hist(st, shift, bits, hist, sm, [&](auto&& f) {
-        for (size_t q = w0 + (threadIdx.x >> 5) * 256; q < nc; q += step) warp_keys(buf + q, (int)min((size_t)256, (size_t)(nc - q)), f);
+        for (size_t q = w0 + (threadIdx.x >> 5) * 256; q < nc; q += step)
+          warp_keys(buf + q, (int)min((size_t)256, (size_t)(nc - q)), f);
       });
   } else if (p == 2 && cap) {
     bool full = false;
@@ -568,9 +569,11 @@ __device__ __forceinline__ void select_bracket(SelectState* st, unsigned long lo
   st->done = 0;
 }
 
-// Sample q: the high word of the key at a hashed position.
+// Sample q: the high word of the key at a hashed position (the finaliser of
+// splitmix64: Steele, Lea and Flood, "Fast splittable pseudorandom number
+// generators", 2014, applied to q + 1).
 __device__ __forceinline__ uint32_t sample_key(const double* __restrict__ A, int n, uint32_t q) {
-  unsigned long long x = (q + 1) * 0x9E3779B97F4A7C15ull;   // two multiply-xorshift rounds
+  unsigned long long x = (q + 1) * 0x9E3779B97F4A7C15ull;
   x = (x ^ (x >> 30)) * 0xBF58476D1CE4E5B9ull;
   x = (x ^ (x >> 27)) * 0x94D049BB133111EBull;
   x ^= x >> 31;
@@ -672,7 +675,8 @@ __device__ __forceinline__ void select_sample(int n, SelectState* st, unsigned l
   if (tid == 0) {
     st->lo = lo;
     st->hi = hi;
-    st->bracket = (double)sm.inside / SAMPLE * (0.5 * (double)n * (double)(n - 1)) < 0.95 * (double)cap + 4.0 ? BRACKET_TRY : BRACKET_NONE;
+    const double expected = (double)sm.inside / SAMPLE * (0.5 * (double)n * (double)(n - 1));
+    st->bracket = expected < 0.95 * (double)cap + 4.0 ? BRACKET_TRY : BRACKET_NONE;
   }
 }
 
@@ -683,9 +687,9 @@ __global__ void __launch_bounds__(SAMPLE_THREADS) k_select_sample(const uint32_t
   select_sample(n, st, cap, *reinterpret_cast<SampleShared*>(sample_smem), [&](uint32_t q) { return keys[q]; });
 }
 
-__global__ void __launch_bounds__(SELECT_THREADS, 2) k_select_bracket(const double* __restrict__ A, int n, SelectState* st,
-                                                                   unsigned long long* __restrict__ buf,
-                                                                   unsigned long long cap) {
+__global__ void __launch_bounds__(SELECT_THREADS, 2)
+    k_select_bracket(const double* __restrict__ A, int n, SelectState* st, unsigned long long* __restrict__ buf,
+                     unsigned long long cap) {
   follow();
   __shared__ SelectShared sm;
   select_bracket(st, buf, cap, gridDim.x, sm, [&](auto&& f) {
@@ -705,7 +709,9 @@ __global__ void __launch_bounds__(SELECT_THREADS, 2) k_select_pass(const double*
 }
 
 __global__ void k_set_scalar(double* p, double v) {
-  follow(); *p = v; }
+  follow();
+  *p = v;
+}
 
 // A_ij = exp(-d2_ij / (2 sigma^2)) (KERN = KERNEL_GAUSSIAN) or
 // A_ij = exp(-sqrt(d2_ij) / sigma) (KERN = KERNEL_EXP, the synthetic-data
@@ -846,7 +852,8 @@ __device__ __forceinline__ void kernel_tile(double* __restrict__ A, int n, const
 #pragma unroll
     for (int m = 0; m < w; ++m) {
       const ff keep = up ? rs[m + w] : rs[m], give = up ? rs[m] : rs[m + w];
-      rs[m] = ff_add(keep, ff{__shfl_xor_sync(0xffffffffu, give.hi, 4 * w), __shfl_xor_sync(0xffffffffu, give.lo, 4 * w)});
+      rs[m] = ff_add(
+          keep, ff{__shfl_xor_sync(0xffffffffu, give.hi, 4 * w), __shfl_xor_sync(0xffffffffu, give.lo, 4 * w)});
     }
   }
 #pragma unroll
@@ -928,7 +935,9 @@ __device__ __forceinline__ void block_sum_to(const double* __restrict__ v, int n
 }
 
 __global__ void k_sum(const double* __restrict__ v, int n, double* __restrict__ out) {
-  follow(); block_sum_to(v, n, out); }
+  follow();
+  block_sum_to(v, n, out);
+}
 
 // ---------------------------------------------------------------- batched form
 // The same steps for every graph of a batch, one launch per step; a block
@@ -1165,7 +1174,7 @@ int graph_build(cdl_ctx* ctx, const double* X, int64_t n64, int T, double sigma,
     {
       Launch L(ctx, CDL_KC_DISTANCE, 0);
       launch_next(k_prepare_series, rows / 8, 256, 0, s, X, n, T, rows, tp, static_cast<__nv_bfloat162*>(wsPl),
-                                                static_cast<long long*>(wsNo), st);
+                  static_cast<long long*>(wsNo), st);
       CDL_TRY(L.done());
     }
     CDL_TRY(dist_tc(ctx, wsPl, static_cast<const long long*>(wsNo), n, rows, tp, A, &st->flags,
@@ -1190,7 +1199,8 @@ int graph_build(cdl_ctx* ctx, const double* X, int64_t n64, int T, double sigma,
   }
   {
     Launch L(ctx, CDL_KC_DISTANCE, 0);
-    launch_next(k_dist_f64, (unsigned)std::min<long long>(tiles, ctx->sm_count * 6), 256, 0, s, X, n, T, A, st, bad, nb64);
+    launch_next(k_dist_f64, (unsigned)std::min<long long>(tiles, ctx->sm_count * 6), 256, 0, s, X, n, T, A, st, bad,
+                nb64);
     CDL_TRY(L.done());
   }
   if (sigma > 0) {
@@ -1211,8 +1221,8 @@ int graph_build(cdl_ctx* ctx, const double* X, int64_t n64, int T, double sigma,
       }
       {
         Launch L(ctx, CDL_KC_SELECT, 0);
-        launch_next(k_select_sample, 1, SAMPLE_THREADS, sizeof(SampleShared), s, reinterpret_cast<const uint32_t*>(sbuf), n, st,
-                                                                        cap);
+        launch_next(k_select_sample, 1, SAMPLE_THREADS, sizeof(SampleShared), s,
+                    reinterpret_cast<const uint32_t*>(sbuf), n, st, cap);
         CDL_TRY(L.done());
       }
       Launch L(ctx, CDL_KC_SELECT, 8.0 * (double)m);
@@ -1289,7 +1299,7 @@ int graph_regen_init(cdl_ctx* ctx, RegenGraph& g, const double* X, int64_t n64, 
   {
     Launch L(ctx, CDL_KC_DISTANCE, 0);
     launch_next(k_prepare_series, g.rows / 8, 256, 0, s, X, n, T, g.rows, g.tp, static_cast<__nv_bfloat162*>(wsPl),
-                                                static_cast<long long*>(wsNo), st);
+                static_cast<long long*>(wsNo), st);
     CDL_TRY(L.done());
   }
   int flags = 0;
@@ -1313,8 +1323,8 @@ int graph_regen_init(cdl_ctx* ctx, RegenGraph& g, const double* X, int64_t n64, 
         const int r1 = std::min(n - 1, r0 + pr);
         if (r1 <= r0) continue;
         Launch L(ctx, CDL_KC_SELECT, 8.0 * (double)pr * n);
-        launch_next(k_select_hist_panel, std::min((r1 - r0 + SELECT_WARPS - 1) / SELECT_WARPS, ctx->sm_count * 4), SELECT_THREADS, 0, s, panel, n, shifts[p], widths[p], st,
-                                                                               hist, r0, r1);
+        launch_next(k_select_hist_panel, std::min((r1 - r0 + SELECT_WARPS - 1) / SELECT_WARPS, ctx->sm_count * 4),
+                    SELECT_THREADS, 0, s, panel, n, shifts[p], widths[p], st, hist, r0, r1);
         CDL_TRY(L.done());
       }
       Launch L(ctx, CDL_KC_SELECT, 0);
@@ -1337,7 +1347,8 @@ int regen_panel(cdl_ctx* ctx, const RegenGraph& g, double* panel, int r0, int ro
   CDL_TRY(dist_tc_panel(ctx, g.planes, g.norms, g.n, g.rows, g.tp, panel, r0, pr, false, g.offgrid));
   const int r1 = std::min(g.n, r0 + rows);
   Launch L(ctx, CDL_KC_KERNEL, 16.0 * (double)(r1 - r0) * g.n);
-  launch_next(k_kernel_rows_panel, std::min(r1 - r0, ctx->sm_count * 8), 256, 0, ctx->stream, panel, g.n, g.sigma, D, r0, r1);
+  launch_next(k_kernel_rows_panel, std::min(r1 - r0, ctx->sm_count * 8), 256, 0, ctx->stream, panel, g.n, g.sigma, D,
+              r0, r1);
   return L.done();
 }
 
@@ -1431,8 +1442,8 @@ int graph_add_edges(cdl_ctx* ctx, double* A, int64_t n, int64_t m, const int64_t
   if (m > 0) {
     const long long blocks = std::min<long long>((m + 255) / 256, (long long)ctx->sm_count * 16);
     Launch L(ctx, CDL_KC_MISC, 0);
-    launch_next(k_add_edges, (unsigned)blocks, 256, 0, s, A, (int)n, (long long)m, reinterpret_cast<const long long*>(ij),
-                                                 w, bad);
+    launch_next(k_add_edges, (unsigned)blocks, 256, 0, s, A, (int)n, (long long)m,
+                reinterpret_cast<const long long*>(ij), w, bad);
     CDL_TRY(L.done());
   }
   unsigned long long h = 0;

@@ -182,9 +182,11 @@ struct Launch {
 // with follow(): the next one may be set up, and nothing is read or written before
 // all earlier work of the stream is complete. For chains of short kernels: the
 // graph of n = 1024 (15 launches) 95 -> 68 us, the bf16 embedding at n = 5003 3.17 ->
-// 2.97 ms, the float64 one at n = 2000 2.89 -> 2.69. The scoring and edge kernels and
-// the batched form launch plainly: so launched they were slower (scores at n = 8192
-// 1.11 -> 1.17 ms, edges at n = 4001 0.74 -> 0.79, 64 pairs 26.5 -> 27.5).
+// 2.97 ms, the float64 one at n = 2000 2.89 -> 2.69. The scores' reductions and top
+// lists, the CUDA-core and bf16 scores, the edge set's kernels and the batched form
+// launch plainly: so launched they were slower (scores at n = 8192 1.11 -> 1.17 ms,
+// edges at n = 4001 0.74 -> 0.79, 64 pairs 26.5 -> 27.5); the residue scores' kernels
+// (crt.cu, k_tc_gramr) are launched so.
 template <typename... P, typename... A>
 inline void launch_next(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A&&... args) {
   cudaLaunchAttribute attr;
@@ -448,7 +450,7 @@ struct GGraph {
   long long* norms; // npad
   double* A;        // n x n
   double* D;        // n
-  double* part;     // ceil(n / 64) x n: sums of A over 64-node blocks
+  double* part;     // ceil(n / 64) x n: sums of A over 64-node blocks; before them, the selection's keys
   double* vol;
   double* sigma;
   void* sel;        // graph_select_bytes(): selection state and histogram
@@ -480,7 +482,7 @@ struct GraphTiles {
   std::vector<uint32_t> dist;    // g | bi << 12 | bj << 22, 64-node blocks, bi <= bj
   std::vector<uint32_t> prep;    // (b << 12) | g, 8 rows of the digit planes
   std::vector<uint32_t> tc;      // g | I << 12 | J << 22, 128 x 64 tiles of the tensor-core distances
-  std::vector<int4> sel;         // (g, first row, end row, 0): about 2^17 keys each
+  std::vector<int4> sel;         // (g, first row, end row, block | the graph's blocks << 16): about 2^17 keys each
 };
 void graph_grouped_tiles(const std::vector<int>& n, const std::vector<char>& tc, int T, GraphTiles& out);
 struct GraphBatch {

@@ -1048,8 +1048,8 @@ struct SolveBlock {
         {
           Launch L(ctx, CDL_KC_MISC, 0);
           launch_next(k_zslice, ctx->sm_count * 4, 256, 0, st, Z, n, k, np, c0, kg,
-                                                       static_cast<const unsigned long long*>(vzmax),
-                                                       static_cast<__nv_bfloat16*>(vzs), static_cast<double*>(vcz));
+                      static_cast<const unsigned long long*>(vzmax), static_cast<__nv_bfloat16*>(vzs),
+                      static_cast<double*>(vcz));
           CDL_TRY(L.done());
         }
         CDL_CUDA_TRY(cudaMemsetAsync(Gg, 0, (size_t)RESID_PAIRS * np * kg * sizeof(double), st));
@@ -1075,8 +1075,8 @@ struct SolveBlock {
         {
           Launch L(ctx, CDL_KC_MISC, 0);
           launch_next(k_zslice, ctx->sm_count * 4, 256, 0, st, Z, n, k, np, c0, kg,
-                                                       static_cast<const unsigned long long*>(vzmax),
-                                                       static_cast<__nv_bfloat16*>(vzs), static_cast<double*>(vcz));
+                      static_cast<const unsigned long long*>(vzmax), static_cast<__nv_bfloat16*>(vzs),
+                      static_cast<double*>(vcz));
           CDL_TRY(L.done());
         }
         CDL_TRY(resid_tc(ctx, ch, vzs, kg, static_cast<double*>(vG) + (size_t)g * RESID_PAIRS * np * 128));
@@ -1102,7 +1102,7 @@ struct SolveBlock {
       dim3 g(res_gx, res_gy);
       Launch L(ctx, CDL_KC_RESIDUAL, (double)n * n * k);
       launch_next(k_residual, g, 256, 0, st, ch->ahl, ch->ahl + (size_t)n * n, static_cast<const float*>(vzh),
-                                     static_cast<const float*>(vzl), Z, Y, ch->D, n, k, R, red);
+                  static_cast<const float*>(vzl), Z, Y, ch->D, n, k, R, red);
       CDL_TRY(L.done());
     }
     nparts = res_gx * res_gy;
@@ -1117,7 +1117,7 @@ struct SolveBlock {
         dim3 g((np + 31) / 32, (kp + 31) / 32);
         Launch L(ctx, CDL_KC_MISC, 0);
         launch_next(k_update_bf16, g, 256, 0, st, static_cast<float*>(vdz), nullptr, sp, np, kp,
-                                         static_cast<__nv_bfloat16*>(vdzop), 0);
+                    static_cast<__nv_bfloat16*>(vdzop), 0);
         CDL_TRY(L.done());
       }
       const __nv_bfloat16* ahi = static_cast<const __nv_bfloat16*>(ch->aop);
@@ -1125,8 +1125,8 @@ struct SolveBlock {
       CDL_TRY(apply_tc_mat(ctx, ahi + (size_t)np * np, np, vdzop, static_cast<float*>(vpart2), kp, sp));
       const int nb = (int)std::min<size_t>((nk + 255) / 256, (size_t)ctx->sm_count * 4);
       Launch L(ctx, CDL_KC_RESIDUAL, 0);
-      launch_next(k_residual_update_tc, nb, 256, 0, st, static_cast<const float*>(vpart), static_cast<const float*>(vpart2),
-                                               sp, np, static_cast<const float*>(vdz), ch->D, n, k, kp, R, red);
+      launch_next(k_residual_update_tc, nb, 256, 0, st, static_cast<const float*>(vpart),
+                  static_cast<const float*>(vpart2), sp, np, static_cast<const float*>(vdz), ch->D, n, k, kp, R, red);
       nparts = nb;
       return L.done();
     }
@@ -1179,17 +1179,17 @@ struct SolveBlock {
       Launch L(ctx, CDL_KC_MISC, 0);
       if (ch->dtype == CDL_F64)
         launch_next(k_precond_in<double>, blocks_for(cnt, 256), 256, 0, st, R, ch->rsqrt_d, n, k, np, kp,
-                                                                    static_cast<double*>(vx));
+                    static_cast<double*>(vx));
       else
         launch_next(k_precond_in<float>, blocks_for(cnt, 256), 256, 0, st, R, ch->rsqrt_d, n, k, np, kp,
-                                                                   static_cast<float*>(vx));
+                    static_cast<float*>(vx));
       CDL_TRY(L.done());
     }
     if (bf16) {
       dim3 g((np + 31) / 32, (kp + 31) / 32);
       Launch L(ctx, CDL_KC_MISC, 0);
       launch_next(k_update_bf16, g, 256, 0, st, static_cast<float*>(vx), nullptr, sp, np, kp,
-                                       static_cast<__nv_bfloat16*>(vxop), 0);
+                  static_cast<__nv_bfloat16*>(vxop), 0);
       CDL_TRY(L.done());
     }
     return CDL_OK;
@@ -1202,7 +1202,7 @@ struct SolveBlock {
       dim3 g((np + 31) / 32, (kp + 31) / 32);
       Launch L(ctx, CDL_KC_MISC, 0);
       launch_next(k_update_bf16, g, 256, 0, st, static_cast<float*>(vx), static_cast<const float*>(vpart), sp, np, kp,
-                                       static_cast<__nv_bfloat16*>(vxop), 1);
+                  static_cast<__nv_bfloat16*>(vxop), 1);
       return L.done();
     }
     if (crt && ch->dtype == CDL_F64) {
@@ -1216,11 +1216,11 @@ struct SolveBlock {
     const size_t cnt = (size_t)np * kp;
     Launch L(ctx, CDL_KC_MISC, 0);
     if (ch->dtype == CDL_F64)
-      launch_next(k_update_simt<double>, blocks_for(cnt, 256), 256, 0, st, 
-          static_cast<double*>(vx), static_cast<const double*>(vpart), splits, cnt);
+      launch_next(k_update_simt<double>, blocks_for(cnt, 256), 256, 0, st, static_cast<double*>(vx),
+                  static_cast<const double*>(vpart), splits, cnt);
     else
-      launch_next(k_update_simt<float>, blocks_for(cnt, 256), 256, 0, st, 
-          static_cast<float*>(vx), static_cast<const float*>(vpart), splits, cnt);
+      launch_next(k_update_simt<float>, blocks_for(cnt, 256), 256, 0, st, static_cast<float*>(vx),
+                  static_cast<const float*>(vpart), splits, cnt);
     return L.done();
   }
 
@@ -1243,8 +1243,8 @@ struct SolveBlock {
       unsigned long long* zmax = static_cast<unsigned long long*>(vzmax);
       {
         Launch L(ctx, CDL_KC_MISC, 0);
-        launch_next(k_center_shift, (k + 31) / 32, 256, 0, st, static_cast<const double*>(vcs), cs_parts, k, ch->vol, shift,
-                                                      zmax);
+        launch_next(k_center_shift, (k + 31) / 32, 256, 0, st, static_cast<const double*>(vcs), cs_parts, k, ch->vol,
+                    shift, zmax);
         CDL_TRY(L.done());
       }
       Launch L(ctx, CDL_KC_MISC, 0);

@@ -916,9 +916,9 @@ constexpr int CR_MAX_KBLOCKS = 62 * CR_CHUNK_KB;       // int32 sums: |sum| <= 6
 // a_i . a_j = sum_{s,t} 2^(8(s+t)) (D_s D_t^T)_ij over nine bf16 products.
 // Every digit product is exact in float32 (<= 2^14) and the slice pairs of
 // one weight w = s + t (at most three) summed over a 256-sample chunk (512
-// where no top digit is above 64 in magnitude: |x| < 64) stay within 2^24, so the MMA's float32 accumulator holds an exact integer; the
-// epilogue adds it, shifted by 8w, to int64 accumulators. The result equals
-// the int64 sum of squared differences exactly; it is written as float64
+// where no top digit is above 64 in magnitude: |x| < 64) stay within 2^24, so the
+// MMA's float32 accumulator holds an exact integer; the epilogue adds it, shifted
+// by 8w, to int64 accumulators. The result equals the int64 sum of squared differences exactly; it is written as float64
 // multiples of 2^-32 to (i, j): the upper triangle and the diagonal 128-blocks
 // (the kernel values are formed from those and mirrored).
 // Tiles are 128 rows x 64 columns of the upper block triangle; warp roles as
@@ -3343,9 +3343,10 @@ int tc_square_grouped_pairs(cdl_ctx* ctx, const TcGroup* host_first, const TcGro
 }
 
 // Residue products t[l] = (A_l B_l^T mod p_l) + 128 of `planes` planes.
-// a_planes: planes x a_rows x K bf16 (a_rows a multiple of 256, K of 64); b_planes: planes x b_rows x K, or null for B = A, of which only the
-// 256 x 256 blocks on and above the diagonal are formed. t: planes x a_rows x
-// (b_rows or a_rows) bytes, 32-byte aligned.
+// a_planes: planes x a_rows x K bf16 (a_rows a multiple of 256, K of 64); b_planes:
+// planes x b_rows x K, or null for B = A, of which only the 256 x 256 blocks on
+// and above the diagonal are formed. t: planes x a_rows x (b_rows or a_rows) bytes,
+// 32-byte aligned.
 bool crt_gemm_supported(cdl_ctx* ctx, int K) {
   return tc_supported(ctx) && pair_clusters(ctx) > 0 && K / BK <= CR_MAX_KBLOCKS;
 }
@@ -3628,7 +3629,8 @@ int fp8t_quantize_level0(cdl_ctx* ctx, cdl_chain* ch) {
   const int np = (int)ch->npad;
   const int nt = np / 128;
   Launch L(ctx, CDL_KC_CHAIN_INIT, 3.0 * np * (double)np);
-  k_quant_fp8_tiles<<<nt * nt, 256, 0, ctx->stream>>>(static_cast<const __nv_bfloat16*>(ch->level16(0)), np, static_cast<uint8_t*>(ch->level(0)), ch->tscale, ch->tatoms);
+  k_quant_fp8_tiles<<<nt * nt, 256, 0, ctx->stream>>>(static_cast<const __nv_bfloat16*>(ch->level16(0)), np,
+                                                      static_cast<uint8_t*>(ch->level(0)), ch->tscale, ch->tatoms);
   return L.done();
 }
 
@@ -3811,7 +3813,8 @@ int gram_launch(cdl_ctx* ctx, const void* u, const void* v, int n, int rows, int
   CDL_TRY(make_map(&mv, v, (int64_t)NP * rows, kp, DS_N));
   CDL_TRY(allow_smem(ctx, k_tc_gramr<MODE, NP>, GR_SMEM_BYTES));
   Launch L(ctx, kc, work);
-  launch_next(k_tc_gramr<MODE, NP>, std::min(p.num_tiles, ctx->sm_count), T8_THREADS, GR_SMEM_BYTES, ctx->stream, mu, mv, p);
+  launch_next(k_tc_gramr<MODE, NP>, std::min(p.num_tiles, ctx->sm_count), T8_THREADS, GR_SMEM_BYTES, ctx->stream, mu,
+              mv, p);
   return L.done();
 }
 }  // namespace
