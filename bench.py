@@ -922,7 +922,7 @@ SEQ_WORKLOAD = "field_n8192_seq4"
 def run_sequence(args):
     """The plain float32 GPU path on a graph sequence: 4 graphs of the 64 x 128
     correlated field (n = 8192, T = 128, AR(1) drift, an 8 x 8 patch shifted in
-    the second transition), each embedded once (float32 chain on CUDA cores,
+    the second transition), each embedded once (float32 chain through residue products,
     d = 12; projection k = 64; solve to 1e-10) and reused by its two pairs,
     then the 3 transitions scored in float32. One step = the whole sequence
     through the C ABI stage by stage; value = transitions scored per second."""
@@ -1017,12 +1017,13 @@ def run_sequence(args):
     if chain[0] is not None:
         cdl.cdl_chain_free(chain[0])
 
-    # the float32 squaring on the CUDA cores against the float32 FMA rate of the
-    # part: 152 SMs x 128 lanes x 2 flop x the maximum SM clock
-    pk, _ = peaks()
-    f32_peak = 152 * 128 * 2 * pk.get("sm_max_mhz", 2070.0) * 1e6 / 1e12
+    # the float32 squarings: eight residue products each on the bf16 tensor cores, with the conversion to residues and
+    # the combination in their time (three launches a squaring; the library counts n^2 (n + 1) of work for it)
+    pk, src = peaks()
+    peak = pk.get("bf16_tflops_sustained", pk.get("bf16_tflops"))
     sq = kc["square"]
-    achieved = sq["work"] / (sq["ms_per_launch"] * 1e-3) / 1e12 if sq["ms_per_launch"] else 0.0
+    products = 8 * G * (d - 1) * float(n) * n * (n + 1.0)
+    achieved = products / (sq["ms_per_step"] * 1e-3) / 1e12 if sq["ms_per_step"] else 0.0
     line = {
         "metric": "graph pairs/s on the n=8192 sequence (plain float32 GPU path)",
         "value": (G - 1) * 1000.0 / step_ms, "unit": "pairs/s", "n_gpus": 1, "steps": args.steps,
@@ -1034,11 +1035,13 @@ def run_sequence(args):
                    "planted_patch_on_top": planted_on_top,
                    "l2": "no flush: each step writes four 537 MB float64 graphs and their 3 GB float32 chains, "
                          "larger than the 129 MB L2"},
-        "roofline": {"kernel": "k_gemm_tn (float32 chain squaring, CUDA cores)", "bound": "alu",
-                     "achieved": achieved, "peak": f32_peak, "unit": "TFLOP/s",
-                     "frac": achieved / f32_peak if f32_peak else None, "traffic": None,
-                     "peak_source": "derived: 152 SMs x 128 float32 lanes x 2 flop x sm_max_mhz",
-                     "work_per_launch": sq["work"], "ms_per_launch": sq["ms_per_launch"]},
+        "roofline": {"kernel": "k_crt_residues + k_tc_crt + k_crt_combine (float32 chain squaring, eight residue "
+                               "products)", "bound": "tensor",
+                     "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+                     "frac": achieved / peak if peak else None, "traffic": None,
+                     "peak_source": f"{src} bf16_tflops_sustained",
+                     "work_per_squaring": products / (G * (d - 1)),
+                     "ms_per_squaring": sq["ms_per_step"] / (G * (d - 1))},
         "cpu_baseline": None,
         "e2e": {"value": (G - 1) / e2e_s, "unit": "pairs/s", "h2d_bytes_per_step": G * n * T * 8,
                 "d2h_bytes_per_step": (G - 1) * (n * 8 + TOPK * 8),
@@ -1294,7 +1297,7 @@ def main():
             peak = pk.get("bf16_tflops_sustained", pk.get("bf16_tflops"))
         elif args.chain in ("fp8", "fp8t"):   # measured bf16 peak x the nominal fp8/bf16 dense ratio (4.5 / 2.25)
             peak = 2.0 * pk.get("bf16_tflops_sustained", pk.get("bf16_tflops"))
-        kname = {"bf16": "k_tc_sq2", "fp8": "k_tc_gemm<fp8>", "fp8t": "k_tc_mx8"}.get(args.chain, "k_gemm_tn")
+        kname = {"bf16": "k_tc_sq2", "fp8": "k_tc_gemm<fp8>", "fp8t": "k_tc_mx8"}.get(args.chain, "k_crt_residues + k_tc_crt + k_crt_combine")
         roof = {"kernel": kname + " (chain squaring)",
                 "bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": (achieved / peak) if peak else None,
