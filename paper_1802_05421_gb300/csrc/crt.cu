@@ -31,6 +31,7 @@
 
 #include "crt.cuh"
 #include "internal.h"
+#include "score_ab.cuh"
 #include "tiles.cuh"
 
 namespace cdl {
@@ -405,14 +406,7 @@ __global__ void __launch_bounds__(128) k_series_residues(const double* __restric
   }
 }
 
-// ---- CAD scores (k_tc_gramr): a = sqrt(vol2) Z2 - sqrt(vol1) Z1, b = sqrt(vol2)
-// Z2 + sqrt(vol1) Z1 in float64.
-__device__ __forceinline__ void score_ab(const double* __restrict__ Z1, const double* __restrict__ Z2, double s1,
-                                         double s2, size_t o, double& a, double& b) {
-  const double w = s2 * Z2[o], v = s1 * Z1[o];
-  a = w - v;
-  b = w + v;
-}
+// ---- CAD scores (k_tc_gramr) on a and b of score_ab.
 
 // What g is chosen from (zeroed before): the largest |a| and |b| as exponent
 // fields, and over the rows' largest |a| and |b| the sums of the exponents and

@@ -24,6 +24,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "score_ab.cuh"
 #include "tiles.cuh"
 
 namespace cdl {
@@ -40,8 +41,9 @@ __device__ __forceinline__ void score_colmax(const double* __restrict__ Z1, cons
   if (idx >= (size_t)n * k) return;
   const int r = (int)(idx % k);
   const double s1 = sqrt(*vol1), s2 = sqrt(*vol2);
-  const double w = s2 * Z2[idx], v = s1 * Z1[idx];
-  const float fa = (float)(fabs(w - v) * (1.0 + 0x1p-20)), fb = (float)(fabs(w + v) * (1.0 + 0x1p-20));
+  double a, b;
+  score_ab(Z1, Z2, s1, s2, idx, a, b);
+  const float fa = (float)(fabs(a) * (1.0 + 0x1p-20)), fb = (float)(fabs(b) * (1.0 + 0x1p-20));
   atomicMax(cmax + r, __float_as_uint(fa));        // non-negative floats order as their bits
   atomicMax(cmax + k + r, __float_as_uint(fb));
 }
@@ -71,10 +73,11 @@ __device__ __forceinline__ void score_prep(const double* __restrict__ Z1, const 
   if (idx >= (size_t)n * k) return;
   const int i = (int)(idx / k), r = (int)(idx % k);
   const double s1 = sqrt(*vol1), s2 = sqrt(*vol2);
-  const double w = s2 * Z2[idx], v = s1 * Z1[idx];
+  double a, b;
+  score_ab(Z1, Z2, s1, s2, idx, a, b);
   const size_t o = (size_t)r * n + i;
-  grid_split(w - v, cmax[r], ah[o], al[o]);
-  grid_split(w + v, cmax[k + r], bh[o], bl[o]);
+  grid_split(a, cmax[r], ah[o], al[o]);
+  grid_split(b, cmax[k + r], bh[o], bl[o]);
 }
 
 __global__ void k_score_colmax(const double* __restrict__ Z1, const double* __restrict__ Z2,
@@ -98,10 +101,11 @@ __device__ __forceinline__ void score_prep64(const double* __restrict__ Z1, cons
   if (idx >= (size_t)n * k) return;
   const int i = (int)(idx / k), r = (int)(idx % k);
   const double s1 = sqrt(*vol1), s2 = sqrt(*vol2);
-  const double w = s2 * Z2[idx], v = s1 * Z1[idx];
+  double a, b;
+  score_ab(Z1, Z2, s1, s2, idx, a, b);
   const size_t o = (size_t)r * n + i;
-  aT[o] = w - v;
-  bT[o] = w + v;
+  aT[o] = a;
+  bT[o] = b;
 }
 
 __global__ void k_score_prep64(const double* __restrict__ Z1, const double* __restrict__ Z2,
@@ -300,12 +304,6 @@ __global__ void k_score_reduce(const double* __restrict__ contrib, int nb, int n
 
 // ---- tensor-core scores (score dtype bf16): slices of u = [a / g | b g] and
 // v = [b g | a / g], and d_i = a_i.b_i, for score_tc.
-__device__ __forceinline__ void tcs_ab(const double* __restrict__ Z1, const double* __restrict__ Z2, double s1,
-                                       double s2, size_t idx, double& a, double& b) {
-  const double w = s2 * Z2[idx], v = s1 * Z1[idx];
-  a = w - v;
-  b = w + v;
-}
 
 // column maxima of |a| (cm[r]) and |b| (cm[k + r]) as float64 bits: maxima of
 // a row chunk per block in shared memory, then one global atomic per column
@@ -321,7 +319,7 @@ __global__ void __launch_bounds__(256) k_tcs_colmax(const double* __restrict__ Z
   const int r0 = blockIdx.x * rows_per_block, r1 = min(n, r0 + rows_per_block);
   for (size_t idx = (size_t)r0 * k + threadIdx.x; idx < (size_t)r1 * k; idx += blockDim.x) {
     double a, b;
-    tcs_ab(Z1, Z2, s1, s2, idx, a, b);
+    score_ab(Z1, Z2, s1, s2, idx, a, b);
     const int r = (int)(idx % k);
     atomicMax(sm + r, (unsigned long long)__double_as_longlong(fabs(a)));
     atomicMax(sm + k + r, (unsigned long long)__double_as_longlong(fabs(b)));
@@ -381,7 +379,7 @@ __global__ void __launch_bounds__(256) k_tcs_slice(const double* __restrict__ Z1
     if (i < n && col < 2 * k) {
       const int r = col < k ? col : col - k;
       double a, b;
-      tcs_ab(Z1, Z2, s1, s2, (size_t)i * k + r, a, b);
+      score_ab(Z1, Z2, s1, s2, (size_t)i * k + r, a, b);
       const double at = a / g[r], bt = b * g[r];            // powers of two: exact
       const double xu = col < k ? at : bt, xv = col < k ? bt : at;
       Nu = llrint(xu * rc * 0x1p48);
@@ -416,7 +414,7 @@ __global__ void __launch_bounds__(256) k_tcs_diag(const double* __restrict__ Z1,
   if (row < n)
     for (int r = lane; r < k; r += 32) {
       double a, b;
-      tcs_ab(Z1, Z2, s1, s2, (size_t)row * k + r, a, b);
+      score_ab(Z1, Z2, s1, s2, (size_t)row * k + r, a, b);
       acc = fma(a, b, acc);
     }
 #pragma unroll
